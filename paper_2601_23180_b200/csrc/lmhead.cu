@@ -7,8 +7,9 @@
 // kernel merges the per-slice partials and computes the drafted-token probabilities.
 //
 // GEMM kernel layout (two CTAs on two SMs work as a pair on one 256 x 256 tile)
-//   M tile  = 256 rows = 4 sequence slots x 64 node slots, 128 rows per CTA of the pair
-//             (T <= 64; missing nodes are zero-filled by the TMA out-of-bounds rule)
+//   M tile  = 256 rows, 128 per CTA of the pair. The rows of the active sequences are packed, row = a * T + node,
+//             so that a chain of 9 nodes costs 9 rows: 64 chains of 9 nodes (128256 x 4096 weights) are 3 M tiles,
+//             where a slot of 64 rows per sequence made them 16 (2571 -> 600 us). Past the last row: zero fill.
 //   N tile  = 256 vocabulary entries, plus one narrower tile (a multiple of 32) for the rest of
 //             the CTA pair's vocabulary range; each CTA loads one half of a tile
 //   K block = 64 bf16 = one 128-byte swizzle row; 4 MMAs of K = 16 per block
@@ -57,7 +58,9 @@ struct __align__(16) LmPartial {
 struct LmParams {
   int T, d, V;
   int n_seq;      // active sequences
-  int n_mt;       // M tiles of 4 sequence slots = ceil(n_seq / 4)
+  int n_mt;       // M tiles of 256 packed rows (of 4 sequence slots)
+  int slots;      // rows are not packed: an M tile is 4 slots of 64 node rows, read through seq_index
+  int wait_rows;  // the packed rows are written by the kernel before this one
   int n_ranges;   // vocabulary ranges of the main part: pair c < n_mt * n_ranges works on M tile c % n_mt, range c / n_mt
   int n_tail;     // pairs beyond those: each sweeps ALL M tiles over its slice of the vocabulary's tail
   int main_units; // 32-column units [0, main_units) belong to the main part, the rest to the tail
@@ -157,18 +160,23 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
   if (warp == 4) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      // sequence slots of this CTA; a slot past the last active sequence re-reads the M tile's
-      // first sequence (its rows are computed and never looked at), which keeps the byte count
-      // of a stage the same in both CTAs
       int stage = 0;
       uint32_t phase = 0;
+      if (p.wait_rows) pdl_wait();
       for (int sweep = 0; sweep < work.n_sweeps; ++sweep) {
-      const int a_first = 4 * (work.mt0 + sweep);
-      int a0 = a_first + 2 * static_cast<int>(rank), a1 = a0 + 1;
-      if (a0 >= p.n_seq) a0 = a_first;
-      if (a1 >= p.n_seq) a1 = a_first;
-      const int s0 = p.seq_index ? __ldg(p.seq_index + a0) : a0;
-      const int s1 = p.seq_index ? __ldg(p.seq_index + a1) : a1;
+      const int row0 = (work.mt0 + sweep) * (2 * LM_BM) + static_cast<int>(rank) * LM_BM;
+      int s0 = 0, s1 = 0;
+      if (p.slots) {
+        // sequence slots of this CTA; a slot past the last active sequence re-reads the M tile's
+        // first sequence (its rows are computed and never looked at), which keeps the byte count
+        // of a stage the same in both CTAs
+        const int a_first = 4 * (work.mt0 + sweep);
+        int a0 = a_first + 2 * static_cast<int>(rank), a1 = a0 + 1;
+        if (a0 >= p.n_seq) a0 = a_first;
+        if (a1 >= p.n_seq) a1 = a_first;
+        s0 = __ldg(p.seq_index + a0);
+        s1 = __ldg(p.seq_index + a1);
+      }
       for (int t = 0; t < tiles.n_tiles; ++t) {
         int n0, nw;
         tiles.tile(t, n0, nw);
@@ -182,8 +190,12 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
           uint8_t* sb = sa + LM_A_BYTES;
           if (rank == 0) mbar_expect_tx(full_bar + stage, tx_pair);
           const uint32_t fb = cluster_map(smem_u32(full_bar + stage), 0);
-          tma_load_3d_pair(sa, &tmap_h, fb, kb * LM_BK, 0, s0);
-          tma_load_3d_pair(sa + LM_BOX_BYTES, &tmap_h, fb, kb * LM_BK, 0, s1);
+          if (p.slots) {
+            tma_load_3d_pair(sa, &tmap_h, fb, kb * LM_BK, 0, s0);
+            tma_load_3d_pair(sa + LM_BOX_BYTES, &tmap_h, fb, kb * LM_BK, 0, s1);
+          } else {
+            tma_load_2d_pair(sa, &tmap_h, fb, kb * LM_BK, row0);
+          }
           for (int j = 0; j < nbox; ++j)
             tma_load_2d_pair(sb + j * LM_BOX_BYTES, &tmap_w, fb, kb * LM_BK, w0 + 64 * j);
           if (++stage == LM_STAGES) { stage = 0; phase ^= 1u; }
@@ -336,12 +348,31 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
   }
 }
 
+// Packs the activation rows of the active sequences (an index list) without gaps: one warp per row. Beside the stream
+// of W it is small: 3 sequences of 61 rows of 5120 are 1.9 MB.
+__global__ void __launch_bounds__(256)
+lmhead_pack_rows_kernel(const uint4* __restrict__ h, const int32_t* __restrict__ seq_index, uint4* __restrict__ out, int T,
+                        int vecs /* 16-byte words per row */, long long n_rows) {
+  pdl_launch_dependents();
+  const int lane = threadIdx.x & 31;
+  const long long r = static_cast<long long>(blockIdx.x) * 8 + (threadIdx.x >> 5);
+  const bool active = r < n_rows;
+  const int a = active ? static_cast<int>(r / T) : 0;
+  const uint4* src = h + (static_cast<long long>(__ldg(seq_index + a)) * T + (active ? r % T : 0)) * vecs;
+  pdl_wait();
+  if (!active) return;
+  uint4* dst = out + r * vecs;
+#pragma unroll 4
+  for (int i = lane; i < vecs; i += 32) dst[i] = __ldg(src + i);
+}
+
 // ---------------------------------------------------------------------------------------
 // Merge of the per-range partials + drafted-token logits.
 // ---------------------------------------------------------------------------------------
 struct LmFinalizeParams {
-  int T, d, V, n_mt, n_ranges;
+  int T, d, V, n_ranges;
   int stride;       // partial rows per vocabulary range
+  int pitch;        // partial rows per active sequence (T: packed rows)
   float scale, c;
   const int32_t* seq_index;
   const LmPartial* partial;
@@ -423,8 +454,8 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
 
   // ---- merge of the per-range partials: own row (all statistics) and parent row (max, sum)
   const size_t stride = static_cast<size_t>(p.stride);
-  const LmPartial* own = p.partial + static_cast<size_t>(a) * 64 + node;
-  const LmPartial* parp = p.partial + static_cast<size_t>(a) * 64 + par;
+  const LmPartial* own = p.partial + static_cast<size_t>(a) * p.pitch + node;
+  const LmPartial* parp = p.partial + static_cast<size_t>(a) * p.pitch + par;
   LmRowAcc ro = {-INFINITY, 0.f, 0.f}, rp = {-INFINITY, 0.f, 0.f};
   float v1 = -INFINITY, v2 = -INFINITY;
   int i1 = -1, i2 = -1;
@@ -485,11 +516,11 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
 }
 
 // ---------------------------------------------------------------------------------------
-// One sequence (batch-1 decoding, the paper's own setting): operands swapped. With at most 64
-// rows the GEMM is bound by streaming W, and the pair kernel above spends half of its ring
-// on H tiles. Here W is the M-side operand (128 vocabulary entries per MMA), the sequence's
+// At most 64 rows (batch-1 decoding, the paper's own setting; a few chains): operands swapped. With so
+// few rows the GEMM is bound by streaming W, and the pair kernel above spends half of its ring
+// on H tiles. Here W is the M-side operand (128 vocabulary entries per MMA), the
 // rows are the N side (16-64 columns), one CTA per SM, and a stage is KPS k-blocks of 16 KB of W plus
-// 2-8 KB of H each, almost all of it W. TMEM lane = vocabulary entry, column = tree node.
+// 2-8 KB of H each, almost all of it W. TMEM lane = vocabulary entry, column = row.
 // A CTA's vocabulary range is a multiple of 16 entries but rarely of 128: its last tile is fetched with
 // a second, lower box (only the rows the range owns; the MMA still spans 128 lanes, the lanes past
 // the range read stale shared memory and are ignored), so the chip streams W once, not the 5-18 %
@@ -509,7 +540,8 @@ constexpr int LW_ROWS = 64;                              // partial rows per voc
 
 struct LmRowsParams {
   LmParams base;
-  int N;            // node columns: T rounded up to 16
+  int n_rows, N;    // rows, and the same rounded up to 16
+  int wait_rows;    // the rows are written by the kernel before this one
   int stages, stage_bytes;
   int tail_rows;    // height of the second W box (a multiple of 16 below 128), 0 = no second box
 };
@@ -647,7 +679,8 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     if (lane == 0) {   // ---------------------------------------------------------- TMA producer
       int stage = 0;
       uint32_t phase = 0;
-      const int seq = p.seq_index ? __ldg(p.seq_index) : 0;     // the one active sequence
+      const int seq = p.seq_index ? __ldg(p.seq_index) : 0;     // one active sequence of several; else packed rows
+      if (sp.wait_rows) pdl_wait();
       const int h_bytes = sp.N * LW_BK * 2;
       for (int t = 0; t < n_tiles; ++t) {
         const int row0 = v_begin + t * LW_BM;
@@ -662,7 +695,7 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
           mbar_expect_tx(full_bar + stage, static_cast<uint32_t>(w_bytes + kc * h_bytes));
           if (KPS == 1) tma_load_2d(sa, tw, full_bar + stage, kb * LW_BK, row0);
           else tma_load_4d(sa, tw, full_bar + stage, 0, 0, kb, row0 >> 3);
-          for (int j = 0; j < kc; ++j)                                                     // nodes past T: zero fill
+          for (int j = 0; j < kc; ++j)                                                     // rows past the last: zero fill
             tma_load_3d(sa + KPS * LW_A_BYTES + j * h_bytes, &tmap_h, full_bar + stage, (kb + j) * LW_BK, 0, seq);
           if (++stage == sp.stages) { stage = 0; phase ^= 1u; }
         }
@@ -734,7 +767,7 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int col = h * 32 + lane;
-        if (col >= p.T) continue;
+        if (col >= sp.n_rows) continue;
         LmColStats q = red[col];
         LmRowAcc a = {q.m, q.s, q.t};
         for (int w2 = 1; w2 < 4; ++w2) {
@@ -758,45 +791,52 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
   }
 }
 
-// One active sequence takes the W-on-M kernel (lmhead_rows_kernel): one CTA and one vocabulary range
-// per SM, LW_ROWS partial rows per range.
-static bool lm_rows_path(int n_seq) { return n_seq == 1; }
 static thread_local int tl_lm_reserved_sms = 0;
 void lm_reserve_sms_once(int n) { tl_lm_reserved_sms = n > 0 ? n : 0; }
 
 struct LmPlan {
-  int n_seq, n_mt;
-  int n_ranges;    // pair kernel: vocabulary ranges of the main part; single-sequence kernel: ranges (= CTAs)
-  int n_tail;      // pair kernel: pairs that sweep all M tiles over a slice of the vocabulary's tail
+  int n_seq;
+  bool few_rows;   // at most 64 rows: lmhead_rows_kernel, one CTA and one vocabulary range per SM
+  bool pack;       // the rows of an index list are gathered into the workspace first
+  bool slots;      // (no workspace to gather into) four slots of 64 node rows per M tile
+  int n_mt;        // M tiles of 256 rows
+  int n_ranges;    // vocabulary ranges of the main part (few_rows: ranges = CTAs)
+  int n_tail;      // pairs that sweep all M tiles over a slice of the vocabulary's tail
   int main_units;  // 32-column units of the main part
-  size_t partial_rows() const { return static_cast<size_t>(n_ranges + n_tail) * n_mt * 2 * LM_BM; }
+  size_t required;   // workspace the call cannot do without
+  size_t pack_bytes; // and what it needs on top of it to pack listed rows
+  size_t partial_bytes() const {
+    return static_cast<size_t>(n_ranges + n_tail) * (few_rows ? LW_ROWS : n_mt * 2 * LM_BM) * sizeof(LmPartial);
+  }
 };
 
-// `max_ws` bounds the partial array (the no-allocation entry point has a fixed one): tail pairs, which
-// cost n_mt x 256 partial rows each, are given up until it fits.
-static int lm_plan(const trispec_lmhead_args* a, LmPlan* pl, size_t max_ws = ~static_cast<size_t>(0)) {
-  if (!a || a->B <= 0 || a->T <= 0 || a->d <= 0 || a->V <= 0) return TRISPEC_ERR_INVALID_ARG;
-  if (a->T > 64 || (a->d % LM_BK) != 0 || a->V < 2) return TRISPEC_ERR_UNSUPPORTED;
-  pl->n_seq = a->seq_index ? a->B_active : a->B;
-  if (pl->n_seq <= 0 || pl->n_seq > a->B) return TRISPEC_ERR_INVALID_ARG;
+// Plans the launch for rows that are packed, or that sit in slots of 64 per sequence. `max_ws` bounds the partial
+// array: tail pairs, which cost a block of partial rows for every M tile each, are given up until it fits.
+static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, size_t max_ws, LmPlan* pl) {
+  const long long rows = static_cast<long long>(n_seq) * a->T;
+  pl->n_seq = n_seq;
+  pl->slots = slots;
+  pl->pack = false;
+  pl->pack_bytes = 0;
   pl->n_tail = 0;
   pl->main_units = (a->V + 31) / 32;
-  if (lm_rows_path(pl->n_seq)) {
+  pl->few_rows = rows <= 64 && !slots;
+  if (pl->few_rows) {
     pl->n_mt = 1;
     const int V16 = (a->V + 15) / 16;
     int sms = device_sm_count() - tl_lm_reserved_sms;
     if (sms < 1) sms = 1;
     pl->n_ranges = sms < V16 ? sms : V16;
-    return TRISPEC_OK;
+    return;
   }
-  pl->n_mt = (pl->n_seq + 3) / 4;
+  pl->n_mt = slots ? (n_seq + 3) / 4 : static_cast<int>((rows + 2 * LM_BM - 1) / (2 * LM_BM));
   const int pairs = device_sm_count() / 2;       // one CTA pair per two SMs
   int r = pairs / pl->n_mt;
   if (r < 1) r = 1;
   const int V32 = (a->V + 31) / 32;
   if (r > V32) r = V32;
   pl->n_ranges = r;
-  // Pairs that the M tiles leave over (74 = 16 x 4 + 10 for 64 sequences) take the tail of the vocabulary,
+  // Pairs that the M tiles leave over (74 = 16 x 4 + 10 for 16 M tiles) take the tail of the vocabulary,
   // every one of them for all M tiles in turn. Balance in whole tiles (a tile costs a k-loop whatever its
   // width): a main pair runs ceil(main_units / r / 8) tiles, a tail pair n_mt x ceil(slice / 8).
   int tail = pairs - pl->n_mt * r;
@@ -824,6 +864,33 @@ static int lm_plan(const trispec_lmhead_args* a, LmPlan* pl, size_t max_ws = ~st
       pl->main_units = V32 - best_slice * tail;
     }
   }
+}
+
+// Rows of all sequences of the batch lie back to back already. Rows of an index list are gathered into the
+// workspace first (a few MB at most beside the hundreds of MB of W) where the caller's workspace has room for
+// them; without (a workspace that was sized for a call without a list, or the entry point that has none) they
+// are read in slots of 64 per sequence. Every call needs the slots' workspace at least, so that how much a
+// call asks for does not depend on how it reads its rows.
+static int lm_plan(const trispec_lmhead_args* a, LmPlan* pl, size_t room, size_t max_ws = ~static_cast<size_t>(0)) {
+  if (!a || a->B <= 0 || a->T <= 0 || a->d <= 0 || a->V <= 0) return TRISPEC_ERR_INVALID_ARG;
+  if (a->T > 64 || (a->d % LM_BK) != 0 || a->V < 2) return TRISPEC_ERR_UNSUPPORTED;
+  const int n_seq = a->seq_index ? a->B_active : a->B;
+  if (n_seq <= 0 || n_seq > a->B) return TRISPEC_ERR_INVALID_ARG;
+  lm_plan_rows(a, n_seq, false, max_ws, pl);
+  pl->required = pl->partial_bytes();
+  if (n_seq == 1) return TRISPEC_OK;
+  LmPlan slots;
+  lm_plan_rows(a, n_seq, true, max_ws, &slots);
+  if (slots.partial_bytes() > pl->required) pl->required = slots.partial_bytes();
+  if (!a->seq_index) return TRISPEC_OK;
+  const size_t pack_bytes = static_cast<size_t>(n_seq) * a->T * a->d * 2;
+  if (room >= pl->required && room - pl->required >= pack_bytes) {
+    pl->pack = true;
+    pl->pack_bytes = pack_bytes;
+  } else {
+    slots.required = pl->required;
+    *pl = slots;
+  }
   return TRISPEC_OK;
 }
 
@@ -832,28 +899,27 @@ static int lm_plan(const trispec_lmhead_args* a, LmPlan* pl, size_t max_ws = ~st
 extern "C" size_t trispec_lmhead_stats_workspace(const trispec_lmhead_args* a) {
   using namespace trispec;
   LmPlan pl;
-  if (lm_plan(a, &pl) != TRISPEC_OK) return 0;
-  if (lm_rows_path(pl.n_seq)) return static_cast<size_t>(pl.n_ranges) * LW_ROWS * sizeof(LmPartial);
-  return pl.partial_rows() * sizeof(LmPartial);
+  if (lm_plan(a, &pl, ~static_cast<size_t>(0)) != TRISPEC_OK) return 0;
+  return pl.required + pl.pack_bytes;
 }
 
 namespace trispec {
-static int lmhead_stats_planned(const trispec_lmhead_args* a, const LmPlan& pl, size_t ws_needed, void* stream);
+static int lmhead_stats_planned(const trispec_lmhead_args* a, const LmPlan& pl, void* stream);
 }
 
 extern "C" int trispec_lmhead_stats(const trispec_lmhead_args* a, void* stream) {
   trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   using namespace trispec;
   LmPlan pl;
-  int rc = lm_plan(a, &pl);
-  const size_t ws_needed = trispec_lmhead_stats_workspace(a);
+  const int rc = lm_plan(a, &pl, a ? a->workspace_bytes : 0);
   tl_lm_reserved_sms = 0;            // a reservation holds for one call
   if (rc != TRISPEC_OK) return rc;
-  return lmhead_stats_planned(a, pl, ws_needed, stream);
+  return lmhead_stats_planned(a, pl, stream);
 }
 
-static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmPlan& pl, size_t ws_needed, void* stream) {
-  const int n_seq = pl.n_seq, n_mt = pl.n_mt, n_ranges = pl.n_ranges;
+static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmPlan& pl, void* stream) {
+  const int n_seq = pl.n_seq, n_ranges = pl.n_ranges;
+  const long long n_rows = static_cast<long long>(n_seq) * a->T;
   int rc = TRISPEC_OK;
   if (!a->h || !a->W || !a->parent || !a->tok || !a->workspace) return TRISPEC_ERR_INVALID_ARG;
   if (!aligned16(a->h) || !aligned16(a->W) || (reinterpret_cast<uintptr_t>(a->workspace) & 255u))
@@ -863,26 +929,13 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   if (!o.max || !o.lse || !o.top1_val || !o.top2_val || !o.p_top1 || !o.p_top2 || !o.top1_idx || !o.top2_idx ||
       !o.draft_logit || !o.p_draft)
     return TRISPEC_ERR_INVALID_ARG;
-  if (a->workspace_bytes < ws_needed) return TRISPEC_ERR_WORKSPACE;
+  if (a->workspace_bytes < pl.required) return TRISPEC_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-  CUtensorMap tm_h, tm_w;
-  {
-    const uint64_t dims[3] = {static_cast<uint64_t>(a->d), static_cast<uint64_t>(a->T), static_cast<uint64_t>(a->B)};
-    const uint64_t strides[2] = {static_cast<uint64_t>(a->d) * 2, static_cast<uint64_t>(a->d) * 2 * a->T};
-    const uint32_t box[3] = {LM_BK, 64, 1};
-    if (!cached_tmap_bf16(&tm_h, a->h, 3, dims, strides, box)) return TRISPEC_ERR_CUDA;
-  }
-  {
-    const uint64_t dims[2] = {static_cast<uint64_t>(a->d), static_cast<uint64_t>(a->V)};
-    const uint64_t strides[1] = {static_cast<uint64_t>(a->d) * 2};
-    const uint32_t box[2] = {LM_BK, 64};
-    if (!cached_tmap_bf16(&tm_w, a->W, 2, dims, strides, box)) return TRISPEC_ERR_CUDA;
-  }
   // the entropy sum costs two more instructions per logit: only computed when it is asked for
   const bool want_entropy = a->out.entropy != nullptr;
   LmFinalizeParams f;
-  f.T = a->T; f.d = a->d; f.V = a->V; f.n_mt = n_mt; f.n_ranges = n_ranges + pl.n_tail;
+  f.T = a->T; f.d = a->d; f.V = a->V; f.n_ranges = n_ranges + pl.n_tail;
   f.scale = a->logit_scale; f.c = a->logit_scale * kLog2e;
   f.seq_index = a->seq_index;
   f.partial = static_cast<LmPartial*>(a->workspace);
@@ -890,16 +943,34 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   f.W = static_cast<const uint16_t*>(a->W);
   f.parent = a->parent; f.tok = a->tok;
   f.out = a->out;
-  if (lm_rows_path(n_seq)) {
+  f.pitch = pl.slots ? 64 : a->T;
+
+  LmParams p;
+  p.T = a->T; p.d = a->d; p.V = a->V;
+  p.n_seq = n_seq; p.n_mt = pl.n_mt; p.n_ranges = n_ranges;
+  p.n_tail = pl.n_tail; p.main_units = pl.main_units;
+  p.slots = pl.slots ? 1 : 0;
+  p.wait_rows = pl.pack ? 1 : 0;
+  p.c = f.c;
+  p.seq_index = a->seq_index;
+  p.partial = static_cast<LmPartial*>(a->workspace);
+  p.dev_status = a->dev_status;
+
+  const void* rows_base = a->h;
+  if (pl.pack) {
+    uint4* packed = reinterpret_cast<uint4*>(static_cast<char*>(a->workspace) + pl.required);
+    rows_base = packed;
+    TRISPEC_CUDA_OK(launch_dependent(lmhead_pack_rows_kernel, static_cast<unsigned>((n_rows + 7) / 8), 256, 0, st, 1,
+                                     static_cast<const uint4*>(a->h), a->seq_index, packed, a->T, a->d / 8, n_rows));
+    count_launch();
+  }
+  if (pl.few_rows) {
     LmRowsParams sp;
-    sp.base.T = a->T; sp.base.d = a->d; sp.base.V = a->V;
-    sp.base.n_seq = 1; sp.base.n_mt = 1; sp.base.n_ranges = n_ranges;
-    sp.base.n_tail = 0; sp.base.main_units = pl.main_units;
-    sp.base.c = f.c;
-    sp.base.seq_index = a->seq_index;
-    sp.base.partial = static_cast<LmPartial*>(a->workspace);
-    sp.base.dev_status = a->dev_status;
-    sp.N = ((a->T + 15) / 16) * 16;
+    sp.base = p;
+    if (pl.pack) sp.base.seq_index = nullptr;
+    sp.n_rows = static_cast<int>(n_rows);
+    sp.wait_rows = p.wait_rows;
+    sp.N = ((sp.n_rows + 15) / 16) * 16;
     const int kps = (a->V % 8) == 0 ? 4 : 1;
     sp.stage_bytes = kps * (LW_A_BYTES + sp.N * LW_BK * 2);
     sp.stages = (216 * 1024) / sp.stage_bytes;
@@ -931,10 +1002,13 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
       }
     }
     {
-      const uint64_t dims[3] = {static_cast<uint64_t>(a->d), static_cast<uint64_t>(a->T), static_cast<uint64_t>(a->B)};
-      const uint64_t strides[2] = {static_cast<uint64_t>(a->d) * 2, static_cast<uint64_t>(a->d) * 2 * a->T};
+      // one active sequence of several: its nodes; otherwise all rows, back to back
+      const bool one = sp.base.seq_index != nullptr;
+      const uint64_t n = static_cast<uint64_t>(n_rows);
+      const uint64_t dims[3] = {static_cast<uint64_t>(a->d), n, one ? static_cast<uint64_t>(a->B) : 1};
+      const uint64_t strides[2] = {static_cast<uint64_t>(a->d) * 2, static_cast<uint64_t>(a->d) * 2 * n};
       const uint32_t box[3] = {LW_BK, static_cast<uint32_t>(sp.N), 1};
-      if (!cached_tmap_bf16(&tm_hn, a->h, 3, dims, strides, box)) return TRISPEC_ERR_CUDA;
+      if (!cached_tmap_bf16(&tm_hn, rows_base, 3, dims, strides, box)) return TRISPEC_ERR_CUDA;
     }
     typedef void (*RowsKernel)(CUtensorMap, CUtensorMap, CUtensorMap, LmRowsParams);
     static const RowsKernel table[2][2] = {{lmhead_rows_kernel<false, 1>, lmhead_rows_kernel<false, 4>},
@@ -948,35 +1022,39 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
                                      static_cast<size_t>(smem_bytes), st, 1, tm_w128, tm_wt, tm_hn, sp));
     count_launch();
     f.stride = LW_ROWS;
-    TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel, static_cast<unsigned>((a->T + 7) / 8),
-                                     LM_FIN_THREADS, 0, st, 1, f, 1));
+    TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel, static_cast<unsigned>((n_rows + 7) / 8),
+                                     LM_FIN_THREADS, 0, st, 1, f, n_seq));
     count_launch();
     return TRISPEC_OK;
   }
-  static bool smem_set[2][64] = {};
-  rc = want_entropy
-           ? ensure_smem_limit(reinterpret_cast<const void*>(lmhead_gemm_kernel<true>), LM_SMEM_BYTES, smem_set[1])
-           : ensure_smem_limit(reinterpret_cast<const void*>(lmhead_gemm_kernel<false>), LM_SMEM_BYTES, smem_set[0]);
-  if (rc != TRISPEC_OK) return rc;
-  LmParams p;
-  p.T = a->T; p.d = a->d; p.V = a->V;
-  p.n_seq = n_seq; p.n_mt = n_mt; p.n_ranges = n_ranges;
-  p.n_tail = pl.n_tail; p.main_units = pl.main_units;
-  p.c = a->logit_scale * kLog2e;
-  p.seq_index = a->seq_index;
-  p.partial = static_cast<LmPartial*>(a->workspace);
-  p.dev_status = a->dev_status;
-  if (want_entropy) {
-    TRISPEC_CUDA_OK(launch_dependent(lmhead_gemm_kernel<true>, static_cast<unsigned>(2 * (n_mt * n_ranges + pl.n_tail)), LM_THREADS,
-                                     LM_SMEM_BYTES, st, 2, tm_h, tm_w, p));
+  CUtensorMap tm_h, tm_w;
+  if (pl.slots) {
+    const uint64_t dims[3] = {static_cast<uint64_t>(a->d), static_cast<uint64_t>(a->T), static_cast<uint64_t>(a->B)};
+    const uint64_t strides[2] = {static_cast<uint64_t>(a->d) * 2, static_cast<uint64_t>(a->d) * 2 * a->T};
+    const uint32_t box[3] = {LM_BK, 64, 1};
+    if (!cached_tmap_bf16(&tm_h, a->h, 3, dims, strides, box)) return TRISPEC_ERR_CUDA;
   } else {
-    TRISPEC_CUDA_OK(launch_dependent(lmhead_gemm_kernel<false>, static_cast<unsigned>(2 * (n_mt * n_ranges + pl.n_tail)), LM_THREADS,
-                                     LM_SMEM_BYTES, st, 2, tm_h, tm_w, p));
+    const uint64_t dims[2] = {static_cast<uint64_t>(a->d), static_cast<uint64_t>(n_rows)};
+    const uint64_t strides[1] = {static_cast<uint64_t>(a->d) * 2};
+    const uint32_t box[2] = {LM_BK, LM_BM};
+    if (!cached_tmap_bf16(&tm_h, rows_base, 2, dims, strides, box)) return TRISPEC_ERR_CUDA;
   }
+  {
+    const uint64_t dims[2] = {static_cast<uint64_t>(a->d), static_cast<uint64_t>(a->V)};
+    const uint64_t strides[1] = {static_cast<uint64_t>(a->d) * 2};
+    const uint32_t box[2] = {LM_BK, 64};
+    if (!cached_tmap_bf16(&tm_w, a->W, 2, dims, strides, box)) return TRISPEC_ERR_CUDA;
+  }
+  static bool smem_set[2][64] = {};
+  typedef void (*GemmKernel)(CUtensorMap, CUtensorMap, LmParams);
+  const GemmKernel kernel = want_entropy ? lmhead_gemm_kernel<true> : lmhead_gemm_kernel<false>;
+  rc = ensure_smem_limit(reinterpret_cast<const void*>(kernel), LM_SMEM_BYTES, smem_set[want_entropy ? 1 : 0]);
+  if (rc != TRISPEC_OK) return rc;
+  TRISPEC_CUDA_OK(launch_dependent(kernel, static_cast<unsigned>(2 * (p.n_mt * n_ranges + pl.n_tail)), LM_THREADS,
+                                   LM_SMEM_BYTES, st, 2, tm_h, tm_w, p));
   count_launch();
-
-  f.stride = n_mt * 2 * LM_BM;
-  TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel, static_cast<unsigned>((n_seq * a->T + 7) / 8),
+  f.stride = p.n_mt * 2 * LM_BM;
+  TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel, static_cast<unsigned>((n_rows + 7) / 8),
                                    LM_FIN_THREADS, 0, st, 1, f, n_seq));
   count_launch();
   return TRISPEC_OK;
@@ -1016,16 +1094,14 @@ extern "C" int trispec_lmhead_stats_noalloc(const trispec_lmhead_args* a, void* 
   using namespace trispec;
   // planned so that the partial array fits the built-in scratch (fewer tail pairs where they would not)
   LmPlan pl;
-  int rc = lm_plan(a, &pl, TRISPEC_NOALLOC_SCRATCH_BYTES);
+  int rc = lm_plan(a, &pl, 0, TRISPEC_NOALLOC_SCRATCH_BYTES);
   if (rc != TRISPEC_OK) return rc;
-  const size_t need = lm_rows_path(pl.n_seq) ? static_cast<size_t>(pl.n_ranges) * LW_ROWS * sizeof(LmPartial)
-                                             : pl.partial_rows() * sizeof(LmPartial);
-  if (need > TRISPEC_NOALLOC_SCRATCH_BYTES) return TRISPEC_ERR_TOO_LARGE;
+  if (pl.required > TRISPEC_NOALLOC_SCRATCH_BYTES) return TRISPEC_ERR_TOO_LARGE;
   void* scratch = nullptr;
   rc = lm_noalloc_scratch(&scratch);
   if (rc != TRISPEC_OK) return rc;
   trispec_lmhead_args b = *a;     // same call, with the built-in array as its workspace
   b.workspace = scratch;
   b.workspace_bytes = TRISPEC_NOALLOC_SCRATCH_BYTES;
-  return lmhead_stats_planned(&b, pl, need, stream);
+  return lmhead_stats_planned(&b, pl, stream);
 }

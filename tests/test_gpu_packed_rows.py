@@ -1,0 +1,68 @@
+"""LM head over packed rows: the rows of all active sequences lie back to back in the M tiles of the GEMM, whatever
+the tree size; rows of an index list are gathered into the workspace, or read in slots of 64 per sequence
+where the workspace has no room for them. Sizes around the 64 rows of the small kernel and the 256 rows of an M tile."""
+import math
+
+import numpy as np
+import pytest
+
+from oracle import trispec_oracle as orc
+from paper_2601_23180_b200 import inputs as gen
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(B, T, listed, d=192, V=3001):
+    cfg = gen.small_variant(gen.CONFIGS["tiny_chain"], B=B, k=T - 1, max_depth=T - 1, d=d, V=V, rho=0.2,
+                            logit_scale=3.6 / (0.02 * math.sqrt(d)), seed=B * 100 + T)
+    inp = gen.make_inputs(cfg, with_attention=False)
+    if listed:
+        inp["seq_index"] = np.random.default_rng(B).permutation(B)[:listed].astype(np.int32)
+    return cfg, inp
+
+
+@pytest.mark.parametrize("B,T,listed", [
+    (7, 9, 0),       # 63 rows: one N tile of the small kernel
+    (8, 8, 0),       # 64
+    (13, 5, 0),      # 65: the pair kernel, one M tile
+    (17, 15, 0),     # 255
+    (32, 8, 0),      # 256
+    (86, 3, 0),      # 258: a second M tile with two rows
+    (40, 13, 0),     # 520: 3 M tiles, two pairs left over for the tail
+    (9, 9, 3),       # 27 of 81 rows, gathered for the small kernel
+    (9, 9, 8),       # 72, gathered for the pair kernel
+    (12, 61, 9),     # 549
+])
+@pytest.mark.parametrize("room", ["full", "slots"])
+def test_lmhead_packed_rows_against_oracle(B, T, listed, room):
+    import torch
+    from paper_2601_23180_b200 import binding as ts
+    import tests.gpu_helpers as H
+    cfg, inp = _inputs(B, T, listed)
+    dev = H.to_device(inp)
+    seqs = list(range(B)) if not listed else [int(s) for s in inp["seq_index"]]
+    st = ts.alloc_stats(B, T, entropy=True)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    a = ts.lmhead_args(dev["h"], dev["W"], dev["parent"], dev["tok"], cfg.logit_scale, st, seq_index=dev["seq_index"],
+                       dev_status=status)
+    need = ts.trispec_lmhead_stats_workspace(a)
+    if room == "slots":
+        if not listed:
+            pytest.skip("rows without a list are packed as they are")
+        need -= listed * T * cfg.d * 2     # what the gathered rows take
+    ws = ts.alloc_workspace(need)
+    a.workspace, a.workspace_bytes = ws.data_ptr(), need
+    ts.trispec_lmhead_stats(a)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    got = {k: v.cpu().numpy() for k, v in st.items()}
+    ref = orc.lmhead_stats(inp["h"], inp["W"], inp["parent"], inp["tok"], cfg.logit_scale, seqs=seqs)
+    n_tie = H.check_stats(got, ref, seqs, T)
+    assert n_tie <= 0.02 * len(seqs) * T + 2
+    for b in set(range(B)) - set(seqs):
+        assert np.isnan(got["lse"][b]).all() and (got["top1_idx"][b] == -1).all()
+    a.workspace_bytes = need - listed * T * cfg.d * 2 - 1 if room == "full" else need - 1
+    n0 = ts.launch_count()
+    with pytest.raises(ts.TrispecError) as e:
+        ts.trispec_lmhead_stats(a)
+    assert e.value.code == 3 and ts.launch_count() == n0
