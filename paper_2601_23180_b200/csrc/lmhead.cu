@@ -118,6 +118,38 @@ struct PairWork {
   }
 };
 
+// Next logit of a scan in ascending vocabulary order (an equal one never displaces): selects, no branches, because the
+// lanes of a warp rarely agree.
+__device__ __forceinline__ void lm_scan2(float v, int i, float& v1, int& i1, float& v2, int& i2) {
+  const bool first = v > v1, second = v > v2;
+  v2 = first ? v1 : (second ? v : v2);
+  i2 = first ? i1 : (second ? i : i2);
+  v1 = first ? v : v1;
+  i1 = first ? i : i1;
+}
+
+// Order-preserving key of (logit, vocabulary entry): larger logit first, lower entry on ties; 0 = no entry. Merging two
+// top-two lists is then three 64-bit minima and maxima.
+__device__ __forceinline__ unsigned long long lm_key(float z, int v) {
+  const uint32_t b = __float_as_uint(z + 0.f);           // -0 ties with +0
+  const uint32_t u = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+  return v < 0 ? 0ull : (static_cast<unsigned long long>(u) << 32) | (0xffffffffu - static_cast<uint32_t>(v));
+}
+__device__ __forceinline__ float lm_key_value(unsigned long long k) {
+  const uint32_t u = static_cast<uint32_t>(k >> 32);
+  return k == 0ull ? -INFINITY : __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
+}
+__device__ __forceinline__ int lm_key_entry(unsigned long long k) {
+  return k == 0ull ? -1 : static_cast<int>(0xffffffffu - static_cast<uint32_t>(k));
+}
+struct LmTop2 { unsigned long long a, b; };              // a >= b
+__device__ __forceinline__ void lm_merge(LmTop2& t, unsigned long long a, unsigned long long b) {
+  const unsigned long long lo = a < t.a ? a : t.a;
+  t.a = a < t.a ? t.a : a;
+  t.b = b < t.b ? t.b : b;
+  t.b = lo < t.b ? t.b : lo;
+}
+
 template <bool kEntropy>
 __global__ void __launch_bounds__(LM_THREADS, 1)
 lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ CUtensorMap tmap_w,
@@ -319,11 +351,7 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
         if (cmax > v2) {
           const int col0 = n0 + c0;
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float v = __uint_as_float(r[j]);
-            if (v > v1) { v2 = v1; i2 = i1; v1 = v; i1 = col0 + j; }
-            else if (v > v2) { v2 = v; i2 = col0 + j; }
-          }
+          for (int j = 0; j < 32; ++j) lm_scan2(__uint_as_float(r[j]), col0 + j, v1, i1, v2, i2);
         }
       }
       tc_fence_before();
@@ -386,26 +414,8 @@ constexpr int LM_FIN_THREADS = 256;   // 8 warps = 8 rows per block
 __device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
 
-// larger value first, lower index on ties; index -1 marks "no entry"
-__device__ __forceinline__ bool lm_better(float va, int ia, float vb, int ib) {
-  return ia >= 0 && (ib < 0 || va > vb || (va == vb && ia < ib));
-}
-__device__ __forceinline__ void lm_top2_insert(float v, int i, float& v1, int& i1, float& v2, int& i2) {
-  if (i < 0) return;
-  if (lm_better(v, i, v1, i1)) { v2 = v1; i2 = i1; v1 = v; i1 = i; }
-  else if (lm_better(v, i, v2, i2)) { v2 = v; i2 = i; }
-}
-
-// running (max, sum of exponentials, sum of exponentials x logit) of a set of vocabulary ranges
-struct LmRowAcc { float m, s, t; };
-__device__ __forceinline__ void lm_fold(LmRowAcc& a, float m, float s, float t, float c) {
-  const float M = fmaxf(a.m, m);
-  const float fa = (a.m == -INFINITY) ? 0.f : ex2f((a.m - M) * c);
-  const float fb = (m == -INFINITY) ? 0.f : ex2f((m - M) * c);
-  a.s = a.s * fa + s * fb;
-  a.t = a.t * fa + t * fb;
-  a.m = M;
-}
+// what a sum relative to maximum m is worth relative to M >= m
+__device__ __forceinline__ float lm_weight(float m, float M, float c) { return (m == -INFINITY) ? 0.f : ex2f((m - M) * c); }
 
 // One warp per (active sequence, node): merges the row's partial statistics and, for a child
 // node, computes the logit of its drafted token in its parent's row (a d-long dot product).
@@ -456,14 +466,16 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
   const size_t stride = static_cast<size_t>(p.stride);
   const LmPartial* own = p.partial + static_cast<size_t>(a) * p.pitch + node;
   const LmPartial* parp = p.partial + static_cast<size_t>(a) * p.pitch + par;
-  LmRowAcc ro = {-INFINITY, 0.f, 0.f}, rp = {-INFINITY, 0.f, 0.f};
-  float v1 = -INFINITY, v2 = -INFINITY;
-  int i1 = -1, i2 = -1;
-  for (int r0 = 0; r0 < p.n_ranges; r0 += 96) {  // three ranges per lane and round, loads first
-    float4 qa[3], qb[3];
-    float2 qp[3];
+  // Up to 148 ranges are five per lane: loaded at once, folded relative to the row's maximum, so that the chains
+  // across the lanes are one maximum, the sums, and the top two as 64-bit keys, side by side.
+  float m_own = -INFINITY, s_own = 0.f, t_own = 0.f, m_par = -INFINITY, s_par = 0.f;
+  LmTop2 top = {0ull, 0ull};
+  constexpr int kPer = 5;
+  for (int r0 = 0; r0 < p.n_ranges; r0 += 32 * kPer) {
+    float4 qa[kPer], qb[kPer];
+    float2 qp[kPer];
 #pragma unroll
-    for (int u = 0; u < 3; ++u) {
+    for (int u = 0; u < kPer; ++u) {
       const int r = r0 + lane + 32 * u;
       qa[u] = make_float4(-INFINITY, 0.f, -INFINITY, -INFINITY);
       qb[u] = make_float4(__int_as_float(-1), __int_as_float(-1), 0.f, 0.f);
@@ -475,27 +487,40 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
         qp[u] = *reinterpret_cast<const float2*>(parp + r * stride);   // m, s of the parent's row
       }
     }
+    float mo = m_own, mp = m_par;
 #pragma unroll
-    for (int u = 0; u < 3; ++u) {
-      lm_fold(ro, qa[u].x, qa[u].y, qb[u].z, p.c);
-      lm_fold(rp, qp[u].x, qp[u].y, 0.f, p.c);
-      lm_top2_insert(qa[u].z, __float_as_int(qb[u].x), v1, i1, v2, i2);
-      lm_top2_insert(qa[u].w, __float_as_int(qb[u].y), v1, i1, v2, i2);
+    for (int u = 0; u < kPer; ++u) { mo = fmaxf(mo, qa[u].x); mp = fmaxf(mp, qp[u].x); }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mo = fmaxf(mo, __shfl_xor_sync(0xffffffffu, mo, o));
+      mp = fmaxf(mp, __shfl_xor_sync(0xffffffffu, mp, o));
+    }
+    const float fo = lm_weight(m_own, mo, p.c), fp = lm_weight(m_par, mp, p.c);
+    s_own *= fo; t_own *= fo; s_par *= fp;
+    m_own = mo; m_par = mp;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const float w = lm_weight(qa[u].x, mo, p.c);
+      s_own = fmaf(qa[u].y, w, s_own);
+      t_own = fmaf(qb[u].z, w, t_own);
+      s_par = fmaf(qp[u].y, lm_weight(qp[u].x, mp, p.c), s_par);
+      lm_merge(top, lm_key(qa[u].z, __float_as_int(qb[u].x)), lm_key(qa[u].w, __float_as_int(qb[u].y)));
     }
   }
+#pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    lm_fold(ro, __shfl_xor_sync(0xffffffffu, ro.m, o), __shfl_xor_sync(0xffffffffu, ro.s, o),
-            __shfl_xor_sync(0xffffffffu, ro.t, o), p.c);
-    lm_fold(rp, __shfl_xor_sync(0xffffffffu, rp.m, o), __shfl_xor_sync(0xffffffffu, rp.s, o), 0.f, p.c);
-    const float ov1 = __shfl_xor_sync(0xffffffffu, v1, o), ov2 = __shfl_xor_sync(0xffffffffu, v2, o);
-    const int oi1 = __shfl_xor_sync(0xffffffffu, i1, o), oi2 = __shfl_xor_sync(0xffffffffu, i2, o);
-    lm_top2_insert(ov1, oi1, v1, i1, v2, i2);
-    lm_top2_insert(ov2, oi2, v1, i1, v2, i2);
+    s_own += __shfl_xor_sync(0xffffffffu, s_own, o);
+    t_own += __shfl_xor_sync(0xffffffffu, t_own, o);
+    s_par += __shfl_xor_sync(0xffffffffu, s_par, o);
+    const unsigned long long a = __shfl_xor_sync(0xffffffffu, top.a, o), b = __shfl_xor_sync(0xffffffffu, top.b, o);
+    lm_merge(top, a, b);
   }
+  const float v1 = lm_key_value(top.a), v2 = lm_key_value(top.b);
+  const int i1 = lm_key_entry(top.a), i2 = lm_key_entry(top.b);
   if (lane == 0) {
-    const float lse = ro.m * p.scale + logf(ro.s);
+    const float lse = m_own * p.scale + logf(s_own);
     const long long o = row0 + node;
-    p.out.max[o] = ro.m * p.scale;
+    p.out.max[o] = m_own * p.scale;
     p.out.lse[o] = lse;
     p.out.top1_val[o] = v1 * p.scale;
     p.out.top2_val[o] = v2 * p.scale;
@@ -504,11 +529,11 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
     p.out.p_top1[o] = expf(v1 * p.scale - lse);
     p.out.p_top2[o] = expf(v2 * p.scale - lse);
     // entropy in nats: H = lse - E_p[z], E_p[z] = scale * sum(e * z_raw) / sum(e); never below 0
-    if (p.out.entropy) p.out.entropy[o] = fmaxf(lse - p.scale * (ro.t / ro.s), 0.f);
+    if (p.out.entropy) p.out.entropy[o] = fmaxf(lse - p.scale * (t_own / s_own), 0.f);
     float dl = __int_as_float(0x7fc00000), pd = dl;
     if (has_draft) {
       dl = dot * p.scale;
-      pd = expf(dl - (rp.m * p.scale + logf(rp.s)));
+      pd = expf(dl - (m_par * p.scale + logf(s_par)));
     }
     p.out.draft_logit[o] = dl;
     p.out.p_draft[o] = pd;
@@ -518,190 +543,141 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
 // ---------------------------------------------------------------------------------------
 // At most 64 rows (batch-1 decoding, the paper's own setting; a few chains): operands swapped. With so
 // few rows the GEMM is bound by streaming W, and the pair kernel above spends half of its ring
-// on H tiles. Here W is the M-side operand (128 vocabulary entries per MMA), the
-// rows are the N side (16-64 columns), one CTA per SM, and a stage is KPS k-blocks of 16 KB of W plus
-// 2-8 KB of H each, almost all of it W. TMEM lane = vocabulary entry, column = row.
-// A CTA's vocabulary range is a multiple of 16 entries but rarely of 128: its last tile is fetched with
-// a second, lower box (only the rows the range owns; the MMA still spans 128 lanes, the lanes past
-// the range read stale shared memory and are ignored), so the chip streams W once, not the 5-18 %
-// more that whole tiles would cost on a launch that is bound by exactly this stream.
-// With KPS = 4 (any vocabulary that is a multiple of 8) W is read through a 4-D view
-// [V/8][d/64][8 rows][64 elements], whose box puts the k-blocks of one group of 8 rows next to each
-// other in the request stream; the stage then holds [16 row groups][KPS k-blocks][8 rows][128 B], and
-// the MMA descriptor of k-block j starts j KB in with KPS KB between row groups. KPS = 1 is the
-// plain 2-D view, the same layout with one k-block.
-// Epilogue: per tile a warp reduces 32 columns at once over its 32 vocabulary entries with
-// transposing shuffle butterflies (top-2 with indices, then the sums of exponentials), after which
-// lane l holds column l's result and folds it into the running statistics it keeps for that column.
+// on H tiles. Here W is the M-side operand, the rows are the N side (16-64 columns), and one CTA per SM takes one
+// vocabulary range. A tile is up to 2 x 128 vocabulary entries, two MMAs that share the k-block of H: a stage is
+// 32 KB of W and 2-8 KB of H, so that up to 160 KB of W are in flight per SM and H, which every SM reads, adds 25 %
+// to what L2 delivers (with 128 entries per tile it was 50 %).
+// A range is cut into tiles of equal height, so that none ends in a tile that is nearly empty and W is streamed once.
+// TMEM lane = vocabulary entry, column = row. Epilogue: warps 0-3 take the first 128 entries of a tile, warps
+// 4-7 the others. A warp passes 32 entries x 16 columns through 2 KB of shared memory, after which a lane holds 16
+// entries of one column and folds them into the running statistics it keeps for that column (the MMAs leave
+// shared memory idle most of the time here; the butterflies over (value, index) tuples that did this before
+// took 5 us for the last tile, which nothing overlaps).
 // ---------------------------------------------------------------------------------------
-constexpr int LW_BM = 128, LW_BK = 64, LW_MAX_STAGES = 12, LW_THREADS = 192;
-constexpr int LW_A_BYTES = LW_BM * LW_BK * 2;           // 16 KB of W per stage
+constexpr int LW_BM = 128, LW_SUBS = 2, LW_BK = 64, LW_MAX_STAGES = 6, LW_EPI_WARPS = 8;
+constexpr int LW_THREADS = 32 * (LW_EPI_WARPS + 2);
+constexpr int LW_A_BYTES = LW_SUBS * LW_BM * LW_BK * 2;  // 32 KB of W per stage
 constexpr int LW_ROWS = 64;                              // partial rows per vocabulary range
+constexpr int LW_XPOSE_BYTES = 2048;                     // 32 entries x 16 columns per epilogue warp
+constexpr int LW_SMEM_BYTES = 227 * 1024;
+constexpr int LW_RING_BYTES = LW_SMEM_BYTES - 1024 /*alignment slack*/ - LW_EPI_WARPS * LW_XPOSE_BYTES - 256 /*barriers*/;
 
 struct LmRowsParams {
   LmParams base;
   int n_rows, N;    // rows, and the same rounded up to 16
   int wait_rows;    // the rows are written by the kernel before this one
+  int n_tiles;      // tiles per vocabulary range
+  int box_rows;     // W rows per copy: the height of half a tile
   int stages, stage_bytes;
-  int tail_rows;    // height of the second W box (a multiple of 16 below 128), 0 = no second box
 };
 
-struct LmColStats { float m, s, t, v1, v2; int i1, i2; };
+struct LmColStats { float m, s, t, v1, v2; int i1, i2; };   // of one column, over the entries a lane has seen
+struct LmColMerge { LmTop2 top; float m, s, t, pad; };     // the same on its way to the other warps
 
-// One 32-column chunk of a tile in the epilogue of lmhead_rows_kernel: r[j] = logit of column col0 + j at this
-// lane's vocabulary entry my_v. Per column: top-2 (value, vocabulary index) and the sum of exponentials over
-// the warp's 32 vocabulary entries, folded into the running statistics `run` of column col0 + lane. A
-// transposing butterfly does all columns at once: in the step with distance o a lane keeps half of the
-// columns it still holds, hands the other half to its partner and merges what it receives, so that after
-// the steps lane l holds column l. NC = 32 columns take five steps; when the tree has at most 16 nodes
-// (NC = 16: chains), four steps leave lanes l and l + 16 with column l over one half of the entries each,
-// and one more exchange merges the halves (lanes 16-31 then hold copies, which nothing reads).
-template <bool kEntropy, int NC>
-__device__ __forceinline__ void lm_rows_chunk_nc(const uint32_t (&r)[32], bool valid, int my_v, int col0, int N, int lane,
-                                                 float c, LmColStats& run) {
-  float v1[NC], v2[NC];
-  int i1[NC], i2[NC];
-#pragma unroll
-  for (int j = 0; j < NC; ++j) {
-    const bool on = valid && (col0 + j < N);
-    v1[j] = on ? __uint_as_float(r[j]) : -INFINITY;
-    i1[j] = on ? my_v : -1;
-    v2[j] = -INFINITY;
-    i2[j] = -1;
-  }
-#pragma unroll
-  for (int o = NC / 2; o > 0; o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < o; ++i) {
-      const float sv1 = up ? v1[i] : v1[i + o], sv2 = up ? v2[i] : v2[i + o];
-      const int si1 = up ? i1[i] : i1[i + o], si2 = up ? i2[i] : i2[i + o];
-      float kv1 = up ? v1[i + o] : v1[i], kv2 = up ? v2[i + o] : v2[i];
-      int ki1 = up ? i1[i + o] : i1[i], ki2 = up ? i2[i + o] : i2[i];
-      const float rv1 = __shfl_xor_sync(0xffffffffu, sv1, o), rv2 = __shfl_xor_sync(0xffffffffu, sv2, o);
-      const int ri1 = __shfl_xor_sync(0xffffffffu, si1, o), ri2 = __shfl_xor_sync(0xffffffffu, si2, o);
-      lm_top2_insert(rv1, ri1, kv1, ki1, kv2, ki2);
-      lm_top2_insert(rv2, ri2, kv1, ki1, kv2, ki2);
-      v1[i] = kv1; v2[i] = kv2; i1[i] = ki1; i2[i] = ki2;
-    }
-  }
-  if (NC == 16) {   // lanes l and l ^ 16 hold the same column over different vocabulary entries
-    const float rv1 = __shfl_xor_sync(0xffffffffu, v1[0], 16), rv2 = __shfl_xor_sync(0xffffffffu, v2[0], 16);
-    const int ri1 = __shfl_xor_sync(0xffffffffu, i1[0], 16), ri2 = __shfl_xor_sync(0xffffffffu, i2[0], 16);
-    lm_top2_insert(rv1, ri1, v1[0], i1[0], v2[0], i2[0]);
-    lm_top2_insert(rv2, ri2, v1[0], i1[0], v2[0], i2[0]);
-  }
-  const float m_t = v1[0];                  // this lane's column: col0 + (lane mod NC)
-  // every lane needs every column's maximum for its exponentials
-  float es[NC], et[NC];
-#pragma unroll
-  for (int j = 0; j < NC; ++j) {
-    const float mj = __shfl_sync(0xffffffffu, m_t, j);
-    const bool on = valid && (col0 + j < N);
-    const float z = __uint_as_float(r[j]);
-    es[j] = on ? ex2f((z - mj) * c) : 0.f;
-    et[j] = (kEntropy && on) ? es[j] * z : 0.f;
-  }
-#pragma unroll
-  for (int o = NC / 2; o > 0; o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < o; ++i) {
-      const float ss = up ? es[i] : es[i + o], ks = up ? es[i + o] : es[i];
-      es[i] = ks + __shfl_xor_sync(0xffffffffu, ss, o);
-      if (kEntropy) {
-        const float st2 = up ? et[i] : et[i + o], kt = up ? et[i + o] : et[i];
-        et[i] = kt + __shfl_xor_sync(0xffffffffu, st2, o);
-      }
-    }
-  }
-  if (NC == 16) {
-    es[0] += __shfl_xor_sync(0xffffffffu, es[0], 16);
-    if (kEntropy) et[0] += __shfl_xor_sync(0xffffffffu, et[0], 16);
-  }
-  // fold the tile's statistics of this lane's column into the running ones
-  LmRowAcc a = {run.m, run.s, run.t};
-  lm_fold(a, m_t, es[0], et[0], c);
-  run.m = a.m; run.s = a.s; run.t = a.t;
-  lm_top2_insert(v1[0], i1[0], run.v1, run.i1, run.v2, run.i2);
-  lm_top2_insert(v2[0], i2[0], run.v1, run.i1, run.v2, run.i2);
-}
+// 16 logits of one column, vocabulary entries v0 + j, of which those below v_end exist.
 template <bool kEntropy>
-__device__ __forceinline__ void lm_rows_chunk(const uint32_t (&r)[32], bool valid, int my_v, int col0, int N, int lane,
-                                              float c, LmColStats& run) {
-  if (N <= 16) lm_rows_chunk_nc<kEntropy, 16>(r, valid, my_v, col0, N, lane, c, run);
-  else lm_rows_chunk_nc<kEntropy, 32>(r, valid, my_v, col0, N, lane, c, run);
+__device__ __forceinline__ void lm_fold16(float (&z)[16], int v0, int v_end, float c, LmColStats& st) {
+  if (v0 + 16 > v_end) {                          // ragged end: entries that do not exist count as -inf
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (v0 + j >= v_end) z[j] = -INFINITY;
+  }
+  float cm[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+  for (int j = 0; j < 16; j += 4) {
+    cm[0] = fmax3(cm[0], z[j], z[j + 1]);
+    cm[1] = fmax3(cm[1], z[j + 2], z[j + 3]);
+  }
+  const float cmax = fmaxf(cm[0], cm[1]);
+  if (cmax > st.m) {
+    const float f = ex2f((st.m - cmax) * c);
+    st.s *= f;
+    if (kEntropy) st.t *= f;
+    st.m = cmax;
+  }
+  const float nmc = (st.m == -INFINITY) ? 0.f : -st.m * c;
+  const float2 c2 = make_float2(c, c), nmc2 = make_float2(nmc, nmc);
+  float2 acc = make_float2(0.f, 0.f), acz = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int j = 0; j < 16; j += 2) {
+    const float2 x = ffma2(make_float2(z[j], z[j + 1]), c2, nmc2);
+    const float2 e = make_float2(ex2f(x.x), ex2f(x.y));
+    acc = fadd2(acc, e);
+    if (kEntropy)                                 // keep 0 * inf out of the sum
+      acz = ffma2(e, make_float2(z[j] == -INFINITY ? 0.f : z[j], z[j + 1] == -INFINITY ? 0.f : z[j + 1]), acz);
+  }
+  st.s += acc.x + acc.y;
+  if (kEntropy) st.t += acz.x + acz.y;
+  if (cmax > st.v2) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) lm_scan2(z[j], v0 + j, st.v1, st.i1, st.v2, st.i2);
+  }
 }
 
-
-template <bool kEntropy, int KPS>
+template <bool kEntropy>
 __global__ void __launch_bounds__(LW_THREADS, 1)
-lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_wt,
-                   const __grid_constant__ CUtensorMap tmap_h, const LmRowsParams sp) {
+lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_h,
+                   const LmRowsParams sp) {
   pdl_launch_dependents();
   const LmParams& p = sp.base;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base_u32 = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (base_u32 - smem_u32(smem_raw));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + sp.stages * sp.stage_bytes);
+  uint8_t* xpose = smem + sp.stages * sp.stage_bytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(xpose + LW_EPI_WARPS * LW_XPOSE_BYTES);
   uint64_t* full_bar = bars;
   uint64_t* empty_bar = bars + LW_MAX_STAGES;
   uint64_t* tmem_full = bars + 2 * LW_MAX_STAGES;
   uint64_t* tmem_empty = bars + 2 * LW_MAX_STAGES + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * LW_MAX_STAGES + 4);
-  LmColStats* red = reinterpret_cast<LmColStats*>(bars + 2 * LW_MAX_STAGES + 6);   // [4 warps][64 columns]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int range = blockIdx.x;
   const int V16 = (p.V + 15) >> 4;
-  const int u0 = static_cast<int>((static_cast<long long>(V16) * range) / p.n_ranges);
-  const int u1 = static_cast<int>((static_cast<long long>(V16) * (range + 1)) / p.n_ranges);
-  const int v_begin = u0 << 4, v_end = min(u1 << 4, p.V);
-  const int n_tiles = (v_end - v_begin + LW_BM - 1) / LW_BM;
+  const int v_begin = static_cast<int>((static_cast<long long>(V16) * range) / p.n_ranges) << 4;
+  const int v_stop = min(static_cast<int>((static_cast<long long>(V16) * (range + 1)) / p.n_ranges) << 4, p.V);
+  const int n_tiles = sp.n_tiles;
   const int n_kb = p.d / LW_BK;
+  // 8-entry units of the range, spread evenly over 2 n_tiles halves
+  const int units = (v_stop - v_begin + 7) >> 3;
+  auto half_begin = [&](int i) { return min(v_begin + 8 * ((units * i) / (LW_SUBS * n_tiles)), v_stop); };
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < sp.stages; ++i) { mbar_init(full_bar + i, 1); mbar_init(empty_bar + i, 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(tmem_full + i, 1); mbar_init(tmem_empty + i, 4); }
+    for (int i = 0; i < 2; ++i) { mbar_init(tmem_full + i, 1); mbar_init(tmem_empty + i, LW_EPI_WARPS); }
     fence_mbar_init();
   }
-  if (warp == 5) {
-    tmem_alloc(tmem_slot, 128);                   // two accumulators of at most 64 columns
+  if (warp == LW_EPI_WARPS + 1) {
+    tmem_alloc(tmem_slot, 256);                   // two buffers of two accumulators of at most 64 columns
     tmem_relinquish();
   }
-  if (warp == 4 && lane == 0) { prefetch_tmap(&tmap_h); prefetch_tmap(&tmap_w); prefetch_tmap(&tmap_wt); }
+  if (warp == LW_EPI_WARPS && lane == 0) { prefetch_tmap(&tmap_h); prefetch_tmap(&tmap_w); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == 4) {
+  if (warp == LW_EPI_WARPS) {
     if (lane == 0) {   // ---------------------------------------------------------- TMA producer
       int stage = 0;
       uint32_t phase = 0;
       const int seq = p.seq_index ? __ldg(p.seq_index) : 0;     // one active sequence of several; else packed rows
       if (sp.wait_rows) pdl_wait();
-      const int h_bytes = sp.N * LW_BK * 2;
+      const uint32_t tx = static_cast<uint32_t>(LW_SUBS * sp.box_rows + sp.N) * (LW_BK * 2);
       for (int t = 0; t < n_tiles; ++t) {
-        const int row0 = v_begin + t * LW_BM;
-        // a box always delivers its full size (rows past V, k-blocks past d: zero fill)
-        const bool low = sp.tail_rows > 0 && v_end - row0 <= sp.tail_rows;
-        const CUtensorMap* tw = low ? &tmap_wt : &tmap_w;
-        const int w_bytes = KPS * (low ? sp.tail_rows : LW_BM) * LW_BK * 2;
-        for (int kb = 0; kb < n_kb; kb += KPS) {
-          const int kc = min(KPS, n_kb - kb);
+        const int w0 = half_begin(LW_SUBS * t), w1 = half_begin(LW_SUBS * t + 1);
+        for (int kb = 0; kb < n_kb; ++kb) {
           mbar_wait(empty_bar + stage, phase ^ 1u, p.dev_status);
           uint8_t* sa = smem + stage * sp.stage_bytes;
-          mbar_expect_tx(full_bar + stage, static_cast<uint32_t>(w_bytes + kc * h_bytes));
-          if (KPS == 1) tma_load_2d(sa, tw, full_bar + stage, kb * LW_BK, row0);
-          else tma_load_4d(sa, tw, full_bar + stage, 0, 0, kb, row0 >> 3);
-          for (int j = 0; j < kc; ++j)                                                     // rows past the last: zero fill
-            tma_load_3d(sa + KPS * LW_A_BYTES + j * h_bytes, &tmap_h, full_bar + stage, (kb + j) * LW_BK, 0, seq);
+          mbar_expect_tx(full_bar + stage, tx);     // a box always delivers its full size (rows past V: zero fill)
+          tma_load_2d(sa, &tmap_w, full_bar + stage, kb * LW_BK, w0);
+          tma_load_2d(sa + LW_A_BYTES / 2, &tmap_w, full_bar + stage, kb * LW_BK, w1);
+          tma_load_3d(sa + LW_A_BYTES, &tmap_h, full_bar + stage, kb * LW_BK, 0, seq);   // rows past the last: zero fill
           if (++stage == sp.stages) { stage = 0; phase ^= 1u; }
         }
       }
     }
-  } else if (warp == 5) {
+  } else if (warp == LW_EPI_WARPS + 1) {
     if (lane == 0) {   // ---------------------------------------------------------- MMA issuer
       int stage = 0;
       uint32_t phase = 0;
@@ -710,17 +686,17 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
         const int buf = t & 1;
         mbar_wait(tmem_empty + buf, ((t >> 1) & 1u) ^ 1u, p.dev_status);
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * 64);
-        for (int kb = 0; kb < n_kb; kb += KPS) {
-          const int kc = min(KPS, n_kb - kb);
+        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * 128);
+        for (int kb = 0; kb < n_kb; ++kb) {
           mbar_wait(full_bar + stage, phase, p.dev_status);
           tc_fence_after();
           const uint32_t sa = base_u32 + stage * sp.stage_bytes;
-          for (int j = 0; j < kc; ++j) {
-            const uint64_t adesc = smem_desc_sw128(sa + j * 1024, KPS * 1024, 16);
-            const uint64_t bdesc = smem_desc_sw128(sa + KPS * LW_A_BYTES + j * (sp.N * LW_BK * 2), 1024, 16);
+          const uint64_t bdesc = smem_desc_sw128(sa + LW_A_BYTES, 1024, 16);
 #pragma unroll
-            for (int k = 0; k < LW_BK / 16; ++k) tc_mma_ss(d_tmem, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | j | k) != 0);
+          for (int u = 0; u < LW_SUBS; ++u) {
+            const uint64_t adesc = smem_desc_sw128(sa + u * (LW_A_BYTES / 2), 1024, 16);
+#pragma unroll
+            for (int k = 0; k < LW_BK / 16; ++k) tc_mma_ss(d_tmem + 64u * u, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0);
           }
           tc_commit(empty_bar + stage);
           if (++stage == sp.stages) { stage = 0; phase ^= 1u; }
@@ -729,11 +705,15 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
       }
     }
   } else {
-    // ------------------------------------------------------------------ epilogue (warps 0-3)
-    // this lane keeps the running statistics of columns `lane` and `lane + 32`
-    LmColStats run[2];
+    // ------------------------------------------------------------------ epilogue (warps 0-7)
+    const int quad = warp & 3, half = warp >> 2;
+    const int col = lane & 15, upper = lane >> 4;           // column within 16, entries 0-15 or 16-31 of the warp's 32
+    // The upper lanes read their entries in the order j ^ 1: entries of other parity lie in the other 16 banks.
+    const int flip = upper;
+    float* xb = reinterpret_cast<float*>(xpose + warp * LW_XPOSE_BYTES);
+    LmColStats run[LW_ROWS / 16];                 // columns 16 h + col, this lane's share of the entries
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < LW_ROWS / 16; ++h) {
       run[h].m = -INFINITY; run[h].s = 0.f; run[h].t = 0.f;
       run[h].v1 = -INFINITY; run[h].v2 = -INFINITY; run[h].i1 = -1; run[h].i2 = -1;
     }
@@ -742,52 +722,90 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
       const int buf = t & 1;
       mbar_wait(tmem_full + buf, (t >> 1) & 1u, p.dev_status);
       tc_fence_after();
-      const int v_lane0 = v_begin + t * LW_BM + warp * 32;    // vocabulary entry of lane 0
-      const bool valid = v_lane0 + lane < v_end;
+      const int v_warp = half_begin(LW_SUBS * t + half) + quad * 32;            // first entry of this warp
+      const int v_end = half_begin(LW_SUBS * t + half + 1);
+      const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(buf * 128 + half * 64);
+      if (v_warp < v_end) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (h * 32 >= sp.N) break;
-        uint32_t r[32];
-        tmem_ld32(tmem_base + (static_cast<uint32_t>(warp * 32) << 16) + static_cast<uint32_t>(buf * 64 + h * 32), r);
-        tc_wait_ld();
-        if (h * 32 + 32 >= sp.N) {                // last chunk read: the accumulator may be overwritten
-          tc_fence_before();
+        for (int h = 0; h < LW_ROWS / 16; ++h) {
+          if (16 * h >= sp.N) break;
+          uint32_t r[16];
+          tmem_ld16(taddr + 16 * h, r);
+          tc_wait_ld();
+          __syncwarp();                           // the block before this one has been read
+#pragma unroll
+          for (int j = 0; j < 4; ++j)             // word (entry e, column c): 16 e + 4 (c / 4 ^ (e / 2) % 4) + c % 4
+            *reinterpret_cast<uint4*>(xb + lane * 16 + ((j ^ ((lane >> 1) & 3)) << 2)) =
+                make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
           __syncwarp();
-          if (lane == 0) mbar_arrive(tmem_empty + buf);
-        }
-        lm_rows_chunk<kEntropy>(r, valid, v_lane0 + lane, h * 32, sp.N, lane, c, run[h]);
-      }
-    }
-    // the four warps covered different vocabulary entries of every tile: merge through shared memory
-    red[warp * 64 + lane] = run[0];
-    red[warp * 64 + 32 + lane] = run[1];
-    asm volatile("bar.sync 2, 128;" ::: "memory");   // the four epilogue warps
-    if (warp == 0) {
-      pdl_wait();   // the partials of the previous pass may still be read until earlier kernels are done
+          float z[16];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int col = h * 32 + lane;
-        if (col >= sp.n_rows) continue;
-        LmColStats q = red[col];
-        LmRowAcc a = {q.m, q.s, q.t};
-        for (int w2 = 1; w2 < 4; ++w2) {
-          const LmColStats o2 = red[w2 * 64 + col];
-          lm_fold(a, o2.m, o2.s, o2.t, c);
-          lm_top2_insert(o2.v1, o2.i1, q.v1, q.i1, q.v2, q.i2);
-          lm_top2_insert(o2.v2, o2.i2, q.v1, q.i1, q.v2, q.i2);
+          for (int j = 0; j < 16; ++j) {
+            const int e = 16 * upper + (j ^ flip);
+            z[j] = xb[e * 16 + (((col >> 2) ^ ((j >> 1) & 3)) << 2) + (col & 3)];
+          }
+#pragma unroll
+          for (int j = 0; j < 16; j += 2) {       // back to ascending entries
+            const float a = z[j], b = z[j + 1];
+            z[j] = flip ? b : a;
+            z[j + 1] = flip ? a : b;
+          }
+          if (v_warp + 16 * upper < v_end) lm_fold16<kEntropy>(z, v_warp + 16 * upper, v_end, c, run[h]);
         }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tmem_empty + buf);
+    }
+    // The lanes l and l + 16 and the eight warps covered different vocabulary entries: merge through the ring's
+    // memory (every copy has landed and every MMA has read it: the last accumulator is complete).
+    LmColMerge* red = reinterpret_cast<LmColMerge*>(smem);          // [8 warps][64 columns]
+#pragma unroll
+    for (int h = 0; h < LW_ROWS / 16; ++h) {
+      if (16 * h >= sp.N) break;
+      const LmColStats q = run[h];
+      LmColMerge o;
+      o.top.a = lm_key(q.v1, q.i1); o.top.b = lm_key(q.v2, q.i2); o.pad = 0.f;
+      const float om = __shfl_xor_sync(0xffffffffu, q.m, 16), os = __shfl_xor_sync(0xffffffffu, q.s, 16);
+      const float ot = kEntropy ? __shfl_xor_sync(0xffffffffu, q.t, 16) : 0.f;
+      const unsigned long long oa = __shfl_xor_sync(0xffffffffu, o.top.a, 16), ob = __shfl_xor_sync(0xffffffffu, o.top.b, 16);
+      lm_merge(o.top, oa, ob);
+      o.m = fmaxf(q.m, om);
+      const float f = lm_weight(q.m, o.m, c), g = lm_weight(om, o.m, c);
+      o.s = fmaf(q.s, f, os * g);
+      o.t = kEntropy ? fmaf(q.t, f, ot * g) : 0.f;
+      if (upper == 0) red[warp * LW_ROWS + 16 * h + col] = o;
+    }
+    asm volatile("bar.sync 2, 256;" ::: "memory");   // the eight epilogue warps
+    if (warp < 2) {
+      const int column = warp * 32 + lane;
+      pdl_wait();   // the partials of the previous pass may still be read until earlier kernels are done
+      if (column < sp.n_rows) {
+        LmColMerge q[LW_EPI_WARPS];
+        LmTop2 top = {0ull, 0ull};
         LmPartial out;
-        out.m = a.m; out.s = a.s; out.v1 = q.v1; out.v2 = q.v2; out.i1 = q.i1; out.i2 = q.i2; out.t = a.t; out.pad = 0;
-        p.partial[static_cast<size_t>(range) * LW_ROWS + col] = out;
+        out.m = -INFINITY; out.s = 0.f; out.t = 0.f; out.pad = 0;
+#pragma unroll
+        for (int w2 = 0; w2 < LW_EPI_WARPS; ++w2) { q[w2] = red[w2 * LW_ROWS + column]; out.m = fmaxf(out.m, q[w2].m); }
+#pragma unroll
+        for (int w2 = 0; w2 < LW_EPI_WARPS; ++w2) {      // relative to the common maximum: no chain from warp to warp
+          const float f = lm_weight(q[w2].m, out.m, c);
+          out.s = fmaf(q[w2].s, f, out.s);
+          if (kEntropy) out.t = fmaf(q[w2].t, f, out.t);
+          lm_merge(top, q[w2].top.a, q[w2].top.b);
+        }
+        out.v1 = lm_key_value(top.a); out.v2 = lm_key_value(top.b);
+        out.i1 = lm_key_entry(top.a); out.i2 = lm_key_entry(top.b);
+        p.partial[static_cast<size_t>(range) * LW_ROWS + column] = out;
       }
     }
   }
   pdl_wait();
   tc_fence_before();
   __syncthreads();
-  if (warp == 5) {
+  if (warp == LW_EPI_WARPS + 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 128);
+    tmem_dealloc(tmem_base, 256);
   }
 }
 
@@ -800,7 +818,8 @@ struct LmPlan {
   bool pack;       // the rows of an index list are gathered into the workspace first
   bool slots;      // (no workspace to gather into) four slots of 64 node rows per M tile
   int n_mt;        // M tiles of 256 rows
-  int n_ranges;    // vocabulary ranges of the main part (few_rows: ranges = CTAs)
+  int n_ranges;    // vocabulary ranges of the main part (few_rows: at most this many)
+  int rows_ctas;   // few_rows: ranges = CTAs
   int n_tail;      // pairs that sweep all M tiles over a slice of the vocabulary's tail
   int main_units;  // 32-column units of the main part
   size_t required;   // workspace the call cannot do without
@@ -827,6 +846,11 @@ static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, si
     int sms = device_sm_count() - tl_lm_reserved_sms;
     if (sms < 1) sms = 1;
     pl->n_ranges = sms < V16 ? sms : V16;
+    pl->rows_ctas = pl->n_ranges;
+    // few units per range: as many ranges as keep the longest one as short, all of the same length where that comes
+    // out even (a small vocabulary's statistics then do not depend on how many SMs the launch was given)
+    const int per = (V16 + sms - 1) / sms;
+    if (per <= 8) pl->rows_ctas = (V16 + per - 1) / per;
     return;
   }
   pl->n_mt = slots ? (n_seq + 3) / 4 : static_cast<int>((rows + 2 * LM_BM - 1) / (2 * LM_BM));
@@ -918,7 +942,7 @@ extern "C" int trispec_lmhead_stats(const trispec_lmhead_args* a, void* stream) 
 }
 
 static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmPlan& pl, void* stream) {
-  const int n_seq = pl.n_seq, n_ranges = pl.n_ranges;
+  const int n_seq = pl.n_seq, n_ranges = pl.few_rows ? pl.rows_ctas : pl.n_ranges;
   const long long n_rows = static_cast<long long>(n_seq) * a->T;
   int rc = TRISPEC_OK;
   if (!a->h || !a->W || !a->parent || !a->tok || !a->workspace) return TRISPEC_ERR_INVALID_ARG;
@@ -971,35 +995,22 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
     sp.n_rows = static_cast<int>(n_rows);
     sp.wait_rows = p.wait_rows;
     sp.N = ((sp.n_rows + 15) / 16) * 16;
-    const int kps = (a->V % 8) == 0 ? 4 : 1;
-    sp.stage_bytes = kps * (LW_A_BYTES + sp.N * LW_BK * 2);
-    sp.stages = (216 * 1024) / sp.stage_bytes;
+    sp.stage_bytes = LW_A_BYTES + sp.N * LW_BK * 2;
+    sp.stages = LW_RING_BYTES / sp.stage_bytes;
     if (sp.stages > LW_MAX_STAGES) sp.stages = LW_MAX_STAGES;
-    const int smem_bytes = sp.stages * sp.stage_bytes + 1024 + 8192;
-    // the longer of the two range lengths (they differ by 16 rows) decides the height of the second box
+    // tiles of equal height: as few as the longest range (in 8-entry units; the lengths differ by two) allows
     {
       const int V16 = (a->V + 15) / 16;
-      const int r_big = ((V16 + n_ranges - 1) / n_ranges) * 16;
-      const int last = r_big - LW_BM * ((r_big + LW_BM - 1) / LW_BM - 1);
-      sp.tail_rows = last < LW_BM ? last : 0;
+      const int u_max = 2 * ((V16 + n_ranges - 1) / n_ranges);
+      sp.n_tiles = (u_max + LW_SUBS * LW_BM / 8 - 1) / (LW_SUBS * LW_BM / 8);
+      sp.box_rows = 8 * ((u_max + LW_SUBS * sp.n_tiles - 1) / (LW_SUBS * sp.n_tiles));
     }
-    CUtensorMap tm_w128, tm_wt, tm_hn;
-    for (int m = 0; m < 2; ++m) {
-      const uint32_t rows = m == 0 ? LW_BM : static_cast<uint32_t>(sp.tail_rows);
-      CUtensorMap* tm = m == 0 ? &tm_w128 : &tm_wt;
-      if (rows == 0) { tm_wt = tm_w128; break; }
-      if (kps == 1) {
-        const uint64_t dims[2] = {static_cast<uint64_t>(a->d), static_cast<uint64_t>(a->V)};
-        const uint64_t strides[1] = {static_cast<uint64_t>(a->d) * 2};
-        const uint32_t box[2] = {LW_BK, rows};
-        if (!cached_tmap_bf16(tm, a->W, 2, dims, strides, box)) return TRISPEC_ERR_CUDA;
-      } else {
-        // [V/8 groups][d/64 k-blocks][8 rows][64 elements]: the k-block index moves 128 B, the row 2 d B
-        const uint64_t dims[4] = {LW_BK, 8, static_cast<uint64_t>(a->d / LW_BK), static_cast<uint64_t>(a->V / 8)};
-        const uint64_t strides[3] = {static_cast<uint64_t>(a->d) * 2, LW_BK * 2, static_cast<uint64_t>(a->d) * 16};
-        const uint32_t box[4] = {LW_BK, 8, static_cast<uint32_t>(kps), rows / 8};
-        if (!cached_tmap_bf16(tm, a->W, 4, dims, strides, box)) return TRISPEC_ERR_CUDA;
-      }
+    CUtensorMap tm_wr, tm_hn;
+    {
+      const uint64_t dims[2] = {static_cast<uint64_t>(a->d), static_cast<uint64_t>(a->V)};
+      const uint64_t strides[1] = {static_cast<uint64_t>(a->d) * 2};
+      const uint32_t box[2] = {LW_BK, static_cast<uint32_t>(sp.box_rows)};
+      if (!cached_tmap_bf16(&tm_wr, a->W, 2, dims, strides, box)) return TRISPEC_ERR_CUDA;
     }
     {
       // one active sequence of several: its nodes; otherwise all rows, back to back
@@ -1010,16 +1021,13 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
       const uint32_t box[3] = {LW_BK, static_cast<uint32_t>(sp.N), 1};
       if (!cached_tmap_bf16(&tm_hn, rows_base, 3, dims, strides, box)) return TRISPEC_ERR_CUDA;
     }
-    typedef void (*RowsKernel)(CUtensorMap, CUtensorMap, CUtensorMap, LmRowsParams);
-    static const RowsKernel table[2][2] = {{lmhead_rows_kernel<false, 1>, lmhead_rows_kernel<false, 4>},
-                                           {lmhead_rows_kernel<true, 1>, lmhead_rows_kernel<true, 4>}};
-    const int wide = kps > 1 ? 1 : 0;
-    const RowsKernel kernel = table[want_entropy ? 1 : 0][wide];
-    static bool smem_set_rows[4][64] = {};
-    rc = ensure_smem_limit(reinterpret_cast<const void*>(kernel), 227 * 1024, smem_set_rows[(want_entropy ? 2 : 0) + wide]);
+    typedef void (*RowsKernel)(CUtensorMap, CUtensorMap, LmRowsParams);
+    const RowsKernel kernel = want_entropy ? lmhead_rows_kernel<true> : lmhead_rows_kernel<false>;
+    static bool smem_set_rows[2][64] = {};
+    rc = ensure_smem_limit(reinterpret_cast<const void*>(kernel), LW_SMEM_BYTES, smem_set_rows[want_entropy ? 1 : 0]);
     if (rc != TRISPEC_OK) return rc;
     TRISPEC_CUDA_OK(launch_dependent(kernel, static_cast<unsigned>(n_ranges), LW_THREADS,
-                                     static_cast<size_t>(smem_bytes), st, 1, tm_w128, tm_wt, tm_hn, sp));
+                                     static_cast<size_t>(LW_SMEM_BYTES), st, 1, tm_wr, tm_hn, sp));
     count_launch();
     f.stride = LW_ROWS;
     TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel, static_cast<unsigned>((n_rows + 7) / 8),
