@@ -631,6 +631,9 @@ static int attn_plan_override() {
   return 0;
 }
 
+static thread_local int tl_attn_splits = 0;
+void attn_splits_once(int splits) { tl_attn_splits = splits; }
+
 static int attn_plan(const trispec_attn_args* a, AttnPlan* pl) {
   if (!a || a->B <= 0 || a->T <= 0 || a->Hq <= 0 || a->Hkv <= 0) return TRISPEC_ERR_INVALID_ARG;
   if (a->D != AT_D || a->T > 64 || a->Hq % a->Hkv != 0) return TRISPEC_ERR_UNSUPPORTED;
@@ -660,6 +663,14 @@ static int attn_plan(const trispec_attn_args* a, AttnPlan* pl) {
   // for that, one wave filled as far as possible; very few (sequence, head) pairs are cut further.
   const long long slots = static_cast<long long>(device_sm_count()) * 2;   // two CTAs per SM (split kernels)
   const int tiles = pl->tiles_max;
+  if (tl_attn_splits > 0) {
+    pl->n_splits = tl_attn_splits;
+    pl->cluster = true;
+    pl->items = static_cast<size_t>(fixed) * pl->n_splits;
+    pl->pieces = false;
+    pl->n_cta = 0;
+    return TRISPEC_OK;
+  }
   int best_s = 0;
   for (int sp = 1; sp <= 8 && !best_s; ++sp)
     if (fixed * sp * 4 >= slots * 5 && tiles / sp >= 32) best_s = sp;
@@ -709,6 +720,20 @@ static int attn_plan(const trispec_attn_args* a, AttnPlan* pl) {
     pl->pieces = ov == 1 || (ov == 0 && uneven && steps_max >= 256 * n_grp);
   }
   return TRISPEC_OK;
+}
+
+int attn_compact_splits(const trispec_attn_args* a, double budget_us, double tile_us, double fixed_us, int max_ctas, int* ctas) {
+  AttnPlan pl;
+  if (attn_plan_override() || attn_plan(a, &pl) != TRISPEC_OK) return 0;
+  const long long fixed = static_cast<long long>(pl.n_seq) * a->Hkv * pl.n_mt;
+  for (int s = 1; s <= 8 && fixed * s <= max_ctas; ++s) {
+    if (s > 1 && pl.tiles_max < 4 * s) break;    // (fewer than four tiles per CTA are never worth a split)
+    if (fixed_us + tile_us * ((pl.tiles_max + s - 1) / s + 1) <= budget_us) {
+      *ctas = static_cast<int>(fixed * s);
+      return s;
+    }
+  }
+  return 0;
 }
 
 int attn_planned_ctas(const trispec_attn_args* a) {

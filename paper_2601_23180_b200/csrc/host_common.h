@@ -93,6 +93,14 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 // CTAs the attention launch for these arguments will use (0 if the arguments are not accepted)
 int attn_planned_ctas(const trispec_attn_args* a);
+// The smallest number of KV splits (1 to 8, merged on chip: no workspace) with which every CTA of the attention ends
+// within `budget_us` at `tile_us` per tile and `fixed_us` besides, in at most `max_ctas` CTAs; 0 if there is none. The
+// number of CTAs goes to `ctas` where there is one.
+int attn_compact_splits(const trispec_attn_args* a, double budget_us, double tile_us, double fixed_us, int max_ctas, int* ctas);
+// KV splits of the next attention launch from this thread (0 = the planner's choice)
+void attn_splits_once(int splits);
+// rows up to which the LM head takes its small-row kernel
+constexpr int LM_FEW_ROWS = 64;
 
 #define TRISPEC_CUDA_OK(expr)                        \
   do {                                               \

@@ -557,7 +557,7 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
 constexpr int LW_BM = 128, LW_SUBS = 2, LW_BK = 64, LW_MAX_STAGES = 6, LW_EPI_WARPS = 8;
 constexpr int LW_THREADS = 32 * (LW_EPI_WARPS + 2);
 constexpr int LW_A_BYTES = LW_SUBS * LW_BM * LW_BK * 2;  // 32 KB of W per stage
-constexpr int LW_ROWS = 64;                              // partial rows per vocabulary range
+constexpr int LW_ROWS = LM_FEW_ROWS;                     // partial rows per vocabulary range
 constexpr int LW_XPOSE_BYTES = 2048;                     // 32 entries x 16 columns per epilogue warp
 constexpr int LW_SMEM_BYTES = 227 * 1024;
 constexpr int LW_RING_BYTES = LW_SMEM_BYTES - 1024 /*alignment slack*/ - LW_EPI_WARPS * LW_XPOSE_BYTES - 256 /*barriers*/;
@@ -839,7 +839,7 @@ static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, si
   pl->pack_bytes = 0;
   pl->n_tail = 0;
   pl->main_units = (a->V + 31) / 32;
-  pl->few_rows = rows <= 64 && !slots;
+  pl->few_rows = rows <= LM_FEW_ROWS && !slots;
   if (pl->few_rows) {
     pl->n_mt = 1;
     const int V16 = (a->V + 15) / 16;

@@ -36,40 +36,70 @@ static int host_pass_streams(HostPassStreams** out) {
 namespace trispec {
 // How a pass arranges its attention and its LM head (they do not depend on each other).
 enum PassForm { PASS_ATTENTION_FIRST = 0, PASS_LM_FIRST = 1, PASS_SIDE_BY_SIDE = 2 };
-static PassForm pass_form(const trispec_attn_args* attn, const trispec_lmhead_args* lm, const trispec_scan_args* scan,
-                          int* attn_ctas_out) {
-  const int lm_seqs = lm->seq_index ? lm->B_active : lm->B;
-  const int attn_ctas = attn ? attn_planned_ctas(attn) : 0;
-  if (attn_ctas_out) *attn_ctas_out = attn_ctas;
-  if (!attn || lm_seqs != 1 || attn_ctas <= 0) return PASS_ATTENTION_FIRST;
-  // TRISPEC_PASS_FORM = attention_first | lm_first | side_by_side overrides the rule below for one active
-  // sequence (a tuning and testing aid, read at every call; side by side still needs at most SMs / 2 CTAs)
-  if (const char* e = getenv("TRISPEC_PASS_FORM")) {
-    if (e[0] == 'a') return PASS_ATTENTION_FIRST;
-    if (e[0] == 'l') return PASS_LM_FIRST;
-    if (e[0] == 's' && attn_ctas * 2 <= device_sm_count() &&
-        !(attn->seq_index && scan && scan->esc_index == attn->seq_index)) return PASS_SIDE_BY_SIDE;
+struct PassPlan {
+  PassForm form;
+  bool beside;        // mask and attention go to the second stream, the LM head leaves them `attn_ctas` SMs
+  int attn_ctas;
+  int attn_splits;    // KV splits of that attention, 0 = what the attention's own planner takes
+};
+static bool stream_is_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
   }
-  // not side by side when the scan's escalation list is written over the index list the attention reads:
+  return status != cudaStreamCaptureStatusNone;
+}
+// `compact`: the attention may be planned for few CTAs beside the LM head. Not while `stream` is captured: the second
+// stream is shared by every caller on the device and should not become part of more captures than it has to.
+static PassPlan pass_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm, const trispec_scan_args* scan,
+                          bool compact = true) {
+  PassPlan pl = {PASS_ATTENTION_FIRST, false, attn ? attn_planned_ctas(attn) : 0, 0};
+  const int lm_seqs = lm->seq_index ? lm->B_active : lm->B;
+  if (!attn || pl.attn_ctas <= 0 || lm_seqs <= 0 || static_cast<long long>(lm_seqs) * lm->T > LM_FEW_ROWS) return pl;
+  const int sms = device_sm_count();
+  // not beside the scan when its escalation list is written over the index list the attention reads:
   // in stream order the scan comes last, side by side it would not
   const bool in_place_list = attn->seq_index && scan && scan->esc_index == attn->seq_index;
-  // Side by side the LM head gives up one SM per attention CTA and takes SMs / (SMs - CTAs) times as long;
-  // one after the other the pass pays the attention (15-25 us at these sizes) and a launch boundary. With the
-  // LM head's time estimated as its bytes of W at 5 TB/s, side by side wins while that extra time stays below
-  // about 40 us (measured on one sequence: 32000 x 2048 weights with 16 and 64 CTAs, 151936 x 2048 with 16 and
-  // 32 CTAs win; 151936 x 2048 with 64 CTAs loses 180 against 152 us; 128256 x 4096 with 32 CTAs is even).
-  // Otherwise the LM head goes first: behind the attention it would stall as a programmatic dependent.
-  const int sms = device_sm_count();
-  const double lm_us = static_cast<double>(lm->V) * lm->d * 2.0 / 5.0e6;
-  if (attn_ctas * 2 <= sms && !in_place_list && lm_us * attn_ctas <= 40.0 * (sms - attn_ctas)) return PASS_SIDE_BY_SIDE;
-  return PASS_LM_FIRST;
+  // TRISPEC_PASS_FORM = attention_first | lm_first | side_by_side overrides the rules below for at most LM_FEW_ROWS
+  // rows (a tuning and testing aid, read at every call; lm_first is then one after the other, and side by
+  // side, with the attention's own plan, still needs at most SMs / 2 CTAs)
+  if (const char* e = getenv("TRISPEC_PASS_FORM")) {
+    if (e[0] == 'a') return pl;
+    if (e[0] == 'l') { pl.form = PASS_LM_FIRST; return pl; }
+    if (e[0] == 's' && pl.attn_ctas * 2 <= sms && !in_place_list) { pl.form = PASS_SIDE_BY_SIDE; pl.beside = true; return pl; }
+  }
+  // With so few rows the LM head is a pure stream of W that does not need every SM to saturate HBM, and the attention
+  // a chain of tiles that does not need bandwidth: the attention runs beside the LM head in as FEW CTAs as end
+  // well before it (a CTA alone on its SM takes about 1.1 us per 64-key tile; W streams at 6 TB/s), one
+  // SM each, as long as that is at most a quarter of the chip. One sequence of 61 nodes, 4096 context tokens, 151936 x 2048
+  // weights: 8 CTAs of 65 tiles beside 140 of the LM head against 64 CTAs after all 148 of it.
+  const double lm_us = static_cast<double>(lm->V) * lm->d * 2.0 / 6.0e6;
+  const int splits = in_place_list || !compact ? 0 : attn_compact_splits(attn, 0.8 * lm_us, 1.1, 6.0, sms / 4, &pl.attn_ctas);
+  if (lm_seqs == 1) {
+    // Behind the attention the LM head would stall as a programmatic dependent, so for one sequence it goes first
+    // whatever the form. What the form is called follows the attention's own plan: side by side where that could
+    // be given one SM per CTA for less than about 40 us of the LM head's time, which then takes SMs / (SMs - CTAs)
+    // times as long.
+    const int own = attn_planned_ctas(attn);
+    const double own_lm_us = lm_us * 6.0 / 5.0;
+    const bool own_fits = own * 2 <= sms && !in_place_list && own_lm_us * own <= 40.0 * (sms - own);
+    pl.form = own_fits ? PASS_SIDE_BY_SIDE : PASS_LM_FIRST;
+    pl.beside = splits > 0 || own_fits;
+  } else if (splits > 0) {
+    pl.form = PASS_SIDE_BY_SIDE;
+    pl.beside = true;
+  }
+  pl.attn_splits = splits;
+  if (splits == 0) pl.attn_ctas = attn_planned_ctas(attn);
+  return pl;
 }
 }  // namespace trispec
 
 extern "C" const char* trispec_verify_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm,
                                            const trispec_scan_args* scan) {
   if (!lm) return "none";
-  switch (trispec::pass_form(attn, lm, scan, nullptr)) {
+  switch (trispec::pass_plan(attn, lm, scan).form) {
     case trispec::PASS_LM_FIRST: return "lm_first";
     case trispec::PASS_SIDE_BY_SIDE: return "side_by_side";
     default: return "attention_first";
@@ -87,16 +117,16 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
   // LM head is a pure stream of W and loses more behind an attention than the hidden latency is worth (one
   // sequence of 4096 context tokens: 166 us against 156 us the other way round), so there the LM head goes
   // first, or the two run side by side (pass_form above).
-  int attn_ctas = 0;
-  const trispec::PassForm form = trispec::pass_form(attn, lm, scan, &attn_ctas);
-  const bool lm_first = form == trispec::PASS_LM_FIRST;
+  const trispec::PassPlan plan =
+      trispec::pass_plan(attn, lm, scan, !trispec::stream_is_capturing(static_cast<cudaStream_t>(stream)));
+  const bool lm_first = plan.form == trispec::PASS_LM_FIRST;
   int rc;
-  // One active sequence and an attention small enough beside the LM head (pass_form): the two run side by
+  // Few rows and an attention that fits beside the LM head (pass_plan): the two run side by
   // side. Mask and attention go to a second stream behind an event recorded on `stream` at the
   // start of the call; the LM head, whose grid is one persistent CTA per SM, leaves them one SM per attention
   // CTA and starts at once, the scan follows it, and `stream` then waits for the second stream: everything
   // the call enqueues is complete before anything enqueued on `stream` after it.
-  if (form == trispec::PASS_SIDE_BY_SIDE) {
+  if (plan.beside) {
     using namespace trispec;
     HostPassStreams* hs = nullptr;
     rc = host_pass_streams(&hs);
@@ -106,19 +136,22 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
     TRISPEC_CUDA_OK(cudaEventRecord(hs->fork, st));
     TRISPEC_CUDA_OK(cudaStreamWaitEvent(hs->copy, hs->fork, 0));
     rc = trispec_build_tree_mask(tree, hs->copy);          // ordinary launch: first kernel of the call
-    if (rc != TRISPEC_OK) return rc;
-    rc = trispec_verify_attn(attn, hs->copy);              // dependent of the mask kernel
-    if (rc != TRISPEC_OK) return rc;
+    if (rc == TRISPEC_OK) {
+      attn_splits_once(plan.attn_splits);
+      rc = trispec_verify_attn(attn, hs->copy);            // dependent of the mask kernel
+      attn_splits_once(0);
+    }
     TRISPEC_CUDA_OK(cudaEventRecord(hs->copied, hs->copy));
-    entry_scope_next_launch_ordinary();                    // first kernel on `stream`
-    lm_reserve_sms_once(attn_ctas);
-    rc = trispec_lmhead_stats(lm, stream);
-    lm_reserve_sms_once(0);
-    if (rc != TRISPEC_OK) return rc;
-    rc = trispec_accept_scan(scan, stream);                // dependent of the LM head's last kernel
-    if (rc != TRISPEC_OK) return rc;
+    if (rc == TRISPEC_OK) {
+      entry_scope_next_launch_ordinary();                  // first kernel on `stream`
+      lm_reserve_sms_once(plan.attn_ctas);
+      rc = trispec_lmhead_stats(lm, stream);
+      lm_reserve_sms_once(0);
+    }
+    if (rc == TRISPEC_OK) rc = trispec_accept_scan(scan, stream);   // dependent of the LM head's last kernel
+    // joined after an argument error too: what has been launched ends before whatever `stream` gets next
     TRISPEC_CUDA_OK(cudaStreamWaitEvent(st, hs->copied, 0));
-    return TRISPEC_OK;
+    return rc;
   }
   rc = trispec_build_tree_mask(tree, stream);
   if (rc != TRISPEC_OK) return rc;
@@ -193,8 +226,8 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
                      {const_cast<void*>(lm->h), io->h, BT * static_cast<size_t>(lm->d) * 2}};
     TRISPEC_CUDA_OK(copy_list(in, 3, cudaMemcpyHostToDevice, st));
   }
-  int attn_ctas = 0;
-  const bool side_by_side = pass_form(attn, lm, scan, &attn_ctas) == PASS_SIDE_BY_SIDE;
+  const PassPlan plan = pass_plan(attn, lm, scan, !stream_is_capturing(st));
+  const bool side_by_side = plan.beside;
   if (side_by_side) TRISPEC_CUDA_OK(cudaEventRecord(hs->inputs, st));
   if (attn) {
     TRISPEC_CUDA_OK(cudaStreamWaitEvent(hs->copy, hs->fork, 0));
@@ -206,22 +239,25 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
   }
   int rc;
   if (side_by_side) {
-    // one active sequence, short context (as in trispec_verify): mask and attention follow their inputs on
+    // few rows (as in trispec_verify): mask and attention follow their inputs on
     // the second stream, the LM head and the scan run on `stream`, which then waits for the second stream
     TRISPEC_CUDA_OK(cudaStreamWaitEvent(hs->copy, hs->inputs, 0));   // the tree's parents have arrived
     rc = trispec_build_tree_mask(tree, hs->copy);
-    if (rc != TRISPEC_OK) return rc;
-    rc = trispec_verify_attn(attn, hs->copy);
-    if (rc != TRISPEC_OK) return rc;
+    if (rc == TRISPEC_OK) {
+      attn_splits_once(plan.attn_splits);
+      rc = trispec_verify_attn(attn, hs->copy);
+      attn_splits_once(0);
+    }
     TRISPEC_CUDA_OK(cudaEventRecord(hs->copied, hs->copy));
-    entry_scope_next_launch_ordinary();                              // first kernel on `stream`
-    lm_reserve_sms_once(attn_ctas);
-    rc = trispec_lmhead_stats(lm, stream);
-    lm_reserve_sms_once(0);
-    if (rc != TRISPEC_OK) return rc;
-    rc = trispec_accept_scan(scan, stream);
-    if (rc != TRISPEC_OK) return rc;
+    if (rc == TRISPEC_OK) {
+      entry_scope_next_launch_ordinary();                            // first kernel on `stream`
+      lm_reserve_sms_once(plan.attn_ctas);
+      rc = trispec_lmhead_stats(lm, stream);
+      lm_reserve_sms_once(0);
+    }
+    if (rc == TRISPEC_OK) rc = trispec_accept_scan(scan, stream);
     TRISPEC_CUDA_OK(cudaStreamWaitEvent(st, hs->copied, 0));
+    if (rc != TRISPEC_OK) return rc;
   } else {
     rc = trispec_build_tree_mask(tree, stream);
     if (rc != TRISPEC_OK) return rc;

@@ -66,3 +66,34 @@ def test_lmhead_packed_rows_against_oracle(B, T, listed, room):
     with pytest.raises(ts.TrispecError) as e:
         ts.trispec_lmhead_stats(a)
     assert e.value.code == 3 and ts.launch_count() == n0
+
+
+@pytest.mark.parametrize("B,k,tree,L,V,d,form", [
+    (1, 60, "random", 1000, 40000, 2048, None),           # two KV splits beside the LM head
+    (3, 8, "chain", 500, 40000, 2048, "side_by_side"),    # three sequences, 27 rows: unsplit
+    (1, 8, "chain", 4096, 8000, 256, "lm_first"),         # the LM head ends long before such an attention: one after the other
+])
+def test_few_row_pass_with_its_attention_beside_the_lm_head(B, k, tree, L, V, d, form):
+    import torch
+    from paper_2601_23180_b200 import binding as ts, runner
+    cfg = gen.small_variant(gen.CONFIGS["proxy_tree"], B=B, k=k, tree=tree, max_depth=min(k, 6), L=L, V=V, d=d, seed=5,
+                            logit_scale=3.6 / (0.02 * math.sqrt(d)))
+    pas = runner.VerifyPass(cfg, gen.make_inputs(cfg))
+    if form:
+        assert ts.trispec_verify_plan(pas.attn_args, pas.lm_args, pas.scan_args) == form
+    ts.trispec_build_tree_mask(pas.tree_args)
+    ts.trispec_verify_attn(pas.attn_args)
+    ts.trispec_lmhead_stats(pas.lm_args)
+    ts.trispec_accept_scan(pas.scan_args)
+    torch.cuda.synchronize()
+    want = pas.o.float().clone(), pas.stats["lse"].clone(), pas.stats["top1_idx"].clone(), pas.scan_out["path"].clone()
+    for _ in range(5):
+        pas.o.fill_(float("nan")); pas.mask.zero_(); pas.stats["lse"].zero_(); pas.stats["top1_idx"].fill_(-7)
+        pas.scan_out["path"].fill_(-9)
+        pas.run()
+        got = pas.o.float().clone(), pas.stats["lse"].clone(), pas.stats["top1_idx"].clone(), pas.scan_out["path"].clone()
+        torch.cuda.synchronize()
+        # two bf16 roundings of outputs of at most about 4 (half a step is 8e-3), as in the parity tests
+        assert (got[0] - want[0]).abs().max().item() <= 2e-2
+        assert (got[1] - want[1]).abs().max().item() <= 1e-4      # fp32 sums in another order, lse of about 30
+        assert torch.equal(got[2], want[2]) and torch.equal(got[3], want[3])
