@@ -101,6 +101,11 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_bar + 7);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // Softmax warps that hold at least one row of the M tile (a chain of 9 nodes with 4 query heads per KV head fills 36
+  // rows, two warps). The others take no part in the tile loop: their rows of P and O are whatever memory holds, never
+  // read, and the exponential unit, which the two CTAs of an SM share, is left to the rows that exist.
+  const int n_rows = min(p.NPT, nn - mtile * p.NPT) * p.G;         // > 0 unless idle_cta
+  const int sm_threads = 32 * ((n_rows + 31) >> 5);
   uint8_t* sPartO = smem;                                               // reuses the K/V ring at the end
   float2* sPartML = reinterpret_cast<float2*>(smem + AT_PART_ML_OFF);
   uint32_t tmem_base = 0;
@@ -118,8 +123,8 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
     asm volatile("bar.arrive 1, 192;" ::: "memory");
   } else {
     if (threadIdx.x == 0) {
-      mbar_init(s_bar, 1); mbar_init(s_free, 128); mbar_init(q_bar, 128);
-      for (int i = 0; i < NP; ++i) { mbar_init(o_bar + i, 1); mbar_init(p_bar + i, 128); }
+      mbar_init(s_bar, 1); mbar_init(s_free, sm_threads); mbar_init(q_bar, sm_threads);
+      for (int i = 0; i < NP; ++i) { mbar_init(o_bar + i, 1); mbar_init(p_bar + i, sm_threads); }
       fence_mbar_init();
     }
     if (warp == 5) {
@@ -253,7 +258,7 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
         }
       }
     }
-  } else {
+  } else if (static_cast<int>(threadIdx.x) < sm_threads) {
     // ------------------------------------------------------------------ softmax (warps 0-3)
     const int row = warp * 32 + lane;
     const int node = mtile * p.NPT + row / p.G;
@@ -390,7 +395,7 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
       if (vrows < AT_BN) {
         mbar_wait(v_full + i % NV, (i / NV) & 1u, p.dev_status);
         uint8_t* sv = sV + (i % NV) * AT_TILE_BYTES;
-        for (int e = threadIdx.x; e < (AT_BN - vrows) * 16; e += 128) {
+        for (int e = threadIdx.x; e < (AT_BN - vrows) * 16; e += sm_threads) {
           const int r = vrows + (e >> 4), c16 = e & 15;
           *reinterpret_cast<uint4*>(sv + (c16 >> 3) * AT_BOX_BYTES + r * 128 + ((c16 & 7) << 4)) = make_uint4(0, 0, 0, 0);
         }
