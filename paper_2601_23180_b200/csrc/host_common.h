@@ -100,7 +100,7 @@ int attn_compact_splits(const trispec_attn_args* a, double budget_us, double til
 // KV splits of the next attention launch from this thread (0 = the planner's choice)
 void attn_splits_once(int splits);
 // rows up to which the LM head takes its small-row kernel
-constexpr int LM_FEW_ROWS = 64;
+constexpr int LM_FEW_ROWS = 128;
 
 #define TRISPEC_CUDA_OK(expr)                        \
   do {                                               \

@@ -541,12 +541,12 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
 }
 
 // ---------------------------------------------------------------------------------------
-// At most 64 rows (batch-1 decoding, the paper's own setting; a few chains): operands swapped. With so
+// At most 128 rows (batch-1 decoding, the paper's own setting; two trees; a batch of chains): operands swapped. With so
 // few rows the GEMM is bound by streaming W, and the pair kernel above spends half of its ring
-// on H tiles. Here W is the M-side operand, the rows are the N side (16-64 columns), and one CTA per SM takes one
+// on H tiles. Here W is the M-side operand, the rows are the N side (16-128 columns), and one CTA per SM takes one
 // vocabulary range. A tile is up to 2 x 128 vocabulary entries, two MMAs that share the k-block of H: a stage is
-// 32 KB of W and 2-8 KB of H, so that up to 160 KB of W are in flight per SM and H, which every SM reads, adds 25 %
-// to what L2 delivers (with 128 entries per tile it was 50 %).
+// 32 KB of W and 2-16 KB of H, so that up to 160 KB of W are in flight per SM and H, which every SM reads, adds 25 %
+// (64 rows) to what L2 delivers (with 128 entries per tile it was 50 %, in the pair kernel it is 100 %).
 // A range is cut into tiles of equal height, so that none ends in a tile that is nearly empty and W is streamed once.
 // TMEM lane = vocabulary entry, column = row. Epilogue: warps 0-3 take the first 128 entries of a tile, warps
 // 4-7 the others. A warp passes 32 entries x 16 columns through 2 KB of shared memory, after which a lane holds 16
@@ -557,7 +557,7 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
 constexpr int LW_BM = 128, LW_SUBS = 2, LW_BK = 64, LW_MAX_STAGES = 6, LW_EPI_WARPS = 8;
 constexpr int LW_THREADS = 32 * (LW_EPI_WARPS + 2);
 constexpr int LW_A_BYTES = LW_SUBS * LW_BM * LW_BK * 2;  // 32 KB of W per stage
-constexpr int LW_ROWS = LM_FEW_ROWS;                     // partial rows per vocabulary range
+constexpr int lw_rows(long long n_rows) { return n_rows <= 64 ? 64 : 128; }   // partial rows per vocabulary range
 constexpr int LW_XPOSE_BYTES = 2048;                     // 32 entries x 16 columns per epilogue warp
 constexpr int LW_SMEM_BYTES = 227 * 1024;
 constexpr int LW_RING_BYTES = LW_SMEM_BYTES - 1024 /*alignment slack*/ - LW_EPI_WARPS * LW_XPOSE_BYTES - 256 /*barriers*/;
@@ -614,7 +614,8 @@ __device__ __forceinline__ void lm_fold16(float (&z)[16], int v0, int v_end, flo
   }
 }
 
-template <bool kEntropy>
+// kRows = 64 or 128: columns that the tensor memory and the statistics are laid out for
+template <bool kEntropy, int kRows>
 __global__ void __launch_bounds__(LW_THREADS, 1)
 lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_h,
                    const LmRowsParams sp) {
@@ -648,7 +649,7 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     fence_mbar_init();
   }
   if (warp == LW_EPI_WARPS + 1) {
-    tmem_alloc(tmem_slot, 256);                   // two buffers of two accumulators of at most 64 columns
+    tmem_alloc(tmem_slot, 4 * kRows);             // two buffers of two accumulators of kRows columns
     tmem_relinquish();
   }
   if (warp == LW_EPI_WARPS && lane == 0) { prefetch_tmap(&tmap_h); prefetch_tmap(&tmap_w); }
@@ -686,7 +687,7 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
         const int buf = t & 1;
         mbar_wait(tmem_empty + buf, ((t >> 1) & 1u) ^ 1u, p.dev_status);
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * 128);
+        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * (2 * kRows));
         for (int kb = 0; kb < n_kb; ++kb) {
           mbar_wait(full_bar + stage, phase, p.dev_status);
           tc_fence_after();
@@ -696,7 +697,7 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
           for (int u = 0; u < LW_SUBS; ++u) {
             const uint64_t adesc = smem_desc_sw128(sa + u * (LW_A_BYTES / 2), 1024, 16);
 #pragma unroll
-            for (int k = 0; k < LW_BK / 16; ++k) tc_mma_ss(d_tmem + 64u * u, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0);
+            for (int k = 0; k < LW_BK / 16; ++k) tc_mma_ss(d_tmem + static_cast<uint32_t>(kRows) * u, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0);
           }
           tc_commit(empty_bar + stage);
           if (++stage == sp.stages) { stage = 0; phase ^= 1u; }
@@ -711,9 +712,9 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     // The upper lanes read their entries in the order j ^ 1: entries of other parity lie in the other 16 banks.
     const int flip = upper;
     float* xb = reinterpret_cast<float*>(xpose + warp * LW_XPOSE_BYTES);
-    LmColStats run[LW_ROWS / 16];                 // columns 16 h + col, this lane's share of the entries
+    LmColStats run[kRows / 16];                 // columns 16 h + col, this lane's share of the entries
 #pragma unroll
-    for (int h = 0; h < LW_ROWS / 16; ++h) {
+    for (int h = 0; h < kRows / 16; ++h) {
       run[h].m = -INFINITY; run[h].s = 0.f; run[h].t = 0.f;
       run[h].v1 = -INFINITY; run[h].v2 = -INFINITY; run[h].i1 = -1; run[h].i2 = -1;
     }
@@ -724,10 +725,10 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
       tc_fence_after();
       const int v_warp = half_begin(LW_SUBS * t + half) + quad * 32;            // first entry of this warp
       const int v_end = half_begin(LW_SUBS * t + half + 1);
-      const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(buf * 128 + half * 64);
+      const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(buf * (2 * kRows) + half * kRows);
       if (v_warp < v_end) {
 #pragma unroll
-        for (int h = 0; h < LW_ROWS / 16; ++h) {
+        for (int h = 0; h < kRows / 16; ++h) {
           if (16 * h >= sp.N) break;
           uint32_t r[16];
           tmem_ld16(taddr + 16 * h, r);
@@ -759,9 +760,9 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     }
     // The lanes l and l + 16 and the eight warps covered different vocabulary entries: merge through the ring's
     // memory (every copy has landed and every MMA has read it: the last accumulator is complete).
-    LmColMerge* red = reinterpret_cast<LmColMerge*>(smem);          // [8 warps][64 columns]
+    LmColMerge* red = reinterpret_cast<LmColMerge*>(smem);          // [8 warps][kRows columns]
 #pragma unroll
-    for (int h = 0; h < LW_ROWS / 16; ++h) {
+    for (int h = 0; h < kRows / 16; ++h) {
       if (16 * h >= sp.N) break;
       const LmColStats q = run[h];
       LmColMerge o;
@@ -774,10 +775,10 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
       const float f = lm_weight(q.m, o.m, c), g = lm_weight(om, o.m, c);
       o.s = fmaf(q.s, f, os * g);
       o.t = kEntropy ? fmaf(q.t, f, ot * g) : 0.f;
-      if (upper == 0) red[warp * LW_ROWS + 16 * h + col] = o;
+      if (upper == 0) red[warp * kRows + 16 * h + col] = o;
     }
     asm volatile("bar.sync 2, 256;" ::: "memory");   // the eight epilogue warps
-    if (warp < 2) {
+    if (warp < kRows / 32) {
       const int column = warp * 32 + lane;
       pdl_wait();   // the partials of the previous pass may still be read until earlier kernels are done
       if (column < sp.n_rows) {
@@ -786,7 +787,7 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
         LmPartial out;
         out.m = -INFINITY; out.s = 0.f; out.t = 0.f; out.pad = 0;
 #pragma unroll
-        for (int w2 = 0; w2 < LW_EPI_WARPS; ++w2) { q[w2] = red[w2 * LW_ROWS + column]; out.m = fmaxf(out.m, q[w2].m); }
+        for (int w2 = 0; w2 < LW_EPI_WARPS; ++w2) { q[w2] = red[w2 * kRows + column]; out.m = fmaxf(out.m, q[w2].m); }
 #pragma unroll
         for (int w2 = 0; w2 < LW_EPI_WARPS; ++w2) {      // relative to the common maximum: no chain from warp to warp
           const float f = lm_weight(q[w2].m, out.m, c);
@@ -796,7 +797,7 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
         }
         out.v1 = lm_key_value(top.a); out.v2 = lm_key_value(top.b);
         out.i1 = lm_key_entry(top.a); out.i2 = lm_key_entry(top.b);
-        p.partial[static_cast<size_t>(range) * LW_ROWS + column] = out;
+        p.partial[static_cast<size_t>(range) * kRows + column] = out;
       }
     }
   }
@@ -805,7 +806,7 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
   __syncthreads();
   if (warp == LW_EPI_WARPS + 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 256);
+    tmem_dealloc(tmem_base, 4 * kRows);
   }
 }
 
@@ -814,18 +815,19 @@ void lm_reserve_sms_once(int n) { tl_lm_reserved_sms = n > 0 ? n : 0; }
 
 struct LmPlan {
   int n_seq;
-  bool few_rows;   // at most 64 rows: lmhead_rows_kernel, one CTA and one vocabulary range per SM
+  bool few_rows;   // at most 128 rows: lmhead_rows_kernel, one CTA and one vocabulary range per SM
   bool pack;       // the rows of an index list are gathered into the workspace first
   bool slots;      // (no workspace to gather into) four slots of 64 node rows per M tile
   int n_mt;        // M tiles of 256 rows
   int n_ranges;    // vocabulary ranges of the main part (few_rows: at most this many)
   int rows_ctas;   // few_rows: ranges = CTAs
+  int part_rows;   // few_rows: partial rows per range
   int n_tail;      // pairs that sweep all M tiles over a slice of the vocabulary's tail
   int main_units;  // 32-column units of the main part
   size_t required;   // workspace the call cannot do without
   size_t pack_bytes; // and what it needs on top of it to pack listed rows
   size_t partial_bytes() const {
-    return static_cast<size_t>(n_ranges + n_tail) * (few_rows ? LW_ROWS : n_mt * 2 * LM_BM) * sizeof(LmPartial);
+    return static_cast<size_t>(n_ranges + n_tail) * (few_rows ? part_rows : n_mt * 2 * LM_BM) * sizeof(LmPartial);
   }
 };
 
@@ -842,6 +844,7 @@ static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, si
   pl->few_rows = rows <= LM_FEW_ROWS && !slots;
   if (pl->few_rows) {
     pl->n_mt = 1;
+    pl->part_rows = lw_rows(rows);
     const int V16 = (a->V + 15) / 16;
     int sms = device_sm_count() - tl_lm_reserved_sms;
     if (sms < 1) sms = 1;
@@ -1022,14 +1025,17 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
       if (!cached_tmap_bf16(&tm_hn, rows_base, 3, dims, strides, box)) return TRISPEC_ERR_CUDA;
     }
     typedef void (*RowsKernel)(CUtensorMap, CUtensorMap, LmRowsParams);
-    const RowsKernel kernel = want_entropy ? lmhead_rows_kernel<true> : lmhead_rows_kernel<false>;
-    static bool smem_set_rows[2][64] = {};
-    rc = ensure_smem_limit(reinterpret_cast<const void*>(kernel), LW_SMEM_BYTES, smem_set_rows[want_entropy ? 1 : 0]);
+    static const RowsKernel table[2][2] = {{lmhead_rows_kernel<false, 64>, lmhead_rows_kernel<false, 128>},
+                                           {lmhead_rows_kernel<true, 64>, lmhead_rows_kernel<true, 128>}};
+    const int wide = pl.part_rows > 64 ? 1 : 0;
+    const RowsKernel kernel = table[want_entropy ? 1 : 0][wide];
+    static bool smem_set_rows[4][64] = {};
+    rc = ensure_smem_limit(reinterpret_cast<const void*>(kernel), LW_SMEM_BYTES, smem_set_rows[(want_entropy ? 2 : 0) + wide]);
     if (rc != TRISPEC_OK) return rc;
     TRISPEC_CUDA_OK(launch_dependent(kernel, static_cast<unsigned>(n_ranges), LW_THREADS,
                                      static_cast<size_t>(LW_SMEM_BYTES), st, 1, tm_wr, tm_hn, sp));
     count_launch();
-    f.stride = LW_ROWS;
+    f.stride = pl.part_rows;
     TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel, static_cast<unsigned>((n_rows + 7) / 8),
                                      LM_FIN_THREADS, 0, st, 1, f, n_seq));
     count_launch();

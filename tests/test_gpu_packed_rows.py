@@ -1,6 +1,6 @@
 """LM head over packed rows: the rows of all active sequences lie back to back in the M tiles of the GEMM, whatever
 the tree size; rows of an index list are gathered into the workspace, or read in slots of 64 per sequence
-where the workspace has no room for them. Sizes around the 64 rows of the small kernel and the 256 rows of an M tile."""
+where the workspace has no room for them. Sizes around the 64 and 128 rows of the small kernel and the 256 rows of an M tile."""
 import math
 
 import numpy as np
@@ -24,13 +24,16 @@ def _inputs(B, T, listed, d=192, V=3001):
 @pytest.mark.parametrize("B,T,listed", [
     (7, 9, 0),       # 63 rows: one N tile of the small kernel
     (8, 8, 0),       # 64
-    (13, 5, 0),      # 65: the pair kernel, one M tile
+    (13, 5, 0),      # 65: the same kernel with 128 columns
+    (16, 8, 0),      # 128
+    (43, 3, 0),      # 129: the pair kernel, one M tile
     (17, 15, 0),     # 255
     (32, 8, 0),      # 256
     (86, 3, 0),      # 258: a second M tile with two rows
     (40, 13, 0),     # 520: 3 M tiles, two pairs left over for the tail
     (9, 9, 3),       # 27 of 81 rows, gathered for the small kernel
-    (9, 9, 8),       # 72, gathered for the pair kernel
+    (9, 9, 8),       # 72, gathered for the small kernel
+    (20, 9, 16),     # 144, gathered for the pair kernel
     (12, 61, 9),     # 549
 ])
 @pytest.mark.parametrize("room", ["full", "slots"])
@@ -71,7 +74,8 @@ def test_lmhead_packed_rows_against_oracle(B, T, listed, room):
 @pytest.mark.parametrize("B,k,tree,L,V,d,form", [
     (1, 60, "random", 1000, 40000, 2048, None),           # two KV splits beside the LM head
     (3, 8, "chain", 500, 40000, 2048, "side_by_side"),    # three sequences, 27 rows: unsplit
-    (1, 8, "chain", 4096, 8000, 256, "lm_first"),         # the LM head ends long before such an attention: one after the other
+    (2, 60, "random", 700, 60000, 2048, "side_by_side"),  # 122 rows
+    (1, 60, "random", 4096, 120000, 2048, "lm_first"),    # 8 CTAs of 65 tiles beside it instead of 64 after it
 ])
 def test_few_row_pass_with_its_attention_beside_the_lm_head(B, k, tree, L, V, d, form):
     import torch
