@@ -7,7 +7,7 @@
 // kernel merges the per-slice partials and computes the drafted-token probabilities.
 //
 // GEMM kernel layout (two CTAs on two SMs work as a pair on one 256 x 256 tile)
-//   M tile  = 256 rows, 128 per CTA of the pair. The rows of the active sequences are packed, row = a * T + node,
+//   M tile  = up to 256 rows, up to 128 per CTA of the pair. The rows of the active sequences are packed, row = a * T + node,
 //             so that a chain of 9 nodes costs 9 rows: 64 chains of 9 nodes (128256 x 4096 weights) are 3 M tiles,
 //             where a slot of 64 rows per sequence made them 16 (2571 -> 600 us). Past the last row: zero fill.
 //   N tile  = 256 vocabulary entries, plus one narrower tile (a multiple of 32) for the rest of
@@ -58,7 +58,8 @@ struct __align__(16) LmPartial {
 struct LmParams {
   int T, d, V;
   int n_seq;      // active sequences
-  int n_mt;       // M tiles of 256 packed rows (of 4 sequence slots)
+  int n_mt;       // M tiles
+  int tile_rows;  // packed rows per M tile, a multiple of 16 up to 256 (4 sequence slots: 256)
   int slots;      // rows are not packed: an M tile is 4 slots of 64 node rows, read through seq_index
   int wait_rows;  // the packed rows are written by the kernel before this one
   int n_ranges;   // vocabulary ranges of the main part: pair c < n_mt * n_ranges works on M tile c % n_mt, range c / n_mt
@@ -179,6 +180,14 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
     for (int i = 0; i < 2; ++i) { mbar_init(tmem_full + i, 1); mbar_init(tmem_empty + i, 8); }
     fence_mbar_init();
   }
+  // Operand rows that no copy writes are zero: nobody reads what comes of them, but multiplying stale data costs power,
+  // and with it clock (16 sequences of 49 nodes, 104 of 128 rows fetched: 1010 us a pass against 985).
+  {
+    const int words = (LM_BM - (p.tile_rows >> 1)) * 8;          // 16-byte words per stage
+    for (int i = threadIdx.x; i < LM_STAGES * words; i += LM_THREADS)
+      *reinterpret_cast<uint4*>(smem + (i / words) * LM_STAGE_BYTES + (p.tile_rows >> 1) * 128 + (i % words) * 16) = make_uint4(0, 0, 0, 0);
+    fence_async_smem();
+  }
   if (warp == 5) {
     tmem_alloc_pair(tmem_slot, 512);
     tmem_relinquish_pair();
@@ -196,7 +205,9 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
       uint32_t phase = 0;
       if (p.wait_rows) pdl_wait();
       for (int sweep = 0; sweep < work.n_sweeps; ++sweep) {
-      const int row0 = (work.mt0 + sweep) * (2 * LM_BM) + static_cast<int>(rank) * LM_BM;
+      // the rows are spread evenly over the M tiles, and only those that a tile has are fetched
+      const int half_rows = p.tile_rows >> 1;
+      const int row0 = (work.mt0 + sweep) * p.tile_rows + static_cast<int>(rank) * half_rows;
       int s0 = 0, s1 = 0;
       if (p.slots) {
         // sequence slots of this CTA; a slot past the last active sequence re-reads the M tile's
@@ -215,7 +226,7 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
         const int nh = nw >> 1;                   // rows of W this CTA stages
         const int nbox = (nh + 63) >> 6;
         const int w0 = n0 + static_cast<int>(rank) * nh;
-        const uint32_t tx_pair = 2u * static_cast<uint32_t>(2 + nbox) * LM_BOX_BYTES;
+        const uint32_t tx_pair = 2u * static_cast<uint32_t>(half_rows + 64 * nbox) * (LM_BK * 2);
         for (int kb = 0; kb < n_kb; ++kb) {
           mbar_wait(empty_bar + stage, phase ^ 1u, p.dev_status);
           uint8_t* sa = smem + stage * LM_STAGE_BYTES;
@@ -271,6 +282,7 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
   } else {
     // ------------------------------------------------------------------ epilogue (warps 0-3)
     const int row = warp * 32 + lane;  // TMEM lane == row of this CTA's half of the M tile
+    const bool no_rows = warp * 32 >= (p.tile_rows >> 1);
     const float c = p.c;
     const uint32_t tmem_empty_leader = cluster_map(smem_u32(tmem_empty), 0);
     for (int sweep = 0; sweep < work.n_sweeps; ++sweep) {
@@ -283,7 +295,7 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
       const int buf = tt & 1;
       mbar_wait(tmem_full + buf, (tt >> 1) & 1u, p.dev_status);
       tc_fence_after();
-      const int ncols = min(nw, p.V - n0);  // valid columns of this tile
+      const int ncols = no_rows ? 0 : min(nw, p.V - n0);  // valid columns of this tile
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(warp * 32) << 16) + static_cast<uint32_t>(buf * LM_BN);
       for (int c0 = 0; c0 < ncols; c0 += 32) {
         uint32_t r[32];
@@ -361,7 +373,8 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
     if (sweep == 0) pdl_wait();   // the partials of the previous pass may still be read until earlier kernels are done
     LmPartial out;
     out.m = m; out.s = s; out.v1 = v1; out.v2 = v2; out.i1 = i1; out.i2 = i2; out.t = tz; out.pad = 0;
-    p.partial[static_cast<size_t>(work.part) * (p.n_mt * 2 * LM_BM) + ((work.mt0 + sweep) * 2 + rank) * LM_BM + row] = out;
+    if (row < (p.tile_rows >> 1))
+      p.partial[static_cast<size_t>(work.part) * (p.n_mt * 2 * LM_BM) + ((work.mt0 + sweep) * 2 + rank) * (p.tile_rows >> 1) + row] = out;
     }   // sweeps
   }
 
@@ -977,6 +990,7 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   p.n_seq = n_seq; p.n_mt = pl.n_mt; p.n_ranges = n_ranges;
   p.n_tail = pl.n_tail; p.main_units = pl.main_units;
   p.slots = pl.slots ? 1 : 0;
+  p.tile_rows = pl.slots ? 2 * LM_BM : static_cast<int>(((n_rows + pl.n_mt - 1) / pl.n_mt + 15) / 16 * 16);
   p.wait_rows = pl.pack ? 1 : 0;
   p.c = f.c;
   p.seq_index = a->seq_index;
@@ -1050,7 +1064,7 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   } else {
     const uint64_t dims[2] = {static_cast<uint64_t>(a->d), static_cast<uint64_t>(n_rows)};
     const uint64_t strides[1] = {static_cast<uint64_t>(a->d) * 2};
-    const uint32_t box[2] = {LM_BK, LM_BM};
+    const uint32_t box[2] = {LM_BK, static_cast<uint32_t>(p.tile_rows / 2)};
     if (!cached_tmap_bf16(&tm_h, rows_base, 2, dims, strides, box)) return TRISPEC_ERR_CUDA;
   }
   {
