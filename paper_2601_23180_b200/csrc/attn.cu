@@ -593,21 +593,37 @@ verify_attn_merge_kernel(const AttnMergeParams p) {
   const int tiles_per_split = max(1, (n_ctx_tiles + p.n_splits - 1) / p.n_splits);
   const int n_valid = max(0, (n_ctx_tiles + tiles_per_split - 1) / tiles_per_split - 1) + 1;
   const size_t item0 = ((static_cast<size_t>(a) * p.Hkv + g) * p.n_mt + mtile) * p.n_splits;
-  float M = -INFINITY;
-  for (int s = 0; s < n_valid; ++s) {
-    const size_t item = item0 + static_cast<size_t>(s);
-    M = fmaxf(M, __ldg(p.part_ml + (item * AT_BM + row) * 2));
-  }
-  float Lsum = 0.f;
+  // Bound by the latency of the partials in L2: four splits' loads go out together, then they are folded (before, a pass
+  // for the maximum and one for the sums, each load behind the last).
+  float M = -INFINITY, Lsum = 0.f;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int s = 0; s < n_valid; ++s) {
-    const size_t item = item0 + static_cast<size_t>(s);
-    const float2 ml = __ldg(reinterpret_cast<const float2*>(p.part_ml + (item * AT_BM + row) * 2));
-    const float wgt = (ml.x == -INFINITY) ? 0.f : ex2f(ml.x - M);
-    Lsum += ml.y * wgt;
-    const float4 v = __ldg(reinterpret_cast<const float4*>(p.part_o + (item * AT_BM + row) * AT_D) + lane);
-    acc.x = fmaf(v.x, wgt, acc.x); acc.y = fmaf(v.y, wgt, acc.y);
-    acc.z = fmaf(v.z, wgt, acc.z); acc.w = fmaf(v.w, wgt, acc.w);
+  for (int s0 = 0; s0 < n_valid; s0 += 4) {
+    float2 ml[4];
+    float4 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      ml[k] = make_float2(-INFINITY, 0.f);
+      v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (s0 + k < n_valid) {
+        const size_t item = item0 + static_cast<size_t>(s0 + k);
+        ml[k] = __ldg(reinterpret_cast<const float2*>(p.part_ml + (item * AT_BM + row) * 2));
+        v[k] = __ldg(reinterpret_cast<const float4*>(p.part_o + (item * AT_BM + row) * AT_D) + lane);
+      }
+    }
+    float Mn = M;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Mn = fmaxf(Mn, ml[k].x);
+    const float keep = (M == -INFINITY) ? 0.f : ex2f(M - Mn);
+    Lsum *= keep;
+    acc.x *= keep; acc.y *= keep; acc.z *= keep; acc.w *= keep;
+    M = Mn;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float wgt = (ml[k].x == -INFINITY) ? 0.f : ex2f(ml[k].x - M);
+      Lsum = fmaf(ml[k].y, wgt, Lsum);
+      acc.x = fmaf(v[k].x, wgt, acc.x); acc.y = fmaf(v[k].y, wgt, acc.y);
+      acc.z = fmaf(v[k].z, wgt, acc.z); acc.w = fmaf(v[k].w, wgt, acc.w);
+    }
   }
   const float inv = 1.f / Lsum;
   uint2 out;
