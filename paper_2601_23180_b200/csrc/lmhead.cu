@@ -363,7 +363,11 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
         if (cmax > v2) {
           const int col0 = n0 + c0;
 #pragma unroll
-          for (int j = 0; j < 32; ++j) lm_scan2(__uint_as_float(r[j]), col0 + j, v1, i1, v2, i2);
+          for (int j = 0; j < 32; ++j) {           // (one row's 32 entries rarely change anything: branches are cheaper)
+            const float v = __uint_as_float(r[j]);
+            if (v > v1) { v2 = v1; i2 = i1; v1 = v; i1 = col0 + j; }
+            else if (v > v2) { v2 = v; i2 = col0 + j; }
+          }
         }
       }
       tc_fence_before();
@@ -577,7 +581,8 @@ constexpr int LW_RING_BYTES = LW_SMEM_BYTES - 1024 /*alignment slack*/ - LW_EPI_
 
 struct LmRowsParams {
   LmParams base;
-  int n_rows, N;    // rows, and the same rounded up to 16
+  int n_rows, N;    // columns that are rows, and the same rounded up to 16
+  int slot_rows;    // > 0: not packed rows but slots of this many (a multiple of 8) per sequence of the index list
   int wait_rows;    // the rows are written by the kernel before this one
   int n_tiles;      // tiles per vocabulary range
   int box_rows;     // W rows per copy: the height of half a tile
@@ -675,9 +680,10 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     if (lane == 0) {   // ---------------------------------------------------------- TMA producer
       int stage = 0;
       uint32_t phase = 0;
-      const int seq = p.seq_index ? __ldg(p.seq_index) : 0;     // one active sequence of several; else packed rows
+      const int n_slots = sp.slot_rows > 0 ? p.n_seq : 1;      // one box per slot; packed rows are one box
+      const int slot_bytes = sp.slot_rows * (LW_BK * 2);
       if (sp.wait_rows) pdl_wait();
-      const uint32_t tx = static_cast<uint32_t>(LW_SUBS * sp.box_rows + sp.N) * (LW_BK * 2);
+      const uint32_t tx = static_cast<uint32_t>(LW_SUBS * sp.box_rows + (sp.slot_rows > 0 ? sp.n_rows : sp.N)) * (LW_BK * 2);
       for (int t = 0; t < n_tiles; ++t) {
         const int w0 = half_begin(LW_SUBS * t), w1 = half_begin(LW_SUBS * t + 1);
         for (int kb = 0; kb < n_kb; ++kb) {
@@ -686,7 +692,9 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
           mbar_expect_tx(full_bar + stage, tx);     // a box always delivers its full size (rows past V: zero fill)
           tma_load_2d(sa, &tmap_w, full_bar + stage, kb * LW_BK, w0);
           tma_load_2d(sa + LW_A_BYTES / 2, &tmap_w, full_bar + stage, kb * LW_BK, w1);
-          tma_load_3d(sa + LW_A_BYTES, &tmap_h, full_bar + stage, kb * LW_BK, 0, seq);   // rows past the last: zero fill
+          for (int a = 0; a < n_slots; ++a)       // rows past the last: zero fill
+            tma_load_3d(sa + LW_A_BYTES + a * slot_bytes, &tmap_h, full_bar + stage, kb * LW_BK, 0,
+                        p.seq_index ? __ldg(p.seq_index + a) : 0);
           if (++stage == sp.stages) { stage = 0; phase ^= 1u; }
         }
       }
@@ -831,6 +839,7 @@ struct LmPlan {
   bool few_rows;   // at most 128 rows: lmhead_rows_kernel, one CTA and one vocabulary range per SM
   bool pack;       // the rows of an index list are gathered into the workspace first
   bool slots;      // (no workspace to gather into) four slots of 64 node rows per M tile
+  int slot_rows;   // few_rows and an index list of several: columns per sequence, read without gathering; 0 = packed
   int n_mt;        // M tiles of 256 rows
   int n_ranges;    // vocabulary ranges of the main part (few_rows: at most this many)
   int rows_ctas;   // few_rows: ranges = CTAs
@@ -844,6 +853,9 @@ struct LmPlan {
   }
 };
 
+// W is streamed from HBM for long enough (about twice L2) that what happens before and after it matters less
+static bool lm_long_stream(const trispec_lmhead_args* a) { return static_cast<long long>(a->V) * a->d * 2 >= (256ll << 20); }
+
 // Plans the launch for rows that are packed, or that sit in slots of 64 per sequence. `max_ws` bounds the partial
 // array: tail pairs, which cost a block of partial rows for every M tile each, are given up until it fits.
 static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, size_t max_ws, LmPlan* pl) {
@@ -854,7 +866,11 @@ static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, si
   pl->pack_bytes = 0;
   pl->n_tail = 0;
   pl->main_units = (a->V + 31) / 32;
-  pl->few_rows = rows <= LM_FEW_ROWS && !slots;
+  // From 65 rows on the small-row kernel's last tile, which nothing overlaps, costs more than the pair kernel's (7 us
+  // at 128 columns): it pays once the stream of W is long (112 rows, 225 MB of W 86 -> 95 us a pass; 72 rows, 622 MB
+  // 142 -> 123 us).
+  pl->few_rows = rows <= (lm_long_stream(a) ? LM_FEW_ROWS : 64) && !slots;
+  pl->slot_rows = 0;
   if (pl->few_rows) {
     pl->n_mt = 1;
     pl->part_rows = lw_rows(rows);
@@ -923,8 +939,20 @@ static int lm_plan(const trispec_lmhead_args* a, LmPlan* pl, size_t room, size_t
   lm_plan_rows(a, n_seq, true, max_ws, &slots);
   if (slots.partial_bytes() > pl->required) pl->required = slots.partial_bytes();
   if (!a->seq_index) return TRISPEC_OK;
+  // A few listed sequences whose rows, rounded up to 8 each, still are at most 128 columns: one copy per sequence and
+  // stage instead of a gather, whose launch would come before the stream of W can start (3 of 5 sequences of 23
+  // nodes, 50257 x 2048 weights: 93.5 us with the gather, 87.5 us in slots of 64 in the pair kernel).
+  const int slot_rows = (a->T + 7) / 8 * 8;
+  if (pl->few_rows && n_seq <= 8 && n_seq * slot_rows <= LM_FEW_ROWS) {
+    pl->slot_rows = slot_rows;
+    pl->part_rows = lw_rows(static_cast<long long>(n_seq) * slot_rows);
+    if (pl->partial_bytes() > pl->required) pl->required = pl->partial_bytes();
+    return TRISPEC_OK;
+  }
   const size_t pack_bytes = static_cast<size_t>(n_seq) * a->T * a->d * 2;
-  if (room >= pl->required && room - pl->required >= pack_bytes) {
+  // The gather is a launch before the stream of W: not for a short stream that it does not make any shorter.
+  const bool worth = pl->few_rows || lm_long_stream(a) || pl->n_mt < slots.n_mt;
+  if (worth && room >= pl->required && room - pl->required >= pack_bytes) {
     pl->pack = true;
     pl->pack_bytes = pack_bytes;
   } else {
@@ -983,7 +1011,7 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   f.W = static_cast<const uint16_t*>(a->W);
   f.parent = a->parent; f.tok = a->tok;
   f.out = a->out;
-  f.pitch = pl.slots ? 64 : a->T;
+  f.pitch = pl.slots ? 64 : (pl.slot_rows > 0 ? pl.slot_rows : a->T);
 
   LmParams p;
   p.T = a->T; p.d = a->d; p.V = a->V;
@@ -1009,7 +1037,8 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
     LmRowsParams sp;
     sp.base = p;
     if (pl.pack) sp.base.seq_index = nullptr;
-    sp.n_rows = static_cast<int>(n_rows);
+    sp.slot_rows = pl.slot_rows;
+    sp.n_rows = pl.slot_rows > 0 ? n_seq * pl.slot_rows : static_cast<int>(n_rows);
     sp.wait_rows = p.wait_rows;
     sp.N = ((sp.n_rows + 15) / 16) * 16;
     sp.stage_bytes = LW_A_BYTES + sp.N * LW_BK * 2;
@@ -1030,12 +1059,12 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
       if (!cached_tmap_bf16(&tm_wr, a->W, 2, dims, strides, box)) return TRISPEC_ERR_CUDA;
     }
     {
-      // one active sequence of several: its nodes; otherwise all rows, back to back
-      const bool one = sp.base.seq_index != nullptr;
-      const uint64_t n = static_cast<uint64_t>(n_rows);
-      const uint64_t dims[3] = {static_cast<uint64_t>(a->d), n, one ? static_cast<uint64_t>(a->B) : 1};
+      // listed sequences: their nodes, one box each; otherwise all rows, back to back
+      const bool listed = sp.base.seq_index != nullptr;
+      const uint64_t n = listed ? static_cast<uint64_t>(a->T) : static_cast<uint64_t>(n_rows);
+      const uint64_t dims[3] = {static_cast<uint64_t>(a->d), n, listed ? static_cast<uint64_t>(a->B) : 1};
       const uint64_t strides[2] = {static_cast<uint64_t>(a->d) * 2, static_cast<uint64_t>(a->d) * 2 * n};
-      const uint32_t box[3] = {LW_BK, static_cast<uint32_t>(sp.N), 1};
+      const uint32_t box[3] = {LW_BK, static_cast<uint32_t>(pl.slot_rows > 0 ? pl.slot_rows : sp.N), 1};
       if (!cached_tmap_bf16(&tm_hn, rows_base, 3, dims, strides, box)) return TRISPEC_ERR_CUDA;
     }
     typedef void (*RowsKernel)(CUtensorMap, CUtensorMap, LmRowsParams);

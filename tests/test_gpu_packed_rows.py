@@ -24,15 +24,17 @@ def _inputs(B, T, listed, d=192, V=3001):
 @pytest.mark.parametrize("B,T,listed", [
     (7, 9, 0),       # 63 rows: one N tile of the small kernel
     (8, 8, 0),       # 64
-    (13, 5, 0),      # 65: the same kernel with 128 columns
+    (13, 5, 0),      # 65: the pair kernel, one M tile
     (16, 8, 0),      # 128
-    (43, 3, 0),      # 129: the pair kernel, one M tile
+    (43, 3, 0),      # 129
     (17, 15, 0),     # 255
     (32, 8, 0),      # 256
     (86, 3, 0),      # 258: a second M tile with two rows
     (40, 13, 0),     # 520: 3 M tiles, two pairs left over for the tail
-    (9, 9, 3),       # 27 of 81 rows, gathered for the small kernel
-    (9, 9, 8),       # 72, gathered for the small kernel
+    (9, 9, 3),       # 27 of 81 rows: the small kernel, three slots of 16 columns
+    (9, 16, 8),      # 128, gathered for the pair kernel
+    (9, 17, 6),      # 102
+    (20, 8, 9),      # 72: more than eight sequences, gathered
     (20, 9, 16),     # 144, gathered for the pair kernel
     (12, 61, 9),     # 549
 ])
@@ -49,10 +51,17 @@ def test_lmhead_packed_rows_against_oracle(B, T, listed, room):
     a = ts.lmhead_args(dev["h"], dev["W"], dev["parent"], dev["tok"], cfg.logit_scale, st, seq_index=dev["seq_index"],
                        dev_status=status)
     need = ts.trispec_lmhead_stats_workspace(a)
+    # Rows of a list are gathered where that saves M tiles, or (small kernel) where they do not fit its columns in slots
+    # of a multiple of 8 for at most eight sequences.
+    rows = listed * T
+    gather = rows > 0 and ((rows + 255) // 256 < (listed + 3) // 4 if rows > 64
+                           else listed > 8 or listed * ((T + 7) // 8 * 8) > 128)
+    gathered = rows * cfg.d * 2 if gather else 0
+    in_place = not gather
     if room == "slots":
-        if not listed:
-            pytest.skip("rows without a list are packed as they are")
-        need -= listed * T * cfg.d * 2     # what the gathered rows take
+        if in_place:
+            pytest.skip("nothing to gather")
+        need -= gathered
     ws = ts.alloc_workspace(need)
     a.workspace, a.workspace_bytes = ws.data_ptr(), need
     ts.trispec_lmhead_stats(a)
@@ -64,17 +73,63 @@ def test_lmhead_packed_rows_against_oracle(B, T, listed, room):
     assert n_tie <= 0.02 * len(seqs) * T + 2
     for b in set(range(B)) - set(seqs):
         assert np.isnan(got["lse"][b]).all() and (got["top1_idx"][b] == -1).all()
-    a.workspace_bytes = need - listed * T * cfg.d * 2 - 1 if room == "full" else need - 1
+    a.workspace_bytes = need - gathered - 1 if room == "full" else need - 1
     n0 = ts.launch_count()
     with pytest.raises(ts.TrispecError) as e:
         ts.trispec_lmhead_stats(a)
     assert e.value.code == 3 and ts.launch_count() == n0
 
 
+@pytest.mark.parametrize("B,T,listed", [
+    (13, 5, 0),      # 65 rows
+    (16, 8, 0),      # 128
+    (9, 25, 3),      # three slots of 32 columns
+    (10, 9, 9),      # 81, gathered
+])
+def test_lmhead_of_up_to_128_rows_over_a_long_stream_of_weights(B, T, listed):
+    """65 to 128 rows take the small kernel only where the weights are 256 MiB or more; an odd vocabulary."""
+    import torch
+    from paper_2601_23180_b200 import binding as ts
+    d, V, scale = 896, 150001, 3.0
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B)
+    W = torch.randn(V, d, generator=g, device="cuda", dtype=torch.bfloat16).mul_(0.02)
+    h = torch.randn(B, T, d, generator=g, device="cuda", dtype=torch.bfloat16)
+    parent = torch.arange(-1, T - 1, dtype=torch.int32, device="cuda").repeat(B, 1).contiguous()
+    tok = torch.randint(0, V, (B, T), generator=g, device="cuda", dtype=torch.int32)
+    seqs = list(range(B)) if not listed else [(3 * i + 1) % B for i in range(listed)]
+    index = torch.tensor(seqs, dtype=torch.int32, device="cuda") if listed else None
+    st = ts.alloc_stats(B, T, entropy=True)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    a = ts.lmhead_args(h, W, parent, tok, scale, st, seq_index=index, dev_status=status)
+    ws = ts.alloc_workspace(ts.trispec_lmhead_stats_workspace(a))
+    a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+    ts.trispec_lmhead_stats(a)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    W64 = W.double()
+    for b in seqs:
+        z = scale * (h[b].double() @ W64.T)
+        lse = torch.logsumexp(z, 1)
+        top = torch.topk(z, 3, dim=1)
+        # fp32 accumulation over d = 896 and 150001 exponentials: about 1e-6 of values of about 13
+        assert (st["lse"][b].double() - lse).abs().max().item() < 1e-4
+        assert (st["top1_val"][b].double() - top.values[:, 0]).abs().max().item() < 1e-4
+        assert (st["top2_val"][b].double() - top.values[:, 1]).abs().max().item() < 1e-4
+        p = torch.softmax(z, 1)
+        assert (st["entropy"][b].double() + (p * torch.log(p)).sum(1)).abs().max().item() < 1e-3
+        clear = top.values[:, 0] - top.values[:, 1] > 1e-4
+        assert torch.equal(st["top1_idx"][b][clear].long(), top.indices[:, 0][clear])
+        clear &= top.values[:, 1] - top.values[:, 2] > 1e-4
+        assert torch.equal(st["top2_idx"][b][clear].long(), top.indices[:, 1][clear])
+        want = torch.stack([z[n - 1, tok[b, n].long()] for n in range(1, T)])
+        assert (st["draft_logit"][b, 1:].double() - want).abs().max().item() < 1e-4
+
+
 @pytest.mark.parametrize("B,k,tree,L,V,d,form", [
     (1, 60, "random", 1000, 40000, 2048, None),           # two KV splits beside the LM head
     (3, 8, "chain", 500, 40000, 2048, "side_by_side"),    # three sequences, 27 rows: unsplit
-    (2, 60, "random", 700, 60000, 2048, "side_by_side"),  # 122 rows
+    (2, 60, "random", 700, 70000, 2048, "side_by_side"),  # 122 rows
     (1, 60, "random", 4096, 120000, 2048, "lm_first"),    # 8 CTAs of 65 tiles beside it instead of 64 after it
 ])
 def test_few_row_pass_with_its_attention_beside_the_lm_head(B, k, tree, L, V, d, form):
