@@ -365,7 +365,7 @@ int trispec_sample_bonus(const trispec_sample_args* a, void* stream);
  * Fused pass: the four calls above on `stream` (one verification round of Algorithm 1 for
  * one verifier): tree mask first, acceptance scan last; the attention and the LM-head
  * statistics, which do not read each other's results, in the order the library finds faster
- * for the shape. `attn` may be NULL to skip attention. For at most 128 active rows whose attention
+ * for the shape. `attn` may be NULL to skip attention. For at most 64 active rows (128 from 256 MiB of W on) whose attention
  * can do with few CTAs the library runs mask + attention on an internal second stream beside the LM head and
  * the scan, and `stream` waits for that stream before the call returns its place in the queue:
  * what the caller sees is unchanged (everything the call enqueues has completed before anything
@@ -377,11 +377,11 @@ int trispec_verify(const trispec_tree_args* tree, const trispec_attn_args* attn,
                    const trispec_lmhead_args* lm, const trispec_scan_args* scan, void* stream);
 /* How a pass with these arguments arranges its attention and its LM head (a diagnostic; host only,
  * nothing is launched; `attn` and `scan` may be NULL): "attention_first" (batches), "lm_first" or
- * "side_by_side" (at most 128 active rows: the second-stream form described above where the LM head can
+ * "side_by_side" (at most 64 active rows (128 from 256 MiB of W on): the second-stream form described above where the LM head can
  * spare the attention's SMs). "lm_first" (one active sequence whose attention is planned for more SMs than that)
  * starts the LM head at once and runs the attention in fewer CTAs beside it, on the second stream as well, where it then
  * still ends before the LM head, and after it otherwise; "none" without `lm`. The environment variable
- * TRISPEC_PASS_FORM = attention_first | lm_first | side_by_side overrides the choice for at most 128 active rows. */
+ * TRISPEC_PASS_FORM = attention_first | lm_first | side_by_side overrides the choice for at most 64 active rows (128 from 256 MiB of W on). */
 const char* trispec_verify_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm,
                                 const trispec_scan_args* scan);
 

@@ -99,8 +99,9 @@ int attn_planned_ctas(const trispec_attn_args* a);
 int attn_compact_splits(const trispec_attn_args* a, double budget_us, double tile_us, double fixed_us, int max_ctas, int* ctas);
 // KV splits of the next attention launch from this thread (0 = the planner's choice)
 void attn_splits_once(int splits);
-// rows up to which the LM head takes its small-row kernel
+// columns of the LM head's small-row kernel, and whether so many active rows take it (from 65 on only with a long W)
 constexpr int LM_FEW_ROWS = 128;
+bool lm_takes_few_rows(const trispec_lmhead_args* a, long long rows);
 
 #define TRISPEC_CUDA_OK(expr)                        \
   do {                                               \

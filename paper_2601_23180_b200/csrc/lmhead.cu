@@ -558,7 +558,7 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
 }
 
 // ---------------------------------------------------------------------------------------
-// At most 128 rows (batch-1 decoding, the paper's own setting; two trees; a batch of chains): operands swapped. With so
+// At most 64 rows, and at most 128 over a long W (batch-1 decoding, the paper's own setting; two trees; a batch of chains): operands swapped. With so
 // few rows the GEMM is bound by streaming W, and the pair kernel above spends half of its ring
 // on H tiles. Here W is the M-side operand, the rows are the N side (16-128 columns), and one CTA per SM takes one
 // vocabulary range. A tile is up to 2 x 128 vocabulary entries, two MMAs that share the k-block of H: a stage is
@@ -856,6 +856,8 @@ struct LmPlan {
 // W is streamed from HBM for long enough (about twice L2) that what happens before and after it matters less
 static bool lm_long_stream(const trispec_lmhead_args* a) { return static_cast<long long>(a->V) * a->d * 2 >= (256ll << 20); }
 
+bool lm_takes_few_rows(const trispec_lmhead_args* a, long long rows) { return rows <= (lm_long_stream(a) ? LM_FEW_ROWS : 64); }
+
 // Plans the launch for rows that are packed, or that sit in slots of 64 per sequence. `max_ws` bounds the partial
 // array: tail pairs, which cost a block of partial rows for every M tile each, are given up until it fits.
 static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, size_t max_ws, LmPlan* pl) {
@@ -869,7 +871,7 @@ static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, si
   // From 65 rows on the small-row kernel's last tile, which nothing overlaps, costs more than the pair kernel's (7 us
   // at 128 columns): it pays once the stream of W is long (112 rows, 225 MB of W 86 -> 95 us a pass; 72 rows, 622 MB
   // 142 -> 123 us).
-  pl->few_rows = rows <= (lm_long_stream(a) ? LM_FEW_ROWS : 64) && !slots;
+  pl->few_rows = lm_takes_few_rows(a, rows) && !slots;
   pl->slot_rows = 0;
   if (pl->few_rows) {
     pl->n_mt = 1;

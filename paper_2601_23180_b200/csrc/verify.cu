@@ -56,12 +56,13 @@ static PassPlan pass_plan(const trispec_attn_args* attn, const trispec_lmhead_ar
                           bool compact = true) {
   PassPlan pl = {PASS_ATTENTION_FIRST, false, attn ? attn_planned_ctas(attn) : 0, 0};
   const int lm_seqs = lm->seq_index ? lm->B_active : lm->B;
-  if (!attn || pl.attn_ctas <= 0 || lm_seqs <= 0 || static_cast<long long>(lm_seqs) * lm->T > LM_FEW_ROWS) return pl;
+  if (!attn || pl.attn_ctas <= 0 || lm_seqs <= 0) return pl;
+  if (!lm_takes_few_rows(lm, static_cast<long long>(lm_seqs) * lm->T)) return pl;      // the pair kernel takes every SM
   const int sms = device_sm_count();
   // not beside the scan when its escalation list is written over the index list the attention reads:
   // in stream order the scan comes last, side by side it would not
   const bool in_place_list = attn->seq_index && scan && scan->esc_index == attn->seq_index;
-  // TRISPEC_PASS_FORM = attention_first | lm_first | side_by_side overrides the rules below for at most LM_FEW_ROWS
+  // TRISPEC_PASS_FORM = attention_first | lm_first | side_by_side overrides the rules below for so few
   // rows (a tuning and testing aid, read at every call; lm_first is then one after the other, and side by
   // side, with the attention's own plan, still needs at most SMs / 2 CTAs)
   if (const char* e = getenv("TRISPEC_PASS_FORM")) {
