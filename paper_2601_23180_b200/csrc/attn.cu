@@ -31,6 +31,13 @@
 // two P buffers (short loops: tile i waits for P V of tile i - 2 only).
 // A sequence may carry fewer than T tree nodes (a pruned tree): rows past its count are not
 // computed and M tiles past it do nothing.
+// In-turn form: one CTA takes all the splits of a (sequence, KV head, M tile) of the cluster form one after the other and
+// merges them itself, with the same arithmetic in the same order: the same bits from an eighth of the CTAs. The fused
+// pass runs it beside an LM head that streams W and can spare few SMs, see there. The CTA is alone on its SM: partials
+// (bf16, as the cluster form exchanges them) 0-3 lie in the other half of tensor memory, 4-6 in the other half of shared
+// memory, and partial 7, if there is one the last, in the K ring. It is bound by the latency of its copies, which the stream
+// of W beside it raises: one P buffer and a V ring of three (beside 151936 x 2048 weights, 65 tiles: 121 us a pass; with
+// two P buffers and a V ring of two 139).
 #include <stdlib.h>
 
 #include "attn_common.cuh"
@@ -41,16 +48,19 @@ namespace trispec {
 // it may overwrite P; with two (and a V ring of two slots instead of three, same shared memory) it
 // waits for tile i - 2, which has long completed: the variant for short tile loops, which are bound
 // by the S -> softmax -> P V chain of a CTA rather than by the bytes in flight.
-template <bool kCluster, int NP>
-__global__ void __launch_bounds__(AT_THREADS, 2)
+enum AttnMerge { MERGE_WORKSPACE = 0, MERGE_CLUSTER = 1, MERGE_IN_TURN = 2 };
+template <int kMerge, int NP>
+__global__ void __launch_bounds__(AT_THREADS, kMerge == MERGE_IN_TURN ? 1 : 2)
 verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                          const __grid_constant__ CUtensorMap tm_kt, const __grid_constant__ CUtensorMap tm_vt,
                          const AttnParams p) {
+  constexpr bool kCluster = kMerge == MERGE_CLUSTER, kInTurn = kMerge == MERGE_IN_TURN;
   pdl_launch_dependents();
   // ---- which work item: the split index varies fastest, so that in cluster mode the CTAs of
   // one cluster are the splits of one (sequence, KV head, M tile) and cluster rank == split
   int idx = blockIdx.x;
-  const int split = idx % p.n_splits; idx /= p.n_splits;
+  const int split = kInTurn ? 0 : idx % p.n_splits;
+  if (!kInTurn) idx /= p.n_splits;
   const int mtile = idx % p.n_mt; idx /= p.n_mt;
   const int g = idx % p.Hkv;
   const int a = idx / p.Hkv;
@@ -70,14 +80,18 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
   const int tiles_per_split = max(1, (n_ctx_tiles + p.n_splits - 1) / p.n_splits);
   const int last_split = max(0, (n_ctx_tiles + tiles_per_split - 1) / tiles_per_split - 1);
   const int t_begin = split * tiles_per_split;
-  const int t_end = min(n_ctx_tiles, t_begin + tiles_per_split);
-  const bool has_tree = (split == last_split);
+  const int t_end = kInTurn ? n_ctx_tiles : min(n_ctx_tiles, t_begin + tiles_per_split);
+  const bool has_tree = kInTurn || (split == last_split);
   const int n_tiles = (t_end - t_begin) + (has_tree ? 1 : 0);   // >= 1 unless this split is empty
 
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base_u32 = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (base_u32 - smem_u32(smem_raw));
-  const bool misaligned = base_u32 - smem_u32(smem_raw) > static_cast<uint32_t>(AT_SMEM_BYTES - AT_SMEM_USED);
+  // first and last tile of a split (the tree tile ends the last one)
+  auto opens_split = [&](int i) { return i == 0 || (kInTurn && i < n_ctx_tiles && i % tiles_per_split == 0); };
+  auto ends_split = [&](int i) { return i == n_tiles - 1 || (kInTurn && i + 1 < n_ctx_tiles && (i + 1) % tiles_per_split == 0); };
+  const uint32_t smem_slack = kInTurn ? AT_TURN_SMEM_BYTES - AT_TURN_SMEM_USED : AT_SMEM_BYTES - AT_SMEM_USED;
+  const bool misaligned = base_u32 - smem_u32(smem_raw) > smem_slack;
   if (misaligned && threadIdx.x == 0 && p.dev_status) atomicExch(p.dev_status, TRISPEC_ERR_SMEM_ALIGN);
   // a split past the end of this sequence's context has nothing to do; in cluster mode it
   // still takes part in the merge (with weight zero), so it may not leave early
@@ -108,6 +122,8 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
   const int sm_threads = 32 * ((n_rows + 31) >> 5);
   uint8_t* sPartO = smem;                                               // reuses the K/V ring at the end
   float2* sPartML = reinterpret_cast<float2*>(smem + AT_PART_ML_OFF);
+  uint8_t* sTurn = smem + AT_SMEM_USED_ALIGNED;                         // in turn: partials 4-6, then (m, l) of all
+  float2* sTurnML = reinterpret_cast<float2*>(sTurn + AT_TURN_SMEM_PARTS * AT_TURN_PART_BYTES);   // [8][128]
   uint32_t tmem_base = 0;
 
   if (!idle_cta) {   // uniform for the whole CTA
@@ -128,7 +144,7 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
       fence_mbar_init();
     }
     if (warp == 5) {
-      tmem_alloc(tmem_slot, AT_TMEM_COLS);
+      tmem_alloc(tmem_slot, kInTurn ? 2 * AT_TMEM_COLS : AT_TMEM_COLS);
       tmem_relinquish();
     }
     tc_fence_before();
@@ -235,12 +251,13 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
           tc_fence_after();
           const uint32_t sv = sV_u + stage * AT_TILE_BYTES;
           const uint32_t sp = sP_u + (next_pv % NP) * AT_P_BYTES;
+          const bool add = !opens_split(next_pv);
 #pragma unroll
           for (int kk = 0; kk < AT_BN / 16; ++kk) {
             const uint64_t ad = smem_desc_sw128(sp + kk * 32, 1024, 16);
             // V: MN-major, 64-dim blocks 8 KB apart (LBO), 8-key groups 1 KB apart (SBO)
             const uint64_t bd = smem_desc_sw128(sv + kk * 2048, 1024, AT_BOX_BYTES);
-            tc_mma_ss(tmem_base + AT_TM_O, ad, bd, idesc_o, (next_pv | kk) != 0);
+            tc_mma_ss(tmem_base + AT_TM_O, ad, bd, idesc_o, add || kk != 0);
           }
           tc_commit(v_empty + stage);
           tc_commit(o_bar + next_pv % NP);
@@ -285,9 +302,11 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
       mbar_arrive(q_bar);
     }
     float m_ref = -INFINITY, l = 0.f;
+    int turn = 0;                                // in turn: the split at hand
 
     for (int i = 0; i < n_tiles; ++i) {
       const bool tree = has_tree && (i == n_tiles - 1);
+      const bool opens = opens_split(i);
       mbar_wait(s_bar, i & 1u, p.dev_status);
       tc_fence_after();
       uint32_t sr[64];
@@ -337,8 +356,9 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
       // previous tile, so that the exponentials below do not wait for that MMA
       bool need = false;
       float f = 1.f;
-      if (i == 0) {
+      if (opens) {
         m_ref = tmax;
+        l = 0.f;
       } else {
         need = tmax > m_ref + kRescaleThreshold;
         if (need) { f = (m_ref == -INFINITY) ? 0.f : ex2f(m_ref - tmax); m_ref = tmax; l *= f; }
@@ -367,7 +387,7 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
         mbar_wait(o_bar + i % NP, ((i / NP) - 1) & 1u, p.dev_status);
         tc_fence_after();
       }
-      if (i > 0) {
+      if (!opens) {
         if (__any_sync(0xffffffffu, need)) {
           if (NP > 1) {   // O is stable only after the previous tile's P V
             mbar_wait(o_bar + (i - 1) % NP, ((i - 1) / NP) & 1u, p.dev_status);
@@ -403,11 +423,101 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
       fence_async_smem();
       tc_fence_before();
       mbar_arrive(p_bar + i % NP);
+      if (kInTurn && ends_split(i)) {
+        // This split's partial, normalised and rounded as the cluster form does it. The next split's first P V, which
+        // overwrites O, comes after its P, and that after these reads.
+        mbar_wait(o_bar + i % NP, (i / NP) & 1u, p.dev_status);
+        tc_fence_after();
+        const float invl = (l > 0.f) ? 1.f / l : 0.f;
+        uint8_t* part = (turn == 7 ? smem : sTurn + (turn - AT_TURN_TMEM_PARTS) * AT_TURN_PART_BYTES) + row * (AT_D * 2);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          uint32_t o0[32], o1[32], pk2[32];
+          tmem_ld32(tmem_base + lane_base + AT_TM_O + c * 64, o0);
+          tmem_ld32(tmem_base + lane_base + AT_TM_O + c * 64 + 32, o1);
+          tc_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            pk2[j] = pack_bf16(__uint_as_float(o0[2 * j]) * invl, __uint_as_float(o0[2 * j + 1]) * invl);
+            pk2[16 + j] = pack_bf16(__uint_as_float(o1[2 * j]) * invl, __uint_as_float(o1[2 * j + 1]) * invl);
+          }
+          if (turn < AT_TURN_TMEM_PARTS) {
+            tmem_st32(tmem_base + lane_base + AT_TMEM_COLS + turn * 64 + c * 32, pk2);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              *reinterpret_cast<uint4*>(part + (((c * 8 + j) ^ (row & 7)) << 4)) =
+                  make_uint4(pk2[4 * j], pk2[4 * j + 1], pk2[4 * j + 2], pk2[4 * j + 3]);
+          }
+        }
+        if (turn < AT_TURN_TMEM_PARTS) tc_wait_st();
+        sTurnML[turn * AT_BM + row] = make_float2(m_ref, l);
+        tc_fence_before();
+        ++turn;
+      }
     }
     // ---------------------------------------------------------------- epilogue
     mbar_wait(o_bar + (n_tiles - 1) % NP, ((n_tiles - 1) / NP) & 1u, p.dev_status);   // the last P V, hence all of them
     tc_fence_after();
-    if (kCluster && p.n_splits == 1) {
+    if (kInTurn) {
+      // merge of this row's partials: the arithmetic of the cluster merge below, in its order
+      pdl_wait();                                // before the first global write
+      const int hq = g * p.G + row % p.G;
+      float wgt[8];
+      float M = -INFINITY, Lsum = 0.f;
+#pragma unroll
+      for (int s = 0; s < 8; ++s)
+        if (s < turn) M = fmaxf(M, sTurnML[s * AT_BM + row].x);
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const float2 ml = s < turn ? sTurnML[s * AT_BM + row] : make_float2(-INFINITY, 0.f);
+        wgt[s] = (ml.x != -INFINITY) ? ex2f(ml.x - M) * ml.y : 0.f;
+        Lsum += wgt[s];
+      }
+      const float inv = 1.f / Lsum;
+      uint16_t* orow = p.o + ((static_cast<size_t>(b) * p.T + (row_valid ? node : 0)) * p.Hq + hq) * AT_D;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {              // 16 dims at a time
+        float acc[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) acc[j] = 0.f;
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+          if (s >= turn) break;                  // (an empty split adds nothing)
+          uint32_t w[8];
+          if (s < AT_TURN_TMEM_PARTS) {
+            tmem_ld8(tmem_base + lane_base + AT_TMEM_COLS + s * 64 + c * 8, w);
+            tc_wait_ld();
+          } else {
+            const uint8_t* part = (s == 7 ? smem : sTurn + (s - AT_TURN_TMEM_PARTS) * AT_TURN_PART_BYTES) + row * (AT_D * 2);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+              const uint4 v = *reinterpret_cast<const uint4*>(part + (((c * 2 + j) ^ (row & 7)) << 4));
+              w[4 * j] = v.x; w[4 * j + 1] = v.y; w[4 * j + 2] = v.z; w[4 * j + 3] = v.w;
+            }
+          }
+          const bool used = sTurnML[s * AT_BM + row].x != -INFINITY;   // a fully masked row's partial counts as 0
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const uint32_t x = used ? w[j] : 0u;
+            acc[2 * j] = fmaf(__uint_as_float(x << 16), wgt[s], acc[2 * j]);
+            acc[2 * j + 1] = fmaf(__uint_as_float(x & 0xffff0000u), wgt[s], acc[2 * j + 1]);
+          }
+        }
+        if (row_valid) {
+#pragma unroll
+          for (int j = 0; j < 16; j += 8) {
+            uint4 out;
+            out.x = pack_bf16(acc[j] * inv, acc[j + 1] * inv);
+            out.y = pack_bf16(acc[j + 2] * inv, acc[j + 3] * inv);
+            out.z = pack_bf16(acc[j + 4] * inv, acc[j + 5] * inv);
+            out.w = pack_bf16(acc[j + 6] * inv, acc[j + 7] * inv);
+            *reinterpret_cast<uint4*>(orow + c * 16 + j) = out;
+          }
+        }
+      }
+      if (row_valid && p.lse) p.lse[(static_cast<size_t>(b) * p.Hq + hq) * p.T + node] = (M + log2f(Lsum)) * kLn2;
+    } else if (kCluster && p.n_splits == 1) {
       // a single split is the whole result: normalise and store it straight from tensor memory
       pdl_wait();                                // before the first global write
       const float invl = (l > 0.f) ? 1.f / l : 0.f;
@@ -482,7 +592,7 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
   __syncthreads();
   if (warp == 5) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, AT_TMEM_COLS);
+    tmem_dealloc(tmem_base, kInTurn ? 2 * AT_TMEM_COLS : AT_TMEM_COLS);
   }
   }   // !idle_cta
 
@@ -652,8 +762,8 @@ static int attn_plan_override() {
   return 0;
 }
 
-static thread_local int tl_attn_splits = 0;
-void attn_splits_once(int splits) { tl_attn_splits = splits; }
+static thread_local bool tl_attn_in_turn = false;
+void attn_in_turn_once(bool on) { tl_attn_in_turn = on; }
 
 static int attn_plan(const trispec_attn_args* a, AttnPlan* pl) {
   if (!a || a->B <= 0 || a->T <= 0 || a->Hq <= 0 || a->Hkv <= 0) return TRISPEC_ERR_INVALID_ARG;
@@ -684,14 +794,6 @@ static int attn_plan(const trispec_attn_args* a, AttnPlan* pl) {
   // for that, one wave filled as far as possible; very few (sequence, head) pairs are cut further.
   const long long slots = static_cast<long long>(device_sm_count()) * 2;   // two CTAs per SM (split kernels)
   const int tiles = pl->tiles_max;
-  if (tl_attn_splits > 0) {
-    pl->n_splits = tl_attn_splits;
-    pl->cluster = true;
-    pl->items = static_cast<size_t>(fixed) * pl->n_splits;
-    pl->pieces = false;
-    pl->n_cta = 0;
-    return TRISPEC_OK;
-  }
   int best_s = 0;
   for (int sp = 1; sp <= 8 && !best_s; ++sp)
     if (fixed * sp * 4 >= slots * 5 && tiles / sp >= 32) best_s = sp;
@@ -743,18 +845,15 @@ static int attn_plan(const trispec_attn_args* a, AttnPlan* pl) {
   return TRISPEC_OK;
 }
 
-int attn_compact_splits(const trispec_attn_args* a, double budget_us, double tile_us, double fixed_us, int max_ctas, int* ctas) {
+int attn_compact_ctas(const trispec_attn_args* a, double budget_us, int max_ctas) {
   AttnPlan pl;
-  if (attn_plan_override() || attn_plan(a, &pl) != TRISPEC_OK) return 0;
-  const long long fixed = static_cast<long long>(pl.n_seq) * a->Hkv * pl.n_mt;
-  for (int s = 1; s <= 8 && fixed * s <= max_ctas; ++s) {
-    if (s > 1 && pl.tiles_max < 4 * s) break;    // (fewer than four tiles per CTA are never worth a split)
-    if (fixed_us + tile_us * ((pl.tiles_max + s - 1) / s + 1) <= budget_us) {
-      *ctas = static_cast<int>(fixed * s);
-      return s;
-    }
-  }
-  return 0;
+  if (attn_plan(a, &pl) != TRISPEC_OK || pl.pieces || !pl.cluster) return 0;
+  const size_t ctas = pl.items / pl.n_splits;
+  if (ctas > static_cast<size_t>(max_ctas)) return 0;
+  // A CTA alone on its SM, launch included (measured: 18.5 us with 9 tiles in 2 splits, 28.7 with 17 in 4, 80.0 with 65 in 8,
+  // 137.4 with 125 in 8). The context's capacity stands for its length, which only the device knows.
+  const double us = 8.5 + 0.96 * (pl.tiles_max + 1) + 1.3 * (pl.n_splits - 1);
+  return us <= budget_us ? static_cast<int>(ctas) : 0;
 }
 
 int attn_planned_ctas(const trispec_attn_args* a) {
@@ -829,11 +928,16 @@ extern "C" int trispec_verify_attn(const trispec_attn_args* a, void* stream) {
   // (128-512) 1005 -> 1023 us, target_escalated (64) 150 -> 154 us, llama_tree (129) unchanged.
   const bool two_p = pl.pieces ? (static_cast<long long>(pl.n_seq) * a->Hkv * pl.n_mt * (pl.tiles_max + 1) / pl.n_cta <= 32)
                                : (pl.tiles_max / pl.n_splits <= 32);
+  const bool in_turn = tl_attn_in_turn && pl.cluster && !pl.pieces && pl.n_splits > 1;
   typedef void (*AttnKernel)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AttnParams);
-  const AttnKernel kernel = pl.cluster ? (two_p ? verify_attn_split_kernel<true, 2> : verify_attn_split_kernel<true, 1>)
-                                       : (two_p ? verify_attn_split_kernel<false, 2> : verify_attn_split_kernel<false, 1>);
-  static bool smem_set[4][64] = {};
-  rc = ensure_smem_limit(reinterpret_cast<const void*>(kernel), AT_SMEM_BYTES, smem_set[(pl.cluster ? 2 : 0) + (two_p ? 1 : 0)]);
+  static const AttnKernel table[5] = {verify_attn_split_kernel<MERGE_WORKSPACE, 1>, verify_attn_split_kernel<MERGE_WORKSPACE, 2>,
+                                      verify_attn_split_kernel<MERGE_CLUSTER, 1>, verify_attn_split_kernel<MERGE_CLUSTER, 2>,
+                                      verify_attn_split_kernel<MERGE_IN_TURN, 1>};
+  const int which = in_turn ? 4 : (pl.cluster ? 2 : 0) + (two_p ? 1 : 0);
+  const AttnKernel kernel = table[which];
+  const int smem_bytes = in_turn ? AT_TURN_SMEM_BYTES : AT_SMEM_BYTES;
+  static bool smem_set[5][64] = {};
+  rc = ensure_smem_limit(reinterpret_cast<const void*>(kernel), smem_bytes, smem_set[which]);
   if (rc != TRISPEC_OK) return rc;
   AttnParams p;
   p.T = a->T; p.Hq = a->Hq; p.Hkv = a->Hkv; p.G = pl.G; p.NPT = pl.NPT; p.n_mt = pl.n_mt;
@@ -855,6 +959,12 @@ extern "C" int trispec_verify_attn(const trispec_attn_args* a, void* stream) {
   if (pl.pieces) {
     const CUtensorMap maps[4] = {tm_k, tm_v, tm_kt, tm_vt};
     return attn_launch_pieces(p, maps, two_p, a->workspace, st);
+  }
+  if (in_turn) {
+    TRISPEC_CUDA_OK(launch_dependent(kernel, static_cast<unsigned>(pl.items / pl.n_splits), AT_THREADS, smem_bytes, st, 1, tm_k, tm_v,
+                                     tm_kt, tm_vt, p));
+    count_launch();
+    return TRISPEC_OK;
   }
   if (pl.cluster) {
     TRISPEC_CUDA_OK(launch_dependent(kernel, static_cast<unsigned>(pl.items), AT_THREADS,

@@ -33,6 +33,14 @@ constexpr int AT_PART_ML2_MAX = AT_BM + 2 * 8;                // n_splits x rows
 static_assert(AT_PART_ML2_OFF + AT_PART_ML2_MAX * 8 <= (AT_STAGES + 2) * AT_TILE_BYTES,
               "partial must fit in the K ring plus the shorter V ring");
 
+// in-turn form (one CTA per SM): the layout above, then the partials it keeps in shared memory and (m, l) of all eight
+constexpr int AT_TURN_TMEM_PARTS = 4, AT_TURN_SMEM_PARTS = 3;    // and the eighth in the K ring
+constexpr int AT_TURN_PART_BYTES = AT_BM * AT_D * 2;             // 16-byte words of a row XORed with row % 8
+constexpr int AT_SMEM_USED_ALIGNED = (AT_SMEM_USED + 1023) / 1024 * 1024;
+constexpr int AT_TURN_SMEM_USED = AT_SMEM_USED_ALIGNED + AT_TURN_SMEM_PARTS * AT_TURN_PART_BYTES + 8 * AT_BM * 8;
+constexpr int AT_TURN_SMEM_BYTES = AT_TURN_SMEM_USED + 1024;
+static_assert(AT_TURN_SMEM_BYTES <= 227 * 1024 && AT_TURN_PART_BYTES <= AT_STAGES * AT_TILE_BYTES, "in-turn partials");
+
 struct AttnParams {
   int T, Hq, Hkv, G, NPT, n_mt, n_splits;
   int paged, max_blocks_per_seq, num_blocks;

@@ -93,12 +93,12 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 // CTAs the attention launch for these arguments will use (0 if the arguments are not accepted)
 int attn_planned_ctas(const trispec_attn_args* a);
-// The smallest number of KV splits (1 to 8, merged on chip: no workspace) with which every CTA of the attention ends
-// within `budget_us` at `tile_us` per tile and `fixed_us` besides, in at most `max_ctas` CTAs; 0 if there is none. The
-// number of CTAs goes to `ctas` where there is one.
-int attn_compact_splits(const trispec_attn_args* a, double budget_us, double tile_us, double fixed_us, int max_ctas, int* ctas);
-// KV splits of the next attention launch from this thread (0 = the planner's choice)
-void attn_splits_once(int splits);
+// CTAs of an attention whose plan merges its splits on chip when each (sequence, KV head, M tile) has one CTA, alone on
+// its SM, that takes the splits in turn (attn.cu); 0 where the plan is another one, where that is more than `max_ctas`
+// CTAs, or where they would take longer than `budget_us`.
+int attn_compact_ctas(const trispec_attn_args* a, double budget_us, int max_ctas);
+// The attention launches of this thread take that form while this is on
+void attn_in_turn_once(bool on);
 // columns of the LM head's small-row kernel, and whether so many active rows take it (from 65 on only with a long W)
 constexpr int LM_FEW_ROWS = 128;
 bool lm_takes_few_rows(const trispec_lmhead_args* a, long long rows);

@@ -40,7 +40,7 @@ struct PassPlan {
   PassForm form;
   bool beside;        // mask and attention go to the second stream, the LM head leaves them `attn_ctas` SMs
   int attn_ctas;
-  int attn_splits;    // KV splits of that attention, 0 = what the attention's own planner takes
+  bool in_turn;       // that attention takes the splits of its plan one after the other, in few CTAs
 };
 static bool stream_is_capturing(cudaStream_t st) {
   cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
@@ -54,7 +54,7 @@ static bool stream_is_capturing(cudaStream_t st) {
 // stream is shared by every caller on the device and should not become part of more captures than it has to.
 static PassPlan pass_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm, const trispec_scan_args* scan,
                           bool compact = true) {
-  PassPlan pl = {PASS_ATTENTION_FIRST, false, attn ? attn_planned_ctas(attn) : 0, 0};
+  PassPlan pl = {PASS_ATTENTION_FIRST, false, attn ? attn_planned_ctas(attn) : 0, false};
   const int lm_seqs = lm->seq_index ? lm->B_active : lm->B;
   if (!attn || pl.attn_ctas <= 0 || lm_seqs <= 0) return pl;
   if (!lm_takes_few_rows(lm, static_cast<long long>(lm_seqs) * lm->T)) return pl;      // the pair kernel takes every SM
@@ -71,28 +71,30 @@ static PassPlan pass_plan(const trispec_attn_args* attn, const trispec_lmhead_ar
     if (e[0] == 's' && pl.attn_ctas * 2 <= sms && !in_place_list) { pl.form = PASS_SIDE_BY_SIDE; pl.beside = true; return pl; }
   }
   // With so few rows the LM head is a pure stream of W that does not need every SM to saturate HBM, and the attention
-  // a chain of tiles that does not need bandwidth: the attention runs beside the LM head in as FEW CTAs as end
-  // well before it (a CTA alone on its SM takes about 1.1 us per 64-key tile; W streams at 6 TB/s), one
-  // SM each, as long as that is at most a quarter of the chip. One sequence of 61 nodes, 4096 context tokens, 151936 x 2048
-  // weights: 8 CTAs of 65 tiles beside 140 of the LM head against 64 CTAs after all 148 of it.
+  // a chain of tiles that does not need bandwidth: the attention runs beside the LM head in as FEW CTAs as it can,
+  // one per (sequence, KV head, M tile), each taking the splits of the attention's own plan in turn (attn.cu: the same
+  // bits), where they end well before the LM head (W streams at 6 TB/s) and are at most a quarter of the chip. One
+  // sequence of 61 nodes, 4096 context tokens, 151936 x 2048 weights: 8 CTAs of 65 tiles beside 140 of the LM head
+  // against 64 CTAs after all 148 of it.
   const double lm_us = static_cast<double>(lm->V) * lm->d * 2.0 / 6.0e6;
-  const int splits = in_place_list || !compact ? 0 : attn_compact_splits(attn, 0.8 * lm_us, 1.1, 6.0, sms / 4, &pl.attn_ctas);
+  const int compact_ctas = in_place_list || !compact ? 0 : attn_compact_ctas(attn, 0.8 * lm_us, sms / 4);
   if (lm_seqs == 1) {
     // Behind the attention the LM head would stall as a programmatic dependent, so for one sequence it goes first
     // whatever the form. What the form is called follows the attention's own plan: side by side where that could
     // be given one SM per CTA for less than about 40 us of the LM head's time, which then takes SMs / (SMs - CTAs)
     // times as long.
-    const int own = attn_planned_ctas(attn);
     const double own_lm_us = lm_us * 6.0 / 5.0;
-    const bool own_fits = own * 2 <= sms && !in_place_list && own_lm_us * own <= 40.0 * (sms - own);
+    const bool own_fits = pl.attn_ctas * 2 <= sms && !in_place_list && own_lm_us * pl.attn_ctas <= 40.0 * (sms - pl.attn_ctas);
     pl.form = own_fits ? PASS_SIDE_BY_SIDE : PASS_LM_FIRST;
-    pl.beside = splits > 0 || own_fits;
-  } else if (splits > 0) {
+    pl.beside = compact_ctas > 0 || own_fits;
+  } else if (compact_ctas > 0) {
     pl.form = PASS_SIDE_BY_SIDE;
     pl.beside = true;
   }
-  pl.attn_splits = splits;
-  if (splits == 0) pl.attn_ctas = attn_planned_ctas(attn);
+  if (compact_ctas > 0) {
+    pl.attn_ctas = compact_ctas;
+    pl.in_turn = true;
+  }
   return pl;
 }
 }  // namespace trispec
@@ -138,9 +140,9 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
     TRISPEC_CUDA_OK(cudaStreamWaitEvent(hs->copy, hs->fork, 0));
     rc = trispec_build_tree_mask(tree, hs->copy);          // ordinary launch: first kernel of the call
     if (rc == TRISPEC_OK) {
-      attn_splits_once(plan.attn_splits);
+      attn_in_turn_once(plan.in_turn);
       rc = trispec_verify_attn(attn, hs->copy);            // dependent of the mask kernel
-      attn_splits_once(0);
+      attn_in_turn_once(false);
     }
     TRISPEC_CUDA_OK(cudaEventRecord(hs->copied, hs->copy));
     if (rc == TRISPEC_OK) {
@@ -245,9 +247,9 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
     TRISPEC_CUDA_OK(cudaStreamWaitEvent(hs->copy, hs->inputs, 0));   // the tree's parents have arrived
     rc = trispec_build_tree_mask(tree, hs->copy);
     if (rc == TRISPEC_OK) {
-      attn_splits_once(plan.attn_splits);
+      attn_in_turn_once(plan.in_turn);
       rc = trispec_verify_attn(attn, hs->copy);
-      attn_splits_once(0);
+      attn_in_turn_once(false);
     }
     TRISPEC_CUDA_OK(cudaEventRecord(hs->copied, hs->copy));
     if (rc == TRISPEC_OK) {
