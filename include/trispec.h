@@ -366,7 +366,7 @@ int trispec_sample_bonus(const trispec_sample_args* a, void* stream);
  * one verifier): tree mask first, acceptance scan last; the attention and the LM-head
  * statistics, which do not read each other's results, in the order the library finds faster
  * for the shape. `attn` may be NULL to skip attention. For at most 64 active rows (128 from 256 MiB of W on) whose attention
- * can do with few CTAs the library runs mask + attention on an internal second stream beside the LM head and
+ * can do with few CTAs the library runs mask + attention on a second stream of its own (one per caller's stream) beside the LM head and
  * the scan, and `stream` waits for that stream before the call returns its place in the queue:
  * what the caller sees is unchanged (everything the call enqueues has completed before anything
  * enqueued on `stream` afterwards starts), but no output buffer of the call may overlap an input
@@ -391,12 +391,13 @@ const char* trispec_verify_plan(const trispec_attn_args* attn, const trispec_lmh
  * from the host, the routing decision goes back to it). The KV cache and the LM-head weights
  * stay resident on the device. Copies the per-round inputs from the host pointers of `io`
  * into the device buffers named by the argument structs (tree->parent, lm->tok, lm->h on
- * `stream`; attn->q, attn->k_tree, attn->v_tree on a stream of the library's own, ordered
+ * `stream`; attn->q, attn->k_tree, attn->v_tree on a second stream of the library's that belongs to `stream`, ordered
  * after everything already on `stream`, so that they overlap the LM-head GEMM), runs the
  * tree mask, the LM-head statistics, the attention and the scan, then copies accept_len,
  * escalate, bonus_tok, last_node and path back to the host pointers. Seen from `stream` the
- * call is one ordered unit of work. The first call on a device creates that stream and two
- * events (host resources, kept until the process exits); no device memory is allocated.
+ * call is one ordered unit of work. The first call on a stream creates that second stream and three
+ * events (host resources; at most 16 per device are kept, until the process exits, and a pass on a further stream that
+ * finds all of them busy runs in stream order); no device memory is allocated.
  * Host pointers should be page-locked for the copies to be asynchronous; the results are
  * valid once `stream` has been synchronised. NULL host input pointers skip that copy.
  * Copies whose host AND device addresses follow each other are merged into one transfer, in

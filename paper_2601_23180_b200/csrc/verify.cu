@@ -1,36 +1,124 @@
 // Fused verify pass: tree mask -> attention -> LM-head statistics -> acceptance scan on one
 // stream (one verification round of Algorithm 1 for one verifier).
 #include <mutex>
+#include <optional>
 #include <stdlib.h>
 
 #include "host_common.h"
 
 namespace trispec {
-// Side stream and events of trispec_verify_host, one set per device, created on first use.
-struct HostPassStreams {
-  cudaStream_t copy = nullptr;
-  cudaEvent_t fork = nullptr, copied = nullptr, inputs = nullptr;
-  bool ready = false;
-  std::mutex enqueue;   // the stream and the events are shared by every caller on this device
+// Second streams (with their events) of the fused passes. A set belongs to one stream of the caller's, so that callers on
+// different streams never wait for each other's work, and a set that is part of a capture is used by that capture only.
+// Per device at most 16, made on first use and kept until the process exits; a set whose work is done is handed on to
+// another stream. A pass that finds none free runs in stream order: the same results without the overlap.
+struct SideStream {
+  cudaStream_t stream = nullptr;
+  cudaEvent_t fork = nullptr, done = nullptr, inputs = nullptr;
+  bool made = false;
+  const void* owner = nullptr;       // the caller's stream
+  unsigned long long used = 0;       // when it was taken last
+  int users = 0;                     // calls that hold it
+  std::mutex enqueue;                // callers that share the owner record and wait on its events one after the other
 };
-static int host_pass_streams(HostPassStreams** out) {
-  static HostPassStreams per_dev[64];
-  static std::mutex mu;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return TRISPEC_ERR_CUDA;
-  if (dev < 0 || dev >= 64) return TRISPEC_ERR_UNSUPPORTED;
-  std::lock_guard<std::mutex> lock(mu);
-  HostPassStreams& h = per_dev[dev];
-  if (!h.ready) {
-    if (cudaStreamCreateWithFlags(&h.copy, cudaStreamNonBlocking) != cudaSuccess) return TRISPEC_ERR_CUDA;
-    if (cudaEventCreateWithFlags(&h.fork, cudaEventDisableTiming) != cudaSuccess) return TRISPEC_ERR_CUDA;
-    if (cudaEventCreateWithFlags(&h.copied, cudaEventDisableTiming) != cudaSuccess) return TRISPEC_ERR_CUDA;
-    if (cudaEventCreateWithFlags(&h.inputs, cudaEventDisableTiming) != cudaSuccess) return TRISPEC_ERR_CUDA;
-    h.ready = true;
+constexpr int kSideStreams = 16;
+struct SidePool {
+  std::mutex mu;
+  unsigned long long clock = 0;
+  SideStream set[kSideStreams];
+};
+
+static bool side_make(SideStream* s) {
+  if (cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess) return false;
+  cudaEvent_t* const ev[3] = {&s->fork, &s->done, &s->inputs};
+  for (int i = 0; i < 3; ++i) {
+    if (cudaEventCreateWithFlags(ev[i], cudaEventDisableTiming) == cudaSuccess) continue;
+    while (i-- > 0) cudaEventDestroy(*ev[i]);
+    cudaStreamDestroy(s->stream);
+    return false;
   }
-  *out = &h;
-  return TRISPEC_OK;
+  s->made = true;
+  return true;
 }
+
+// The set for a pass on `st` while this object lives; operator-> of one without a set may not be used.
+class SideLease {
+ public:
+  explicit SideLease(cudaStream_t st) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+    // looking a stream over, and making one, must not disturb a capture of another thread's
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    take(pools()[dev], st);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (s_) s_->enqueue.lock();
+  }
+  ~SideLease() {
+    if (!s_) return;
+    s_->enqueue.unlock();
+    std::lock_guard<std::mutex> lock(pool_->mu);
+    --s_->users;
+  }
+  SideLease(const SideLease&) = delete;
+  SideLease& operator=(const SideLease&) = delete;
+  explicit operator bool() const { return s_ != nullptr; }
+  SideStream* operator->() const { return s_; }
+
+ private:
+  static SidePool* pools() {
+    static SidePool per_dev[64];
+    return per_dev;
+  }
+  // the id of the capture `st` is part of, 0 if it is in none; false where that cannot be told or the capture is broken
+  static bool capture_of(cudaStream_t st, unsigned long long* id) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    *id = 0;
+    if (cudaStreamGetCaptureInfo(st, &status, id) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (status == cudaStreamCaptureStatusNone) *id = 0;
+    return status != cudaStreamCaptureStatusInvalidated;
+  }
+  void take(SidePool& pool, cudaStream_t st) {
+    unsigned long long capture = 0, theirs = 0;
+    static thread_local char per_thread;       // (one handle stands for every thread's default stream)
+    const void* const id = st == cudaStreamPerThread ? static_cast<const void*>(&per_thread) : st;
+    if (!capture_of(st, &capture)) return;
+    std::lock_guard<std::mutex> lock(pool.mu);
+    SideStream* got = nullptr;
+    for (SideStream& s : pool.set)
+      if (s.made && s.owner == id) {
+        // (a set that an earlier capture of the owner's has not given back yet stays with it)
+        if (!capture_of(s.stream, &theirs) || (theirs != 0 && theirs != capture)) return;
+        got = &s;
+        break;
+      }
+    for (int i = 0; i < kSideStreams && !got; ++i)
+      if (!pool.set[i].made) {
+        if (!side_make(&pool.set[i])) {
+          cudaGetLastError();
+          return;
+        }
+        got = &pool.set[i];
+      }
+    if (!got) {
+      for (SideStream& s : pool.set) {
+        if (s.users > 0 || (got && got->used < s.used) || !capture_of(s.stream, &theirs) || theirs != 0) continue;
+        if (cudaStreamQuery(s.stream) == cudaSuccess) got = &s;
+        else cudaGetLastError();
+      }
+      if (!got) return;
+    }
+    got->owner = id;
+    got->used = ++pool.clock;
+    ++got->users;
+    pool_ = &pool;
+    s_ = got;
+  }
+  SidePool* pool_ = nullptr;
+  SideStream* s_ = nullptr;
+};
 }  // namespace trispec
 
 namespace trispec {
@@ -42,18 +130,7 @@ struct PassPlan {
   int attn_ctas;
   bool in_turn;       // that attention takes the splits of its plan one after the other, in few CTAs
 };
-static bool stream_is_capturing(cudaStream_t st) {
-  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return status != cudaStreamCaptureStatusNone;
-}
-// `compact`: the attention may be planned for few CTAs beside the LM head. Not while `stream` is captured: the second
-// stream is shared by every caller on the device and should not become part of more captures than it has to.
-static PassPlan pass_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm, const trispec_scan_args* scan,
-                          bool compact = true) {
+static PassPlan pass_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm, const trispec_scan_args* scan) {
   PassPlan pl = {PASS_ATTENTION_FIRST, false, attn ? attn_planned_ctas(attn) : 0, false};
   const int lm_seqs = lm->seq_index ? lm->B_active : lm->B;
   if (!attn || pl.attn_ctas <= 0 || lm_seqs <= 0) return pl;
@@ -77,7 +154,7 @@ static PassPlan pass_plan(const trispec_attn_args* attn, const trispec_lmhead_ar
   // sequence of 61 nodes, 4096 context tokens, 151936 x 2048 weights: 8 CTAs of 65 tiles beside 140 of the LM head
   // against 64 CTAs after all 148 of it.
   const double lm_us = static_cast<double>(lm->V) * lm->d * 2.0 / 6.0e6;
-  const int compact_ctas = in_place_list || !compact ? 0 : attn_compact_ctas(attn, 0.8 * lm_us, sms / 4);
+  const int compact_ctas = in_place_list ? 0 : attn_compact_ctas(attn, 0.8 * lm_us, sms / 4);
   if (lm_seqs == 1) {
     // Behind the attention the LM head would stall as a programmatic dependent, so for one sequence it goes first
     // whatever the form. What the form is called follows the attention's own plan: side by side where that could
@@ -119,9 +196,8 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
   // arrive within a microsecond of the attention's end, whenever it started). For one active sequence the
   // LM head is a pure stream of W and loses more behind an attention than the hidden latency is worth (one
   // sequence of 4096 context tokens: 166 us against 156 us the other way round), so there the LM head goes
-  // first, or the two run side by side (pass_form above).
-  const trispec::PassPlan plan =
-      trispec::pass_plan(attn, lm, scan, !trispec::stream_is_capturing(static_cast<cudaStream_t>(stream)));
+  // first, or the two run side by side (pass_plan above).
+  const trispec::PassPlan plan = trispec::pass_plan(attn, lm, scan);
   const bool lm_first = plan.form == trispec::PASS_LM_FIRST;
   int rc;
   // Few rows and an attention that fits beside the LM head (pass_plan): the two run side by
@@ -131,30 +207,29 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
   // the call enqueues is complete before anything enqueued on `stream` after it.
   if (plan.beside) {
     using namespace trispec;
-    HostPassStreams* hs = nullptr;
-    rc = host_pass_streams(&hs);
-    if (rc != TRISPEC_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    std::unique_lock<std::mutex> enqueue_lock(hs->enqueue);
-    TRISPEC_CUDA_OK(cudaEventRecord(hs->fork, st));
-    TRISPEC_CUDA_OK(cudaStreamWaitEvent(hs->copy, hs->fork, 0));
-    rc = trispec_build_tree_mask(tree, hs->copy);          // ordinary launch: first kernel of the call
-    if (rc == TRISPEC_OK) {
-      attn_in_turn_once(plan.in_turn);
-      rc = trispec_verify_attn(attn, hs->copy);            // dependent of the mask kernel
-      attn_in_turn_once(false);
+    SideLease side(st);
+    if (side) {
+      TRISPEC_CUDA_OK(cudaEventRecord(side->fork, st));
+      TRISPEC_CUDA_OK(cudaStreamWaitEvent(side->stream, side->fork, 0));
+      rc = trispec_build_tree_mask(tree, side->stream);      // ordinary launch: first kernel of the call
+      if (rc == TRISPEC_OK) {
+        attn_in_turn_once(plan.in_turn);
+        rc = trispec_verify_attn(attn, side->stream);        // dependent of the mask kernel
+        attn_in_turn_once(false);
+      }
+      TRISPEC_CUDA_OK(cudaEventRecord(side->done, side->stream));
+      if (rc == TRISPEC_OK) {
+        entry_scope_next_launch_ordinary();                  // first kernel on `stream`
+        lm_reserve_sms_once(plan.attn_ctas);
+        rc = trispec_lmhead_stats(lm, stream);
+        lm_reserve_sms_once(0);
+      }
+      if (rc == TRISPEC_OK) rc = trispec_accept_scan(scan, stream);   // dependent of the LM head's last kernel
+      // joined after an argument error too: what has been launched ends before whatever `stream` gets next
+      TRISPEC_CUDA_OK(cudaStreamWaitEvent(st, side->done, 0));
+      return rc;
     }
-    TRISPEC_CUDA_OK(cudaEventRecord(hs->copied, hs->copy));
-    if (rc == TRISPEC_OK) {
-      entry_scope_next_launch_ordinary();                  // first kernel on `stream`
-      lm_reserve_sms_once(plan.attn_ctas);
-      rc = trispec_lmhead_stats(lm, stream);
-      lm_reserve_sms_once(0);
-    }
-    if (rc == TRISPEC_OK) rc = trispec_accept_scan(scan, stream);   // dependent of the LM head's last kernel
-    // joined after an argument error too: what has been launched ends before whatever `stream` gets next
-    TRISPEC_CUDA_OK(cudaStreamWaitEvent(st, hs->copied, 0));
-    return rc;
   }
   rc = trispec_build_tree_mask(tree, stream);
   if (rc != TRISPEC_OK) return rc;
@@ -210,18 +285,12 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
     }
     return cudaSuccess;
   };
-  HostPassStreams* hs = nullptr;
-  std::unique_lock<std::mutex> enqueue_lock;
-  if (attn) {
-    int rc = host_pass_streams(&hs);
-    if (rc != TRISPEC_OK) return rc;
-    // one caller at a time records and waits on the shared events (host threads driving
-    // different streams of one device would otherwise pick up each other's records)
-    enqueue_lock = std::unique_lock<std::mutex>(hs->enqueue);
-    // the side stream may not overwrite q / k_tree / v_tree before earlier work on `stream`
-    // (a previous pass reading them) is done
-    TRISPEC_CUDA_OK(cudaEventRecord(hs->fork, st));
-  }
+  // the attention's inputs are copied on a second stream (in stream order where there is none free); it may not overwrite
+  // q / k_tree / v_tree before earlier work on `stream` (a previous pass reading them) is done
+  std::optional<SideLease> side;
+  if (attn) side.emplace(st);
+  const bool forked = side && *side;
+  if (forked) TRISPEC_CUDA_OK(cudaEventRecord((*side)->fork, st));
   // what the LM head needs goes first through the copy engine
   {
     CopyReq in[3] = {{const_cast<int32_t*>(tree->parent), io->parent, BT * 4},
@@ -229,29 +298,29 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
                      {const_cast<void*>(lm->h), io->h, BT * static_cast<size_t>(lm->d) * 2}};
     TRISPEC_CUDA_OK(copy_list(in, 3, cudaMemcpyHostToDevice, st));
   }
-  const PassPlan plan = pass_plan(attn, lm, scan, !stream_is_capturing(st));
-  const bool side_by_side = plan.beside;
-  if (side_by_side) TRISPEC_CUDA_OK(cudaEventRecord(hs->inputs, st));
+  const PassPlan plan = pass_plan(attn, lm, scan);
+  const bool side_by_side = plan.beside && forked;
+  if (side_by_side) TRISPEC_CUDA_OK(cudaEventRecord((*side)->inputs, st));
   if (attn) {
-    TRISPEC_CUDA_OK(cudaStreamWaitEvent(hs->copy, hs->fork, 0));
+    if (forked) TRISPEC_CUDA_OK(cudaStreamWaitEvent((*side)->stream, (*side)->fork, 0));
     CopyReq in[3] = {{const_cast<void*>(attn->q), io->q, BT * static_cast<size_t>(attn->Hq) * attn->D * 2},
                      {const_cast<void*>(attn->k_tree), io->k_tree, BT * static_cast<size_t>(attn->Hkv) * attn->D * 2},
                      {const_cast<void*>(attn->v_tree), io->v_tree, BT * static_cast<size_t>(attn->Hkv) * attn->D * 2}};
-    TRISPEC_CUDA_OK(copy_list(in, 3, cudaMemcpyHostToDevice, hs->copy));
-    if (!side_by_side) TRISPEC_CUDA_OK(cudaEventRecord(hs->copied, hs->copy));
+    TRISPEC_CUDA_OK(copy_list(in, 3, cudaMemcpyHostToDevice, forked ? (*side)->stream : st));
+    if (forked && !side_by_side) TRISPEC_CUDA_OK(cudaEventRecord((*side)->done, (*side)->stream));
   }
   int rc;
   if (side_by_side) {
     // few rows (as in trispec_verify): mask and attention follow their inputs on
     // the second stream, the LM head and the scan run on `stream`, which then waits for the second stream
-    TRISPEC_CUDA_OK(cudaStreamWaitEvent(hs->copy, hs->inputs, 0));   // the tree's parents have arrived
-    rc = trispec_build_tree_mask(tree, hs->copy);
+    TRISPEC_CUDA_OK(cudaStreamWaitEvent((*side)->stream, (*side)->inputs, 0));   // the tree's parents have arrived
+    rc = trispec_build_tree_mask(tree, (*side)->stream);
     if (rc == TRISPEC_OK) {
       attn_in_turn_once(plan.in_turn);
-      rc = trispec_verify_attn(attn, hs->copy);
+      rc = trispec_verify_attn(attn, (*side)->stream);
       attn_in_turn_once(false);
     }
-    TRISPEC_CUDA_OK(cudaEventRecord(hs->copied, hs->copy));
+    TRISPEC_CUDA_OK(cudaEventRecord((*side)->done, (*side)->stream));
     if (rc == TRISPEC_OK) {
       entry_scope_next_launch_ordinary();                            // first kernel on `stream`
       lm_reserve_sms_once(plan.attn_ctas);
@@ -259,7 +328,7 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
       lm_reserve_sms_once(0);
     }
     if (rc == TRISPEC_OK) rc = trispec_accept_scan(scan, stream);
-    TRISPEC_CUDA_OK(cudaStreamWaitEvent(st, hs->copied, 0));
+    TRISPEC_CUDA_OK(cudaStreamWaitEvent(st, (*side)->done, 0));
     if (rc != TRISPEC_OK) return rc;
   } else {
     rc = trispec_build_tree_mask(tree, stream);
@@ -267,7 +336,7 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
     rc = trispec_lmhead_stats(lm, stream);
     if (rc != TRISPEC_OK) return rc;
     if (attn) {
-      TRISPEC_CUDA_OK(cudaStreamWaitEvent(st, hs->copied, 0));
+      if (forked) TRISPEC_CUDA_OK(cudaStreamWaitEvent(st, (*side)->done, 0));
       rc = trispec_verify_attn(attn, stream);
       if (rc != TRISPEC_OK) return rc;
     }

@@ -1,5 +1,6 @@
 """The fused pass of few rows, whose attention runs beside the LM head in one CTA per (sequence, KV head, M tile)
-that takes the splits of the attention's own plan in turn: the same bits as the attention called by itself."""
+that takes the splits of the attention's own plan in turn: the same bits as the attention called by itself, on the
+second stream of each caller's stream, captured or not."""
 import math
 
 import pytest
@@ -81,6 +82,21 @@ class Pass:
         from paper_2601_23180_b200 import binding as ts
         ts.trispec_verify(self.tree_args, self.attn_args, self.lm_args, self.scan_args, stream)
 
+    def from_host(self, stream=None):
+        """The pass with its per-round inputs in pinned memory; the device copies are spoiled first."""
+        import torch
+        from paper_2601_23180_b200 import binding as ts
+        names = dict(parent=self.parent, tok=self.tok, h=self.h, q=self.q, k_tree=self.kt, v_tree=self.vt)
+        if not hasattr(self, "pinned"):
+            self.pinned = {n: t.cpu().pin_memory() for n, t in names.items()}
+            self.back = {n: torch.zeros(self.out[n].shape, dtype=self.out[n].dtype).pin_memory()
+                         for n in ("accept_len", "bonus_tok", "last_node", "path", "escalate")}
+            self.io = ts.host_io(**self.pinned, **self.back)
+        with torch.cuda.stream(stream):
+            for t in names.values():
+                t.zero_()
+        ts.trispec_verify_host(self.io, self.tree_args, self.attn_args, self.lm_args, self.scan_args, stream)
+
     def snapshot(self):
         import torch
         torch.cuda.synchronize()
@@ -145,3 +161,134 @@ def test_fused_pass_gives_the_attentions_own_bits(kw):
         x, y = p.o[b, :n].double(), p.attention64(b)
         # P rounded to bf16 relative to each split's maximum, partials and the result to bf16: 2^-9 each, at most
         assert (torch.linalg.norm(x - y) / torch.linalg.norm(y)).item() <= 3 * 2.0 ** -9
+
+
+CHAINS = dict(T=9, Hq=32, Hkv=8, cap=256, lens=[256, 100, 31], d=2048, V=40000)      # 27 rows, 24 CTAs
+ONE = dict(T=9, Hq=16, Hkv=8, cap=512, lens=[512], d=2048, V=32000)
+
+
+def _want(p):
+    p.spoil()
+    p.separate()
+    return p.snapshot()
+
+
+@pytest.mark.parametrize("call", ["fused", "from_host"])
+def test_a_pass_does_not_wait_for_another_callers_stream(call):
+    import torch
+    a, b = Pass(**CHAINS), Pass(**dict(CHAINS, seed=4))
+    sa, sb = torch.cuda.Stream(), torch.cuda.Stream()
+    want = [_want(a), _want(b)]
+    for p, s in ((a, sa), (b, sb)):
+        getattr(p, call)(s)
+        torch.cuda.synchronize()
+        p.spoil()
+    torch.cuda.synchronize()
+    reached = torch.cuda.Event()
+    with torch.cuda.stream(sa):
+        torch.cuda._sleep(400_000_000)             # about 0.2 s
+        reached.record()
+    getattr(a, call)(sa)
+    getattr(b, call)(sb)
+    sb.synchronize()
+    assert not reached.query()                     # b's pass is done and a's has not begun
+    got = [a.snapshot(), b.snapshot()]
+    assert_same_attention(got[0], want[0])
+    assert_same_attention(got[1], want[1])
+
+
+@pytest.mark.parametrize("kw", [CHAINS, ONE, dict(T=61, Hq=16, Hkv=8, cap=4096, lens=[4096])])
+def test_captured_pass_beside_an_eager_one(kw):
+    """A pass under capture, and between two of its calls an eager pass on another stream: neither disturbs the other."""
+    import torch
+    p, q = Pass(**kw), Pass(**dict(CHAINS, seed=4))
+    want_p, want_q = _want(p), _want(q)
+    sp, sq = torch.cuda.Stream(), torch.cuda.Stream()
+    for x, s in ((p, sp), (q, sq)):
+        x.fused(s)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    q.spoil()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=sp):
+        p.fused(sp)
+        q.fused(sq)
+        p.fused(sp)
+    assert_same_attention(q.snapshot(), want_q)
+    for _ in range(3):
+        p.spoil()
+        torch.cuda.synchronize()
+        graph.replay()
+        assert_same_attention(p.snapshot(), want_p)
+    p.spoil()
+    torch.cuda.synchronize()
+    p.fused(sp)                                    # the stream's second stream is usable again after the capture
+    assert_same_attention(p.snapshot(), want_p)
+    del graph
+
+
+def test_more_busy_streams_than_second_streams():
+    import torch
+    tiny = dict(T=9, Hq=8, Hkv=8, cap=128, lens=[100], d=64, V=3000)
+    passes = [Pass(**dict(tiny, seed=i)) for i in range(20)]
+    want = [_want(p) for p in passes]
+    for rounds in range(2):
+        for p in passes:
+            p.spoil()
+        torch.cuda.synchronize()
+        gate, opened = torch.cuda.Stream(), torch.cuda.Event()
+        with torch.cuda.stream(gate):
+            torch.cuda._sleep(20_000_000)
+            opened.record()
+        streams = [torch.cuda.Stream() for _ in passes]
+        for p, s in zip(passes, streams):
+            s.wait_event(opened)                   # all twenty are pending at once
+            p.fused(s)
+        torch.cuda.synchronize()
+        for p, w in zip(passes, want):
+            assert_same_attention(p.snapshot(), w)
+
+
+def test_threads_on_streams_of_their_own_and_on_a_shared_one():
+    import threading
+    import torch
+    passes = [Pass(**dict(kw, seed=i)) for i, kw in enumerate((CHAINS, ONE, CHAINS, ONE))]
+    want = [_want(p) for p in passes]
+    shared = torch.cuda.Stream()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream(), shared, shared]
+    for p in passes:
+        p.spoil()
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(p, s, call):
+        try:
+            for _ in range(40):
+                getattr(p, call)(s)
+        except Exception as e:                     # (reported by the main thread)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(p, s, c))
+               for p, s, c in zip(passes, streams, ("fused", "from_host", "from_host", "fused"))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors
+    for p, w in zip(passes, want):
+        assert_same_attention(p.snapshot(), w)
+
+
+@pytest.mark.parametrize("kw", [CHAINS, dict(CHAINS, listed=[2, 0]), ONE, dict(T=61, Hq=16, Hkv=8, cap=704, lens=[700, 333])])
+def test_host_buffer_pass_of_several_sequences(kw):
+    import torch
+    p = Pass(**kw)
+    want = _want(p)
+    for s in (torch.cuda.current_stream(), torch.cuda.Stream()):
+        for _ in range(3):
+            p.spoil()
+            torch.cuda.synchronize()
+            p.from_host(s)
+            assert_same_attention(p.snapshot(), want)
+            for n, t in p.back.items():
+                assert torch.equal(t, p.out[n].cpu()), n
