@@ -584,6 +584,10 @@ struct LmRowsParams {
   int n_rows, N;    // columns that are rows, and the same rounded up to 16
   int slot_rows;    // > 0: not packed rows but slots of this many (a multiple of 8) per sequence of the index list
   int wait_rows;    // the rows are written by the kernel before this one
+  // SMs are left free for an attention beside this kernel: the kernels after it may not start before its last copies are
+  // on their way. Their blocks, waiting on those SMs, kept the attention's CTAs off until this kernel's end wherever it
+  // was placed first (the pass of one sequence, 61 nodes, 4096 tokens, 151936 x 2048, behind other work: 197 -> 133 us).
+  int late_dependents;
   int n_tiles;      // tiles per vocabulary range
   int box_rows;     // W rows per copy: the height of half a tile
   int stages, stage_bytes;
@@ -637,7 +641,7 @@ template <bool kEntropy, int kRows>
 __global__ void __launch_bounds__(LW_THREADS, 1)
 lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_h,
                    const LmRowsParams sp) {
-  pdl_launch_dependents();
+  if (!sp.late_dependents) pdl_launch_dependents();
   const LmParams& p = sp.base;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base_u32 = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -698,6 +702,7 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
           if (++stage == sp.stages) { stage = 0; phase ^= 1u; }
         }
       }
+      if (sp.late_dependents) pdl_launch_dependents();
     }
   } else if (warp == LW_EPI_WARPS + 1) {
     if (lane == 0) {   // ---------------------------------------------------------- MMA issuer
@@ -839,6 +844,7 @@ struct LmPlan {
   bool few_rows;   // at most 128 rows: lmhead_rows_kernel, one CTA and one vocabulary range per SM
   bool pack;       // the rows of an index list are gathered into the workspace first
   bool slots;      // (no workspace to gather into) four slots of 64 node rows per M tile
+  bool reserved;   // few_rows: SMs are left to an attention that runs beside it
   int slot_rows;   // few_rows and an index list of several: columns per sequence, read without gathering; 0 = packed
   int n_mt;        // M tiles of 256 rows
   int n_ranges;    // vocabulary ranges of the main part (few_rows: at most this many)
@@ -873,11 +879,13 @@ static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, si
   // 142 -> 123 us).
   pl->few_rows = lm_takes_few_rows(a, rows) && !slots;
   pl->slot_rows = 0;
+  pl->reserved = false;
   if (pl->few_rows) {
     pl->n_mt = 1;
     pl->part_rows = lw_rows(rows);
     const int V16 = (a->V + 15) / 16;
     int sms = device_sm_count() - tl_lm_reserved_sms;
+    pl->reserved = tl_lm_reserved_sms > 0;
     if (sms < 1) sms = 1;
     pl->n_ranges = sms < V16 ? sms : V16;
     pl->rows_ctas = pl->n_ranges;
@@ -1042,6 +1050,7 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
     sp.slot_rows = pl.slot_rows;
     sp.n_rows = pl.slot_rows > 0 ? n_seq * pl.slot_rows : static_cast<int>(n_rows);
     sp.wait_rows = p.wait_rows;
+    sp.late_dependents = pl.reserved ? 1 : 0;
     sp.N = ((sp.n_rows + 15) / 16) * 16;
     sp.stage_bytes = LW_A_BYTES + sp.N * LW_BK * 2;
     sp.stages = LW_RING_BYTES / sp.stage_bytes;
