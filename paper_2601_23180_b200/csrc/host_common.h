@@ -55,8 +55,8 @@ bool entry_scope_next_launch_is_dependent();
 // The next launch inside the current scope is an ordinary one again (after work was moved to or joined from
 // another stream, where "the kernel before it" is not the kernel enqueued last).
 void entry_scope_next_launch_ordinary();
-// SMs the single-sequence LM head leaves free on its next launch from this thread (0 = none); consumed by
-// that launch. The fused pass sets it when a small attention runs beside the LM head on a second stream.
+// SMs the LM head's small-row kernel leaves free on its next launch from this thread (0 = none); consumed by
+// that launch. The fused pass sets it when the attention runs beside the LM head on a second stream.
 void lm_reserve_sms_once(int n);
 
 template <typename... KArgs, typename... Args>

@@ -67,7 +67,8 @@ struct LmParams {
   int main_units; // 32-column units [0, main_units) belong to the main part, the rest to the tail
   float c;        // logit_scale * log2(e)
   const int32_t* seq_index;
-  LmPartial* partial;  // [n_ranges + n_tail][n_mt * 256]
+  int part_rows;       // rows of a vocabulary range's partials: n_mt * tile_rows
+  LmPartial* partial;  // [n_ranges + n_tail][part_rows]
   int32_t* dev_status;
 };
 
@@ -378,7 +379,7 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
     LmPartial out;
     out.m = m; out.s = s; out.v1 = v1; out.v2 = v2; out.i1 = i1; out.i2 = i2; out.t = tz; out.pad = 0;
     if (row < (p.tile_rows >> 1))
-      p.partial[static_cast<size_t>(work.part) * (p.n_mt * 2 * LM_BM) + ((work.mt0 + sweep) * 2 + rank) * (p.tile_rows >> 1) + row] = out;
+      p.partial[static_cast<size_t>(work.part) * p.part_rows + ((work.mt0 + sweep) * 2 + rank) * (p.tile_rows >> 1) + row] = out;
     }   // sweeps
   }
 
@@ -574,7 +575,7 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
 constexpr int LW_BM = 128, LW_SUBS = 2, LW_BK = 64, LW_MAX_STAGES = 6, LW_EPI_WARPS = 8;
 constexpr int LW_THREADS = 32 * (LW_EPI_WARPS + 2);
 constexpr int LW_A_BYTES = LW_SUBS * LW_BM * LW_BK * 2;  // 32 KB of W per stage
-constexpr int lw_rows(long long n_rows) { return n_rows <= 64 ? 64 : 128; }   // partial rows per vocabulary range
+constexpr int lw_rows(long long n_rows) { return n_rows <= 64 ? 64 : static_cast<int>((n_rows + 15) / 16 * 16); }   // partial rows per range
 constexpr int LW_XPOSE_BYTES = 2048;                     // 32 entries x 16 columns per epilogue warp
 constexpr int LW_SMEM_BYTES = 227 * 1024;
 constexpr int LW_RING_BYTES = LW_SMEM_BYTES - 1024 /*alignment slack*/ - LW_EPI_WARPS * LW_XPOSE_BYTES - 256 /*barriers*/;
@@ -823,7 +824,7 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
         }
         out.v1 = lm_key_value(top.a); out.v2 = lm_key_value(top.b);
         out.i1 = lm_key_entry(top.a); out.i2 = lm_key_entry(top.b);
-        p.partial[static_cast<size_t>(range) * kRows + column] = out;
+        p.partial[static_cast<size_t>(range) * p.part_rows + column] = out;
       }
     }
   }
@@ -847,15 +848,15 @@ struct LmPlan {
   bool reserved;   // few_rows: SMs are left to an attention that runs beside it
   int slot_rows;   // few_rows and an index list of several: columns per sequence, read without gathering; 0 = packed
   int n_mt;        // M tiles of 256 rows
-  int n_ranges;    // vocabulary ranges of the main part (few_rows: at most this many)
-  int rows_ctas;   // few_rows: ranges = CTAs
-  int part_rows;   // few_rows: partial rows per range
+  int n_ranges;    // vocabulary ranges of the main part (few_rows: one per CTA, at most this many)
+  int tile_rows;   // rows per M tile (the rows are spread evenly over the tiles)
+  int part_rows;   // partial rows per vocabulary range
   int n_tail;      // pairs that sweep all M tiles over a slice of the vocabulary's tail
   int main_units;  // 32-column units of the main part
   size_t required;   // workspace the call cannot do without
   size_t pack_bytes; // and what it needs on top of it to pack listed rows
   size_t partial_bytes() const {
-    return static_cast<size_t>(n_ranges + n_tail) * (few_rows ? part_rows : n_mt * 2 * LM_BM) * sizeof(LmPartial);
+    return static_cast<size_t>(n_ranges + n_tail) * part_rows * sizeof(LmPartial);
   }
 };
 
@@ -864,8 +865,13 @@ static bool lm_long_stream(const trispec_lmhead_args* a) { return static_cast<lo
 
 bool lm_takes_few_rows(const trispec_lmhead_args* a, long long rows) { return rows <= (lm_long_stream(a) ? LM_FEW_ROWS : 64); }
 
+static int lm_ranges_within(size_t max_ws, int part_rows, int ranges) {
+  const size_t fit = max_ws / (static_cast<size_t>(part_rows) * sizeof(LmPartial));
+  return fit >= static_cast<size_t>(ranges) ? ranges : (fit > 0 ? static_cast<int>(fit) : 1);
+}
 // Plans the launch for rows that are packed, or that sit in slots of 64 per sequence. `max_ws` bounds the partial
-// array: tail pairs, which cost a block of partial rows for every M tile each, are given up until it fits.
+// array: tail pairs, which cost a block of partial rows for every M tile each, are given up until it fits, and packed rows
+// are cut into fewer ranges.
 static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, size_t max_ws, LmPlan* pl) {
   const long long rows = static_cast<long long>(n_seq) * a->T;
   pl->n_seq = n_seq;
@@ -882,32 +888,31 @@ static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, si
   pl->reserved = false;
   if (pl->few_rows) {
     pl->n_mt = 1;
+    pl->tile_rows = 0;
     pl->part_rows = lw_rows(rows);
     const int V16 = (a->V + 15) / 16;
     int sms = device_sm_count() - tl_lm_reserved_sms;
     pl->reserved = tl_lm_reserved_sms > 0;
     if (sms < 1) sms = 1;
     pl->n_ranges = sms < V16 ? sms : V16;
-    pl->rows_ctas = pl->n_ranges;
-    // few units per range: as many ranges as keep the longest one as short, all of the same length where that comes
-    // out even (a small vocabulary's statistics then do not depend on how many SMs the launch was given)
-    const int per = (V16 + sms - 1) / sms;
-    if (per <= 8) pl->rows_ctas = (V16 + per - 1) / per;
     return;
   }
   pl->n_mt = slots ? (n_seq + 3) / 4 : static_cast<int>((rows + 2 * LM_BM - 1) / (2 * LM_BM));
+  pl->tile_rows = slots ? 2 * LM_BM : static_cast<int>(((rows + pl->n_mt - 1) / pl->n_mt + 15) / 16 * 16);
+  pl->part_rows = pl->n_mt * pl->tile_rows;
   const int pairs = device_sm_count() / 2;       // one CTA pair per two SMs
   int r = pairs / pl->n_mt;
   if (r < 1) r = 1;
   const int V32 = (a->V + 31) / 32;
   if (r > V32) r = V32;
+  if (!slots) r = lm_ranges_within(max_ws, pl->part_rows, r);
   pl->n_ranges = r;
   // Pairs that the M tiles leave over (74 = 16 x 4 + 10 for 16 M tiles) take the tail of the vocabulary,
   // every one of them for all M tiles in turn. Balance in whole tiles (a tile costs a k-loop whatever its
   // width): a main pair runs ceil(main_units / r / 8) tiles, a tail pair n_mt x ceil(slice / 8).
   int tail = pairs - pl->n_mt * r;
   if (pl->n_mt < 2 || tail < 1 || pl->n_mt * r > pairs) tail = 0;
-  while (tail > 0 && static_cast<size_t>(r + tail) * pl->n_mt * 2 * LM_BM * sizeof(LmPartial) > max_ws) --tail;
+  while (tail > 0 && static_cast<size_t>(r + tail) * pl->part_rows * sizeof(LmPartial) > max_ws) --tail;
   if (tail > 0) {
     int best_slice = 0, best_cost = (V32 / r + 7) / 8 + 1;    // without a tail: the longest main range
     {
@@ -942,21 +947,28 @@ static int lm_plan(const trispec_lmhead_args* a, LmPlan* pl, size_t room, size_t
   if (a->T > 64 || (a->d % LM_BK) != 0 || a->V < 2) return TRISPEC_ERR_UNSUPPORTED;
   const int n_seq = a->seq_index ? a->B_active : a->B;
   if (n_seq <= 0 || n_seq > a->B) return TRISPEC_ERR_INVALID_ARG;
-  lm_plan_rows(a, n_seq, false, max_ws, pl);
-  pl->required = pl->partial_bytes();
-  if (n_seq == 1) return TRISPEC_OK;
+  if (n_seq == 1) {
+    lm_plan_rows(a, n_seq, false, max_ws, pl);
+    pl->required = pl->partial_bytes();
+    return TRISPEC_OK;
+  }
+  // the slots' workspace is what a call of several sequences asks for, however it reads its rows (a packed plan that would
+  // take more, one M tile of more than 248 rows from 9 to 12 sequences, has 72 ranges instead of 74)
   LmPlan slots;
   lm_plan_rows(a, n_seq, true, max_ws, &slots);
-  if (slots.partial_bytes() > pl->required) pl->required = slots.partial_bytes();
+  const size_t required = slots.partial_bytes();
+  lm_plan_rows(a, n_seq, false, required, pl);
+  pl->required = slots.required = required;
+  if (pl->few_rows) pl->n_ranges = lm_ranges_within(required, pl->part_rows, pl->n_ranges);
   if (!a->seq_index) return TRISPEC_OK;
   // A few listed sequences whose rows, rounded up to 8 each, still are at most 128 columns: one copy per sequence and
-  // stage instead of a gather, whose launch would come before the stream of W can start (3 of 5 sequences of 23
-  // nodes, 50257 x 2048 weights: 93.5 us with the gather, 87.5 us in slots of 64 in the pair kernel).
+  // stage instead of a gather, whose launch would come before the stream of W can start (3 of 5 sequences
+  // of 23 nodes, 50257 x 2048 weights: 93.5 us with the gather, 87.5 us in slots of 64 in the pair kernel).
   const int slot_rows = (a->T + 7) / 8 * 8;
   if (pl->few_rows && n_seq <= 8 && n_seq * slot_rows <= LM_FEW_ROWS) {
     pl->slot_rows = slot_rows;
     pl->part_rows = lw_rows(static_cast<long long>(n_seq) * slot_rows);
-    if (pl->partial_bytes() > pl->required) pl->required = pl->partial_bytes();
+    pl->n_ranges = lm_ranges_within(required, pl->part_rows, pl->n_ranges);
     return TRISPEC_OK;
   }
   const size_t pack_bytes = static_cast<size_t>(n_seq) * a->T * a->d * 2;
@@ -966,7 +978,6 @@ static int lm_plan(const trispec_lmhead_args* a, LmPlan* pl, size_t room, size_t
     pl->pack = true;
     pl->pack_bytes = pack_bytes;
   } else {
-    slots.required = pl->required;
     *pl = slots;
   }
   return TRISPEC_OK;
@@ -996,7 +1007,14 @@ extern "C" int trispec_lmhead_stats(const trispec_lmhead_args* a, void* stream) 
 }
 
 static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmPlan& pl, void* stream) {
-  const int n_seq = pl.n_seq, n_ranges = pl.few_rows ? pl.rows_ctas : pl.n_ranges;
+  int n_ranges = pl.n_ranges;
+  if (pl.few_rows) {
+    // few units per range: as many ranges as keep the longest one as short, all of the same length where that comes
+    // out even (a small vocabulary's statistics then do not depend on how many SMs the launch was given)
+    const int V16 = (a->V + 15) / 16, per = (V16 + n_ranges - 1) / n_ranges;
+    if (per <= 8) n_ranges = (V16 + per - 1) / per;
+  }
+  const int n_seq = pl.n_seq;
   const long long n_rows = static_cast<long long>(n_seq) * a->T;
   int rc = TRISPEC_OK;
   if (!a->h || !a->W || !a->parent || !a->tok || !a->workspace) return TRISPEC_ERR_INVALID_ARG;
@@ -1028,7 +1046,8 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   p.n_seq = n_seq; p.n_mt = pl.n_mt; p.n_ranges = n_ranges;
   p.n_tail = pl.n_tail; p.main_units = pl.main_units;
   p.slots = pl.slots ? 1 : 0;
-  p.tile_rows = pl.slots ? 2 * LM_BM : static_cast<int>(((n_rows + pl.n_mt - 1) / pl.n_mt + 15) / 16 * 16);
+  p.tile_rows = pl.tile_rows;
+  p.part_rows = pl.part_rows;
   p.wait_rows = pl.pack ? 1 : 0;
   p.c = f.c;
   p.seq_index = a->seq_index;
@@ -1081,7 +1100,7 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
     typedef void (*RowsKernel)(CUtensorMap, CUtensorMap, LmRowsParams);
     static const RowsKernel table[2][2] = {{lmhead_rows_kernel<false, 64>, lmhead_rows_kernel<false, 128>},
                                            {lmhead_rows_kernel<true, 64>, lmhead_rows_kernel<true, 128>}};
-    const int wide = pl.part_rows > 64 ? 1 : 0;
+    const int wide = sp.n_rows > 64 ? 1 : 0;
     const RowsKernel kernel = table[want_entropy ? 1 : 0][wide];
     static bool smem_set_rows[4][64] = {};
     rc = ensure_smem_limit(reinterpret_cast<const void*>(kernel), LW_SMEM_BYTES, smem_set_rows[(want_entropy ? 2 : 0) + wide]);
@@ -1121,7 +1140,7 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   TRISPEC_CUDA_OK(launch_dependent(kernel, static_cast<unsigned>(2 * (p.n_mt * n_ranges + pl.n_tail)), LM_THREADS,
                                    LM_SMEM_BYTES, st, 2, tm_h, tm_w, p));
   count_launch();
-  f.stride = p.n_mt * 2 * LM_BM;
+  f.stride = pl.part_rows;
   TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel, static_cast<unsigned>((n_rows + 7) / 8),
                                    LM_FIN_THREADS, 0, st, 1, f, n_seq));
   count_launch();

@@ -1,0 +1,59 @@
+"""LM head with the least workspace that a call may bring, whatever way its rows are read."""
+import math
+
+import numpy as np
+import pytest
+
+from oracle import trispec_oracle as orc
+from paper_2601_23180_b200 import inputs as gen
+
+pytestmark = pytest.mark.gpu
+
+
+def _call(B, T, listed, d, V, seed=7):
+    import torch
+    import tests.gpu_helpers as H
+    from paper_2601_23180_b200 import binding as ts
+    cfg = gen.small_variant(gen.CONFIGS["tiny_chain"], B=B, k=T - 1, max_depth=T - 1, d=d, V=V, rho=0.2,
+                            logit_scale=3.6 / (0.02 * math.sqrt(d)), seed=seed)
+    inp = gen.make_inputs(cfg, with_attention=False)
+    if listed:
+        inp["seq_index"] = np.random.default_rng(B).permutation(B)[:listed].astype(np.int32)
+    dev = H.to_device(inp)
+    st = ts.alloc_stats(B, T, entropy=True)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    a = ts.lmhead_args(dev["h"], dev["W"], dev["parent"], dev["tok"], cfg.logit_scale, st, seq_index=dev["seq_index"],
+                       dev_status=status)
+    a._held += (dev,)
+    return cfg, inp, a, st, status
+
+
+def _check(cfg, inp, st, status, T, B):
+    import tests.gpu_helpers as H
+    assert int(status.item()) == 0
+    seqs = list(range(B)) if inp.get("seq_index") is None else [int(s) for s in inp["seq_index"]]
+    got = {k: v.cpu().numpy() for k, v in st.items()}
+    ref = orc.lmhead_stats(inp["h"], inp["W"], inp["parent"], inp["tok"], cfg.logit_scale, seqs=seqs)
+    assert H.check_stats(got, ref, seqs, T) <= 0.02 * len(seqs) * T + 2
+    for b in set(range(B)) - set(seqs):
+        assert np.isnan(got["lse"][b]).all() and (got["top1_idx"][b] == -1).all()
+
+
+@pytest.mark.parametrize("B,T,d,V", [
+    (12, 21, 192, 3001),       # 252 packed rows: 72 vocabulary ranges instead of 74
+    (9, 9, 192, 3001),
+    (33, 31, 64, 20011),       # 1023: four M tiles of 256, nine in slots
+    (24, 53, 64, 20011),       # 1272: five M tiles, whose tail pairs have to fit as well
+    (12, 10, 2048, 65552),     # 120 rows over 256 MiB of W: the small-row kernel with 144 ranges
+])
+def test_lmhead_with_the_workspace_of_the_slots(B, T, d, V):
+    import torch
+    from paper_2601_23180_b200 import binding as ts
+    cfg, inp, a, st, status = _call(B, T, 0, d, V)
+    need = ts.trispec_lmhead_stats_workspace(a)
+    ws = torch.full((need + 4096,), 0x5A, dtype=torch.uint8, device="cuda")
+    a.workspace, a.workspace_bytes = ws.data_ptr(), need
+    ts.trispec_lmhead_stats(a)
+    torch.cuda.synchronize()
+    assert (ws[need:] == 0x5A).all()
+    _check(cfg, inp, st, status, T, B)
