@@ -99,9 +99,9 @@ int attn_planned_ctas(const trispec_attn_args* a);
 int attn_compact_ctas(const trispec_attn_args* a, double budget_us, int max_ctas);
 // The attention launches of this thread take that form while this is on
 void attn_in_turn_once(bool on);
-// columns of the LM head's small-row kernel, and whether so many active rows take it (from 65 on only with a long W)
+// columns of the LM head's small-row kernel, and whether a call with these arguments (its workspace's size among them) takes it
 constexpr int LM_FEW_ROWS = 128;
-bool lm_takes_few_rows(const trispec_lmhead_args* a, long long rows);
+bool lm_runs_small_rows(const trispec_lmhead_args* a);
 
 #define TRISPEC_CUDA_OK(expr)                        \
   do {                                               \

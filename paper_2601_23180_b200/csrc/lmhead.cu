@@ -863,7 +863,7 @@ struct LmPlan {
 // W is streamed from HBM for long enough (about twice L2) that what happens before and after it matters less
 static bool lm_long_stream(const trispec_lmhead_args* a) { return static_cast<long long>(a->V) * a->d * 2 >= (256ll << 20); }
 
-bool lm_takes_few_rows(const trispec_lmhead_args* a, long long rows) { return rows <= (lm_long_stream(a) ? LM_FEW_ROWS : 64); }
+static bool lm_takes_few_rows(const trispec_lmhead_args* a, long long rows) { return rows <= (lm_long_stream(a) ? LM_FEW_ROWS : 64); }
 
 static int lm_ranges_within(size_t max_ws, int part_rows, int ranges) {
   const size_t fit = max_ws / (static_cast<size_t>(part_rows) * sizeof(LmPartial));
@@ -993,6 +993,10 @@ extern "C" size_t trispec_lmhead_stats_workspace(const trispec_lmhead_args* a) {
 }
 
 namespace trispec {
+bool lm_runs_small_rows(const trispec_lmhead_args* a) {
+  LmPlan pl;
+  return lm_plan(a, &pl, a->workspace_bytes) == TRISPEC_OK && pl.few_rows;
+}
 static int lmhead_stats_planned(const trispec_lmhead_args* a, const LmPlan& pl, void* stream);
 }
 

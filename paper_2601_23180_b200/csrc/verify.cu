@@ -133,8 +133,7 @@ struct PassPlan {
 static PassPlan pass_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm, const trispec_scan_args* scan) {
   PassPlan pl = {PASS_ATTENTION_FIRST, false, attn ? attn_planned_ctas(attn) : 0, false};
   const int lm_seqs = lm->seq_index ? lm->B_active : lm->B;
-  if (!attn || pl.attn_ctas <= 0 || lm_seqs <= 0) return pl;
-  if (!lm_takes_few_rows(lm, static_cast<long long>(lm_seqs) * lm->T)) return pl;      // the pair kernel takes every SM
+  if (!attn || pl.attn_ctas <= 0 || !lm_runs_small_rows(lm)) return pl;      // the pair kernel takes every SM
   const int sms = device_sm_count();
   // not beside the scan when its escalation list is written over the index list the attention reads:
   // in stream order the scan comes last, side by side it would not

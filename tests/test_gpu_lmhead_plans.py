@@ -57,3 +57,39 @@ def test_lmhead_with_the_workspace_of_the_slots(B, T, d, V):
     torch.cuda.synchronize()
     assert (ws[need:] == 0x5A).all()
     _check(cfg, inp, st, status, T, B)
+
+
+@pytest.mark.parametrize("B,T,listed", [(20, 5, 12), (12, 6, 10)])     # 60 rows of more than eight sequences
+@pytest.mark.parametrize("room", ["gathered", "slots"])
+def test_few_listed_rows_with_and_without_room_to_gather(B, T, listed, room):
+    import torch
+    from paper_2601_23180_b200 import binding as ts
+    cfg, inp, a, st, status = _call(B, T, listed, 192, 3001)
+    need = ts.trispec_lmhead_stats_workspace(a) - (0 if room == "gathered" else listed * T * 192 * 2)
+    ws = torch.full((need + 4096,), 0x5A, dtype=torch.uint8, device="cuda")
+    a.workspace, a.workspace_bytes = ws.data_ptr(), need
+    n0 = ts.launch_count()
+    ts.trispec_lmhead_stats(a)
+    torch.cuda.synchronize()
+    assert ts.launch_count() - n0 == (3 if room == "gathered" else 2)
+    assert (ws[need:] == 0x5A).all()
+    _check(cfg, inp, st, status, T, B)
+
+
+@pytest.mark.parametrize("room", ["gathered", "slots"])
+def test_fused_pass_of_listed_rows_with_and_without_room_to_gather(room):
+    import torch
+    from paper_2601_23180_b200 import binding as ts
+    from tests.test_gpu_beside import Pass, assert_same_attention
+    p = Pass(T=6, Hq=8, Hkv=1, cap=256, lens=[200 + i for i in range(12)], listed=[11, 3, 0, 7, 5, 1, 9, 2, 8, 4], V=60000)
+    if room == "slots":
+        p.lm_args.workspace_bytes -= 60 * 2048 * 2
+    assert ts.trispec_verify_plan(p.attn_args, p.lm_args, p.scan_args) == ("side_by_side" if room == "gathered" else
+                                                                         "attention_first")
+    p.spoil()
+    p.separate()
+    want = p.snapshot()
+    for _ in range(3):
+        p.spoil()
+        p.fused()
+        assert_same_attention(p.snapshot(), want)

@@ -3,6 +3,7 @@
 import pytest
 
 from paper_2601_23180_b200 import binding as ts
+from paper_2601_23180_b200 import inputs as gen
 
 
 def _lm(B, T, d, V, listed=0):
@@ -23,3 +24,17 @@ def test_several_sequences_ask_for_the_workspace_of_their_slots_and_no_more(B, T
     # with an index list, room for the gathered rows comes on top of it
     rows = B * T * d * 2
     assert ts.trispec_lmhead_stats_workspace(_lm(B, T, d, V, B)) == 24 * 3 * 256 * 32 + rows
+
+
+def test_pass_form_asks_which_kernel_the_lm_head_takes():
+    """Ten listed sequences of six nodes are gathered for the small-row kernel; a workspace that was sized without a
+    list leaves them in slots in the pair kernel, which takes every SM: nothing runs beside it."""
+    cfg = gen.small_variant(gen.CONFIGS["tiny_chain"], B=12, L=256, Hq=8, Hkv=1)
+    t = ts.AttnArgs()
+    t.B, t.T, t.Hq, t.Hkv, t.D, t.scale = cfg.B, 6, cfg.Hq, cfg.Hkv, cfg.D, 1.0
+    t.kv_layout, t.Lmax, t.B_active, t.seq_index = ts.KV_CONTIGUOUS, cfg.L, 10, 1
+    lm = _lm(12, 6, 2048, 60000, 10)
+    lm.workspace_bytes = ts.trispec_lmhead_stats_workspace(lm)
+    assert ts.trispec_verify_plan(t, lm) == "side_by_side"
+    lm.workspace_bytes = ts.trispec_lmhead_stats_workspace(_lm(12, 6, 2048, 60000))
+    assert ts.trispec_verify_plan(t, lm) == "attention_first"
