@@ -961,11 +961,11 @@ static int lm_plan(const trispec_lmhead_args* a, LmPlan* pl, size_t room, size_t
   pl->required = slots.required = required;
   if (pl->few_rows) pl->n_ranges = lm_ranges_within(required, pl->part_rows, pl->n_ranges);
   if (!a->seq_index) return TRISPEC_OK;
-  // A few listed sequences whose rows, rounded up to 8 each, still are at most 128 columns: one copy per sequence and
-  // stage instead of a gather, whose launch would come before the stream of W can start (3 of 5 sequences
+  // A few listed sequences whose rows, rounded up to 8 each, still are columns of the small-row kernel: one copy per
+  // sequence and stage instead of a gather, whose launch would come before the stream of W can start (3 of 5 sequences
   // of 23 nodes, 50257 x 2048 weights: 93.5 us with the gather, 87.5 us in slots of 64 in the pair kernel).
   const int slot_rows = (a->T + 7) / 8 * 8;
-  if (pl->few_rows && n_seq <= 8 && n_seq * slot_rows <= LM_FEW_ROWS) {
+  if (pl->few_rows && n_seq <= 8 && lm_takes_few_rows(a, static_cast<long long>(n_seq) * slot_rows)) {
     pl->slot_rows = slot_rows;
     pl->part_rows = lw_rows(static_cast<long long>(n_seq) * slot_rows);
     pl->n_ranges = lm_ranges_within(required, pl->part_rows, pl->n_ranges);

@@ -93,3 +93,21 @@ def test_fused_pass_of_listed_rows_with_and_without_room_to_gather(room):
         p.spoil()
         p.fused()
         assert_same_attention(p.snapshot(), want)
+
+
+@pytest.mark.parametrize("B,T,listed,launches", [
+    (8, 9, 7, 3),      # 63 rows, but 112 columns in slots: gathered, over a short W
+    (9, 12, 5, 3),     # 60 rows, 80 columns
+    (9, 16, 4, 2),     # 64 rows, 64 columns: read in slots
+])
+def test_slots_of_the_small_row_kernel_are_counted_in_columns(B, T, listed, launches):
+    import torch
+    from paper_2601_23180_b200 import binding as ts
+    cfg, inp, a, st, status = _call(B, T, listed, 192, 3001)
+    ws = ts.alloc_workspace(ts.trispec_lmhead_stats_workspace(a))
+    a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+    n0 = ts.launch_count()
+    ts.trispec_lmhead_stats(a)
+    torch.cuda.synchronize()
+    assert ts.launch_count() - n0 == launches
+    _check(cfg, inp, st, status, T, B)
