@@ -313,11 +313,11 @@ esc_compact_kernel(const uint8_t* __restrict__ escalate, int B, int32_t* __restr
   if (tid == 0 && (!block_count || blockIdx.x == gridDim.x - 1)) *n_escalated = running;
 }
 
-}  // namespace trispec
-
-extern "C" int trispec_accept_scan(const trispec_scan_args* a, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
-  using namespace trispec;
+// acceptance rule: the Bernoulli inputs select Eq. 6 when the rule field is left at its default
+static int scan_rule(const trispec_scan_args* a) {
+  return a->accept_rule == TRISPEC_ACCEPT_GREEDY && a->q_draft ? TRISPEC_ACCEPT_STOCHASTIC : a->accept_rule;
+}
+int scan_check(const trispec_scan_args* a) {
   if (!a || a->B <= 0 || a->T <= 0) return TRISPEC_ERR_INVALID_ARG;
   if (a->T > 64) return TRISPEC_ERR_UNSUPPORTED;
   if (!a->parent || !a->tok || !a->in.top1_idx || !a->accept_len || !a->bonus_tok || !a->path || !a->last_node ||
@@ -332,14 +332,22 @@ extern "C" int trispec_accept_scan(const trispec_scan_args* a, void* stream) {
   }
   if ((a->n_escalated == nullptr) != (a->esc_index == nullptr)) return TRISPEC_ERR_INVALID_ARG;
   if ((a->q_draft == nullptr) != (a->u_accept == nullptr)) return TRISPEC_ERR_INVALID_ARG;
-  // acceptance rule: the Bernoulli inputs select Eq. 6 when the rule field is left at its default
-  int rule = a->accept_rule;
-  if (rule == TRISPEC_ACCEPT_GREEDY && a->q_draft) rule = TRISPEC_ACCEPT_STOCHASTIC;
+  const int rule = scan_rule(a);
   if (rule < TRISPEC_ACCEPT_GREEDY || rule > TRISPEC_ACCEPT_TOKEN_SPECIFIC) return TRISPEC_ERR_INVALID_ARG;
   if (rule == TRISPEC_ACCEPT_STOCHASTIC && (!a->q_draft || !a->in.p_draft)) return TRISPEC_ERR_INVALID_ARG;
   if (rule == TRISPEC_ACCEPT_TOKEN_SPECIFIC &&
       (!a->in.p_draft || !a->in.p_top1 || !(a->alpha >= 0.f && a->alpha <= 1.f)))
     return TRISPEC_ERR_INVALID_ARG;
+  return TRISPEC_OK;
+}
+}  // namespace trispec
+
+extern "C" int trispec_accept_scan(const trispec_scan_args* a, void* stream) {
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
+  using namespace trispec;
+  const int rc = scan_check(a);
+  if (rc != TRISPEC_OK) return rc;
+  const int rule = scan_rule(a);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // kernel instance for (criterion, acceptance rule); TARGET mode reads no feature: margin instance
   const int crit = (a->mode == TRISPEC_MODE_PROXY) ? a->criterion : TRISPEC_CRIT_MARGIN;

@@ -880,12 +880,11 @@ extern "C" const char* trispec_verify_attn_plan(const trispec_attn_args* a) {
   return pl.pieces ? "pieces" : (pl.cluster ? "cluster" : "splits");
 }
 
-extern "C" int trispec_verify_attn(const trispec_attn_args* a, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
-  using namespace trispec;
-  AttnPlan pl;
-  int rc = attn_plan(a, &pl);
+namespace trispec {
+static int attn_checked_plan(const trispec_attn_args* a, AttnPlan* plan) {
+  const int rc = attn_plan(a, plan);
   if (rc != TRISPEC_OK) return rc;
+  const AttnPlan& pl = *plan;
   if (!a->q || !a->k_tree || !a->v_tree || !a->ctx_len || !a->mask || !a->o) return TRISPEC_ERR_INVALID_ARG;
   if ((pl.pieces || !pl.cluster) && !a->workspace) return TRISPEC_ERR_INVALID_ARG;
   if (pl.tiles_max > 0 && (!a->k_cache || !a->v_cache)) return TRISPEC_ERR_INVALID_ARG;
@@ -895,6 +894,20 @@ extern "C" int trispec_verify_attn(const trispec_attn_args* a, void* stream) {
     return TRISPEC_ERR_INVALID_ARG;
   if (!(a->scale > 0.f) || !isfinite(a->scale)) return TRISPEC_ERR_INVALID_ARG;
   if (a->workspace_bytes < trispec_verify_attn_workspace(a)) return TRISPEC_ERR_WORKSPACE;
+  return TRISPEC_OK;
+}
+int attn_check(const trispec_attn_args* a) {
+  AttnPlan pl;
+  return attn_checked_plan(a, &pl);
+}
+}  // namespace trispec
+
+extern "C" int trispec_verify_attn(const trispec_attn_args* a, void* stream) {
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
+  using namespace trispec;
+  AttnPlan pl;
+  int rc = attn_checked_plan(a, &pl);
+  if (rc != TRISPEC_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
   const uint64_t D = AT_D, Hkv = a->Hkv, T = a->T, B = a->B;

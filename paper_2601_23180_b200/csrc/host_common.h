@@ -91,6 +91,11 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 #endif
 
+// What an entry point refuses, without launching anything (the fused passes ask all their steps first)
+int tree_mask_check(const trispec_tree_args* a);
+int attn_check(const trispec_attn_args* a);
+int lmhead_check(const trispec_lmhead_args* a);
+int scan_check(const trispec_scan_args* a);
 // CTAs the attention launch for these arguments will use (0 if the arguments are not accepted)
 int attn_planned_ctas(const trispec_attn_args* a);
 // CTAs of an attention whose plan merges its splits on chip when each (sequence, KV head, M tile) has one CTA, alone on

@@ -997,6 +997,23 @@ bool lm_runs_small_rows(const trispec_lmhead_args* a) {
   LmPlan pl;
   return lm_plan(a, &pl, a->workspace_bytes) == TRISPEC_OK && pl.few_rows;
 }
+static int lm_check_planned(const trispec_lmhead_args* a, const LmPlan& pl) {
+  if (!a->h || !a->W || !a->parent || !a->tok || !a->workspace) return TRISPEC_ERR_INVALID_ARG;
+  if (!aligned16(a->h) || !aligned16(a->W) || (reinterpret_cast<uintptr_t>(a->workspace) & 255u))
+    return TRISPEC_ERR_INVALID_ARG;
+  if (!(a->logit_scale > 0.f) || !isfinite(a->logit_scale)) return TRISPEC_ERR_INVALID_ARG;
+  const trispec_stats& o = a->out;
+  if (!o.max || !o.lse || !o.top1_val || !o.top2_val || !o.p_top1 || !o.p_top2 || !o.top1_idx || !o.top2_idx ||
+      !o.draft_logit || !o.p_draft)
+    return TRISPEC_ERR_INVALID_ARG;
+  if (a->workspace_bytes < pl.required) return TRISPEC_ERR_WORKSPACE;
+  return TRISPEC_OK;
+}
+int lmhead_check(const trispec_lmhead_args* a) {
+  LmPlan pl;
+  const int rc = lm_plan(a, &pl, a ? a->workspace_bytes : 0);
+  return rc != TRISPEC_OK ? rc : lm_check_planned(a, pl);
+}
 static int lmhead_stats_planned(const trispec_lmhead_args* a, const LmPlan& pl, void* stream);
 }
 
@@ -1020,16 +1037,8 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   }
   const int n_seq = pl.n_seq;
   const long long n_rows = static_cast<long long>(n_seq) * a->T;
-  int rc = TRISPEC_OK;
-  if (!a->h || !a->W || !a->parent || !a->tok || !a->workspace) return TRISPEC_ERR_INVALID_ARG;
-  if (!aligned16(a->h) || !aligned16(a->W) || (reinterpret_cast<uintptr_t>(a->workspace) & 255u))
-    return TRISPEC_ERR_INVALID_ARG;
-  if (!(a->logit_scale > 0.f) || !isfinite(a->logit_scale)) return TRISPEC_ERR_INVALID_ARG;
-  const trispec_stats& o = a->out;
-  if (!o.max || !o.lse || !o.top1_val || !o.top2_val || !o.p_top1 || !o.p_top2 || !o.top1_idx || !o.top2_idx ||
-      !o.draft_logit || !o.p_draft)
-    return TRISPEC_ERR_INVALID_ARG;
-  if (a->workspace_bytes < pl.required) return TRISPEC_ERR_WORKSPACE;
+  int rc = lm_check_planned(a, pl);
+  if (rc != TRISPEC_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
   // the entropy sum costs two more instructions per logit: only computed when it is asked for

@@ -177,11 +177,16 @@ tree_mask_block_kernel(const int32_t* __restrict__ parent, uint64_t* __restrict_
 
 }  // namespace trispec
 
+int trispec::tree_mask_check(const trispec_tree_args* a) {
+  if (!a || !a->parent || !a->mask || a->B <= 0 || a->T <= 0) return TRISPEC_ERR_INVALID_ARG;
+  return a->T > 64 ? TRISPEC_ERR_UNSUPPORTED : TRISPEC_OK;
+}
+
 extern "C" int trispec_build_tree_mask(const trispec_tree_args* a, void* stream) {
   trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   using namespace trispec;
-  if (!a || !a->parent || !a->mask || a->B <= 0 || a->T <= 0) return TRISPEC_ERR_INVALID_ARG;
-  if (a->T > 64) return TRISPEC_ERR_UNSUPPORTED;
+  const int rc = tree_mask_check(a);
+  if (rc != TRISPEC_OK) return rc;
   const long long n = a->B;
   if (n >= 2048) {   // enough sequences to fill the chip with a thread each
     unsigned grid = static_cast<unsigned>((n + kMaskBlockSeqs - 1) / kMaskBlockSeqs);

@@ -173,6 +173,19 @@ static PassPlan pass_plan(const trispec_attn_args* attn, const trispec_lmhead_ar
   }
   return pl;
 }
+
+// Argument errors of any step are found before anything is launched.
+static int pass_check(const trispec_tree_args* tree, const trispec_attn_args* attn, const trispec_lmhead_args* lm,
+                      const trispec_scan_args* scan, const PassPlan& plan) {
+  int rc = tree_mask_check(tree);
+  if (rc == TRISPEC_OK && attn) rc = attn_check(attn);
+  if (rc == TRISPEC_OK) {
+    lm_reserve_sms_once(plan.beside ? plan.attn_ctas : 0);
+    rc = lmhead_check(lm);
+    lm_reserve_sms_once(0);
+  }
+  return rc == TRISPEC_OK ? scan_check(scan) : rc;
+}
 }  // namespace trispec
 
 extern "C" const char* trispec_verify_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm,
@@ -198,7 +211,8 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
   // first, or the two run side by side (pass_plan above).
   const trispec::PassPlan plan = trispec::pass_plan(attn, lm, scan);
   const bool lm_first = plan.form == trispec::PASS_LM_FIRST;
-  int rc;
+  int rc = trispec::pass_check(tree, attn, lm, scan, plan);
+  if (rc != TRISPEC_OK) return rc;
   // Few rows and an attention that fits beside the LM head (pass_plan): the two run side by
   // side. Mask and attention go to a second stream behind an event recorded on `stream` at the
   // start of the call; the LM head, whose grid is one persistent CTA per SM, leaves them one SM per attention
@@ -225,7 +239,7 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
         lm_reserve_sms_once(0);
       }
       if (rc == TRISPEC_OK) rc = trispec_accept_scan(scan, stream);   // dependent of the LM head's last kernel
-      // joined after an argument error too: what has been launched ends before whatever `stream` gets next
+      // joined after an error too: what has been launched ends before whatever `stream` gets next
       TRISPEC_CUDA_OK(cudaStreamWaitEvent(st, side->done, 0));
       return rc;
     }
@@ -236,6 +250,8 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
     rc = trispec_verify_attn(attn, stream);
     if (rc != TRISPEC_OK) return rc;
   }
+  // (a pass that would have left SMs free, but found no second stream, keeps the LM head's plan: the same bits)
+  trispec::lm_reserve_sms_once(plan.beside ? plan.attn_ctas : 0);
   rc = trispec_lmhead_stats(lm, stream);
   if (rc != TRISPEC_OK) return rc;
   if (lm_first) {
@@ -259,6 +275,9 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
   // the copies below land in the buffers the structs name: they must describe one and the same pass
   if (tree->parent != lm->parent || tree->parent != scan->parent || lm->tok != scan->tok)
     return TRISPEC_ERR_INVALID_ARG;
+  const PassPlan plan = pass_plan(attn, lm, scan);
+  int rc = pass_check(tree, attn, lm, scan, plan);
+  if (rc != TRISPEC_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t BT = static_cast<size_t>(tree->B) * tree->T;
   // A copy list is issued with neighbours merged: requests whose source AND destination follow
@@ -297,7 +316,6 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
                      {const_cast<void*>(lm->h), io->h, BT * static_cast<size_t>(lm->d) * 2}};
     TRISPEC_CUDA_OK(copy_list(in, 3, cudaMemcpyHostToDevice, st));
   }
-  const PassPlan plan = pass_plan(attn, lm, scan);
   const bool side_by_side = plan.beside && forked;
   if (side_by_side) TRISPEC_CUDA_OK(cudaEventRecord((*side)->inputs, st));
   if (attn) {
@@ -308,7 +326,6 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
     TRISPEC_CUDA_OK(copy_list(in, 3, cudaMemcpyHostToDevice, forked ? (*side)->stream : st));
     if (forked && !side_by_side) TRISPEC_CUDA_OK(cudaEventRecord((*side)->done, (*side)->stream));
   }
-  int rc;
   if (side_by_side) {
     // few rows (as in trispec_verify): mask and attention follow their inputs on
     // the second stream, the LM head and the scan run on `stream`, which then waits for the second stream
@@ -332,6 +349,7 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
   } else {
     rc = trispec_build_tree_mask(tree, stream);
     if (rc != TRISPEC_OK) return rc;
+    lm_reserve_sms_once(plan.beside ? plan.attn_ctas : 0);   // (as in trispec_verify)
     rc = trispec_lmhead_stats(lm, stream);
     if (rc != TRISPEC_OK) return rc;
     if (attn) {

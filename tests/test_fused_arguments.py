@@ -1,0 +1,73 @@
+"""What the fused passes decide on the host before anything is launched; addresses are never followed."""
+import ctypes
+
+import pytest
+
+from paper_2601_23180_b200 import binding as ts
+
+
+class Args:
+    """Argument structs of one pass whose buffers lie 256 MiB apart at made-up addresses."""
+
+    def __init__(self, B=1, T=9, Hq=16, Hkv=8, cap=512, d=2048, V=32000, listed=0):
+        self.at = 1 << 40
+        t, a, l, s = ts.TreeArgs(), ts.AttnArgs(), ts.LmheadArgs(), ts.ScanArgs()
+        t.B, t.T, t.parent, t.mask, t.depth = B, T, self.new(), self.new(), self.new()
+        a.B, a.T, a.Hq, a.Hkv, a.D, a.scale = B, T, Hq, Hkv, 128, 0.1
+        a.kv_layout, a.Lmax = ts.KV_CONTIGUOUS, cap
+        for f in ("q", "k_tree", "v_tree", "k_cache", "v_cache", "ctx_len", "o", "lse"):
+            setattr(a, f, self.new())
+        a.mask = t.mask
+        l.B, l.T, l.d, l.V, l.logit_scale = B, T, d, V, 1.0
+        l.h, l.W, l.parent, l.tok = self.new(), self.new(), t.parent, self.new()
+        for f in ("max", "lse", "top1_val", "top2_val", "p_top1", "p_top2", "top1_idx", "top2_idx", "draft_logit", "p_draft"):
+            setattr(l.out, f, self.new())
+        s.B, s.T, s.lam, s.parent, s.tok, s.stats = B, T, 0.5, t.parent, l.tok, l.out
+        for f in ("accept_len", "bonus_tok", "path", "last_node", "escalate", "n_escalated", "esc_index"):
+            setattr(s, f, self.new())
+        if listed:
+            a.seq_index = l.seq_index = self.new()
+            a.B_active = l.B_active = listed
+        a.workspace, a.workspace_bytes = self.new(), ts.trispec_verify_attn_workspace(a)
+        l.workspace, l.workspace_bytes = self.new(), ts.trispec_lmhead_stats_workspace(l)
+        self.tree, self.attn, self.lm, self.scan = t, a, l, s
+
+    def new(self):
+        self.at += 256 << 20
+        return self.at
+
+    def call(self, host):
+        lib, r = ts._lib, ctypes.byref
+        structs = (r(self.tree), r(self.attn), r(self.lm), r(self.scan), None)
+        return lib.trispec_verify_host(r(ts.HostIO()), *structs) if host else lib.trispec_verify(*structs)
+
+    def form(self):
+        return ts.trispec_verify_plan(self.attn, self.lm, self.scan)
+
+
+@pytest.mark.parametrize("host", [False, True])
+@pytest.mark.parametrize("shape", [dict(), dict(B=8, T=61, cap=4096), dict(V=151936, T=61, cap=4096)],
+                         ids=["beside", "attention_first", "in_turn"])
+@pytest.mark.parametrize("step,field,value,code", [
+    ("tree", "mask", None, 1), ("attn", "o", None, 1), ("attn", "scale", 0.0, 1), ("attn", "q", 4096 + 8, 1),
+    ("attn", "D", 64, 2), ("lm", "W", None, 1), ("lm", "workspace_bytes", 256, 3), ("lm", "d", 100, 2),
+    ("scan", "path", None, 1), ("scan", "criterion", 9, 1), ("scan", "u_accept", 4096, 1),
+])
+def test_an_argument_error_of_any_step_is_found_before_the_first_launch(host, shape, step, field, value, code):
+    p = Args(**shape)
+    setattr(getattr(p, step), field, value)
+    n0 = ts.launch_count()
+    assert p.call(host) == code
+    assert ts.launch_count() == n0
+
+
+@pytest.mark.parametrize("B", [1, 4])
+def test_a_fused_pass_asks_for_the_attentions_workspace(B):
+    """The split plan of a long context merges through the workspace, whatever form the pass would take."""
+    p = Args(B=B, T=9, Hq=8, Hkv=1, cap=16384, V=151936)
+    assert p.attn.workspace_bytes > 0
+    p.attn.workspace_bytes -= 1
+    assert p.call(False) == 3 and p.call(True) == 3
+    p.attn.workspace_bytes += 1
+    p.attn.workspace = None
+    assert p.call(False) == 1
