@@ -130,21 +130,106 @@ struct PassPlan {
   int attn_ctas;
   bool in_turn;       // that attention takes the splits of its plan one after the other, in few CTAs
 };
-static PassPlan pass_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm, const trispec_scan_args* scan) {
+
+// The memory that one of the two streams of a pass reads and writes.
+class Footprint {
+ public:
+  void reads(const void* p, size_t bytes) { add(p, bytes, false); }
+  void writes(const void* p, size_t bytes) { add(p, bytes, true); }
+  bool clashes(const Footprint& o) const {
+    for (int i = 0; i < n_; ++i)
+      for (int j = 0; j < o.n_; ++j) {
+        const Span &a = span_[i], &b = o.span_[j];
+        if ((a.written || b.written) && a.at < b.at + b.bytes && b.at < a.at + a.bytes) return true;
+      }
+    return false;
+  }
+
+ private:
+  struct Span { uintptr_t at; size_t bytes; bool written; };
+  void add(const void* p, size_t bytes, bool written) {
+    if (p && bytes > 0 && n_ < kMax) span_[n_++] = {reinterpret_cast<uintptr_t>(p), bytes, written};
+  }
+  static constexpr int kMax = 48;     // 16 arrays on one side, 37 on the other
+  Span span_[kMax];
+  int n_ = 0;
+};
+
+// Whether the steps that would run beside each other share memory that one of them writes (a workspace used by both, an
+// escalation list written over the index list that the attention reads): in stream order that is no conflict.
+static bool pass_shares_memory(const trispec_tree_args* tree, const trispec_attn_args* attn, const trispec_lmhead_args* lm,
+                               const trispec_scan_args* scan) {
+  Footprint beside, main;
+  if (tree) {
+    const size_t n = static_cast<size_t>(tree->B) * tree->T;
+    beside.reads(tree->parent, n * 4);
+    beside.writes(tree->mask, n * 8);
+    beside.writes(tree->depth, n * 4);
+  }
+  {
+    const size_t B = attn->B, T = attn->T, Hq = attn->Hq, Hkv = attn->Hkv, D = attn->D;
+    const bool paged = attn->kv_layout == TRISPEC_KV_PAGED;
+    const size_t kv = (paged ? static_cast<size_t>(attn->num_blocks) * attn->block_size : B * attn->Lmax) * Hkv * D * 2;
+    beside.reads(attn->q, B * T * Hq * D * 2);
+    beside.reads(attn->k_tree, B * T * Hkv * D * 2);
+    beside.reads(attn->v_tree, B * T * Hkv * D * 2);
+    beside.reads(attn->k_cache, kv);
+    beside.reads(attn->v_cache, kv);
+    if (paged) beside.reads(attn->block_table, B * attn->max_blocks_per_seq * 4);
+    beside.reads(attn->ctx_len, B * 4);
+    beside.reads(attn->mask, B * T * 8);
+    if (attn->seq_index) beside.reads(attn->seq_index, static_cast<size_t>(attn->B_active) * 4);
+    beside.reads(attn->n_nodes, B * 4);
+    beside.writes(attn->o, B * T * Hq * D * 2);
+    beside.writes(attn->lse, B * T * Hq * 4);
+    beside.writes(attn->workspace, trispec_verify_attn_workspace(attn));
+  }
+  {
+    const size_t n = static_cast<size_t>(lm->B) * lm->T;
+    main.reads(lm->h, n * lm->d * 2);
+    main.reads(lm->W, static_cast<size_t>(lm->V) * lm->d * 2);
+    main.reads(lm->parent, n * 4);
+    main.reads(lm->tok, n * 4);
+    if (lm->seq_index) main.reads(lm->seq_index, static_cast<size_t>(lm->B_active) * 4);
+    const trispec_stats& o = lm->out;
+    const void* const out[11] = {o.max, o.lse, o.top1_val, o.top2_val, o.p_top1, o.p_top2, o.top1_idx, o.top2_idx,
+                                 o.draft_logit, o.p_draft, o.entropy};
+    for (const void* p : out) main.writes(p, n * 4);
+    const size_t need = trispec_lmhead_stats_workspace(lm);
+    main.writes(lm->workspace, need < lm->workspace_bytes ? need : lm->workspace_bytes);
+  }
+  if (scan) {
+    const size_t B = scan->B, n = B * scan->T;
+    const trispec_stats& in = scan->in;
+    const void* const by_node[9] = {scan->parent, scan->tok, scan->q_draft, scan->u_accept, in.top1_idx, in.p_top1,
+                                    in.p_top2, in.entropy, in.p_draft};
+    for (const void* p : by_node) main.reads(p, n * 4);
+    main.reads(scan->active, B);
+    main.reads(scan->start_node, B * 4);
+    const void* const by_sequence[5] = {scan->accept_len, scan->bonus_tok, scan->last_node, scan->near_thr, scan->esc_index};
+    for (const void* p : by_sequence) main.writes(p, B * 4);
+    main.writes(scan->path, n * 4);
+    main.writes(scan->escalate, B);
+    main.writes(scan->n_escalated, 4);
+    main.writes(scan->compact_scratch, (B + 65535) / 65536 * 4);
+  }
+  return beside.clashes(main) || (scan && scan->esc_index && attn->seq_index == scan->esc_index);
+}
+
+static PassPlan pass_plan(const trispec_tree_args* tree, const trispec_attn_args* attn, const trispec_lmhead_args* lm,
+                          const trispec_scan_args* scan) {
   PassPlan pl = {PASS_ATTENTION_FIRST, false, attn ? attn_planned_ctas(attn) : 0, false};
   const int lm_seqs = lm->seq_index ? lm->B_active : lm->B;
   if (!attn || pl.attn_ctas <= 0 || !lm_runs_small_rows(lm)) return pl;      // the pair kernel takes every SM
   const int sms = device_sm_count();
-  // not beside the scan when its escalation list is written over the index list the attention reads:
-  // in stream order the scan comes last, side by side it would not
-  const bool in_place_list = attn->seq_index && scan && scan->esc_index == attn->seq_index;
+  const bool in_order = pass_shares_memory(tree, attn, lm, scan);
   // TRISPEC_PASS_FORM = attention_first | lm_first | side_by_side overrides the rules below for so few
   // rows (a tuning and testing aid, read at every call; lm_first is then one after the other, and side by
   // side, with the attention's own plan, still needs at most SMs / 2 CTAs)
   if (const char* e = getenv("TRISPEC_PASS_FORM")) {
     if (e[0] == 'a') return pl;
     if (e[0] == 'l') { pl.form = PASS_LM_FIRST; return pl; }
-    if (e[0] == 's' && pl.attn_ctas * 2 <= sms && !in_place_list) { pl.form = PASS_SIDE_BY_SIDE; pl.beside = true; return pl; }
+    if (e[0] == 's' && pl.attn_ctas * 2 <= sms && !in_order) { pl.form = PASS_SIDE_BY_SIDE; pl.beside = true; return pl; }
   }
   // With so few rows the LM head is a pure stream of W that does not need every SM to saturate HBM, and the attention
   // a chain of tiles that does not need bandwidth: the attention runs beside the LM head in as FEW CTAs as it can,
@@ -153,14 +238,14 @@ static PassPlan pass_plan(const trispec_attn_args* attn, const trispec_lmhead_ar
   // sequence of 61 nodes, 4096 context tokens, 151936 x 2048 weights: 8 CTAs of 65 tiles beside 140 of the LM head
   // against 64 CTAs after all 148 of it.
   const double lm_us = static_cast<double>(lm->V) * lm->d * 2.0 / 6.0e6;
-  const int compact_ctas = in_place_list ? 0 : attn_compact_ctas(attn, 0.8 * lm_us, sms / 4);
+  const int compact_ctas = in_order ? 0 : attn_compact_ctas(attn, 0.8 * lm_us, sms / 4);
   if (lm_seqs == 1) {
     // Behind the attention the LM head would stall as a programmatic dependent, so for one sequence it goes first
     // whatever the form. What the form is called follows the attention's own plan: side by side where that could
     // be given one SM per CTA for less than about 40 us of the LM head's time, which then takes SMs / (SMs - CTAs)
     // times as long.
     const double own_lm_us = lm_us * 6.0 / 5.0;
-    const bool own_fits = pl.attn_ctas * 2 <= sms && !in_place_list && own_lm_us * pl.attn_ctas <= 40.0 * (sms - pl.attn_ctas);
+    const bool own_fits = pl.attn_ctas * 2 <= sms && !in_order && own_lm_us * pl.attn_ctas <= 40.0 * (sms - pl.attn_ctas);
     pl.form = own_fits ? PASS_SIDE_BY_SIDE : PASS_LM_FIRST;
     pl.beside = compact_ctas > 0 || own_fits;
   } else if (compact_ctas > 0) {
@@ -191,7 +276,7 @@ static int pass_check(const trispec_tree_args* tree, const trispec_attn_args* at
 extern "C" const char* trispec_verify_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm,
                                            const trispec_scan_args* scan) {
   if (!lm) return "none";
-  switch (trispec::pass_plan(attn, lm, scan).form) {
+  switch (trispec::pass_plan(nullptr, attn, lm, scan).form) {
     case trispec::PASS_LM_FIRST: return "lm_first";
     case trispec::PASS_SIDE_BY_SIDE: return "side_by_side";
     default: return "attention_first";
@@ -209,7 +294,7 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
   // LM head is a pure stream of W and loses more behind an attention than the hidden latency is worth (one
   // sequence of 4096 context tokens: 166 us against 156 us the other way round), so there the LM head goes
   // first, or the two run side by side (pass_plan above).
-  const trispec::PassPlan plan = trispec::pass_plan(attn, lm, scan);
+  const trispec::PassPlan plan = trispec::pass_plan(tree, attn, lm, scan);
   const bool lm_first = plan.form == trispec::PASS_LM_FIRST;
   int rc = trispec::pass_check(tree, attn, lm, scan, plan);
   if (rc != TRISPEC_OK) return rc;
@@ -275,7 +360,7 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
   // the copies below land in the buffers the structs name: they must describe one and the same pass
   if (tree->parent != lm->parent || tree->parent != scan->parent || lm->tok != scan->tok)
     return TRISPEC_ERR_INVALID_ARG;
-  const PassPlan plan = pass_plan(attn, lm, scan);
+  const PassPlan plan = pass_plan(tree, attn, lm, scan);
   int rc = pass_check(tree, attn, lm, scan, plan);
   if (rc != TRISPEC_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);

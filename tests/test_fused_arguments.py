@@ -71,3 +71,36 @@ def test_a_fused_pass_asks_for_the_attentions_workspace(B):
     p.attn.workspace_bytes += 1
     p.attn.workspace = None
     assert p.call(False) == 1
+
+
+@pytest.mark.parametrize("shape", [dict(), dict(B=4, listed=1), dict(B=3, V=151936)])
+def test_steps_that_share_written_memory_run_in_stream_order(shape):
+    in_order = "attention_first" if shape.get("B") == 3 else "lm_first"
+    p = Args(**shape)
+    assert p.form() == "side_by_side"
+    n = p.scan.B * 4
+    if p.attn.seq_index:
+        for at in (p.attn.seq_index, p.attn.seq_index - n + 4, p.attn.seq_index - 4):
+            p.scan.esc_index = at
+            assert p.form() == (in_order if at + n > p.attn.seq_index else "side_by_side"), at
+        p.scan.esc_index = p.attn.seq_index + 4                 # behind the one listed entry
+        assert p.form() == "side_by_side"
+    p.lm.workspace, keep = p.attn.o, p.lm.workspace
+    assert p.form() == in_order
+    p.lm.workspace = keep
+    p.scan.path, keep = p.attn.ctx_len, p.scan.path
+    assert p.form() == in_order
+    p.scan.path = keep
+    p.scan.last_node, keep = p.attn.mask + 8, p.scan.last_node
+    assert p.form() == in_order
+    p.scan.last_node = keep
+    assert p.form() == "side_by_side"
+
+
+def test_a_workspace_shared_by_the_attention_and_the_lm_head():
+    p = Args(B=1, T=9, Hq=8, Hkv=1, cap=8192)                   # 16 splits through the workspace, 16 CTAs
+    assert p.attn.workspace_bytes > 0 and p.form() == "side_by_side"
+    p.lm.workspace = p.attn.workspace
+    assert p.form() == "lm_first"
+    p.lm.workspace = p.attn.workspace + p.attn.workspace_bytes  # one buffer, one part each
+    assert p.form() == "side_by_side"

@@ -292,3 +292,33 @@ def test_host_buffer_pass_of_several_sequences(kw):
             assert_same_attention(p.snapshot(), want)
             for n, t in p.back.items():
                 assert torch.equal(t, p.out[n].cpu()), n
+
+
+@pytest.mark.parametrize("what", ["workspace", "list"])
+def test_pass_whose_steps_share_memory_runs_in_order(what):
+    """One workspace for both steps; the escalation list written one entry before the list that the attention reads."""
+    import torch
+    from paper_2601_23180_b200 import binding as ts
+    if what == "workspace":
+        p = Pass(T=9, Hq=8, Hkv=1, cap=8192, lens=[8000], V=32000)
+        ws = ts.alloc_workspace(max(p.attn_args.workspace_bytes, p.lm_args.workspace_bytes))
+        for a in (p.attn_args, p.lm_args):
+            a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+    else:
+        p = Pass(**dict(CHAINS, listed=[2, 0]))
+        buf = torch.tensor([-1, 2, 0, -1], dtype=torch.int32, device="cuda")
+        for a in (p.attn_args, p.lm_args):
+            a.seq_index = buf[1:].data_ptr()
+        p.scan_args.esc_index = buf.data_ptr()
+    want = None
+    for call in (p.separate, p.fused, p.fused, p.fused):
+        p.spoil()
+        if what == "list":
+            buf.copy_(torch.tensor([-1, 2, 0, -1], dtype=torch.int32))
+        call()
+        got = p.snapshot()
+        if want is not None:
+            assert_same_attention(got, want)
+        want = want or got
+    if what == "list":
+        assert int(p.out["n_escalated"].item()) == int((buf[:3] >= 0).sum().item())
