@@ -377,15 +377,22 @@ int trispec_sample_bonus(const trispec_sample_args* a, void* stream);
  * ------------------------------------------------------------------------------------- */
 int trispec_verify(const trispec_tree_args* tree, const trispec_attn_args* attn,
                    const trispec_lmhead_args* lm, const trispec_scan_args* scan, void* stream);
-/* How a pass with these arguments arranges its attention and its LM head (a diagnostic; host only,
- * nothing is launched; `attn` and `scan` may be NULL): "attention_first" (batches), "lm_first" or
- * "side_by_side" (at most 64 active rows (128 from 256 MiB of W on): the second-stream form described above where the LM head can
- * spare the attention's SMs). "lm_first" (one active sequence whose attention is planned for more SMs than that)
- * starts the LM head at once and runs the attention in fewer CTAs beside it, on the second stream as well, where it then
- * still ends before the LM head, and after it otherwise; "none" without `lm`. The environment variable
- * TRISPEC_PASS_FORM = attention_first | lm_first | side_by_side overrides the choice for at most 64 active rows (128 from 256 MiB of W on). */
+/* How a pass with these arguments arranges its attention and its LM head (diagnostics; host only,
+ * nothing is launched; `attn` and `scan` may be NULL; captured and eager passes are arranged alike).
+ * trispec_verify_plan: "attention_first" (batches); for at most 64 active rows (128 from 256 MiB of W
+ * on) also "side_by_side" (the LM head can spare the SMs of the attention) or "lm_first" (one active
+ * sequence whose attention is planned for more SMs than that: the LM head starts at once, the
+ * attention runs in few CTAs beside it where it then still ends in time, and after it otherwise);
+ * "none" without `lm`. The environment variable TRISPEC_PASS_FORM = attention_first | lm_first |
+ * side_by_side overrides the choice for so few rows.
+ * trispec_verify_beside: the number of CTAs in which the attention runs on the second stream, beside
+ * the LM head, or 0 where the steps run in stream order. Memory that a step shares with the `tree`
+ * of the call, and a second stream that is not to be had, are the only reasons to run in stream
+ * order that these answers do not see. */
 const char* trispec_verify_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm,
                                 const trispec_scan_args* scan);
+int trispec_verify_beside(const trispec_attn_args* attn, const trispec_lmhead_args* lm,
+                          const trispec_scan_args* scan);
 
 /* ---------------------------------------------------------------------------------------
  * The same pass for callers whose per-round data lives in HOST memory (one verification

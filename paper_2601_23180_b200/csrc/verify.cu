@@ -241,9 +241,9 @@ static PassPlan pass_plan(const trispec_tree_args* tree, const trispec_attn_args
   const int compact_ctas = in_order ? 0 : attn_compact_ctas(attn, 0.8 * lm_us, sms / 4);
   if (lm_seqs == 1) {
     // Behind the attention the LM head would stall as a programmatic dependent, so for one sequence it goes first
-    // whatever the form. What the form is called follows the attention's own plan: side by side where that could
-    // be given one SM per CTA for less than about 40 us of the LM head's time, which then takes SMs / (SMs - CTAs)
-    // times as long.
+    // whatever the form. The attention's own plan runs side by side where it can be given one SM per CTA for less
+    // than about 40 us of the LM head's time, which then takes SMs / (SMs - CTAs) times as long. (Where only its form
+    // in few CTAs does, the pass still is called LM head first.)
     const double own_lm_us = lm_us * 6.0 / 5.0;
     const bool own_fits = pl.attn_ctas * 2 <= sms && !in_order && own_lm_us * pl.attn_ctas <= 40.0 * (sms - pl.attn_ctas);
     pl.form = own_fits ? PASS_SIDE_BY_SIDE : PASS_LM_FIRST;
@@ -281,6 +281,12 @@ extern "C" const char* trispec_verify_plan(const trispec_attn_args* attn, const 
     case trispec::PASS_SIDE_BY_SIDE: return "side_by_side";
     default: return "attention_first";
   }
+}
+
+extern "C" int trispec_verify_beside(const trispec_attn_args* attn, const trispec_lmhead_args* lm, const trispec_scan_args* scan) {
+  if (!lm) return 0;
+  const trispec::PassPlan plan = trispec::pass_plan(nullptr, attn, lm, scan);
+  return plan.beside ? plan.attn_ctas : 0;
 }
 
 extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_args* attn,

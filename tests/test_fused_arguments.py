@@ -104,3 +104,23 @@ def test_a_workspace_shared_by_the_attention_and_the_lm_head():
     assert p.form() == "lm_first"
     p.lm.workspace = p.attn.workspace + p.attn.workspace_bytes  # one buffer, one part each
     assert p.form() == "side_by_side"
+
+
+@pytest.mark.parametrize("shape,form,ctas", [
+    (dict(), "side_by_side", 16),                                            # the attention's own 8 x 2 splits
+    (dict(V=151936), "side_by_side", 8),                                     # a long W: one CTA per KV head
+    (dict(T=61, cap=4096, V=151936), "lm_first", 8),                         # 8 x 8 splits in turn
+    (dict(T=61, cap=8192, V=151936), "lm_first", 0),                         # 16 splits through the workspace
+    (dict(T=61, Hq=64, cap=8192, d=5120, V=151936), "lm_first", 32),
+    (dict(B=3, V=151936), "side_by_side", 24),
+    (dict(B=2, T=61, cap=704, V=151936), "side_by_side", 16),
+    (dict(B=8, T=61, cap=4096, V=151936), "attention_first", 0),
+    (dict(B=12, T=5, listed=9, cap=256, V=151936), "attention_first", 0),    # 72 CTAs
+])
+def test_the_plan_tells_what_runs_beside_the_lm_head(shape, form, ctas):
+    p = Args(**shape)
+    assert p.form() == form
+    assert ts.trispec_verify_beside(p.attn, p.lm, p.scan) == ctas
+    p.scan.path = p.attn.ctx_len
+    assert ts.trispec_verify_beside(p.attn, p.lm, p.scan) == 0
+    assert ts.trispec_verify_beside(None, p.lm, p.scan) == 0

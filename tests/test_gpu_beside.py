@@ -148,7 +148,12 @@ def assert_same_attention(got, want):
 ])
 def test_fused_pass_gives_the_attentions_own_bits(kw):
     import torch
+    from paper_2601_23180_b200 import binding as ts
     p = Pass(**kw)
+    per_tile = min(64, 128 * kw["Hkv"] // kw["Hq"])
+    ctas = len(p.seqs) * kw["Hkv"] * ((kw["T"] + per_tile - 1) // per_tile)
+    items = ctas if kw["cap"] <= 4096 and ctas <= 148 // 4 else 0
+    assert ts.trispec_verify_beside(p.attn_args, p.lm_args, p.scan_args) == items
     p.spoil()
     p.separate()
     want = p.snapshot()
