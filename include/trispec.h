@@ -65,7 +65,8 @@ typedef enum {
   TRISPEC_ERR_TOO_LARGE = 8,       /* problem needs more than the library's built-in scratch */
   TRISPEC_ERR_NO_ROOM = 9,         /* dev_status: a KV commit would exceed a sequence's capacity; skipped */
   TRISPEC_ERR_BAD_LENGTH = 10,     /* dev_status: ctx_len[b] outside [0, capacity], clamped to it */
-  TRISPEC_ERR_BAD_TREE = 11        /* dev_status: parent[] of some sequence is not a tree (see entry 1) */
+  TRISPEC_ERR_BAD_TREE = 11,       /* dev_status: parent[] of some sequence is not a tree (see entry 1) */
+  TRISPEC_ERR_BAD_INDEX = 12       /* dev_status: seq_index entry outside [0, B), nothing is computed for it */
 } trispec_status;
 
 #define TRISPEC_MODE_PROXY 0   /* margin rule of Eq. 8-9 applied (proxy verifier) */
@@ -120,7 +121,8 @@ int trispec_build_tree_mask(const trispec_tree_args* a, void* stream);
  *    ctx_len [B] int32, 0 <= ctx_len[b] <= Lmax (contiguous) or 64 * max_blocks_per_seq; a
  *      value outside that range is clamped to it and dev_status receives TRISPEC_ERR_BAD_LENGTH.
  *    seq_index (optional, int32 [B_active], device): only these sequences are computed;
- *      NULL = all B (then B_active is ignored).
+ *      NULL = all B (then B_active is ignored). An entry outside [0, B) is skipped and
+ *      dev_status receives TRISPEC_ERR_BAD_INDEX.
  *    lse (optional) f32 [B][Hq][T]: log-sum-exp of the scaled scores.
  *    n_nodes (optional, int32 [B], device): sequence b has only its first n_nodes[b] tree
  *      nodes (a pruned tree: n_keep of trispec_prune_tree, the branches that are passed on to

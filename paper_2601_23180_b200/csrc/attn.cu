@@ -64,16 +64,18 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
   const int mtile = idx % p.n_mt; idx /= p.n_mt;
   const int g = idx % p.Hkv;
   const int a = idx / p.Hkv;
-  const int b = p.seq_index ? __ldg(p.seq_index + a) : a;
+  // a sequence that does not exist has no nodes: its CTAs do nothing
+  const int listed = attn_sequence(p.seq_index, a, p.B), b = max(listed, 0);
+  if (listed < 0 && threadIdx.x == 0 && p.dev_status) atomicExch(p.dev_status, TRISPEC_ERR_BAD_INDEX);
   // a length outside [0, capacity] (a stale or corrupt entry) is clamped and flagged: the block
   // table row and the cache are never read past their ends
-  int L = __ldg(p.ctx_len + b);
+  int L = listed < 0 ? 0 : __ldg(p.ctx_len + b);
   if (L < 0 || L > p.Lcap) {
     if (threadIdx.x == 0 && p.dev_status) atomicExch(p.dev_status, TRISPEC_ERR_BAD_LENGTH);
     L = max(0, min(L, p.Lcap));
   }
   // a pruned tree has fewer nodes: rows past them are not computed, M tiles past them do nothing
-  const int nn = p.n_nodes ? max(0, min(p.T, __ldg(p.n_nodes + b))) : p.T;
+  const int nn = listed < 0 ? 0 : (p.n_nodes ? max(0, min(p.T, __ldg(p.n_nodes + b))) : p.T);
   const int n_ctx_tiles = (L + AT_BN - 1) / AT_BN;
   // every sequence spreads its own context tiles evenly over the splits, so that the CTAs that
   // merge with each other finish together whatever the sequence's length
@@ -675,7 +677,7 @@ verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_
 // Merge of the KV splits: one warp per output row (sequence, node, query head).
 // ---------------------------------------------------------------------------------------
 struct AttnMergeParams {
-  int T, Hq, Hkv, G, NPT, n_mt, n_splits, n_seq, Lcap;
+  int B, T, Hq, Hkv, G, NPT, n_mt, n_splits, n_seq, Lcap;
   const int32_t *ctx_len, *seq_index, *n_nodes;
   const float *part_o, *part_ml;
   uint16_t* o;   // bf16 [B][T][Hq][128]
@@ -693,7 +695,8 @@ verify_attn_merge_kernel(const AttnMergeParams p) {
   const int hq = static_cast<int>(w % p.Hq);
   const int node = static_cast<int>((w / p.Hq) % p.T);
   const int a = static_cast<int>(w / (static_cast<long long>(p.Hq) * p.T));
-  const int b = p.seq_index ? __ldg(p.seq_index + a) : a;
+  const int b = attn_sequence(p.seq_index, a, p.B);
+  if (b < 0) return;
   if (p.n_nodes && node >= __ldg(p.n_nodes + b)) return;   // not a node of this (pruned) tree
   const int g = hq / p.G, j = hq % p.G;
   const int mtile = node / p.NPT;
@@ -953,7 +956,7 @@ extern "C" int trispec_verify_attn(const trispec_attn_args* a, void* stream) {
   rc = ensure_smem_limit(reinterpret_cast<const void*>(kernel), smem_bytes, smem_set[which]);
   if (rc != TRISPEC_OK) return rc;
   AttnParams p;
-  p.T = a->T; p.Hq = a->Hq; p.Hkv = a->Hkv; p.G = pl.G; p.NPT = pl.NPT; p.n_mt = pl.n_mt;
+  p.B = a->B; p.T = a->T; p.Hq = a->Hq; p.Hkv = a->Hkv; p.G = pl.G; p.NPT = pl.NPT; p.n_mt = pl.n_mt;
   p.n_splits = pl.n_splits;
   p.paged = (a->kv_layout == TRISPEC_KV_PAGED); p.max_blocks_per_seq = a->max_blocks_per_seq;
   p.num_blocks = a->num_blocks;
@@ -991,7 +994,7 @@ extern "C" int trispec_verify_attn(const trispec_attn_args* a, void* stream) {
   count_launch();
 
   AttnMergeParams m;
-  m.T = a->T; m.Hq = a->Hq; m.Hkv = a->Hkv; m.G = pl.G; m.NPT = pl.NPT; m.n_mt = pl.n_mt;
+  m.B = a->B; m.T = a->T; m.Hq = a->Hq; m.Hkv = a->Hkv; m.G = pl.G; m.NPT = pl.NPT; m.n_mt = pl.n_mt;
   m.n_splits = pl.n_splits; m.n_seq = pl.n_seq; m.Lcap = p.Lcap;
   m.ctx_len = a->ctx_len; m.seq_index = a->seq_index; m.n_nodes = a->n_nodes;
   m.part_o = p.part_o; m.part_ml = p.part_ml;

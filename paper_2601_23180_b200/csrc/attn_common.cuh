@@ -42,7 +42,7 @@ constexpr int AT_TURN_SMEM_BYTES = AT_TURN_SMEM_USED + 1024;
 static_assert(AT_TURN_SMEM_BYTES <= 227 * 1024 && AT_TURN_PART_BYTES <= AT_STAGES * AT_TILE_BYTES, "in-turn partials");
 
 struct AttnParams {
-  int T, Hq, Hkv, G, NPT, n_mt, n_splits;
+  int B, T, Hq, Hkv, G, NPT, n_mt, n_splits;
   int paged, max_blocks_per_seq, num_blocks;
   int Lcap;         // capacity of a sequence's context: Lmax, or 64 x max_blocks_per_seq
   float scale_log2;
@@ -59,6 +59,12 @@ struct AttnParams {
   int n_seq;        // active sequences (at most 128)
   int n_cta;        // CTAs of the launch: CTA c walks tiles [c W / n_cta, (c + 1) W / n_cta) of the work
 };
+
+// Entry a of the index list (or a itself); one outside [0, B) is -1.
+__device__ __forceinline__ int attn_sequence(const int32_t* seq_index, int a, int B) {
+  const int b = seq_index ? __ldg(seq_index + a) : a;
+  return static_cast<unsigned>(b) < static_cast<unsigned>(B) ? b : -1;
+}
 
 __device__ __forceinline__ uint4 ld_cluster_u4(uint32_t addr) {
   uint4 v;

@@ -49,13 +49,15 @@ __device__ __forceinline__ WorkMap load_work_map(const AttnParams& p, int lane, 
     const int a = j * 32 + lane;
     int L = 0, nn = 0;
     if (a < p.n_seq) {
-      const int b = p.seq_index ? __ldg(p.seq_index + a) : a;
-      L = __ldg(p.ctx_len + b);
+      // a sequence that does not exist has no nodes, hence no steps
+      const int listed = attn_sequence(p.seq_index, a, p.B), b = max(listed, 0);
+      if (listed < 0 && flag_bad && p.dev_status) atomicExch(p.dev_status, TRISPEC_ERR_BAD_INDEX);
+      L = listed < 0 ? 0 : __ldg(p.ctx_len + b);
       if (L < 0 || L > p.Lcap) {
         if (flag_bad && p.dev_status) atomicExch(p.dev_status, TRISPEC_ERR_BAD_LENGTH);
         L = max(0, min(L, p.Lcap));
       }
-      nn = p.n_nodes ? max(0, min(p.T, __ldg(p.n_nodes + b))) : p.T;
+      nn = listed < 0 ? 0 : (p.n_nodes ? max(0, min(p.T, __ldg(p.n_nodes + b))) : p.T);
     }
     w.L[j] = L;
     w.nn[j] = nn;

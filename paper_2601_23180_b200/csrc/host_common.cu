@@ -137,6 +137,7 @@ extern "C" const char* trispec_status_string(int s) {
     case TRISPEC_ERR_NO_ROOM: return "no room in the KV cache for the committed rows (device status)";
     case TRISPEC_ERR_BAD_LENGTH: return "context length out of range (device status)";
     case TRISPEC_ERR_BAD_TREE: return "parent array is not a tree (device status)";
+    case TRISPEC_ERR_BAD_INDEX: return "sequence index out of range (device status)";
     case TRISPEC_ERR_TOO_LARGE: return "problem exceeds the built-in scratch of the no-allocation entry point";
     default: return "unknown status";
   }

@@ -397,14 +397,16 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
 // Packs the activation rows of the active sequences (an index list) without gaps: one warp per row. Beside the stream
 // of W it is small: 3 sequences of 61 rows of 5120 are 1.9 MB.
 __global__ void __launch_bounds__(256)
-lmhead_pack_rows_kernel(const uint4* __restrict__ h, const int32_t* __restrict__ seq_index, uint4* __restrict__ out, int T,
+lmhead_pack_rows_kernel(const uint4* __restrict__ h, const int32_t* __restrict__ seq_index, uint4* __restrict__ out, int B, int T,
                         int vecs /* 16-byte words per row */, long long n_rows) {
   pdl_launch_dependents();
   const int lane = threadIdx.x & 31;
   const long long r = static_cast<long long>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   const bool active = r < n_rows;
   const int a = active ? static_cast<int>(r / T) : 0;
-  const uint4* src = h + (static_cast<long long>(__ldg(seq_index + a)) * T + (active ? r % T : 0)) * vecs;
+  const int seq = __ldg(seq_index + a);
+  const bool there = static_cast<unsigned>(seq) < static_cast<unsigned>(B);   // (finalize skips a sequence that is not)
+  const uint4* src = h + (static_cast<long long>(there ? seq : 0) * T + (active ? r % T : 0)) * vecs;
   pdl_wait();
   if (!active) return;
   uint4* dst = out + r * vecs;
@@ -416,7 +418,7 @@ lmhead_pack_rows_kernel(const uint4* __restrict__ h, const int32_t* __restrict__
 // Merge of the per-range partials + drafted-token logits.
 // ---------------------------------------------------------------------------------------
 struct LmFinalizeParams {
-  int T, d, V, n_ranges;
+  int B, T, d, V, n_ranges;
   int stride;       // partial rows per vocabulary range
   int pitch;        // partial rows per active sequence (T: packed rows)
   float scale, c;
@@ -424,6 +426,7 @@ struct LmFinalizeParams {
   const LmPartial* partial;
   const uint16_t *h, *W;
   const int32_t *parent, *tok;
+  int32_t* dev_status;
   trispec_stats out;
 };
 
@@ -446,9 +449,14 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
   const int lane = threadIdx.x & 31;
   const long long w = static_cast<long long>(blockIdx.x) * (LM_FIN_THREADS / 32) + (threadIdx.x >> 5);
   const int T = p.T;
-  const bool active = w < static_cast<long long>(n_seq) * T;
+  bool active = w < static_cast<long long>(n_seq) * T;
   const int a = active ? static_cast<int>(w / T) : 0, node = active ? static_cast<int>(w % T) : 0;
-  const int seq = p.seq_index ? __ldg(p.seq_index + a) : a;
+  int seq = p.seq_index ? __ldg(p.seq_index + a) : a;
+  if (static_cast<unsigned>(seq) >= static_cast<unsigned>(p.B)) {   // no such sequence: its rows are computed and dropped
+    if (active && lane == 0 && p.dev_status) atomicExch(p.dev_status, TRISPEC_ERR_BAD_INDEX);
+    active = false;
+    seq = 0;
+  }
   const long long row0 = static_cast<long long>(seq) * T;
 
   // ---- drafted-token logit z[parent(node)][tok[node]]: inputs only
@@ -1044,13 +1052,13 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   // the entropy sum costs two more instructions per logit: only computed when it is asked for
   const bool want_entropy = a->out.entropy != nullptr;
   LmFinalizeParams f;
-  f.T = a->T; f.d = a->d; f.V = a->V; f.n_ranges = n_ranges + pl.n_tail;
+  f.B = a->B; f.T = a->T; f.d = a->d; f.V = a->V; f.n_ranges = n_ranges + pl.n_tail;
   f.scale = a->logit_scale; f.c = a->logit_scale * kLog2e;
   f.seq_index = a->seq_index;
   f.partial = static_cast<LmPartial*>(a->workspace);
   f.h = static_cast<const uint16_t*>(a->h);
   f.W = static_cast<const uint16_t*>(a->W);
-  f.parent = a->parent; f.tok = a->tok;
+  f.parent = a->parent; f.tok = a->tok; f.dev_status = a->dev_status;
   f.out = a->out;
   f.pitch = pl.slots ? 64 : (pl.slot_rows > 0 ? pl.slot_rows : a->T);
 
@@ -1072,7 +1080,7 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
     uint4* packed = reinterpret_cast<uint4*>(static_cast<char*>(a->workspace) + pl.required);
     rows_base = packed;
     TRISPEC_CUDA_OK(launch_dependent(lmhead_pack_rows_kernel, static_cast<unsigned>((n_rows + 7) / 8), 256, 0, st, 1,
-                                     static_cast<const uint4*>(a->h), a->seq_index, packed, a->T, a->d / 8, n_rows));
+                                     static_cast<const uint4*>(a->h), a->seq_index, packed, a->B, a->T, a->d / 8, n_rows));
     count_launch();
   }
   if (pl.few_rows) {

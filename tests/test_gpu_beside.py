@@ -37,7 +37,7 @@ class Pass:
         self.parent = i32([[-1] + [(7 * i + 3 * b) % i for i in range(1, T)] for b in range(B)])
         self.tok = torch.randint(0, V, (B, T), generator=g, device="cuda", dtype=torch.int32)
         self.W, self.h = normal(V, d).mul_(0.02), normal(B, T, d)
-        self.seqs = list(range(B)) if listed is None else listed
+        self.seqs = list(range(B)) if listed is None else [x for x in listed if 0 <= x < B]
         self.index = None if listed is None else i32(listed)
         self.nodes = None if n_nodes is None else i32(n_nodes)
         self.n_nodes = n_nodes or [T] * B
@@ -97,10 +97,10 @@ class Pass:
                 t.zero_()
         ts.trispec_verify_host(self.io, self.tree_args, self.attn_args, self.lm_args, self.scan_args, stream)
 
-    def snapshot(self):
+    def snapshot(self, status=0):
         import torch
         torch.cuda.synchronize()
-        assert int(self.status.item()) == 0
+        assert int(self.status.item()) == status
         return dict(o=self.o.view(torch.int16).clone(), lse=self.lse.view(torch.int32).clone(), mask=self.mask.clone(),
                     **{"s_" + k: v.clone() for k, v in self.stats.items()}, **{"d_" + k: v.clone() for k, v in self.out.items()})
 
@@ -327,3 +327,58 @@ def test_pass_whose_steps_share_memory_runs_in_order(what):
         want = want or got
     if what == "list":
         assert int(p.out["n_escalated"].item()) == int((buf[:3] >= 0).sum().item())
+
+
+@pytest.mark.parametrize("kw,plan,room", [
+    (dict(T=9, Hq=32, Hkv=8, cap=256, lens=[256, 100, 31, 200], listed=[2, -1, 0, 4], V=40000), None, "full"),
+    (dict(T=6, Hq=8, Hkv=1, cap=256, lens=[200] * 12, listed=[11, -1, 0, 7, 5, 12, 9, 2, -7, 4], V=60000), None, "full"),
+    (dict(T=6, Hq=8, Hkv=1, cap=256, lens=[200] * 12, listed=[11, -1, 0, 7, 5, 12, 9, 2, -7, 4], V=60000), None, "slots"),
+    (dict(T=30, Hq=16, Hkv=8, cap=700, lens=[700] * 12, listed=[11, -1, 0, 7, 5, 12, 9, 2, 1 << 30, 4], d=192, V=3001),
+     None, "full"),
+    (dict(T=61, Hq=64, Hkv=8, cap=4096, lens=[4000] * 4, listed=[3, -1, 1], d=192, V=3001, target=True), "splits", "full"),
+    (dict(T=30, Hq=16, Hkv=8, cap=700, lens=[700] * 4, listed=[3, -1, 1, 4], d=192, V=3001), "pieces", "full"),
+], ids=["beside", "gathered", "slots", "packed", "workspace", "pieces"])
+def test_listed_sequences_that_do_not_exist_are_skipped_and_reported(kw, plan, room, monkeypatch):
+    import torch
+    from paper_2601_23180_b200 import binding as ts
+    if plan:
+        monkeypatch.setenv("TRISPEC_ATTN_PLAN", plan)
+    good = Pass(**dict(kw, listed=[x for x in kw["listed"] if 0 <= x < len(kw["lens"])]))
+    p = Pass(**kw)
+    if plan:
+        assert ts.trispec_verify_attn_plan(p.attn_args) == plan
+    if room == "slots":
+        p.lm_args.workspace_bytes -= len(kw["listed"]) * kw["T"] * 2048 * 2
+    want = _want(good)
+    for call in (p.separate, p.fused):
+        p.spoil()
+        p.status.zero_()
+        call()
+        p.snapshot(status=12)
+        for b in range(p.B):
+            if b not in p.seqs:                        # as spoil() left them
+                assert torch.isnan(p.o[b].float()).all() and (p.stats["lse"][b] == 0).all()
+                continue
+            x, y = p.o[b].float(), p.attention64(b).float()
+            # two bf16 steps of outputs of at most about 4, as in the parity tests
+            assert (x - y).abs().max().item() <= 2e-2
+            assert (p.stats["lse"][b] - good.stats["lse"][b]).abs().max().item() <= 1e-4
+            assert torch.equal(p.stats["top1_idx"][b], want["s_top1_idx"][b])
+            assert torch.equal(p.out["path"][b], want["d_path"][b])
+
+
+@pytest.mark.parametrize("kw", [CHAINS, dict(T=61, Hq=16, Hkv=8, cap=4096, lens=[3000], paged=True)])
+def test_stochastic_pass_beside(kw):
+    import torch
+    from paper_2601_23180_b200 import binding as ts
+    p = Pass(**kw)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    q = torch.rand(p.B, p.T, generator=g, device="cuda") * 1e-4 + 1e-6
+    u = torch.rand(p.B, p.T, generator=g, device="cuda")
+    p.scan_args = ts.scan_args(p.stats, p.parent, p.tok, 0.0, ts.MODE_PROXY, p.out, active=p.active, q_draft=q, u_accept=u)
+    want = _want(p)
+    for _ in range(3):
+        p.spoil()
+        p.fused()
+        assert_same_attention(p.snapshot(), want)
