@@ -46,11 +46,7 @@ class SideLease {
   explicit SideLease(cudaStream_t st) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
-    // looking a stream over, and making one, must not disturb a capture of another thread's
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
     take(pools()[dev], st);
-    cudaThreadExchangeStreamCaptureMode(&mode);
     if (s_) s_->enqueue.lock();
   }
   ~SideLease() {
@@ -80,6 +76,22 @@ class SideLease {
     if (status == cudaStreamCaptureStatusNone) *id = 0;
     return status != cudaStreamCaptureStatusInvalidated;
   }
+  // a set that belongs to nobody yet, or the one of those whose work is done that was taken the longest ago
+  static SideStream* fresh(SidePool& pool) {
+    SideStream* got = nullptr;
+    unsigned long long theirs = 0;
+    for (SideStream& s : pool.set) {
+      if (!s.made) {
+        if (side_make(&s)) return &s;
+        cudaGetLastError();
+        return nullptr;
+      }
+      if (s.users > 0 || (got && got->used < s.used) || !capture_of(s.stream, &theirs) || theirs != 0) continue;
+      if (cudaStreamQuery(s.stream) == cudaSuccess) got = &s;
+      else cudaGetLastError();
+    }
+    return got;
+  }
   void take(SidePool& pool, cudaStream_t st) {
     unsigned long long capture = 0, theirs = 0;
     static thread_local char per_thread;       // (one handle stands for every thread's default stream)
@@ -94,20 +106,12 @@ class SideLease {
         got = &s;
         break;
       }
-    for (int i = 0; i < kSideStreams && !got; ++i)
-      if (!pool.set[i].made) {
-        if (!side_make(&pool.set[i])) {
-          cudaGetLastError();
-          return;
-        }
-        got = &pool.set[i];
-      }
     if (!got) {
-      for (SideStream& s : pool.set) {
-        if (s.users > 0 || (got && got->used < s.used) || !capture_of(s.stream, &theirs) || theirs != 0) continue;
-        if (cudaStreamQuery(s.stream) == cudaSuccess) got = &s;
-        else cudaGetLastError();
-      }
+      // making a stream, and asking one for its state, must not disturb a capture of this or another thread's
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      got = fresh(pool);
+      cudaThreadExchangeStreamCaptureMode(&mode);
       if (!got) return;
     }
     got->owner = id;

@@ -229,7 +229,16 @@ def test_captured_pass_beside_an_eager_one(kw):
     torch.cuda.synchronize()
     p.fused(sp)                                    # the stream's second stream is usable again after the capture
     assert_same_attention(p.snapshot(), want_p)
-    del graph
+    first = torch.cuda.CUDAGraph()
+    fresh = torch.cuda.Stream()                    # a stream that the library meets under capture
+    with torch.cuda.graph(first, stream=fresh):
+        p.fused(fresh)
+    p.spoil()
+    torch.cuda.synchronize()
+    first.replay()
+    graph.replay()
+    assert_same_attention(p.snapshot(), want_p)
+    del graph, first
 
 
 def test_more_busy_streams_than_second_streams():
