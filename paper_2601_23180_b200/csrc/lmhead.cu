@@ -13,9 +13,9 @@
 //   N tile  = 256 vocabulary entries, plus one narrower tile (a multiple of 32) for the rest of
 //             the CTA pair's vocabulary range; each CTA loads one half of a tile
 //   K block = 64 bf16 = one 128-byte swizzle row; 4 MMAs of K = 16 per block
-//   Per k-block a CTA stages its own 128 rows of H (16 KB) and half of the W tile (16 KB):
-//   32 KB for 128 x 256 x 64 multiply-adds per SM, against 48 KB when every SM works
-//   alone. The pipeline is bound by how fast W tiles reach shared memory, so this is what
+//   Per k-block a CTA stages its own half of the M tile's rows of H (up to 128, 16 KB) and half
+//   of the W tile (16 KB): 32 KB for 128 x 256 x 64 multiply-adds per SM, against 48 KB when
+//   every SM works alone. The pipeline is bound by how fast W tiles reach shared memory, so this is what
 //   lifts the tensor-core duty cycle.
 //   warps 0-3: epilogue (one TMEM lane = one row per thread), warp 4: TMA producer,
 //   warp 5: TMEM owner; in the leader CTA (cluster rank 0) one of its threads issues the
@@ -567,8 +567,8 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
 }
 
 // ---------------------------------------------------------------------------------------
-// At most 64 rows, and at most 128 over a long W (batch-1 decoding, the paper's own setting; two trees; a batch of chains): operands swapped. With so
-// few rows the GEMM is bound by streaming W, and the pair kernel above spends half of its ring
+// At most 64 columns, and at most 128 over a long W (batch-1 decoding, the paper's own setting; two trees; a batch of
+// chains): operands swapped. With so few rows the GEMM is bound by streaming W, and the pair kernel above spends half of its ring
 // on H tiles. Here W is the M-side operand, the rows are the N side (16-128 columns), and one CTA per SM takes one
 // vocabulary range. A tile is up to 2 x 128 vocabulary entries, two MMAs that share the k-block of H: a stage is
 // 32 KB of W and 2-16 KB of H, so that up to 160 KB of W are in flight per SM and H, which every SM reads, adds 25 %
@@ -583,7 +583,8 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
 constexpr int LW_BM = 128, LW_SUBS = 2, LW_BK = 64, LW_MAX_STAGES = 6, LW_EPI_WARPS = 8;
 constexpr int LW_THREADS = 32 * (LW_EPI_WARPS + 2);
 constexpr int LW_A_BYTES = LW_SUBS * LW_BM * LW_BK * 2;  // 32 KB of W per stage
-constexpr int lw_rows(long long n_rows) { return n_rows <= 64 ? 64 : static_cast<int>((n_rows + 15) / 16 * 16); }   // partial rows per range
+// partial rows per vocabulary range
+constexpr int lw_rows(long long n_rows) { return n_rows <= 64 ? 64 : static_cast<int>((n_rows + 15) / 16 * 16); }
 constexpr int LW_XPOSE_BYTES = 2048;                     // 32 entries x 16 columns per epilogue warp
 constexpr int LW_SMEM_BYTES = 227 * 1024;
 constexpr int LW_RING_BYTES = LW_SMEM_BYTES - 1024 /*alignment slack*/ - LW_EPI_WARPS * LW_XPOSE_BYTES - 256 /*barriers*/;
@@ -732,7 +733,8 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
           for (int u = 0; u < LW_SUBS; ++u) {
             const uint64_t adesc = smem_desc_sw128(sa + u * (LW_A_BYTES / 2), 1024, 16);
 #pragma unroll
-            for (int k = 0; k < LW_BK / 16; ++k) tc_mma_ss(d_tmem + static_cast<uint32_t>(kRows) * u, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0);
+            for (int k = 0; k < LW_BK / 16; ++k)
+              tc_mma_ss(d_tmem + static_cast<uint32_t>(kRows) * u, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0);
           }
           tc_commit(empty_bar + stage);
           if (++stage == sp.stages) { stage = 0; phase ^= 1u; }
@@ -871,7 +873,9 @@ struct LmPlan {
 // W is streamed from HBM for long enough (about twice L2) that what happens before and after it matters less
 static bool lm_long_stream(const trispec_lmhead_args* a) { return static_cast<long long>(a->V) * a->d * 2 >= (256ll << 20); }
 
-static bool lm_takes_few_rows(const trispec_lmhead_args* a, long long rows) { return rows <= (lm_long_stream(a) ? LM_FEW_ROWS : 64); }
+static bool lm_takes_few_rows(const trispec_lmhead_args* a, long long columns) {
+  return columns <= (lm_long_stream(a) ? LM_FEW_ROWS : 64);
+}
 
 static int lm_ranges_within(size_t max_ws, int part_rows, int ranges) {
   const size_t fit = max_ws / (static_cast<size_t>(part_rows) * sizeof(LmPartial));
