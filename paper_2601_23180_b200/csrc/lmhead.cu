@@ -98,11 +98,13 @@ struct TileIter {
 
 // What a CTA pair works on. A main pair computes one M tile over one vocabulary range (one sweep). When
 // the M tiles do not divide the pairs of the chip, the pairs left over take the tail of the vocabulary:
-// each of them sweeps all M tiles, one after the other, over its own slice of that tail, which is
-// short enough to stay in L2 between the sweeps; the main ranges shrink accordingly, so that every
+// each of them takes all M tiles over its own slice of that tail, one W tile after the other and on each of them one M tile
+// after the other, so that W comes from HBM once (M tile by M tile the slices, 84 MB with 16 M tiles, did not stay in L2
+// beside the main stream: 2.05 GB of DRAM reads for 0.64, an eighth of the energy of a launch that runs at the power limit;
+// 3904 rows, 151936 x 2048 weights: 1862 -> 1780 us). The main ranges shrink accordingly, so that every
 // pair of the chip runs about the same number of tiles.
 struct PairWork {
-  int n_sweeps, mt0, part;      // M tile of sweep s = mt0 + s; `part` = row block of the partial array
+  int n_sweeps, mt0, part;      // M tiles mt0 .. mt0 + n_sweeps - 1; `part` = row block of the partial array
   TileIter tiles;
   __device__ PairWork(const LmParams& p, int pair)
       : n_sweeps(1), mt0(0), part(0), tiles(0, 0, 1, 0) {
@@ -205,9 +207,12 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
       int stage = 0;
       uint32_t phase = 0;
       if (p.wait_rows) pdl_wait();
-      for (int sweep = 0; sweep < work.n_sweeps; ++sweep) {
       // the rows are spread evenly over the M tiles, and only those that a tile has are fetched
       const int half_rows = p.tile_rows >> 1;
+      for (int t = 0; t < tiles.n_tiles; ++t) {
+      int n0, nw;
+      tiles.tile(t, n0, nw);
+      for (int sweep = 0; sweep < work.n_sweeps; ++sweep) {
       const int row0 = (work.mt0 + sweep) * p.tile_rows + static_cast<int>(rank) * half_rows;
       int s0 = 0, s1 = 0;
       if (p.slots) {
@@ -221,9 +226,6 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
         s0 = __ldg(p.seq_index + a0);
         s1 = __ldg(p.seq_index + a1);
       }
-      for (int t = 0; t < tiles.n_tiles; ++t) {
-        int n0, nw;
-        tiles.tile(t, n0, nw);
         const int nh = nw >> 1;                   // rows of W this CTA stages
         const int nbox = (nh + 63) >> 6;
         const int w0 = n0 + static_cast<int>(rank) * nh;
@@ -244,8 +246,8 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
             tma_load_2d_pair(sb + j * LM_BOX_BYTES, &tmap_w, fb, kb * LM_BK, w0 + 64 * j);
           if (++stage == LM_STAGES) { stage = 0; phase ^= 1u; }
         }
-      }
       }   // sweeps
+      }
     }
   } else if (warp == 5) {
     // ------------------------------------------------------------------ MMA issuer (leader CTA)
@@ -254,7 +256,7 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
       uint32_t phase = 0;
       const int n_all = work.n_sweeps * tiles.n_tiles;      // the accumulator buffers alternate over all sweeps
       for (int tt = 0; tt < n_all; ++tt) {
-        const int t = tt % tiles.n_tiles;
+        const int t = tt / work.n_sweeps;
         int n0, nw;
         tiles.tile(t, n0, nw);
         const int buf = tt & 1;
@@ -286,14 +288,25 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
     const bool no_rows = warp * 32 >= (p.tile_rows >> 1);
     const float c = p.c;
     const uint32_t tmem_empty_leader = cluster_map(smem_u32(tmem_empty), 0);
-    for (int sweep = 0; sweep < work.n_sweeps; ++sweep) {
     float m = -INFINITY, s = 0.f, tz = 0.f, v1 = -INFINITY, v2 = -INFINITY;
     int i1 = -1, i2 = -1;
-    for (int t = 0; t < tiles.n_tiles; ++t) {
+    for (int t = 0, tt = 0; t < tiles.n_tiles; ++t)
+    for (int sweep = 0; sweep < work.n_sweeps; ++sweep, ++tt) {
       int n0, nw;
       tiles.tile(t, n0, nw);
-      const int tt = sweep * tiles.n_tiles + t;
       const int buf = tt & 1;
+      // several M tiles: this row's statistics over the tiles so far wait in its place of the partials
+      LmPartial* const place = p.partial + static_cast<size_t>(work.part) * p.part_rows +
+                               ((work.mt0 + sweep) * 2 + rank) * (p.tile_rows >> 1) + row;
+      const bool mine = row < (p.tile_rows >> 1);
+      if (work.n_sweeps > 1) {
+        m = -INFINITY; s = 0.f; tz = 0.f; v1 = -INFINITY; v2 = -INFINITY;
+        i1 = -1; i2 = -1;
+        if (t > 0 && mine) {
+          const LmPartial q = *place;
+          m = q.m; s = q.s; v1 = q.v1; v2 = q.v2; i1 = q.i1; i2 = q.i2; tz = q.t;
+        }
+      }
       mbar_wait(tmem_full + buf, (tt >> 1) & 1u, p.dev_status);
       tc_fence_after();
       const int ncols = no_rows ? 0 : min(nw, p.V - n0);  // valid columns of this tile
@@ -374,13 +387,13 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(tmem_empty_leader + static_cast<uint32_t>(buf) * 8u);
+      if (work.n_sweeps > 1 || t == tiles.n_tiles - 1) {
+        if (tt == 0 || work.n_sweeps == 1) pdl_wait();   // the previous pass's partials may be read until earlier kernels are done
+        LmPartial out;
+        out.m = m; out.s = s; out.v1 = v1; out.v2 = v2; out.i1 = i1; out.i2 = i2; out.t = tz; out.pad = 0;
+        if (mine) *place = out;
+      }
     }
-    if (sweep == 0) pdl_wait();   // the partials of the previous pass may still be read until earlier kernels are done
-    LmPartial out;
-    out.m = m; out.s = s; out.v1 = v1; out.v2 = v2; out.i1 = i1; out.i2 = i2; out.t = tz; out.pad = 0;
-    if (row < (p.tile_rows >> 1))
-      p.partial[static_cast<size_t>(work.part) * p.part_rows + ((work.mt0 + sweep) * 2 + rank) * (p.tile_rows >> 1) + row] = out;
-    }   // sweeps
   }
 
   pdl_wait();
