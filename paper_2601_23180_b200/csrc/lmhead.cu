@@ -154,6 +154,60 @@ __device__ __forceinline__ void lm_merge(LmTop2& t, unsigned long long a, unsign
   t.b = lo < t.b ? t.b : lo;
 }
 
+struct LmRowStats { float m, s, t, v1, v2; int i1, i2; };    // of a row (or a column) over the entries a lane has seen
+
+// 32 logits of a row, vocabulary entries v0 + j, of which the first nv exist.
+template <bool kEntropy>
+__device__ __forceinline__ void lm_fold32(uint32_t (&r)[32], int v0, int nv, float c, LmRowStats& st) {
+  if (nv < 32) {                                  // ragged end of the vocabulary: columns past V count as -inf
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (j >= nv) r[j] = __float_as_uint(-INFINITY);
+  }
+  // maxima of groups of eight: three-input max and, below, packed fp32 pairs halve the instruction count
+  float gm[4];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    const float* z = reinterpret_cast<const float*>(r + 8 * g);
+    gm[g] = fmaxf(fmax3(fmax3(z[0], z[1], z[2]), z[3], z[4]), fmax3(z[5], z[6], z[7]));
+  }
+  const float cmax = fmaxf(fmax3(gm[0], gm[1], gm[2]), gm[3]);
+  if (cmax > st.m) {
+    const float f = ex2f((st.m - cmax) * c);
+    st.s *= f;
+    if (kEntropy) st.t *= f;
+    st.m = cmax;
+  }
+  const float nmc = -st.m * c;
+  const float2 c2 = make_float2(c, c), nmc2 = make_float2(nmc, nmc);
+  float2 acc2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  float2 acz2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+  for (int j = 0; j < 32; j += 2) {
+    float2 z = make_float2(__uint_as_float(r[j]), __uint_as_float(r[j + 1]));
+    const float2 x = ffma2(z, c2, nmc2);
+    const float2 e = make_float2(ex2f(x.x), ex2f(x.y));
+    acc2[(j >> 1) & 1] = fadd2(acc2[(j >> 1) & 1], e);
+    if (kEntropy) {
+      if (nv < 32) {                              // masked columns hold -inf with e = 0: keep 0 * inf out of the sum
+        if (j >= nv) z.x = 0.f;
+        if (j + 1 >= nv) z.y = 0.f;
+      }
+      acz2[(j >> 1) & 1] = ffma2(e, z, acz2[(j >> 1) & 1]);
+    }
+  }
+  st.s += (acc2[0].x + acc2[0].y) + (acc2[1].x + acc2[1].y);
+  if (kEntropy) st.t += (acz2[0].x + acz2[0].y) + (acz2[1].x + acz2[1].y);
+  // The top two change once every few hundred entries of a row, but among a warp's 32 rows about once per 32 columns: eight
+  // entries at a time, without branches between them (a branch per entry took 1000 of the 1500 clocks of 32 columns).
+#pragma unroll
+  for (int g = 0; g < 4; ++g)
+    if (gm[g] > st.v2) {
+#pragma unroll
+      for (int j = 8 * g; j < 8 * g + 8; ++j) lm_scan2(__uint_as_float(r[j]), v0 + j, st.v1, st.i1, st.v2, st.i2);
+    }
+}
+
 template <bool kEntropy>
 __global__ void __launch_bounds__(LM_THREADS, 1)
 lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ CUtensorMap tmap_w,
@@ -288,8 +342,7 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
     const bool no_rows = warp * 32 >= (p.tile_rows >> 1);
     const float c = p.c;
     const uint32_t tmem_empty_leader = cluster_map(smem_u32(tmem_empty), 0);
-    float m = -INFINITY, s = 0.f, tz = 0.f, v1 = -INFINITY, v2 = -INFINITY;
-    int i1 = -1, i2 = -1;
+    LmRowStats st = {-INFINITY, 0.f, 0.f, -INFINITY, -INFINITY, -1, -1};
     for (int t = 0, tt = 0; t < tiles.n_tiles; ++t)
     for (int sweep = 0; sweep < work.n_sweeps; ++sweep, ++tt) {
       int n0, nw;
@@ -300,88 +353,27 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
                                ((work.mt0 + sweep) * 2 + rank) * (p.tile_rows >> 1) + row;
       const bool mine = row < (p.tile_rows >> 1);
       if (work.n_sweeps > 1) {
-        m = -INFINITY; s = 0.f; tz = 0.f; v1 = -INFINITY; v2 = -INFINITY;
-        i1 = -1; i2 = -1;
+        st = {-INFINITY, 0.f, 0.f, -INFINITY, -INFINITY, -1, -1};
         if (t > 0 && mine) {
           const LmPartial q = *place;
-          m = q.m; s = q.s; v1 = q.v1; v2 = q.v2; i1 = q.i1; i2 = q.i2; tz = q.t;
+          st = {q.m, q.s, q.t, q.v1, q.v2, q.i1, q.i2};
         }
       }
       mbar_wait(tmem_full + buf, (tt >> 1) & 1u, p.dev_status);
       tc_fence_after();
       const int ncols = no_rows ? 0 : min(nw, p.V - n0);  // valid columns of this tile
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(warp * 32) << 16) + static_cast<uint32_t>(buf * LM_BN);
-      for (int c0 = 0; c0 < ncols; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld32(taddr + c0, r);
-        tc_wait_ld();
-        const int nv = ncols - c0;  // >= 1
-        float cmax = -INFINITY;
-        if (nv >= 32) {
-          // whole chunk valid: three-input max and packed fp32 pairs halve the instruction count
-          float cm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-          for (int j = 0; j < 32; j += 8) {
-            cm[0] = fmax3(cm[0], __uint_as_float(r[j]), __uint_as_float(r[j + 1]));
-            cm[1] = fmax3(cm[1], __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
-            cm[2] = fmax3(cm[2], __uint_as_float(r[j + 4]), __uint_as_float(r[j + 5]));
-            cm[3] = fmax3(cm[3], __uint_as_float(r[j + 6]), __uint_as_float(r[j + 7]));
-          }
-          cmax = fmaxf(fmaxf(cm[0], cm[1]), fmaxf(cm[2], cm[3]));
-          if (cmax > m) {
-            const float f = ex2f((m - cmax) * c);
-            s *= f;
-            tz *= f;
-            m = cmax;
-          }
-          const float nmc = -m * c;
-          const float2 c2 = make_float2(c, c), nmc2 = make_float2(nmc, nmc);
-          float2 acc2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-          float2 acz2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            const float2 z = make_float2(__uint_as_float(r[j]), __uint_as_float(r[j + 1]));
-            const float2 x = ffma2(z, c2, nmc2);
-            const float2 e = make_float2(ex2f(x.x), ex2f(x.y));
-            acc2[(j >> 1) & 1] = fadd2(acc2[(j >> 1) & 1], e);
-            if (kEntropy) acz2[(j >> 1) & 1] = ffma2(e, z, acz2[(j >> 1) & 1]);
-          }
-          s += (acc2[0].x + acc2[0].y) + (acc2[1].x + acc2[1].y);
-          if (kEntropy) tz += (acz2[0].x + acz2[0].y) + (acz2[1].x + acz2[1].y);
-        } else {
-          // ragged end of the vocabulary: columns past V count as -inf
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            float v = __uint_as_float(r[j]);
-            if (j >= nv) { v = -INFINITY; r[j] = __float_as_uint(v); }
-            cmax = fmaxf(cmax, v);
-          }
-          if (cmax > m) {
-            const float f = ex2f((m - cmax) * c);
-            s *= f;
-            tz *= f;
-            m = cmax;
-          }
-          const float mc = m * c;
-          float acc = 0.f, acz = 0.f;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float e = ex2f(fmaf(__uint_as_float(r[j]), c, -mc));
-            acc += e;
-            // masked columns hold -inf with e = 0: keep 0 * inf out of the sum
-            if (kEntropy) acz = fmaf(e, (j < nv) ? __uint_as_float(r[j]) : 0.f, acz);
-          }
-          s += acc;
-          tz += acz;
-        }
-        if (cmax > v2) {
-          const int col0 = n0 + c0;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {           // (one row's 32 entries rarely change anything: branches are cheaper)
-            const float v = __uint_as_float(r[j]);
-            if (v > v1) { v2 = v1; i2 = i1; v1 = v; i1 = col0 + j; }
-            else if (v > v2) { v2 = v; i2 = col0 + j; }
-          }
+      // The next 32 columns are on their way to registers while the warp folds the ones at hand.
+      uint32_t ra[32], rb[32];
+      if (ncols > 0) tmem_ld32(taddr, ra);
+      for (int c0 = 0; c0 < ncols; c0 += 64) {
+        tc_wait_ld(ra);
+        if (c0 + 32 < ncols) tmem_ld32(taddr + c0 + 32, rb);
+        lm_fold32<kEntropy>(ra, n0 + c0, ncols - c0, c, st);
+        if (c0 + 32 < ncols) {
+          tc_wait_ld(rb);
+          if (c0 + 64 < ncols) tmem_ld32(taddr + c0 + 64, ra);
+          lm_fold32<kEntropy>(rb, n0 + c0 + 32, ncols - c0 - 32, c, st);
         }
       }
       tc_fence_before();
@@ -390,7 +382,7 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
       if (work.n_sweeps > 1 || t == tiles.n_tiles - 1) {
         if (tt == 0 || work.n_sweeps == 1) pdl_wait();   // the previous pass's partials may be read until earlier kernels are done
         LmPartial out;
-        out.m = m; out.s = s; out.v1 = v1; out.v2 = v2; out.i1 = i1; out.i2 = i2; out.t = tz; out.pad = 0;
+        out.m = st.m; out.s = st.s; out.v1 = st.v1; out.v2 = st.v2; out.i1 = st.i1; out.i2 = st.i2; out.t = st.t; out.pad = 0;
         if (mine) *place = out;
       }
     }
