@@ -34,7 +34,7 @@
  *     that gave up, an index or length outside its range, a malformed tree); the kernels never
  *     trap and never read or write outside the caller's arrays because of such a value.
  *   - Ordering. A call may read any of its inputs as soon as its first kernel starts, and that
- *     kernel is an ordinary stream-ordered launch: whatever was enqueued on `stream` before the
+ *     kernel does nothing before what was enqueued ahead of it has completed: whatever was enqueued on `stream` before the
  *     call - the caller's own kernels and copies, or an earlier call of this library such as a
  *     KV commit, a pruning step or the scan that wrote an escalation list - has completed by
  *     then. One exception is the caller's to avoid: a kernel that uses programmatic dependent
@@ -368,9 +368,10 @@ int trispec_sample_bonus(const trispec_sample_args* a, void* stream);
  * one verifier): tree mask first, acceptance scan last; the attention and the LM-head
  * statistics, which do not read each other's results, in the order the library finds faster
  * for the shape. `attn` may be NULL to skip attention. For at most 64 active rows (128 from 256 MiB
- * of W on) whose attention can do with few CTAs the library runs mask + attention on a second
- * stream of its own (one per caller's stream) beside the LM head and the scan, and `stream` waits
- * for that stream before the call returns its place in the queue: everything the call enqueues has
+ * of W on) whose attention can do with few CTAs, masks, attention and LM head share a launch; where
+ * the attention's own plan is given the SMs, mask + attention run on a second
+ * stream of the library's own (one per caller's stream) beside the LM head and the scan, and `stream` waits
+ * for that stream before the call returns its place in the queue. Either way everything the call enqueues has
  * completed before anything enqueued on `stream` afterwards starts. Attention, masks and decisions
  * are bit for bit those of the four calls; the statistics' sums may be taken over other vocabulary
  * ranges (the LM head leaves the attention some SMs), so that their last bits can differ. Steps that
@@ -387,8 +388,8 @@ int trispec_verify(const trispec_tree_args* tree, const trispec_attn_args* attn,
  * attention runs in few CTAs beside it where it then still ends in time, and after it otherwise);
  * "none" without `lm`. The environment variable TRISPEC_PASS_FORM = attention_first | lm_first |
  * side_by_side overrides the choice for so few rows.
- * trispec_verify_beside: the number of CTAs in which the attention runs on the second stream, beside
- * the LM head, or 0 where the steps run in stream order. Memory that a step shares with the `tree`
+ * trispec_verify_beside: the number of CTAs that the attention needs beside the LM head (it may be
+ * given two for each of a few), or 0 where the steps run in stream order. Memory that a step shares with the `tree`
  * of the call, and a second stream that is not to be had, are the only reasons to run in stream
  * order that these answers do not see. */
 const char* trispec_verify_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm,

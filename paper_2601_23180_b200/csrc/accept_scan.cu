@@ -16,9 +16,9 @@ constexpr int kScanThreads = 256;  // 8 sequences per block
 // the proxy feature the routing criterion looks at (margin of Eq. 8 by default)
 template <int kCrit>
 __device__ __forceinline__ float scan_feature(const trispec_scan_args& a, long long idx) {
-  if (kCrit == TRISPEC_CRIT_TOP1) return __ldg(a.in.p_top1 + idx);
-  if (kCrit == TRISPEC_CRIT_ENTROPY) return __ldg(a.in.entropy + idx);
-  return __ldg(a.in.p_top1 + idx) - __ldg(a.in.p_top2 + idx);
+  if (kCrit == TRISPEC_CRIT_TOP1) return __ldcg(a.in.p_top1 + idx);
+  if (kCrit == TRISPEC_CRIT_ENTROPY) return __ldcg(a.in.entropy + idx);
+  return __ldcg(a.in.p_top1 + idx) - __ldcg(a.in.p_top2 + idx);
 }
 
 // The walk of one sequence by one warp; writes the sequence's outputs and returns its escalation flag.
@@ -27,13 +27,14 @@ __device__ __forceinline__ float scan_feature(const trispec_scan_args& a, long l
 // kAccept: TRISPEC_ACCEPT_GREEDY (arg-max match), _STOCHASTIC (Eq. 6 at temperature 1) or
 // _TOKEN_SPECIFIC (the token-specific deferral rule of the SpecCascade baselines).
 template <int kCrit, int kAccept>
-__device__ __forceinline__ int scan_sequence(const trispec_scan_args& a, const long long b, const int lane) {
+__device__ __forceinline__ int scan_sequence(const trispec_scan_args& a, const long long b, const int lane, const bool write = true) {
   const int T = a.T;
   const long long base = b * T;
   int32_t* path = a.path + base;
   const bool has0 = lane < T, has1 = lane + 32 < T;
 
-  if (a.active && a.active[b] == 0) {
+  if (a.active && __ldcg(a.active + b) == 0) {
+    if (!write) return 0;
     if (has0) path[lane] = -1;
     if (has1) path[lane + 32] = -1;
     if (lane == 0) {
@@ -57,12 +58,12 @@ __device__ __forceinline__ int scan_sequence(const trispec_scan_args& a, const l
   // (1 - alpha) times its parent's) and the probability of the nodes' own drafted tokens
   float pt0 = 0.f, pt1 = 0.f, pd0 = -1.f, pd1 = -1.f;
   if (token_rule) {
-    if (has0) { pt0 = __ldg(a.in.p_top1 + base + lane); if (lane > 0) pd0 = __ldg(a.in.p_draft + base + lane); }
-    if (has1) { pt1 = __ldg(a.in.p_top1 + base + lane + 32); pd1 = __ldg(a.in.p_draft + base + lane + 32); }
+    if (has0) { pt0 = __ldcg(a.in.p_top1 + base + lane); if (lane > 0) pd0 = __ldcg(a.in.p_draft + base + lane); }
+    if (has1) { pt1 = __ldcg(a.in.p_top1 + base + lane + 32); pd1 = __ldcg(a.in.p_draft + base + lane + 32); }
   }
   if (has0) {
-    par0 = __ldg(a.parent + base + lane); tok0 = __ldg(a.tok + base + lane);
-    top0 = __ldg(a.in.top1_idx + base + lane);
+    par0 = __ldcg(a.parent + base + lane); tok0 = __ldcg(a.tok + base + lane);
+    top0 = __ldcg(a.in.top1_idx + base + lane);
     if (proxy) {
       const float f = scan_feature<kCrit>(a, base + lane);
       tr0 = (kCrit == TRISPEC_CRIT_ENTROPY) ? (f <= a.lambda) : (f >= a.lambda);
@@ -70,8 +71,8 @@ __device__ __forceinline__ int scan_sequence(const trispec_scan_args& a, const l
     }
   }
   if (has1) {
-    par1 = __ldg(a.parent + base + lane + 32); tok1 = __ldg(a.tok + base + lane + 32);
-    top1v = __ldg(a.in.top1_idx + base + lane + 32);
+    par1 = __ldcg(a.parent + base + lane + 32); tok1 = __ldcg(a.tok + base + lane + 32);
+    top1v = __ldcg(a.in.top1_idx + base + lane + 32);
     if (proxy) {
       const float f = scan_feature<kCrit>(a, base + lane + 32);
       tr1 = (kCrit == TRISPEC_CRIT_ENTROPY) ? (f <= a.lambda) : (f >= a.lambda);
@@ -87,19 +88,19 @@ __device__ __forceinline__ int scan_sequence(const trispec_scan_args& a, const l
   if (stochastic) {
     bool ps0 = false, ps1 = false;
     if (has0 && lane > 0) {
-      const float q = __ldg(a.q_draft + base + lane), pd = __ldg(a.in.p_draft + base + lane);
-      ps0 = __ldg(a.u_accept + base + lane) < ((q > 0.f) ? fminf(1.f, pd / q) : 1.f);
+      const float q = __ldcg(a.q_draft + base + lane), pd = __ldcg(a.in.p_draft + base + lane);
+      ps0 = __ldcg(a.u_accept + base + lane) < ((q > 0.f) ? fminf(1.f, pd / q) : 1.f);
     }
     if (has1) {
-      const float q = __ldg(a.q_draft + base + lane + 32), pd = __ldg(a.in.p_draft + base + lane + 32);
-      ps1 = __ldg(a.u_accept + base + lane + 32) < ((q > 0.f) ? fminf(1.f, pd / q) : 1.f);
+      const float q = __ldcg(a.q_draft + base + lane + 32), pd = __ldcg(a.in.p_draft + base + lane + 32);
+      ps1 = __ldcg(a.u_accept + base + lane + 32) < ((q > 0.f) ? fminf(1.f, pd / q) : 1.f);
     }
     passes = __ballot_sync(0xffffffffu, ps0) | (static_cast<unsigned long long>(__ballot_sync(0xffffffffu, ps1)) << 32);
   }
   // the compaction kernel only writes the leading entries of esc_index
-  if (a.esc_index && lane == 0) a.esc_index[b] = -1;
+  if (write && a.esc_index && lane == 0) a.esc_index[b] = -1;
 
-  int cur = a.start_node ? a.start_node[b] : 0;
+  int cur = a.start_node ? __ldcg(a.start_node + b) : 0;
   if (cur < 0 || cur >= T) cur = 0;
   int n = 0, esc = 0, bonus = -1, near = 0;
   int path0 = -1, path1 = -1;   // entries `lane` and `lane + 32` of the accepted path
@@ -134,6 +135,8 @@ __device__ __forceinline__ int scan_sequence(const trispec_scan_args& a, const l
     ++n;
     cur = nxt;
   }
+  asm volatile("" ::"r"(path0), "r"(path1), "r"(bonus), "r"(near));   // (computed whether they are written or not)
+  if (!write) return esc;
   if (has0) path[lane] = path0;
   if (has1) path[lane + 32] = path1;
   if (lane == 0) {
@@ -149,8 +152,8 @@ __device__ __forceinline__ int scan_sequence(const trispec_scan_args& a, const l
 template <int kCrit, int kAccept>
 __global__ void __launch_bounds__(kScanThreads)
 accept_scan_kernel(trispec_scan_args a) {
-  pdl_launch_dependents();
   pdl_wait();
+  pdl_launch_dependents();
   const int lane = threadIdx.x & 31;
   const long long b = static_cast<long long>(blockIdx.x) * (kScanThreads / 32) + (threadIdx.x >> 5);
   if (b >= a.B) return;
@@ -163,12 +166,20 @@ accept_scan_kernel(trispec_scan_args a) {
 constexpr int kScanSmallMax = 32;
 template <int kCrit, int kAccept>
 __global__ void __launch_bounds__(32 * kScanSmallMax)
-accept_scan_small_kernel(trispec_scan_args a) {
+accept_scan_small_kernel(trispec_scan_args a, int rehearse) {
   __shared__ int s_esc[kScanSmallMax];
-  pdl_launch_dependents();
-  pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int esc = (warp < a.B) ? scan_sequence<kCrit, kAccept>(a, warp, lane) : 0;
+  int esc = 0;
+  // Behind another kernel of the same call the scan runs twice, the first time before the wait and without writing: that
+  // brings its code into the instruction cache (the loads bypass L1).
+#pragma unroll 1
+  for (int run = rehearse ? 0 : 1; run < 2; ++run) {
+    if (run == 1) {
+      pdl_wait();
+      pdl_launch_dependents();
+    }
+    if (warp < a.B) esc = scan_sequence<kCrit, kAccept>(a, warp, lane, run == 1);
+  }
   if (lane == 0) s_esc[warp] = esc;
   __syncthreads();
   if (warp == 0 && a.esc_index) {
@@ -343,7 +354,7 @@ int scan_check(const trispec_scan_args* a) {
 }  // namespace trispec
 
 extern "C" int trispec_accept_scan(const trispec_scan_args* a, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
+  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
   using namespace trispec;
   const int rc = scan_check(a);
   if (rc != TRISPEC_OK) return rc;
@@ -353,16 +364,19 @@ extern "C" int trispec_accept_scan(const trispec_scan_args* a, void* stream) {
   const int crit = (a->mode == TRISPEC_MODE_PROXY) ? a->criterion : TRISPEC_CRIT_MARGIN;
   const int which = crit * 3 + rule;
   typedef void (*ScanKernel)(trispec_scan_args);
+  typedef void (*SmallScanKernel)(trispec_scan_args, int);
 #define TRISPEC_SCAN_ROW(K, C) K<C, TRISPEC_ACCEPT_GREEDY>, K<C, TRISPEC_ACCEPT_STOCHASTIC>, K<C, TRISPEC_ACCEPT_TOKEN_SPECIFIC>
-  static const ScanKernel small_k[9] = {TRISPEC_SCAN_ROW(accept_scan_small_kernel, TRISPEC_CRIT_MARGIN),
+  static const SmallScanKernel small_k[9] = {TRISPEC_SCAN_ROW(accept_scan_small_kernel, TRISPEC_CRIT_MARGIN),
                                         TRISPEC_SCAN_ROW(accept_scan_small_kernel, TRISPEC_CRIT_TOP1),
                                         TRISPEC_SCAN_ROW(accept_scan_small_kernel, TRISPEC_CRIT_ENTROPY)};
   static const ScanKernel big_k[9] = {TRISPEC_SCAN_ROW(accept_scan_kernel, TRISPEC_CRIT_MARGIN),
                                       TRISPEC_SCAN_ROW(accept_scan_kernel, TRISPEC_CRIT_TOP1),
                                       TRISPEC_SCAN_ROW(accept_scan_kernel, TRISPEC_CRIT_ENTROPY)};
 #undef TRISPEC_SCAN_ROW
+  const int rehearse = entry_scope_launched() ? 1 : 0;    // its inputs are complete but for what this call computes
+  launch_first_early(st);
   if (a->B <= kScanSmallMax) {
-    TRISPEC_CUDA_OK(launch_dependent(small_k[which], 1u, static_cast<unsigned>(32 * a->B), 0, st, 1, *a));
+    TRISPEC_CUDA_OK(launch_dependent(small_k[which], 1u, static_cast<unsigned>(32 * a->B), 0, st, 1, *a, rehearse));
     count_launch();
     return TRISPEC_OK;
   }

@@ -38,7 +38,8 @@ constexpr int AT_TURN_TMEM_PARTS = 4, AT_TURN_SMEM_PARTS = 3;    // and the eigh
 constexpr int AT_TURN_PART_BYTES = AT_BM * AT_D * 2;             // 16-byte words of a row XORed with row % 8
 constexpr int AT_SMEM_USED_ALIGNED = (AT_SMEM_USED + 1023) / 1024 * 1024;
 constexpr int AT_TURN_SMEM_USED = AT_SMEM_USED_ALIGNED + AT_TURN_SMEM_PARTS * AT_TURN_PART_BYTES + 8 * AT_BM * 8;
-constexpr int AT_TURN_SMEM_BYTES = AT_TURN_SMEM_USED + 1024;
+constexpr int AT_TURN_MASK_OFF = AT_TURN_SMEM_USED;              // the tree's mask, where the CTA computes it
+constexpr int AT_TURN_SMEM_BYTES = AT_TURN_SMEM_USED + 64 * 8 + 1024;
 static_assert(AT_TURN_SMEM_BYTES <= 227 * 1024 && AT_TURN_PART_BYTES <= AT_STAGES * AT_TILE_BYTES, "in-turn partials");
 
 struct AttnParams {
@@ -55,6 +56,8 @@ struct AttnParams {
   uint16_t* o;      // bf16 [B][T][Hq][128]  (cluster mode writes the result itself)
   float* lse;       // [B][Hq][T] or null
   int32_t* dev_status;
+  const int32_t* parent;   // in turn: the CTA computes the mask of its tree from these, or null = `mask`
+  int first;        // this is the call's first kernel, launched early (pdl_enter)
   // persistent kernel only
   int n_seq;        // active sequences (at most 128)
   int n_cta;        // CTAs of the launch: CTA c walks tiles [c W / n_cta, (c + 1) W / n_cta) of the work
@@ -84,6 +87,20 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return r;
 }
 
+}  // namespace trispec
+
+// An attention in turn (attn_split.cuh) that shares a launch with the LM head's small-row kernel
+namespace trispec {
+struct AttnBeside {
+  CUtensorMap k, v, kt, vt;
+  AttnParams p;
+  int ctas;         // CTAs of the launch that are the attention's: the first ones
+  bool pair;        // two per (sequence, KV head, M tile), a cluster
+  bool masks;       // the launch computes the tree masks as well
+  trispec_tree_args tree;
+};
+int attn_beside(const trispec_attn_args* a, const trispec_tree_args* tree, bool pair, AttnBeside* out);
+int lmhead_stats_beside(const trispec_lmhead_args* a, const AttnBeside& beside, void* stream);
 }  // namespace trispec
 
 // the persistent form (attn_pieces.cu)

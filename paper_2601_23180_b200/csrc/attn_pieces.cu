@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2)
 verify_attn_pieces_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                           const __grid_constant__ CUtensorMap tm_kt, const __grid_constant__ CUtensorMap tm_vt,
                           const AttnParams p) {
-  pdl_launch_dependents();
+  pdl_enter(p.first);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // The loader and the issuer warp each keep a copy of the work map (registers) and walk this CTA's
   // pieces with it; the softmax warps get every piece from the issuer through a two-entry mailbox in
@@ -152,7 +152,10 @@ verify_attn_pieces_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
   uint8_t* smem = smem_raw + (base_u32 - smem_u32(smem_raw));
   const bool misaligned = base_u32 - smem_u32(smem_raw) > static_cast<uint32_t>(AT_SMEM_BYTES - AT_SMEM_USED);
   if (misaligned && threadIdx.x == 0 && p.dev_status) atomicExch(p.dev_status, TRISPEC_ERR_SMEM_ALIGN);
-  if (w_begin >= w_end || misaligned) return;    // nothing to do (fewer steps than CTAs): the merge kernel knows
+  if (w_begin >= w_end || misaligned) {          // nothing to do (fewer steps than CTAs): the merge kernel knows
+    pdl_wait();                                  // (no grid ends before the one ahead of it)
+    return;
+  }
 
   constexpr int NV = (NP == 2) ? 2 : 3;         // V ring slots: K ring + V ring + P buffers = 112 KB either way
   uint8_t* sK = smem;                           // [AT_STAGES] K tiles
@@ -617,13 +620,16 @@ verify_attn_pieces_merge_kernel(const AttnParams p) {
     const int pj = __shfl_sync(0xffffffffu, wm.pre[j], a & 31);
     if (j == (a >> 5)) { L = Lj; nn = nj; pre = pj; }
   }
-  if (mtile * p.NPT >= nn) return;               // no node of this (pruned) tree in the M tile
+  const bool none = mtile * p.NPT >= nn;         // no node of this (pruned) tree in the M tile
   const int n_it = (L + AT_BN - 1) / AT_BN + 1;
   const long long W = wm.total;
   const int n_grp = p.n_cta / p.n_mt;
   const long long x = pre + static_cast<long long>(g) * n_it;                 // first global step of the (sequence, head)
   const int r_first = cta_of_step(W, n_grp, x), r_last = cta_of_step(W, n_grp, x + n_it - 1);
-  if (r_first == r_last) return;                 // one piece: stored by the first kernel
+  if (none || r_first == r_last) {               // one piece: stored by the first kernel
+    pdl_wait();                                  // (no grid ends before the one ahead of it)
+    return;
+  }
   const int b = p.seq_index ? __ldg(p.seq_index + a) : a;
   pdl_wait();                                    // the partials come from the kernel before
   const int n_rows = min(min(AT_BM, p.NPT * p.G), (quarter + 1) * (AT_BM / AP_MERGE_BLOCKS));

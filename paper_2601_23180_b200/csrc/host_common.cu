@@ -13,15 +13,32 @@ void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 namespace {
 thread_local int tl_scope_depth = 0;
 thread_local bool tl_scope_launched = false;
+thread_local bool tl_scope_early = false;       // the next launch is the call's first and may be made early
+thread_local bool tl_scope_ordinary = false;    // ... may not: it follows an event of another stream
 }  // namespace
 EntryScope::EntryScope() {
-  if (tl_scope_depth++ == 0) tl_scope_launched = false;
+  if (tl_scope_depth++ == 0) tl_scope_launched = tl_scope_early = tl_scope_ordinary = false;
 }
 EntryScope::~EntryScope() { --tl_scope_depth; }
-void entry_scope_next_launch_ordinary() { tl_scope_launched = false; }
+void entry_scope_next_launch_ordinary() {
+  tl_scope_launched = false;
+  tl_scope_ordinary = true;
+}
+bool entry_scope_launched() { return tl_scope_depth > 0 && tl_scope_launched; }
+bool entry_scope_outermost() { return tl_scope_depth == 1; }
+bool launch_first_early(cudaStream_t st) {
+  if (tl_scope_depth == 0 || tl_scope_launched || tl_scope_ordinary) return false;
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return tl_scope_early = status == cudaStreamCaptureStatusNone;
+}
 bool entry_scope_next_launch_is_dependent() {
-  const bool dependent = tl_scope_depth > 0 && tl_scope_launched;
+  const bool dependent = tl_scope_depth > 0 && (tl_scope_launched || tl_scope_early);
   tl_scope_launched = true;
+  tl_scope_early = tl_scope_ordinary = false;
   return dependent;
 }
 
@@ -54,9 +71,15 @@ bool encode_tmap_bf16(CUtensorMap* out, const void* base, int rank, const uint64
     es[i] = 1;
   }
   for (int i = 0; i + 1 < rank; ++i) gstr[i] = strides_bytes[i];
-  CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), gdim, gstr, bx, es,
+  const auto encode = [&] {
+    return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), gdim, gstr, bx, es,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = encode();
+  // the driver's call wants a context, which a thread has only once the runtime has had something to do on it
+  int dev = 0;
+  if (r == CUDA_ERROR_INVALID_CONTEXT && cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess) r = encode();
   return r == CUDA_SUCCESS;
 }
 

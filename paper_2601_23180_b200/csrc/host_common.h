@@ -29,11 +29,12 @@ int device_sm_count();
 int ensure_smem_limit(const void* func, int bytes, bool* done_per_device /* [64] */);
 
 // Programmatic dependent launch inside one call of the library. The FIRST kernel a public entry
-// point launches is an ordinary launch: it starts once everything enqueued on the stream before
+// point launches does nothing before everything enqueued on the stream before
 // the call has completed and its writes are visible, so every input of the call (activations,
 // the KV cache and its lengths, index arrays written by an earlier call such as the escalation
 // list, pruned-tree node counts or committed lengths) may be read by any kernel of the call at
-// any time. Every LATER kernel of the same call is launched as a programmatic dependent of the
+// any time. It is an ordinary launch, or (launch_first_early below) it is on the SMs already but waits before anything else and
+// only then lets its own dependents start. Every LATER kernel of the same call is launched as a programmatic dependent of the
 // kernel before it: its CTAs may be scheduled as soon as all CTAs of that kernel have called
 // pdl_launch_dependents() (they do so at their start) and resources are free, so launch latency,
 // prologues and tails inside a call overlap. Such a kernel calls pdl_wait() before its first read
@@ -52,6 +53,15 @@ struct EntryScope {
 // True if a kernel was already launched inside the current outermost scope (the next launch may
 // then be a programmatic dependent); records that a launch happens now.
 bool entry_scope_next_launch_is_dependent();
+// To be called right before the launch of a kernel that waits (pdl_wait) before anything else and before it lets its dependents
+// start. True if that launch is the call's first and may be made while the kernel before it on the stream still runs: not under
+// capture, not behind an event of another stream. What this hides is the launch (a pass of five short sequences 60.7 -> 59.1 us).
+// The wait is for the kernel before it on the stream, which stands for all earlier work because no kernel of the library
+// ends before the one ahead of it has (every one waits, also where it has nothing to do).
+bool launch_first_early(cudaStream_t st);
+// Whether the current call has launched a kernel already; whether it is not part of another one
+bool entry_scope_launched();
+bool entry_scope_outermost();
 // The next launch inside the current scope is an ordinary one again (after work was moved to or joined from
 // another stream, where "the kernel before it" is not the kernel enqueued last).
 void entry_scope_next_launch_ordinary();
@@ -89,6 +99,11 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, uns
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The start of a kernel that may be the first of a call: `first` = launch_first_early()
+__device__ __forceinline__ void pdl_enter(int first) {
+  if (first) pdl_wait();
+  pdl_launch_dependents();
+}
 #endif
 
 // What an entry point refuses, without launching anything (the fused passes ask all their steps first)
@@ -99,9 +114,10 @@ int scan_check(const trispec_scan_args* a);
 // CTAs the attention launch for these arguments will use (0 if the arguments are not accepted)
 int attn_planned_ctas(const trispec_attn_args* a);
 // CTAs of an attention whose plan merges its splits on chip when each (sequence, KV head, M tile) has one CTA, alone on
-// its SM, that takes the splits in turn (attn.cu); 0 where the plan is another one, where that is more than `max_ctas`
-// CTAs, or where they would take longer than `budget_us`.
-int attn_compact_ctas(const trispec_attn_args* a, double budget_us, int max_ctas);
+// its SM, that takes the splits in turn (attn_split.cuh); 0 where the plan is another one, where that is more than `max_ctas`
+// CTAs, or where they would take longer than `budget_us`. `pair` (may be null): a pass that has both in one launch gives every item two CTAs
+// (the answer is the number of CTAs that end in time, twice the items where one each does not).
+int attn_compact_ctas(const trispec_attn_args* a, double budget_us, int max_ctas, bool* pair);
 // The attention launches of this thread take that form while this is on
 void attn_in_turn_once(bool on);
 // columns of the LM head's small-row kernel, and whether a call with these arguments (its workspace's size among them) takes it

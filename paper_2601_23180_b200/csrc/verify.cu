@@ -4,7 +4,7 @@
 #include <optional>
 #include <stdlib.h>
 
-#include "host_common.h"
+#include "attn_common.cuh"
 
 namespace trispec {
 // Second streams (with their events) of the fused passes. A set belongs to one stream of the caller's, so that callers on
@@ -133,6 +133,7 @@ struct PassPlan {
   bool beside;        // mask and attention go to the second stream, the LM head leaves them `attn_ctas` SMs
   int attn_ctas;
   bool in_turn;       // that attention takes the splits of its plan one after the other, in few CTAs
+  bool pair;          // two CTAs per item, in the LM head's launch
 };
 
 // The memory that one of the two streams of a pass reads and writes.
@@ -220,9 +221,10 @@ static bool pass_shares_memory(const trispec_tree_args* tree, const trispec_attn
   return beside.clashes(main) || (scan && scan->esc_index && attn->seq_index == scan->esc_index);
 }
 
+// `one_launch`: the attention in turn and the LM head share a launch (everything is on the device already).
 static PassPlan pass_plan(const trispec_tree_args* tree, const trispec_attn_args* attn, const trispec_lmhead_args* lm,
-                          const trispec_scan_args* scan) {
-  PassPlan pl = {PASS_ATTENTION_FIRST, false, attn ? attn_planned_ctas(attn) : 0, false};
+                          const trispec_scan_args* scan, bool one_launch = true) {
+  PassPlan pl = {PASS_ATTENTION_FIRST, false, attn ? attn_planned_ctas(attn) : 0, false, false};
   const int lm_seqs = lm->seq_index ? lm->B_active : lm->B;
   if (!attn || pl.attn_ctas <= 0 || !lm_runs_small_rows(lm)) return pl;      // the pair kernel takes every SM
   const int sms = device_sm_count();
@@ -242,7 +244,7 @@ static PassPlan pass_plan(const trispec_tree_args* tree, const trispec_attn_args
   // sequence of 61 nodes, 4096 context tokens, 151936 x 2048 weights: 8 CTAs of 65 tiles beside 140 of the LM head
   // against 64 CTAs after all 148 of it.
   const double lm_us = static_cast<double>(lm->V) * lm->d * 2.0 / 6.0e6;
-  const int compact_ctas = in_order ? 0 : attn_compact_ctas(attn, 0.8 * lm_us, sms / 4);
+  const int compact_ctas = in_order ? 0 : attn_compact_ctas(attn, 0.8 * lm_us, sms / 4, one_launch ? &pl.pair : nullptr);
   if (lm_seqs == 1) {
     // Behind the attention the LM head would stall as a programmatic dependent, so for one sequence it goes first
     // whatever the form. The attention's own plan runs side by side where it can be given one SM per CTA for less
@@ -295,7 +297,7 @@ extern "C" int trispec_verify_beside(const trispec_attn_args* attn, const trispe
 
 extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_args* attn,
                               const trispec_lmhead_args* lm, const trispec_scan_args* scan, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
+  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
   if (!tree || !lm || !scan) return TRISPEC_ERR_INVALID_ARG;
   // The attention and the LM head do not depend on each other, so their order is free. A kernel launched as
   // a programmatic dependent gets its launch latency and prologue hidden, but its loads make almost no
@@ -308,8 +310,17 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
   const bool lm_first = plan.form == trispec::PASS_LM_FIRST;
   int rc = trispec::pass_check(tree, attn, lm, scan, plan);
   if (rc != TRISPEC_OK) return rc;
-  // Few rows and an attention that fits beside the LM head (pass_plan): the two run side by
-  // side. Mask and attention go to a second stream behind an event recorded on `stream` at the
+  // Few rows and an attention in turn that fits beside the LM head (pass_plan): masks, attention and LM head in one launch, the
+  // scan behind its merge. (On a second stream, forked and joined by events, until now: one short chain 36.4 -> 31.0 us a pass,
+  // host 29 -> 18 us a call.)
+  if (plan.in_turn) {
+    trispec::AttnBeside beside;
+    rc = trispec::attn_beside(attn, tree, plan.pair, &beside);
+    if (rc == TRISPEC_OK && !beside.masks) rc = trispec_build_tree_mask(tree, stream);
+    if (rc == TRISPEC_OK) rc = trispec::lmhead_stats_beside(lm, beside, stream);
+    return rc == TRISPEC_OK ? trispec_accept_scan(scan, stream) : rc;
+  }
+  // The attention's own plan beside the LM head: mask and attention go to a second stream behind an event recorded on `stream` at the
   // start of the call; the LM head, whose grid is one persistent CTA per SM, leaves them one SM per attention
   // CTA and starts at once, the scan follows it, and `stream` then waits for the second stream: everything
   // the call enqueues is complete before anything enqueued on `stream` after it.
@@ -320,11 +331,10 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
     if (side) {
       TRISPEC_CUDA_OK(cudaEventRecord(side->fork, st));
       TRISPEC_CUDA_OK(cudaStreamWaitEvent(side->stream, side->fork, 0));
-      rc = trispec_build_tree_mask(tree, side->stream);      // ordinary launch: first kernel of the call
+      entry_scope_next_launch_ordinary();                    // (behind the event)
+      rc = trispec_build_tree_mask(tree, side->stream);
       if (rc == TRISPEC_OK) {
-        attn_in_turn_once(plan.in_turn);
         rc = trispec_verify_attn(attn, side->stream);        // dependent of the mask kernel
-        attn_in_turn_once(false);
       }
       TRISPEC_CUDA_OK(cudaEventRecord(side->done, side->stream));
       if (rc == TRISPEC_OK) {
@@ -364,13 +374,13 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
 extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree_args* tree,
                                    const trispec_attn_args* attn, const trispec_lmhead_args* lm,
                                    const trispec_scan_args* scan, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
+  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
   using namespace trispec;
   if (!io || !tree || !lm || !scan) return TRISPEC_ERR_INVALID_ARG;
   // the copies below land in the buffers the structs name: they must describe one and the same pass
   if (tree->parent != lm->parent || tree->parent != scan->parent || lm->tok != scan->tok)
     return TRISPEC_ERR_INVALID_ARG;
-  const PassPlan plan = pass_plan(tree, attn, lm, scan);
+  const PassPlan plan = pass_plan(tree, attn, lm, scan, false);
   int rc = pass_check(tree, attn, lm, scan, plan);
   if (rc != TRISPEC_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -425,6 +435,7 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
     // few rows (as in trispec_verify): mask and attention follow their inputs on
     // the second stream, the LM head and the scan run on `stream`, which then waits for the second stream
     TRISPEC_CUDA_OK(cudaStreamWaitEvent((*side)->stream, (*side)->inputs, 0));   // the tree's parents have arrived
+    entry_scope_next_launch_ordinary();                              // (behind the events)
     rc = trispec_build_tree_mask(tree, (*side)->stream);
     if (rc == TRISPEC_OK) {
       attn_in_turn_once(plan.in_turn);
@@ -442,6 +453,7 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
     TRISPEC_CUDA_OK(cudaStreamWaitEvent(st, (*side)->done, 0));
     if (rc != TRISPEC_OK) return rc;
   } else {
+    entry_scope_next_launch_ordinary();                      // (behind the copies)
     rc = trispec_build_tree_mask(tree, stream);
     if (rc != TRISPEC_OK) return rc;
     lm_reserve_sms_once(plan.beside ? plan.attn_ctas : 0);   // (as in trispec_verify)
