@@ -915,6 +915,180 @@ lmhead_rows_beside_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gr
   }
 }
 
+// ---------------------------------------------------------------------------------------
+// More rows than the small-row kernel takes, in tiles that leave a quarter of the pair kernel's M lanes or more empty: operands
+// swapped in a CTA pair. W is the M side (256 vocabulary entries per tile, 128 per CTA), the rows are the N side, exactly as
+// many columns as there are (to 16): no MMA cycle goes to padding (312 rows run as 2 x 160 columns instead of 2 x 256 lanes).
+// What bounds both kernels beside the power limit is how fast L2 delivers operands (about 53 of 64 bytes per clock and SM);
+// the statistics cross the lanes through shared memory as in the small-row kernel, twice the work per logit of the pair
+// kernel's, hidden behind the MMAs of 32 k-blocks and more. Both CTAs' statistics meet through distributed shared memory, so
+// that a range still is one row block of the partials. Up to 8 stages of 16 KB of W and up to 12 KB of H per CTA.
+// ---------------------------------------------------------------------------------------
+constexpr int LC_EPI_WARPS = 8, LC_THREADS = 32 * (LC_EPI_WARPS + 2), LC_MAX_STAGES = 8, LC_MAX_COLS = 256;
+constexpr int LC_A_BYTES = 128 * LM_BK * 2;                        // 16 KB: this CTA's half of the W tile
+constexpr int LC_RING_BYTES = LW_SMEM_BYTES - 1024 - LC_EPI_WARPS * LW_XPOSE_BYTES - 256;
+
+struct LmColsParams {
+  LmParams base;    // tile_rows: columns of a tile, a multiple of 16
+  int n_rows;
+  int stages, stage_bytes;
+};
+
+template <bool kEntropy>
+__global__ void __launch_bounds__(LC_THREADS, 1)
+lmhead_cols_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_h, const LmColsParams sp) {
+  if (!sp.base.first) pdl_launch_dependents();
+  const LmParams& p = sp.base;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base_u32 = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* smem = smem_raw + (base_u32 - smem_u32(smem_raw));
+  uint8_t* xpose = smem + sp.stages * sp.stage_bytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(xpose + LC_EPI_WARPS * LW_XPOSE_BYTES);
+  uint64_t* full_bar = bars;                          // (used in the leader)
+  uint64_t* empty_bar = bars + LC_MAX_STAGES;
+  uint64_t* tmem_full = bars + 2 * LC_MAX_STAGES;
+  uint64_t* tmem_empty = bars + 2 * LC_MAX_STAGES + 2;   // (used in the leader)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * LC_MAX_STAGES + 4);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();            // 0 = leader
+  const PairWork work(p, blockIdx.x >> 1);
+  const TileIter& tiles = work.tiles;
+  const int n_kb = p.d / LM_BK;
+  const int cols = p.tile_rows, half_cols = cols >> 1;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < sp.stages; ++i) { mbar_init(full_bar + i, 1); mbar_init(empty_bar + i, 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(tmem_full + i, 1); mbar_init(tmem_empty + i, 2 * LC_EPI_WARPS); }
+    fence_mbar_init();
+  }
+  if (warp == LC_EPI_WARPS + 1) {
+    tmem_alloc_pair(tmem_slot, 512);
+    tmem_relinquish_pair();
+  }
+  if (warp == LC_EPI_WARPS && lane == 0) { prefetch_tmap(&tmap_h); prefetch_tmap(&tmap_w); }
+  tc_fence_before();
+  cluster_sync_all();                                 // both CTAs' barriers and TMEM are ready
+  tc_fence_after();
+  if (p.first) pdl_wait();                            // what is above needs nothing from earlier kernels
+  const uint32_t tmem_base = *tmem_slot;
+  LmColMerge* red = reinterpret_cast<LmColMerge*>(smem);           // [4 warps][columns], in the ring's memory at the end
+
+  if (warp == LC_EPI_WARPS) {
+    if (lane == 0) {   // ---------------------------------------------------------- TMA producer
+      int stage = 0;
+      uint32_t phase = 0;
+      if (p.first) pdl_launch_dependents();
+      if (p.wait_rows) pdl_wait();
+      const int row0 = work.mt0 * cols + static_cast<int>(rank) * half_cols;
+      for (int t = 0; t < tiles.n_tiles; ++t) {
+        int n0, nw;
+        tiles.tile(t, n0, nw);
+        const int nh = nw >> 1, nbox = (nh + 63) >> 6;
+        const int w0 = n0 + static_cast<int>(rank) * nh;
+        const uint32_t tx_pair = 2u * static_cast<uint32_t>(half_cols + 64 * nbox) * (LM_BK * 2);
+        for (int kb = 0; kb < n_kb; ++kb) {
+          mbar_wait(empty_bar + stage, phase ^ 1u, p.dev_status);
+          uint8_t* sa = smem + stage * sp.stage_bytes;
+          if (rank == 0) mbar_expect_tx(full_bar + stage, tx_pair);
+          const uint32_t fb = cluster_map(smem_u32(full_bar + stage), 0);
+          for (int j = 0; j < nbox; ++j) tma_load_2d_pair(sa + j * LM_BOX_BYTES, &tmap_w, fb, kb * LM_BK, w0 + 64 * j);
+          tma_load_2d_pair(sa + LC_A_BYTES, &tmap_h, fb, kb * LM_BK, row0);
+          if (++stage == sp.stages) { stage = 0; phase ^= 1u; }
+        }
+      }
+    }
+  } else if (warp == LC_EPI_WARPS + 1) {
+    if (lane == 0 && rank == 0) {   // --------------------------------------------- MMA issuer (leader CTA)
+      int stage = 0;
+      uint32_t phase = 0;
+      const uint32_t idesc = idesc_bf16(256, cols, false, false);
+      for (int t = 0; t < tiles.n_tiles; ++t) {
+        const int buf = t & 1;
+        mbar_wait(tmem_empty + buf, ((t >> 1) & 1u) ^ 1u, p.dev_status);
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * LC_MAX_COLS);
+        for (int kb = 0; kb < n_kb; ++kb) {
+          mbar_wait(full_bar + stage, phase, p.dev_status);
+          tc_fence_after();
+          const uint32_t sa = base_u32 + stage * sp.stage_bytes;
+          const uint64_t adesc = smem_desc_sw128(sa, 1024, 16), bdesc = smem_desc_sw128(sa + LC_A_BYTES, 1024, 16);
+#pragma unroll
+          for (int k = 0; k < LM_BK / 16; ++k) tc_mma_ss_pair(d_tmem, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0);
+          tc_commit_pair(empty_bar + stage, 3);
+          if (++stage == sp.stages) { stage = 0; phase ^= 1u; }
+        }
+        tc_commit_pair(tmem_full + buf, 3);
+      }
+    }
+  } else {
+    // ------------------------------------------------------------------ epilogue (warps 0-7)
+    const int quad = warp & 3, side = warp >> 2;              // lanes of tensor memory; every other block of 16 columns
+    const int col = lane & 15, upper = lane >> 4;
+    float* xb = reinterpret_cast<float*>(xpose + warp * LW_XPOSE_BYTES);
+    const float c = p.c;
+    const uint32_t tmem_empty_leader = cluster_map(smem_u32(tmem_empty), 0);
+    LmColStats run[LC_MAX_COLS / 32];                         // columns 32 h + 16 side + col
+#pragma unroll
+    for (int h = 0; h < LC_MAX_COLS / 32; ++h) {
+      run[h].m = -INFINITY; run[h].s = 0.f; run[h].t = 0.f;
+      run[h].v1 = -INFINITY; run[h].v2 = -INFINITY; run[h].i1 = -1; run[h].i2 = -1;
+    }
+    for (int t = 0; t < tiles.n_tiles; ++t) {
+      int n0, nw;
+      tiles.tile(t, n0, nw);
+      const int buf = t & 1;
+      mbar_wait(tmem_full + buf, (t >> 1) & 1u, p.dev_status);
+      tc_fence_after();
+      const int v_first = n0 + static_cast<int>(rank) * (nw >> 1), v_end = min(v_first + (nw >> 1), p.V), v_warp = v_first + quad * 32;
+      const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(buf * LC_MAX_COLS + 16 * side);
+      if (v_warp < v_end && 16 * side < cols) {
+        uint32_t r[16];
+        tmem_ld16(taddr, r);
+#pragma unroll
+        for (int h = 0; h < LC_MAX_COLS / 32; ++h) {
+          if (32 * h + 16 * side >= cols) break;
+          float z[16];
+          lm_block16(r, taddr + 32 * (h + 1), 32 * (h + 1) + 16 * side < cols, xb, lane, z);
+          if (v_warp + 16 * upper < v_end) lm_fold16<kEntropy>(z, v_warp + 16 * upper, v_end, c, run[h]);
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(tmem_empty_leader + static_cast<uint32_t>(buf) * 8u);
+    }
+#pragma unroll
+    for (int h = 0; h < LC_MAX_COLS / 32; ++h) {
+      if (32 * h + 16 * side >= cols) break;
+      const LmColMerge o = lm_merge_halves<kEntropy>(run[h], c);
+      if (upper == 0) red[quad * LC_MAX_COLS + 32 * h + 16 * side + col] = o;
+    }
+  }
+  tc_fence_before();
+  cluster_sync_all();    // both CTAs' statistics are in shared memory; the leader's MMAs and commits on the peer are over
+  if (warp == LC_EPI_WARPS + 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem_base, 512);
+  }
+  pdl_wait();            // the partials of the previous pass may still be read until earlier kernels are done
+  // a column's eight shares, four of them the peer's; each CTA merges half of the columns
+  for (int column = static_cast<int>(rank) * half_cols + threadIdx.x; column < (static_cast<int>(rank) + 1) * half_cols; column += LC_THREADS) {
+    const int row = work.mt0 * cols + column;
+    if (row >= sp.n_rows) break;
+    LmColMerge q[8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const uint32_t at = cluster_map(smem_u32(red + (s & 3) * LC_MAX_COLS + column), s >> 2);
+      const uint4 a = ld_cluster_u4(at), b = ld_cluster_u4(at + 16);
+      q[s].top.a = (static_cast<unsigned long long>(a.y) << 32) | a.x;
+      q[s].top.b = (static_cast<unsigned long long>(a.w) << 32) | a.z;
+      q[s].m = __uint_as_float(b.x); q[s].s = __uint_as_float(b.y); q[s].t = __uint_as_float(b.z);
+    }
+    p.partial[static_cast<size_t>(work.part) * p.part_rows + row] = lm_merge_shares<kEntropy>(q, p.c);
+  }
+  cluster_sync_all();    // nobody leaves while its shared memory may still be read
+}
+
 static thread_local int tl_lm_reserved_sms = 0;
 void lm_reserve_sms_once(int n) { tl_lm_reserved_sms = n > 0 ? n : 0; }
 
@@ -923,6 +1097,7 @@ struct LmPlan {
   bool few_rows;   // at most 128 rows: lmhead_rows_kernel, one CTA and one vocabulary range per SM
   bool pack;       // the rows of an index list are gathered into the workspace first
   bool slots;      // (no workspace to gather into) four slots of 64 node rows per M tile
+  bool cols;       // lmhead_cols_kernel: the rows of an M tile are the columns
   int slot_rows;   // few_rows and an index list of several: columns per sequence, read without gathering; 0 = packed
   int n_mt;        // M tiles of 256 rows
   int n_ranges;    // vocabulary ranges of the main part (few_rows: one per CTA, at most this many)
@@ -964,6 +1139,7 @@ static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, si
   // 142 -> 123 us).
   pl->few_rows = lm_takes_few_rows(a, rows) && !slots;
   pl->slot_rows = 0;
+  pl->cols = false;
   if (pl->few_rows) {
     pl->n_mt = 1;
     pl->tile_rows = 0;
@@ -990,6 +1166,11 @@ static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, si
   int tail = pairs - pl->n_mt * r;
   if (pl->n_mt < 2 || tail < 1 || pl->n_mt * r > pairs) tail = 0;
   while (tail > 0 && static_cast<size_t>(r + tail) * pl->part_rows * sizeof(LmPartial) > max_ws) --tail;
+  // Rows as columns where the M tiles would be a quarter padding or more, over rows long enough to hide the heavier statistics
+  // (LM head alone, pair kernel against this one: 183 rows of 5120 345 and 327 us, 312 of 4096 394 and 368, 576 of 4096 575 and
+  // 563, 150 of 2048 137 and 133; 784 of 4096, a fifth padding, 752 and 749; 488 of 2048 262 and 278; 150 of 1024 31 and 42).
+  pl->cols = !slots && pl->tile_rows <= 192 && a->d >= 2048 && lm_long_stream(a);
+  if (pl->cols) tail = 0;
   if (tail > 0) {
     int best_slice = 0, best_cost = (V32 / r + 7) / 8 + 1;    // without a tail: the longest main range
     {
@@ -1249,6 +1430,25 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
     const uint64_t strides[1] = {static_cast<uint64_t>(a->d) * 2};
     const uint32_t box[2] = {LM_BK, 64};
     if (!cached_tmap_bf16(&tm_w, a->W, 2, dims, strides, box)) return TRISPEC_ERR_CUDA;
+  }
+  if (pl.cols) {
+    LmColsParams sp;
+    sp.base = p;
+    sp.n_rows = static_cast<int>(n_rows);
+    sp.stage_bytes = LC_A_BYTES + p.tile_rows / 2 * (LM_BK * 2);
+    sp.stages = LC_RING_BYTES / sp.stage_bytes < LC_MAX_STAGES ? LC_RING_BYTES / sp.stage_bytes : LC_MAX_STAGES;
+    typedef void (*ColsKernel)(CUtensorMap, CUtensorMap, LmColsParams);
+    const ColsKernel kernel = want_entropy ? lmhead_cols_kernel<true> : lmhead_cols_kernel<false>;
+    static bool smem_set_cols[2][64] = {};
+    rc = ensure_smem_limit(reinterpret_cast<const void*>(kernel), LW_SMEM_BYTES, smem_set_cols[want_entropy ? 1 : 0]);
+    if (rc != TRISPEC_OK) return rc;
+    TRISPEC_CUDA_OK(launch_dependent(kernel, static_cast<unsigned>(2 * p.n_mt * n_ranges), LC_THREADS, static_cast<size_t>(LW_SMEM_BYTES),
+                                     st, 2, tm_w, tm_h, sp));
+    count_launch();
+    f.stride = pl.part_rows;
+    TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel, static_cast<unsigned>((n_rows + 7) / 8), LM_FIN_THREADS, 0, st, 1, f, n_seq));
+    count_launch();
+    return TRISPEC_OK;
   }
   static bool smem_set[2][64] = {};
   typedef void (*GemmKernel)(CUtensorMap, CUtensorMap, LmParams);
