@@ -30,11 +30,12 @@ RECORD = os.path.join(PKG, "..", "profiles", "dram_traffic.json")
 _COMMON = ["csrc/sm100.cuh", "csrc/host_common.h"]
 SOURCES = {
     "lmhead_gemm_kernel": ["csrc/lmhead.cu"] + _COMMON,
+    "lmhead_cols_kernel": ["csrc/lmhead.cu"] + _COMMON,
     "lmhead_rows_kernel": ["csrc/lmhead.cu"] + _COMMON,
-    "verify_attn_split_kernel": ["csrc/attn.cu", "csrc/attn_common.cuh"] + _COMMON,
+    "verify_attn_split_kernel": ["csrc/attn.cu", "csrc/attn_split.cuh", "csrc/attn_common.cuh"] + _COMMON,
     "verify_attn_pieces_kernel": ["csrc/attn_pieces.cu", "csrc/attn_common.cuh"] + _COMMON,
     "accept_scan_kernel": ["csrc/accept_scan.cu", "csrc/host_common.h"],
-    "tree_mask_block_kernel": ["csrc/tree_mask.cu", "csrc/host_common.h"],
+    "tree_mask_block_kernel": ["csrc/tree_mask.cu", "csrc/tree_mask.cuh", "csrc/host_common.h"],
 }
 
 _UNIT = {"byte": 1.0, "Kbyte": 1e3, "Mbyte": 1e6, "Gbyte": 1e9, "Tbyte": 1e12}
