@@ -34,7 +34,7 @@
  *     that gave up, an index or length outside its range, a malformed tree); the kernels never
  *     trap and never read or write outside the caller's arrays because of such a value.
  *   - Ordering. A call may read any of its inputs as soon as its first kernel starts, and that
- *     kernel does nothing before what was enqueued ahead of it has completed: whatever was enqueued on `stream` before the
+ *     kernel is an ordinary stream-ordered launch: whatever was enqueued on `stream` before the
  *     call - the caller's own kernels and copies, or an earlier call of this library such as a
  *     KV commit, a pruning step or the scan that wrote an escalation list - has completed by
  *     then. One exception is the caller's to avoid: a kernel that uses programmatic dependent

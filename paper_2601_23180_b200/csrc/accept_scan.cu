@@ -152,8 +152,8 @@ __device__ __forceinline__ int scan_sequence(const trispec_scan_args& a, const l
 template <int kCrit, int kAccept>
 __global__ void __launch_bounds__(kScanThreads)
 accept_scan_kernel(trispec_scan_args a) {
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const long long b = static_cast<long long>(blockIdx.x) * (kScanThreads / 32) + (threadIdx.x >> 5);
   if (b >= a.B) return;
@@ -168,16 +168,14 @@ template <int kCrit, int kAccept>
 __global__ void __launch_bounds__(32 * kScanSmallMax)
 accept_scan_small_kernel(trispec_scan_args a, int rehearse) {
   __shared__ int s_esc[kScanSmallMax];
+  pdl_launch_dependents();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int esc = 0;
   // Behind another kernel of the same call the scan runs twice, the first time before the wait and without writing: that
   // brings its code into the instruction cache (the loads bypass L1).
 #pragma unroll 1
   for (int run = rehearse ? 0 : 1; run < 2; ++run) {
-    if (run == 1) {
-      pdl_wait();
-      pdl_launch_dependents();
-    }
+    if (run == 1) pdl_wait();
     if (warp < a.B) esc = scan_sequence<kCrit, kAccept>(a, warp, lane, run == 1);
   }
   if (lane == 0) s_esc[warp] = esc;
@@ -354,7 +352,7 @@ int scan_check(const trispec_scan_args* a) {
 }  // namespace trispec
 
 extern "C" int trispec_accept_scan(const trispec_scan_args* a, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   using namespace trispec;
   const int rc = scan_check(a);
   if (rc != TRISPEC_OK) return rc;
@@ -374,7 +372,6 @@ extern "C" int trispec_accept_scan(const trispec_scan_args* a, void* stream) {
                                       TRISPEC_SCAN_ROW(accept_scan_kernel, TRISPEC_CRIT_ENTROPY)};
 #undef TRISPEC_SCAN_ROW
   const int rehearse = entry_scope_launched() ? 1 : 0;    // its inputs are complete but for what this call computes
-  launch_first_early(st);
   if (a->B <= kScanSmallMax) {
     TRISPEC_CUDA_OK(launch_dependent(small_k[which], 1u, static_cast<unsigned>(32 * a->B), 0, st, 1, *a, rehearse));
     count_launch();

@@ -10,7 +10,7 @@ __global__ void __launch_bounds__(AT_THREADS, kMerge == MERGE_IN_TURN ? 1 : 2)
 verify_attn_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                          const __grid_constant__ CUtensorMap tm_kt, const __grid_constant__ CUtensorMap tm_vt,
                          const AttnParams p) {
-  pdl_enter(p.first);
+  pdl_launch_dependents();
   attn_split_cta<kMerge, NP>(tm_k, tm_v, tm_kt, tm_vt, p, blockIdx.x);
 }
 
@@ -305,7 +305,6 @@ static AttnParams attn_params(const trispec_attn_args* a, const AttnPlan& pl) {
   p.dev_status = a->dev_status;
   p.n_seq = pl.n_seq;
   p.parent = nullptr;
-  p.first = 0;
   p.n_cta = pl.n_cta;
   return p;
 }
@@ -328,7 +327,7 @@ int attn_beside(const trispec_attn_args* a, const trispec_tree_args* tree, bool 
 }  // namespace trispec
 
 extern "C" int trispec_verify_attn(const trispec_attn_args* a, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   using namespace trispec;
   AttnPlan pl;
   int rc = attn_checked_plan(a, &pl);
@@ -354,8 +353,7 @@ extern "C" int trispec_verify_attn(const trispec_attn_args* a, void* stream) {
   static bool smem_set[5][64] = {};
   rc = ensure_smem_limit(reinterpret_cast<const void*>(kernel), smem_bytes, smem_set[which]);
   if (rc != TRISPEC_OK) return rc;
-  AttnParams p = attn_params(a, pl);
-  p.first = launch_first_early(st);
+  const AttnParams p = attn_params(a, pl);
   if (pl.pieces) {
     const CUtensorMap maps[4] = {tm_k, tm_v, tm_kt, tm_vt};
     return attn_launch_pieces(p, maps, two_p, a->workspace, st);

@@ -57,7 +57,6 @@ struct AttnParams {
   float* lse;       // [B][Hq][T] or null
   int32_t* dev_status;
   const int32_t* parent;   // in turn: the CTA computes the mask of its tree from these, or null = `mask`
-  int first;        // this is the call's first kernel, launched early (pdl_enter)
   // persistent kernel only
   int n_seq;        // active sequences (at most 128)
   int n_cta;        // CTAs of the launch: CTA c walks tiles [c W / n_cta, (c + 1) W / n_cta) of the work

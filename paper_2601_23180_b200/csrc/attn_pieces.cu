@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2)
 verify_attn_pieces_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                           const __grid_constant__ CUtensorMap tm_kt, const __grid_constant__ CUtensorMap tm_vt,
                           const AttnParams p) {
-  pdl_enter(p.first);
+  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // The loader and the issuer warp each keep a copy of the work map (registers) and walk this CTA's
   // pieces with it; the softmax warps get every piece from the issuer through a two-entry mailbox in

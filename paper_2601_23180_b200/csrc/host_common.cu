@@ -13,32 +13,17 @@ void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 namespace {
 thread_local int tl_scope_depth = 0;
 thread_local bool tl_scope_launched = false;
-thread_local bool tl_scope_early = false;       // the next launch is the call's first and may be made early
-thread_local bool tl_scope_ordinary = false;    // ... may not: it follows an event of another stream
 }  // namespace
 EntryScope::EntryScope() {
-  if (tl_scope_depth++ == 0) tl_scope_launched = tl_scope_early = tl_scope_ordinary = false;
+  if (tl_scope_depth++ == 0) tl_scope_launched = false;
 }
 EntryScope::~EntryScope() { --tl_scope_depth; }
-void entry_scope_next_launch_ordinary() {
-  tl_scope_launched = false;
-  tl_scope_ordinary = true;
-}
+void entry_scope_next_launch_ordinary() { tl_scope_launched = false; }
 bool entry_scope_launched() { return tl_scope_depth > 0 && tl_scope_launched; }
 bool entry_scope_outermost() { return tl_scope_depth == 1; }
-bool launch_first_early(cudaStream_t st) {
-  if (tl_scope_depth == 0 || tl_scope_launched || tl_scope_ordinary) return false;
-  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return tl_scope_early = status == cudaStreamCaptureStatusNone;
-}
 bool entry_scope_next_launch_is_dependent() {
-  const bool dependent = tl_scope_depth > 0 && (tl_scope_launched || tl_scope_early);
+  const bool dependent = tl_scope_depth > 0 && tl_scope_launched;
   tl_scope_launched = true;
-  tl_scope_early = tl_scope_ordinary = false;
   return dependent;
 }
 

@@ -42,8 +42,8 @@ __device__ __forceinline__ int commit_rows(const CommitParams& p, int b, int L) 
 
 __global__ void __launch_bounds__(kCommitThreads)
 kv_commit_kernel(const CommitParams p) {
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   const int b = blockIdx.x;
   const int L = __ldg(p.ctx_len + b);
   const int rows = commit_rows(p, b, L);
@@ -103,7 +103,7 @@ kv_commit_len_kernel(const CommitParams p) {
 }  // namespace trispec
 
 extern "C" int trispec_commit_kv(const trispec_commit_args* a, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   using namespace trispec;
   if (!a || a->B <= 0 || a->T <= 0 || a->Hkv <= 0) return TRISPEC_ERR_INVALID_ARG;
   if (a->D != 128 || a->T > 64) return TRISPEC_ERR_UNSUPPORTED;
@@ -131,7 +131,6 @@ extern "C" int trispec_commit_kv(const trispec_commit_args* a, void* stream) {
   p.block_table = a->block_table; p.ctx_len = a->ctx_len; p.path = a->path; p.accept_len = a->accept_len;
   p.active = a->active; p.ctx_len_out = a->ctx_len_out; p.dev_status = a->dev_status;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  launch_first_early(st);
   TRISPEC_CUDA_OK(launch_dependent(kv_commit_kernel, static_cast<unsigned>(a->B), kCommitThreads, 0, st, 1, p));
   count_launch();
   TRISPEC_CUDA_OK(launch_dependent(kv_commit_len_kernel, static_cast<unsigned>((a->B + 255) / 256), 256, 0, st, 1, p));

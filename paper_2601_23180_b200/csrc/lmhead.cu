@@ -60,7 +60,6 @@ struct LmParams {
   int tile_rows;  // packed rows per M tile, a multiple of 16 up to 256 (4 sequence slots: 256)
   int slots;      // rows are not packed: an M tile is 4 slots of 64 node rows, read through seq_index
   int wait_rows;  // the packed rows are written by the kernel before this one
-  int first;      // this is the call's first kernel, launched early (pdl_enter)
   int n_ranges;   // vocabulary ranges of the main part: pair c < n_mt * n_ranges works on M tile c % n_mt, range c / n_mt
   int n_tail;     // pairs beyond those: each sweeps ALL M tiles over its slice of the vocabulary's tail
   int main_units; // 32-column units [0, main_units) belong to the main part, the rest to the tail
@@ -211,7 +210,7 @@ template <bool kEntropy>
 __global__ void __launch_bounds__(LM_THREADS, 1)
 lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ CUtensorMap tmap_w,
                    const LmParams p) {
-  if (!p.first) pdl_launch_dependents();
+  pdl_launch_dependents();
   extern __shared__ uint8_t smem_raw[];
   // the dynamic window starts at the same offset in both CTAs of the pair, so the aligned
   // layouts coincide, as the paired MMA requires
@@ -252,7 +251,6 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
   tc_fence_before();
   cluster_sync_all();                             // both CTAs' barriers and TMEM are ready
   tc_fence_after();
-  if (p.first) pdl_wait();                        // what is above needs nothing from earlier kernels
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 4) {
@@ -260,7 +258,6 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
     if (lane == 0) {
       int stage = 0;
       uint32_t phase = 0;
-      if (p.first) pdl_launch_dependents();
       if (p.wait_rows) pdl_wait();
       // the rows are spread evenly over the M tiles, and only those that a tile has are fetched
       const int half_rows = p.tile_rows >> 1;
@@ -404,8 +401,8 @@ lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_cons
 // of W it is small: 3 sequences of 61 rows of 5120 are 1.9 MB.
 __global__ void __launch_bounds__(256)
 lmhead_pack_rows_kernel(const uint4* __restrict__ h, const int32_t* __restrict__ seq_index, uint4* __restrict__ out, int B, int T,
-                        int vecs /* 16-byte words per row */, long long n_rows, int first) {
-  pdl_enter(first);
+                        int vecs /* 16-byte words per row */, long long n_rows) {
+  pdl_launch_dependents();
   const int lane = threadIdx.x & 31;
   const long long r = static_cast<long long>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   const bool active = r < n_rows;
@@ -759,7 +756,6 @@ __device__ __forceinline__ void lm_rows_cta(const CUtensorMap& tmap_w, const CUt
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (p.first) pdl_wait();                        // what is above needs nothing from earlier kernels
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == LW_EPI_WARPS) {
@@ -896,7 +892,7 @@ lmhead_rows_beside_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gr
                           const __grid_constant__ AttnBeside at) {
   const int block = blockIdx.x;
   if (block < at.ctas) {
-    pdl_enter(sp.base.first);
+    pdl_launch_dependents();
     const int spare = static_cast<int>(threadIdx.x >> 5) - AT_THREADS / 32;
     if (spare == 0 && at.masks) attn_mask_warp<kPair>(at.p, block);
     if (spare == 1 && at.masks) {                      // what the tree step returns, of all sequences
@@ -937,7 +933,7 @@ struct LmColsParams {
 template <bool kEntropy>
 __global__ void __launch_bounds__(LC_THREADS, 1)
 lmhead_cols_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_h, const LmColsParams sp) {
-  if (!sp.base.first) pdl_launch_dependents();
+  pdl_launch_dependents();
   const LmParams& p = sp.base;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base_u32 = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -970,7 +966,6 @@ lmhead_cols_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
   tc_fence_before();
   cluster_sync_all();                                 // both CTAs' barriers and TMEM are ready
   tc_fence_after();
-  if (p.first) pdl_wait();                            // what is above needs nothing from earlier kernels
   const uint32_t tmem_base = *tmem_slot;
   LmColMerge* red = reinterpret_cast<LmColMerge*>(smem);           // [4 warps][columns], in the ring's memory at the end
 
@@ -978,7 +973,6 @@ lmhead_cols_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     if (lane == 0) {   // ---------------------------------------------------------- TMA producer
       int stage = 0;
       uint32_t phase = 0;
-      if (p.first) pdl_launch_dependents();
       if (p.wait_rows) pdl_wait();
       const int row0 = work.mt0 * cols + static_cast<int>(rank) * half_cols;
       for (int t = 0; t < tiles.n_tiles; ++t) {
@@ -1285,7 +1279,7 @@ int lmhead_stats_beside(const trispec_lmhead_args* a, const AttnBeside& beside, 
 }
 
 extern "C" int trispec_lmhead_stats(const trispec_lmhead_args* a, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   using namespace trispec;
   LmPlan pl;
   const int rc = lm_plan(a, &pl, a ? a->workspace_bytes : 0);
@@ -1331,7 +1325,6 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   p.tile_rows = pl.tile_rows;
   p.part_rows = pl.part_rows;
   p.wait_rows = pl.pack ? 1 : 0;
-  p.first = launch_first_early(st);     // (the pass in which it is not the first has launched the mask kernel)
   p.c = f.c;
   p.seq_index = a->seq_index;
   p.partial = static_cast<LmPartial*>(a->workspace);
@@ -1342,9 +1335,8 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
     uint4* packed = reinterpret_cast<uint4*>(static_cast<char*>(a->workspace) + pl.required);
     rows_base = packed;
     TRISPEC_CUDA_OK(launch_dependent(lmhead_pack_rows_kernel, static_cast<unsigned>((n_rows + 7) / 8), 256, 0, st, 1,
-                                     static_cast<const uint4*>(a->h), a->seq_index, packed, a->B, a->T, a->d / 8, n_rows, p.first));
+                                     static_cast<const uint4*>(a->h), a->seq_index, packed, a->B, a->T, a->d / 8, n_rows));
     count_launch();
-    p.first = 0;
   }
   if (pl.few_rows) {
     LmRowsParams sp;
@@ -1495,7 +1487,7 @@ static int lm_noalloc_scratch(void** out) {
 }  // namespace trispec
 
 extern "C" int trispec_lmhead_stats_noalloc(const trispec_lmhead_args* a, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   using namespace trispec;
   // planned so that the partial array fits the built-in scratch (fewer tail pairs where they would not)
   LmPlan pl;

@@ -29,8 +29,8 @@ __device__ __forceinline__ unsigned long long prune_pack_mask(unsigned long long
 
 __global__ void __launch_bounds__(kPruneThreads)
 prune_tree_kernel(trispec_prune_args a) {
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const long long b = static_cast<long long>(blockIdx.x) * (kPruneThreads / 32) + (threadIdx.x >> 5);
   if (b >= a.B) return;
@@ -86,7 +86,7 @@ prune_tree_kernel(trispec_prune_args a) {
 }  // namespace trispec
 
 extern "C" int trispec_prune_tree(const trispec_prune_args* a, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   using namespace trispec;
   if (!a || a->B <= 0 || a->T <= 0) return TRISPEC_ERR_INVALID_ARG;
   if (a->T > 64) return TRISPEC_ERR_UNSUPPORTED;
@@ -95,7 +95,6 @@ extern "C" int trispec_prune_tree(const trispec_prune_args* a, void* stream) {
   if (a->parent_out == a->parent || a->tok_out == a->tok || a->mask_out == a->mask) return TRISPEC_ERR_INVALID_ARG;
   const int per_block = kPruneThreads / 32;
   const unsigned grid = static_cast<unsigned>((static_cast<long long>(a->B) + per_block - 1) / per_block);
-  launch_first_early(static_cast<cudaStream_t>(stream));
   TRISPEC_CUDA_OK(launch_dependent(prune_tree_kernel, grid, kPruneThreads, 0, static_cast<cudaStream_t>(stream), 1, *a));
   count_launch();
   return TRISPEC_OK;

@@ -59,8 +59,8 @@ __device__ __forceinline__ float gumbel_from_word(unsigned int w) {
 
 __global__ void __launch_bounds__(256)
 sample_gather_kernel(const SampleParams p) {
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   const int b = blockIdx.x;
   const bool live = b < p.B && __ldg(p.bonus_tok + b) == -2;
   int node = live ? __ldg(p.last_node + b) : 0;
@@ -452,7 +452,7 @@ extern "C" size_t trispec_sample_bonus_workspace(const trispec_sample_args* a) {
 }
 
 extern "C" int trispec_sample_bonus(const trispec_sample_args* a, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   using namespace trispec;
   int n_mt, n_ranges;
   int rc = sample_plan(a, &n_mt, &n_ranges);
@@ -489,7 +489,6 @@ extern "C" int trispec_sample_bonus(const trispec_sample_args* a, void* stream) 
     const uint32_t box[2] = {SM_BK, 64};
     if (!cached_tmap_bf16(&tm_w, a->W, 2, dims, strides, box)) return TRISPEC_ERR_CUDA;
   }
-  launch_first_early(st);
   TRISPEC_CUDA_OK(launch_dependent(sample_gather_kernel, static_cast<unsigned>(n_mt * SM_BM), 256, 0, st, 1, p));
   count_launch();
   if (a->B <= SW_MAX_SEQ * SW_MAX_GROUPS) {

@@ -13,8 +13,8 @@ constexpr int kMaskSeqPerWarp = 2;  // sequences per warp: their loads are issue
 __global__ void __launch_bounds__(kMaskThreads)
 tree_mask_kernel(const int32_t* __restrict__ parent, uint64_t* __restrict__ mask, int32_t* __restrict__ depth,
                  long long n_seq, int T, int32_t* __restrict__ status) {
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const long long w = static_cast<long long>(blockIdx.x) * (kMaskThreads / 32) + (threadIdx.x >> 5);
   const long long b0 = w * kMaskSeqPerWarp;
@@ -69,8 +69,8 @@ tree_mask_block_kernel(const int32_t* __restrict__ parent, uint64_t* __restrict_
                        long long n_seq, int T, int32_t* __restrict__ status) {
   __shared__ signed char sPar[64 * kMaskParPitch];
   __shared__ unsigned long long sMask[kMaskBlockSeqs * kMaskSeqPitch];
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   const long long s0 = static_cast<long long>(blockIdx.x) * kMaskBlockSeqs;
   const int n_here = static_cast<int>(min(static_cast<long long>(kMaskBlockSeqs), n_seq - s0));
   const int n_elem = n_here * T;
@@ -157,14 +157,13 @@ int trispec::tree_mask_check(const trispec_tree_args* a) {
 }
 
 extern "C" int trispec_build_tree_mask(const trispec_tree_args* a, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   using namespace trispec;
   const int rc = tree_mask_check(a);
   if (rc != TRISPEC_OK) return rc;
   const long long n = a->B;
   if (n >= 2048) {   // enough sequences to fill the chip with a thread each
     unsigned grid = static_cast<unsigned>((n + kMaskBlockSeqs - 1) / kMaskBlockSeqs);
-    launch_first_early(static_cast<cudaStream_t>(stream));
     TRISPEC_CUDA_OK(launch_dependent(tree_mask_block_kernel, grid, kMaskBlockThreads, 0,
                                      static_cast<cudaStream_t>(stream), 1, a->parent, a->mask, a->depth, n, a->T,
                                      a->dev_status));
@@ -173,7 +172,6 @@ extern "C" int trispec_build_tree_mask(const trispec_tree_args* a, void* stream)
   }
   const int per_block = (kMaskThreads / 32) * kMaskSeqPerWarp;
   unsigned grid = static_cast<unsigned>((n + per_block - 1) / per_block);
-  launch_first_early(static_cast<cudaStream_t>(stream));
   TRISPEC_CUDA_OK(launch_dependent(tree_mask_kernel, grid, kMaskThreads, 0, static_cast<cudaStream_t>(stream), 1,
                                    a->parent, a->mask, a->depth, n, a->T, a->dev_status));
   count_launch();

@@ -297,7 +297,7 @@ extern "C" int trispec_verify_beside(const trispec_attn_args* attn, const trispe
 
 extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_args* attn,
                               const trispec_lmhead_args* lm, const trispec_scan_args* scan, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   if (!tree || !lm || !scan) return TRISPEC_ERR_INVALID_ARG;
   // The attention and the LM head do not depend on each other, so their order is free. A kernel launched as
   // a programmatic dependent gets its launch latency and prologue hidden, but its loads make almost no
@@ -331,8 +331,7 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
     if (side) {
       TRISPEC_CUDA_OK(cudaEventRecord(side->fork, st));
       TRISPEC_CUDA_OK(cudaStreamWaitEvent(side->stream, side->fork, 0));
-      entry_scope_next_launch_ordinary();                    // (behind the event)
-      rc = trispec_build_tree_mask(tree, side->stream);
+      rc = trispec_build_tree_mask(tree, side->stream);      // ordinary launch: first kernel of the call
       if (rc == TRISPEC_OK) {
         rc = trispec_verify_attn(attn, side->stream);        // dependent of the mask kernel
       }
@@ -374,7 +373,7 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
 extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree_args* tree,
                                    const trispec_attn_args* attn, const trispec_lmhead_args* lm,
                                    const trispec_scan_args* scan, void* stream) {
-  trispec::EntryScope entry_scope;   // the first kernel launched below waits for all earlier work on the stream
+  trispec::EntryScope entry_scope;   // the first kernel launched below is an ordinary launch
   using namespace trispec;
   if (!io || !tree || !lm || !scan) return TRISPEC_ERR_INVALID_ARG;
   // the copies below land in the buffers the structs name: they must describe one and the same pass
@@ -435,7 +434,6 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
     // few rows (as in trispec_verify): mask and attention follow their inputs on
     // the second stream, the LM head and the scan run on `stream`, which then waits for the second stream
     TRISPEC_CUDA_OK(cudaStreamWaitEvent((*side)->stream, (*side)->inputs, 0));   // the tree's parents have arrived
-    entry_scope_next_launch_ordinary();                              // (behind the events)
     rc = trispec_build_tree_mask(tree, (*side)->stream);
     if (rc == TRISPEC_OK) {
       attn_in_turn_once(plan.in_turn);
@@ -453,7 +451,6 @@ extern "C" int trispec_verify_host(const trispec_host_io* io, const trispec_tree
     TRISPEC_CUDA_OK(cudaStreamWaitEvent(st, (*side)->done, 0));
     if (rc != TRISPEC_OK) return rc;
   } else {
-    entry_scope_next_launch_ordinary();                      // (behind the copies)
     rc = trispec_build_tree_mask(tree, stream);
     if (rc != TRISPEC_OK) return rc;
     lm_reserve_sms_once(plan.beside ? plan.attn_ctas : 0);   // (as in trispec_verify)

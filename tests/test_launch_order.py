@@ -1,0 +1,57 @@
+"""How a call's launches are ordered behind earlier work, seen from the requests to the CUDA runtime."""
+from tests.host_launches import requests
+
+EVERY_CALL = """
+S = 77                                            # the caller's stream
+forms = dict(one_launch=dict(), in_turn=dict(T=61, cap=4096, V=151936), two_streams=dict(T=9, Hq=8, Hkv=1, cap=8192),
+             lm_first=dict(T=61, cap=8192, V=151936), batch=dict(B=8, T=61, cap=4096), pieces=dict(B=40, T=61, cap=32768),
+             listed=dict(B=12, T=61, listed=5, cap=700, V=151936), columns=dict(B=3, T=61, cap=700, d=5120, V=151936), many=dict(B=3000, T=9, cap=64))
+for name, kw in forms.items():
+    p = Args(**kw)
+    structs = (r(p.tree), r(p.attn), r(p.lm), r(p.scan), S)
+    call("verify_" + name, lib.trispec_verify(*structs))
+    call("host_" + name, lib.trispec_verify_host(r(ts.HostIO()), *structs))
+    call("mask_" + name, lib.trispec_build_tree_mask(r(p.tree), S))
+    call("attn_" + name, lib.trispec_verify_attn(r(p.attn), S))
+    call("lmhead_" + name, lib.trispec_lmhead_stats(r(p.lm), S))
+    call("scan_" + name, lib.trispec_accept_scan(r(p.scan), S))
+    if name == "one_launch":
+        call("noalloc", lib.trispec_lmhead_stats_noalloc(r(p.lm), S))
+    c = ts.CommitArgs()
+    c.B, c.T, c.Hkv, c.D, c.kv_layout, c.Lmax = p.attn.B, p.attn.T, p.attn.Hkv, 128, ts.KV_CONTIGUOUS, p.attn.Lmax
+    for f in ("k_tree", "v_tree", "k_cache", "v_cache", "ctx_len"):
+        setattr(c, f, getattr(p.attn, f))
+    c.path, c.accept_len, c.ctx_len_out = p.scan.path, p.scan.accept_len, p.new()
+    call("commit_" + name, lib.trispec_commit_kv(r(c), S))
+    u = ts.PruneArgs()
+    u.B, u.T, u.parent, u.tok, u.mask = p.tree.B, p.tree.T, p.tree.parent, p.lm.tok, p.tree.mask
+    for f in ("root", "n_keep", "node_map", "parent_out", "tok_out", "mask_out"):
+        setattr(u, f, p.new())
+    call("prune_" + name, lib.trispec_prune_tree(r(u), S))
+    b = ts.SampleArgs()
+    b.B, b.T, b.d, b.V, b.logit_scale = p.lm.B, p.lm.T, p.lm.d, p.lm.V, 1.0
+    b.h, b.W, b.last_node, b.bonus_tok = p.lm.h, p.lm.W, p.scan.last_node, p.scan.bonus_tok
+    b.workspace, b.workspace_bytes = p.new(), ts.trispec_sample_bonus_workspace(b)
+    call("sample_" + name, lib.trispec_sample_bonus(r(b), S))
+"""
+
+
+def test_the_first_kernel_of_every_call_is_an_ordinary_launch(tmp_path):
+    """A programmatic dependent waits for the kernel right ahead of it; a call's first kernel has to wait for everything
+    on its stream, whatever the caller put there last."""
+    calls = requests(tmp_path, EVERY_CALL)
+    assert len(calls) == 9 * 9 + 1
+    kernels = set()
+    for name, log in calls.items():
+        launches = [x for what, _, x in log if what == "launch"]
+        kernels |= {x.kernel for x in launches}
+        assert launches, name
+        for stream in {x.stream for x in launches}:
+            own = [x for x in launches if x.stream == stream]
+            assert not own[0].dependent, (name, own[0].kernel)
+        # the kernels inside a call are dependents of each other
+        if name.startswith("verify_") and "streams" not in name:
+            assert all(x.dependent for x in launches[1:]), name
+    for part in ("rows_beside", "lmhead_cols", "lmhead_gemm", "attn_pieces_kernel", "attn_split", "attn_merge", "tree_mask_block",
+                 "esc_compact", "sample_gather", "pack_rows", "prune_tree", "kv_commit_kernel"):
+        assert any(part in k for k in kernels), part
