@@ -20,7 +20,6 @@ EntryScope::EntryScope() {
 EntryScope::~EntryScope() { --tl_scope_depth; }
 void entry_scope_next_launch_ordinary() { tl_scope_launched = false; }
 bool entry_scope_launched() { return tl_scope_depth > 0 && tl_scope_launched; }
-bool entry_scope_outermost() { return tl_scope_depth == 1; }
 bool entry_scope_next_launch_is_dependent() {
   const bool dependent = tl_scope_depth > 0 && tl_scope_launched;
   tl_scope_launched = true;

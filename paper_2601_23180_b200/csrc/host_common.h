@@ -54,9 +54,8 @@ struct EntryScope {
 // True if a kernel was already launched inside the current outermost scope (the next launch may
 // then be a programmatic dependent); records that a launch happens now.
 bool entry_scope_next_launch_is_dependent();
-// Whether the current call has launched a kernel already; whether it is not part of another one
+// Whether the current call has launched a kernel already
 bool entry_scope_launched();
-bool entry_scope_outermost();
 // The next launch inside the current scope is an ordinary one again (after work was moved to or joined from
 // another stream, where "the kernel before it" is not the kernel enqueued last).
 void entry_scope_next_launch_ordinary();

@@ -425,8 +425,6 @@ struct LmFinalizeParams {
   int stride;       // partial rows per vocabulary range
   int pitch;        // partial rows per active sequence (T: packed rows)
   int rehearse;     // run the merge once before the wait
-  int last;         // the call's last kernel: the next call's first one may come once this one's wait is over, not before (LM
-                    // head after LM head, 61 rows, 32000 x 1024 weights: 29 us, with the next one there early 39)
   float scale, c;
   const int32_t* seq_index;
   const LmPartial* partial;
@@ -451,7 +449,7 @@ __device__ __forceinline__ float lm_weight(float m, float M, float c) { return (
 // the node's row and of the parent's row in one go and the warp folds them by shuffles.
 __global__ void __launch_bounds__(LM_FIN_THREADS)
 lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
-  if (!p.last) pdl_launch_dependents();
+  pdl_launch_dependents();
   const int lane = threadIdx.x & 31;
   const long long w = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int T = p.T;
@@ -503,7 +501,6 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
   for (int run = p.rehearse ? 0 : 1; run < 2; ++run) {
   if (run == 1) {
     pdl_wait();                                  // the partials come from the GEMM kernel
-    if (p.last) pdl_launch_dependents();
     if (!active) return;
   }
   // Up to 148 ranges are five per lane: loaded at once, folded relative to the row's maximum, so that the chains
@@ -1313,7 +1310,6 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   f.W = static_cast<const uint16_t*>(a->W);
   f.parent = a->parent; f.tok = a->tok; f.dev_status = a->dev_status;
   f.out = a->out;
-  f.last = entry_scope_outermost() ? 1 : 0;
   f.rehearse = pl.few_rows ? 0 : 1;
   f.pitch = pl.slots ? 64 : (pl.slot_rows > 0 ? pl.slot_rows : a->T);
 
