@@ -424,7 +424,6 @@ struct LmFinalizeParams {
   int B, T, d, V, n_ranges;
   int stride;       // partial rows per vocabulary range
   int pitch;        // partial rows per active sequence (T: packed rows)
-  int rehearse;     // run the merge once before the wait
   float scale, c;
   const int32_t* seq_index;
   const LmPartial* partial;
@@ -447,6 +446,11 @@ __device__ __forceinline__ float lm_weight(float m, float M, float c) { return (
 // The dot product needs only the kernel's inputs, so it runs before the wait for the GEMM and
 // overlaps that kernel's tail; after the wait every lane loads its share of the partials of
 // the node's row and of the parent's row in one go and the warp folds them by shuffles.
+// Bound by latency. (Going over the partials once before the wait, to have code and pages at hand, gave nothing beside the pair
+// kernel: 150 rows, 50257 x 1024 weights, 34.8 us either way.) kCg: loads that bypass L1, where the blocks come to wait on the SMs
+// of an attention in the same launch (one chain of 9 nodes 34.1 -> 33.4 us a pass); elsewhere they cost 1 to 4 us (LM head alone,
+// 32000 x 1024 weights, 18 rows 21.3 -> 23.9 us, 61 rows 25.1 -> 28.7; 9 rows, 32000 x 2048, 31.6 -> 32.6).
+template <bool kCg>
 __global__ void __launch_bounds__(LM_FIN_THREADS)
 lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
   pdl_launch_dependents();
@@ -489,20 +493,13 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
   }
   if (!has_draft) par = node;                    // a valid row to load; the result is not used
 
+  pdl_wait();                                    // the partials come from the GEMM kernel
+  if (!active) return;
+
   // ---- merge of the per-range partials: own row (all statistics) and parent row (max, sum)
   const size_t stride = static_cast<size_t>(p.stride);
   const LmPartial* own = p.partial + static_cast<size_t>(a) * p.pitch + node;
   const LmPartial* parp = p.partial + static_cast<size_t>(a) * p.pitch + par;
-  // Beside the pair kernel the blocks are resident early, and the merge runs twice: the first time before the wait, over whatever
-  // the partials hold then, so that its code and its pages are at hand (the loads bypass L1, nothing is stored; 150 rows, 50257 x
-  // 1024 weights: 36.6 -> 33.3 us). Beside the small-row kernel, which takes all shared memory, the blocks only start at that
-  // kernel's end, and a rehearsal would come on top (a pass of two sequences 90 -> 98 us).
-#pragma unroll 1
-  for (int run = p.rehearse ? 0 : 1; run < 2; ++run) {
-  if (run == 1) {
-    pdl_wait();                                  // the partials come from the GEMM kernel
-    if (!active) return;
-  }
   // Up to 148 ranges are five per lane: loaded at once, folded relative to the row's maximum, so that the chains
   // across the lanes are one maximum, the sums, and the top two as 64-bit keys, side by side.
   float m_own = -INFINITY, s_own = 0.f, t_own = 0.f, m_par = -INFINITY, s_par = 0.f;
@@ -519,9 +516,10 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
       qp[u] = make_float2(-INFINITY, 0.f);
       if (r < p.n_ranges) {
         const float4* q4 = reinterpret_cast<const float4*>(own + r * stride);
-        qa[u] = __ldcg(q4);                      // m, s, v1, v2
-        qb[u] = __ldcg(q4 + 1);                  // i1, i2, t, pad
-        qp[u] = __ldcg(reinterpret_cast<const float2*>(parp + r * stride));   // m, s of the parent's row
+        const float2* qp2 = reinterpret_cast<const float2*>(parp + r * stride);
+        qa[u] = kCg ? __ldcg(q4) : q4[0];        // m, s, v1, v2
+        qb[u] = kCg ? __ldcg(q4 + 1) : q4[1];    // i1, i2, t, pad
+        qp[u] = kCg ? __ldcg(qp2) : *qp2;        // m, s of the parent's row
       }
     }
     float mo = m_own, mp = m_par;
@@ -554,13 +552,8 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
   }
   const float v1 = lm_key_value(top.a), v2 = lm_key_value(top.b);
   const int i1 = lm_key_entry(top.a), i2 = lm_key_entry(top.b);
-  const float lse = m_own * p.scale + logf(s_own);
-  const float p1 = expf(v1 * p.scale - lse), p2 = expf(v2 * p.scale - lse);
-  // entropy in nats: H = lse - E_p[z], E_p[z] = scale * sum(e * z_raw) / sum(e); never below 0
-  const float entropy = fmaxf(lse - p.scale * (t_own / s_own), 0.f);
-  const float dl = dot * p.scale, pd = expf(dl - (m_par * p.scale + logf(s_par)));
-  asm volatile("" ::"f"(p1), "f"(p2), "f"(entropy), "f"(pd), "r"(i1), "r"(i2));   // (computed in both runs)
-  if (run == 1 && lane == 0) {
+  if (lane == 0) {
+    const float lse = m_own * p.scale + logf(s_own);
     const long long o = row0 + node;
     p.out.max[o] = m_own * p.scale;
     p.out.lse[o] = lse;
@@ -568,12 +561,17 @@ lmhead_finalize_kernel(const LmFinalizeParams p, int n_seq) {
     p.out.top2_val[o] = v2 * p.scale;
     p.out.top1_idx[o] = i1;
     p.out.top2_idx[o] = i2;
-    p.out.p_top1[o] = p1;
-    p.out.p_top2[o] = p2;
-    if (p.out.entropy) p.out.entropy[o] = entropy;
-    p.out.draft_logit[o] = has_draft ? dl : __int_as_float(0x7fc00000);
-    p.out.p_draft[o] = has_draft ? pd : __int_as_float(0x7fc00000);
-  }
+    p.out.p_top1[o] = expf(v1 * p.scale - lse);
+    p.out.p_top2[o] = expf(v2 * p.scale - lse);
+    // entropy in nats: H = lse - E_p[z], E_p[z] = scale * sum(e * z_raw) / sum(e); never below 0
+    if (p.out.entropy) p.out.entropy[o] = fmaxf(lse - p.scale * (t_own / s_own), 0.f);
+    float dl = __int_as_float(0x7fc00000), pd = dl;
+    if (has_draft) {
+      dl = dot * p.scale;
+      pd = expf(dl - (m_par * p.scale + logf(s_par)));
+    }
+    p.out.draft_logit[o] = dl;
+    p.out.p_draft[o] = pd;
   }
 }
 
@@ -1310,7 +1308,6 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
   f.W = static_cast<const uint16_t*>(a->W);
   f.parent = a->parent; f.tok = a->tok; f.dev_status = a->dev_status;
   f.out = a->out;
-  f.rehearse = pl.few_rows ? 0 : 1;
   f.pitch = pl.slots ? 64 : (pl.slot_rows > 0 ? pl.slot_rows : a->T);
 
   LmParams p;
@@ -1397,7 +1394,8 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
     count_launch();
     f.stride = pl.part_rows;
     // one row per block: as many SMs as rows fetch the merge's operands (LM head alone, 9 rows: 31.7 -> 30.1 us, 61: 110.7 -> 107.3)
-    TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel, static_cast<unsigned>(n_rows), 32, 0, st, 1, f, n_seq));
+    TRISPEC_CUDA_OK(launch_dependent(beside ? lmhead_finalize_kernel<true> : lmhead_finalize_kernel<false>, static_cast<unsigned>(n_rows),
+                                     32, 0, st, 1, f, n_seq));
     count_launch();
     return TRISPEC_OK;
   }
@@ -1434,7 +1432,7 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
                                      st, 2, tm_w, tm_h, sp));
     count_launch();
     f.stride = pl.part_rows;
-    TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel, static_cast<unsigned>((n_rows + 7) / 8), LM_FIN_THREADS, 0, st, 1, f, n_seq));
+    TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel<false>, static_cast<unsigned>((n_rows + 7) / 8), LM_FIN_THREADS, 0, st, 1, f, n_seq));
     count_launch();
     return TRISPEC_OK;
   }
@@ -1447,7 +1445,7 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
                                    LM_SMEM_BYTES, st, 2, tm_h, tm_w, p));
   count_launch();
   f.stride = pl.part_rows;
-  TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel, static_cast<unsigned>((n_rows + 7) / 8),
+  TRISPEC_CUDA_OK(launch_dependent(lmhead_finalize_kernel<false>, static_cast<unsigned>((n_rows + 7) / 8),
                                    LM_FIN_THREADS, 0, st, 1, f, n_seq));
   count_launch();
   return TRISPEC_OK;
