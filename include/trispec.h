@@ -388,10 +388,10 @@ int trispec_verify(const trispec_tree_args* tree, const trispec_attn_args* attn,
  * attention runs in few CTAs beside it where it then still ends in time, and after it otherwise);
  * "none" without `lm`. The environment variable TRISPEC_PASS_FORM = attention_first | lm_first |
  * side_by_side overrides the choice for so few rows.
- * trispec_verify_beside: the number of CTAs that the attention needs beside the LM head (it may be
- * given two for each of a few), or 0 where the steps run in stream order. Memory that a step shares with the `tree`
- * of the call, and a second stream that is not to be had, are the only reasons to run in stream
- * order that these answers do not see. */
+ * trispec_verify_beside: the number of CTAs in which the attention of trispec_verify runs beside the LM
+ * head, in its launch or on the second stream, or 0 where the steps run in stream order. Memory that a
+ * step shares with the `tree` of the call, and a second stream that is not to be had, are the only
+ * reasons to run in stream order that these answers do not see. */
 const char* trispec_verify_plan(const trispec_attn_args* attn, const trispec_lmhead_args* lm,
                                 const trispec_scan_args* scan);
 int trispec_verify_beside(const trispec_attn_args* attn, const trispec_lmhead_args* lm,

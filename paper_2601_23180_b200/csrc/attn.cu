@@ -201,13 +201,14 @@ int attn_compact_ctas(const trispec_attn_args* a, double budget_us, int max_ctas
   // nodes at 4096 tokens beside 151936 x 2048 weights: 131 -> 117 us a pass; 64 query heads at 8192 tokens, 64 CTAs: 258 -> 317).
   const bool two = pair && pl.n_splits >= 2 && 4 * ctas <= static_cast<size_t>(max_ctas);
   if (two) *pair = true;
+  const int launched = static_cast<int>(two ? 2 * ctas : ctas);
   // A CTA alone on its SM, launch included (measured: 18.5 us with 9 tiles in 2 splits, 28.7 with 17 in 4, 80.0 with 65 in 8,
   // 137.4 with 125 in 8). The context's capacity stands for its length, which only the device knows.
   const double us = 8.5 + 0.96 * (pl.tiles_max + 1) + 1.3 * (pl.n_splits - 1);
-  if (us <= budget_us) return static_cast<int>(ctas);
+  if (us <= budget_us) return launched;
   const int own = (pl.n_splits + 1) / 2;         // splits of a pair's longer half
   const double half = static_cast<double>(own) * ((pl.tiles_max + pl.n_splits - 1) / pl.n_splits);
-  if (two && 8.5 + 0.96 * (half + 1) + 1.3 * own <= budget_us) return static_cast<int>(2 * ctas);
+  if (two && 8.5 + 0.96 * (half + 1) + 1.3 * own <= budget_us) return launched;
   if (pair) *pair = false;
   return 0;
 }

@@ -104,8 +104,8 @@ int scan_check(const trispec_scan_args* a);
 int attn_planned_ctas(const trispec_attn_args* a);
 // CTAs of an attention whose plan merges its splits on chip when each (sequence, KV head, M tile) has one CTA, alone on
 // its SM, that takes the splits in turn (attn_split.cuh); 0 where the plan is another one, where that is more than `max_ctas`
-// CTAs, or where they would take longer than `budget_us`. `pair` (may be null): a pass that has both in one launch gives every item two CTAs
-// (the answer is the number of CTAs that end in time, twice the items where one each does not).
+// CTAs, or where they would take longer than `budget_us`. `pair` (may be null) allows, and then says, that a launch shared with the
+// LM head gives each of a few items two CTAs; both of them count.
 int attn_compact_ctas(const trispec_attn_args* a, double budget_us, int max_ctas, bool* pair);
 // The attention launches of this thread take that form while this is on
 void attn_in_turn_once(bool on);

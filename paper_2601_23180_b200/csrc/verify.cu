@@ -130,9 +130,10 @@ namespace trispec {
 enum PassForm { PASS_ATTENTION_FIRST = 0, PASS_LM_FIRST = 1, PASS_SIDE_BY_SIDE = 2 };
 struct PassPlan {
   PassForm form;
-  bool beside;        // mask and attention go to the second stream, the LM head leaves them `attn_ctas` SMs
+  bool beside;        // the attention runs beside the LM head, which leaves it `attn_ctas` SMs
   int attn_ctas;
-  bool in_turn;       // that attention takes the splits of its plan one after the other, in few CTAs
+  bool in_turn;       // that attention takes the splits of its plan one after the other, in few CTAs: in the LM head's launch (in
+                      // trispec_verify_host on the second stream, as the attention's own plan always is)
   bool pair;          // two CTAs per item, in the LM head's launch
 };
 
@@ -239,10 +240,10 @@ static PassPlan pass_plan(const trispec_tree_args* tree, const trispec_attn_args
   }
   // With so few rows the LM head is a pure stream of W that does not need every SM to saturate HBM, and the attention
   // a chain of tiles that does not need bandwidth: the attention runs beside the LM head in as FEW CTAs as it can,
-  // one per (sequence, KV head, M tile), each taking the splits of the attention's own plan in turn (attn.cu: the same
-  // bits), where they end well before the LM head (W streams at 6 TB/s) and are at most a quarter of the chip. One
-  // sequence of 61 nodes, 4096 context tokens, 151936 x 2048 weights: 8 CTAs of 65 tiles beside 140 of the LM head
-  // against 64 CTAs after all 148 of it.
+  // one or two per (sequence, KV head, M tile), each taking the splits of the attention's own plan in turn (attn_split.cuh: the
+  // same bits), where they end well before the LM head (W streams at 6 TB/s) and are at most a quarter of the chip. One
+  // sequence of 61 nodes, 4096 context tokens, 151936 x 2048 weights: 8 pairs of CTAs, 65 tiles each, beside 132 CTAs of the LM
+  // head, 117 us a pass (8 single CTAs beside 140 of it, 126 us).
   const double lm_us = static_cast<double>(lm->V) * lm->d * 2.0 / 6.0e6;
   const int compact_ctas = in_order ? 0 : attn_compact_ctas(attn, 0.8 * lm_us, sms / 4, one_launch ? &pl.pair : nullptr);
   if (lm_seqs == 1) {

@@ -108,8 +108,8 @@ def test_a_workspace_shared_by_the_attention_and_the_lm_head():
 
 @pytest.mark.parametrize("shape,form,ctas", [
     (dict(), "side_by_side", 16),                                            # the attention's own 8 x 2 splits
-    (dict(V=151936), "side_by_side", 8),                                     # a long W: one CTA per KV head
-    (dict(T=61, cap=4096, V=151936), "lm_first", 8),                         # 8 x 8 splits in turn
+    (dict(V=151936), "side_by_side", 16),                                    # a long W: a pair of CTAs per KV head
+    (dict(T=61, cap=4096, V=151936), "lm_first", 16),                        # 8 x 8 splits in turn, in pairs
     (dict(T=61, cap=8192, V=151936), "lm_first", 0),                         # 16 splits through the workspace
     (dict(T=61, Hq=64, cap=8192, d=5120, V=151936), "lm_first", 32),
     (dict(B=3, V=151936), "side_by_side", 24),

@@ -152,8 +152,8 @@ def test_fused_pass_gives_the_attentions_own_bits(kw):
     p = Pass(**kw)
     per_tile = min(64, 128 * kw["Hkv"] // kw["Hq"])
     ctas = len(p.seqs) * kw["Hkv"] * ((kw["T"] + per_tile - 1) // per_tile)
-    items = ctas if kw["cap"] <= 4096 and ctas <= 148 // 4 else 0
-    assert ts.trispec_verify_beside(p.attn_args, p.lm_args, p.scan_args) == items
+    in_turn = ctas * (2 if 4 * ctas <= 148 // 4 else 1)                    # (every plan here has two splits or more)
+    assert ts.trispec_verify_beside(p.attn_args, p.lm_args, p.scan_args) == (in_turn if kw["cap"] <= 4096 and ctas <= 148 // 4 else 0)
     p.spoil()
     p.separate()
     want = p.snapshot()

@@ -55,3 +55,21 @@ def test_the_first_kernel_of_every_call_is_an_ordinary_launch(tmp_path):
     for part in ("rows_beside", "lmhead_cols", "lmhead_gemm", "attn_pieces_kernel", "attn_split", "attn_merge", "tree_mask_block",
                  "esc_compact", "sample_gather", "pack_rows", "prune_tree", "kv_commit_kernel"):
         assert any(part in k for k in kernels), part
+
+
+BESIDE = """
+for name, kw in dict(one_each_would_do=dict(d=8192), two_each=dict(d=4096), one_each=dict(B=3, d=8192),
+                     second_stream=dict(Hq=8, Hkv=1, cap=8192)).items():
+    p = Args(**dict(kw, V=15872))
+    call(name + ":%d" % ts.trispec_verify_beside(p.attn, p.lm, p.scan), lib.trispec_verify(r(p.tree), r(p.attn), r(p.lm), r(p.scan), 77))
+"""
+
+
+def test_the_answer_beside_the_lm_head_is_the_number_of_ctas_launched(tmp_path):
+    """992 units of 16 vocabulary entries are 124 ranges of 8 wherever the LM head is left 124 to 141 SMs."""
+    for name, log in requests(tmp_path, BESIDE).items():
+        launches = [x for what, _, x in log if what == "launch"]
+        rows = next(x for x in launches if "lmhead_rows" in x.kernel)
+        attn = [x.grid for x in launches if "attn_split" in x.kernel]
+        assert ("rows_beside" in rows.kernel) != bool(attn)
+        assert int(name.split(":")[1]) == (attn[0] if attn else rows.grid - 124) > 0, name
