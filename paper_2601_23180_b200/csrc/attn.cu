@@ -319,9 +319,11 @@ int attn_beside(const trispec_attn_args* a, const trispec_tree_args* tree, bool 
   out->p = attn_params(a, pl);
   out->pair = pair;
   // the masks of a decode batch: by the same launch, where the attention reads what the tree step writes
-  out->masks = tree->mask == a->mask && tree->B == a->B && tree->T == a->T && tree->B < 2048;
-  out->tree = *tree;
-  out->p.parent = out->masks ? tree->parent : nullptr;
+  out->masks = tree && tree->mask == a->mask && tree->B == a->B && tree->T == a->T && tree->B < 2048;
+  if (out->masks) {
+    out->tree = *tree;
+    out->p.parent = tree->parent;
+  }
   out->ctas = static_cast<int>(pl.items / pl.n_splits) * (pair ? 2 : 1);
   return TRISPEC_OK;
 }

@@ -98,6 +98,7 @@ struct AttnBeside {
   bool masks;       // the launch computes the tree masks as well
   trispec_tree_args tree;
 };
+// `tree`: null where the masks are another launch's whatever the arguments are
 int attn_beside(const trispec_attn_args* a, const trispec_tree_args* tree, bool pair, AttnBeside* out);
 int lmhead_stats_beside(const trispec_lmhead_args* a, const AttnBeside& beside, void* stream);
 }  // namespace trispec

@@ -161,35 +161,47 @@ class Footprint {
   int n_ = 0;
 };
 
+static void tree_footprint(Footprint* f, const trispec_tree_args* tree) {
+  const size_t n = static_cast<size_t>(tree->B) * tree->T;
+  f->reads(tree->parent, n * 4);
+  f->writes(tree->mask, n * 8);
+  f->writes(tree->depth, n * 4);
+}
+static void attn_footprint(Footprint* f, const trispec_attn_args* attn) {
+  const size_t B = attn->B, T = attn->T, Hq = attn->Hq, Hkv = attn->Hkv, D = attn->D;
+  const bool paged = attn->kv_layout == TRISPEC_KV_PAGED;
+  const size_t kv = (paged ? static_cast<size_t>(attn->num_blocks) * attn->block_size : B * attn->Lmax) * Hkv * D * 2;
+  f->reads(attn->q, B * T * Hq * D * 2);
+  f->reads(attn->k_tree, B * T * Hkv * D * 2);
+  f->reads(attn->v_tree, B * T * Hkv * D * 2);
+  f->reads(attn->k_cache, kv);
+  f->reads(attn->v_cache, kv);
+  if (paged) f->reads(attn->block_table, B * attn->max_blocks_per_seq * 4);
+  f->reads(attn->ctx_len, B * 4);
+  if (attn->seq_index) f->reads(attn->seq_index, static_cast<size_t>(attn->B_active) * 4);
+  f->reads(attn->n_nodes, B * 4);
+  f->writes(attn->o, B * T * Hq * D * 2);
+  f->writes(attn->lse, B * T * Hq * 4);
+  f->writes(attn->workspace, trispec_verify_attn_workspace(attn));
+}
+
+// Whether the tree step and the attention share more than the mask: then the one comes after the other, also where a launch of
+// both would compute the masks on the way.
+static bool tree_shares_memory(const trispec_tree_args* tree, const trispec_attn_args* attn) {
+  Footprint masks, attention;
+  tree_footprint(&masks, tree);
+  attn_footprint(&attention, attn);
+  return masks.clashes(attention);
+}
+
 // Whether the steps that would run beside each other share memory that one of them writes (a workspace used by both, an
 // escalation list written over the index list that the attention reads): in stream order that is no conflict.
 static bool pass_shares_memory(const trispec_tree_args* tree, const trispec_attn_args* attn, const trispec_lmhead_args* lm,
                                const trispec_scan_args* scan) {
   Footprint beside, main;
-  if (tree) {
-    const size_t n = static_cast<size_t>(tree->B) * tree->T;
-    beside.reads(tree->parent, n * 4);
-    beside.writes(tree->mask, n * 8);
-    beside.writes(tree->depth, n * 4);
-  }
-  {
-    const size_t B = attn->B, T = attn->T, Hq = attn->Hq, Hkv = attn->Hkv, D = attn->D;
-    const bool paged = attn->kv_layout == TRISPEC_KV_PAGED;
-    const size_t kv = (paged ? static_cast<size_t>(attn->num_blocks) * attn->block_size : B * attn->Lmax) * Hkv * D * 2;
-    beside.reads(attn->q, B * T * Hq * D * 2);
-    beside.reads(attn->k_tree, B * T * Hkv * D * 2);
-    beside.reads(attn->v_tree, B * T * Hkv * D * 2);
-    beside.reads(attn->k_cache, kv);
-    beside.reads(attn->v_cache, kv);
-    if (paged) beside.reads(attn->block_table, B * attn->max_blocks_per_seq * 4);
-    beside.reads(attn->ctx_len, B * 4);
-    beside.reads(attn->mask, B * T * 8);
-    if (attn->seq_index) beside.reads(attn->seq_index, static_cast<size_t>(attn->B_active) * 4);
-    beside.reads(attn->n_nodes, B * 4);
-    beside.writes(attn->o, B * T * Hq * D * 2);
-    beside.writes(attn->lse, B * T * Hq * 4);
-    beside.writes(attn->workspace, trispec_verify_attn_workspace(attn));
-  }
+  if (tree) tree_footprint(&beside, tree);
+  attn_footprint(&beside, attn);
+  beside.reads(attn->mask, static_cast<size_t>(attn->B) * attn->T * 8);
   {
     const size_t n = static_cast<size_t>(lm->B) * lm->T;
     main.reads(lm->h, n * lm->d * 2);
@@ -316,7 +328,7 @@ extern "C" int trispec_verify(const trispec_tree_args* tree, const trispec_attn_
   // host 29 -> 18 us a call.)
   if (plan.in_turn) {
     trispec::AttnBeside beside;
-    rc = trispec::attn_beside(attn, tree, plan.pair, &beside);
+    rc = trispec::attn_beside(attn, trispec::tree_shares_memory(tree, attn) ? nullptr : tree, plan.pair, &beside);
     if (rc == TRISPEC_OK && !beside.masks) rc = trispec_build_tree_mask(tree, stream);
     if (rc == TRISPEC_OK) rc = trispec::lmhead_stats_beside(lm, beside, stream);
     return rc == TRISPEC_OK ? trispec_accept_scan(scan, stream) : rc;

@@ -73,3 +73,23 @@ def test_the_answer_beside_the_lm_head_is_the_number_of_ctas_launched(tmp_path):
         attn = [x.grid for x in launches if "attn_split" in x.kernel]
         assert ("rows_beside" in rows.kernel) != bool(attn)
         assert int(name.split(":")[1]) == (attn[0] if attn else rows.grid - 124) > 0, name
+
+
+SHARED = """
+for name in ("apart", "depth_in_lse", "parents_in_o", "depth_in_n_nodes", "other_mask", "other_batch"):
+    p = Args(B=2, V=151936)
+    if name == "depth_in_lse": p.tree.depth = p.attn.lse
+    if name == "parents_in_o": p.tree.parent = p.attn.o + 64
+    if name == "depth_in_n_nodes": p.attn.n_nodes = p.tree.depth
+    if name == "other_mask": p.attn.mask = p.new()
+    if name == "other_batch": p.tree.B = 3
+    call(name, lib.trispec_verify(r(p.tree), r(p.attn), r(p.lm), r(p.scan), 77))
+"""
+
+
+def test_masks_come_first_where_the_tree_step_shares_memory_with_the_attention(tmp_path):
+    """In the launch that has masks and attention they run at the same time: only where neither writes what the other touches."""
+    for name, log in requests(tmp_path, SHARED).items():
+        kernels = [x.kernel for what, _, x in log if what == "launch"]
+        assert ["tree_mask" in k for k in kernels].index(False) == (0 if name == "apart" else 1), name
+        assert any("rows_beside" in k for k in kernels), name
