@@ -1,6 +1,6 @@
-"""The fused pass of few rows, whose attention runs beside the LM head in one CTA per (sequence, KV head, M tile)
-that takes the splits of the attention's own plan in turn: the same bits as the attention called by itself, on the
-second stream of each caller's stream, captured or not."""
+"""The fused pass of few rows, whose attention runs beside the LM head: in its launch, in one or two CTAs per (sequence, KV
+head, M tile) that take the splits of the attention's own plan in turn, or by that plan on the second stream of the caller's
+stream; the same bits as the attention called by itself, captured or not. The host-buffer pass always takes the second stream."""
 import math
 
 import pytest
@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 class Pass:
     """One pass with inputs drawn on the GPU. Capacity `cap` tokens per sequence, lengths `lens`."""
 
-    def __init__(self, T, Hq, Hkv, cap, lens, listed=None, n_nodes=None, paged=False, d=2048, V=151936, seed=3, target=False):
+    def __init__(self, T, Hq, Hkv, cap, lens, listed=None, n_nodes=None, paged=False, d=2048, V=151936, seed=3, target=False,
+                 entropy=True):
         import torch
         from paper_2601_23180_b200 import binding as ts
         B = len(lens)
@@ -46,7 +47,7 @@ class Pass:
         self.depth = torch.zeros((B, T), dtype=torch.int32, device="cuda")
         self.o = torch.zeros((B, T, Hq, 128), dtype=torch.bfloat16, device="cuda")
         self.lse = torch.zeros((B, Hq, T), dtype=torch.float32, device="cuda")
-        self.stats, self.out = ts.alloc_stats(B, T), ts.alloc_scan_out(B, T)
+        self.stats, self.out = ts.alloc_stats(B, T, entropy=entropy), ts.alloc_scan_out(B, T)
         self.tree_args = ts.tree_args(self.parent, self.mask, self.depth, dev_status=self.status)
         self.attn_args = ts.attn_args(self.q, self.kt, self.vt, self.mask, self.kc, self.vc, self.ctx, self.scale, self.o,
                                       block_table=self.table, seq_index=self.index, lse=self.lse, dev_status=self.status,
@@ -68,6 +69,7 @@ class Pass:
         self.o.fill_(float("nan"))
         self.lse.fill_(float("nan"))
         self.mask.zero_()
+        self.depth.fill_(-7)
         for v in list(self.stats.values()) + list(self.out.values()):
             v.zero_()
 
@@ -102,6 +104,7 @@ class Pass:
         torch.cuda.synchronize()
         assert int(self.status.item()) == status
         return dict(o=self.o.view(torch.int16).clone(), lse=self.lse.view(torch.int32).clone(), mask=self.mask.clone(),
+                    depth=self.depth.clone(),
                     **{"s_" + k: v.clone() for k, v in self.stats.items()}, **{"d_" + k: v.clone() for k, v in self.out.items()})
 
     def attention64(self, b):
@@ -123,10 +126,23 @@ class Pass:
 
 
 def assert_same_attention(got, want):
-    for k in ("o", "lse", "mask", "s_top1_idx", "d_path", "d_accept_len", "d_escalate"):
+    for k in ("o", "lse", "mask", "depth", "s_top1_idx", "d_path", "d_accept_len", "d_escalate"):
         assert bool((got[k] == want[k]).all()), k
     # sums over other ranges of the vocabulary: fp32 sums of 150000 terms, lse of about 15
     assert (got["s_lse"] - want["s_lse"]).abs().max().item() <= 1e-4
+    if "s_entropy" in want:                        # and E[z] of values of up to 40 on top of it
+        assert (got["s_entropy"] - want["s_entropy"]).abs().max().item() <= 1e-3
+
+
+def launches(call, *args):
+    from paper_2601_23180_b200 import binding as ts
+    n0 = ts.launch_count()
+    call(*args)
+    return ts.launch_count() - n0
+
+
+# launches that a fused pass saves: masks, attention and LM head in one; the attention and the LM head; none
+ONE_LAUNCH, MASKS_APART, SECOND_STREAM = 2, 1, 0
 
 
 @pytest.mark.parametrize("kw", [
@@ -143,6 +159,8 @@ def assert_same_attention(got, want):
     dict(T=61, Hq=16, Hkv=8, cap=2048, lens=[2048, 900], n_nodes=[40, 1]),  # pruned trees
     dict(T=61, Hq=64, Hkv=4, cap=2048, lens=[1024, 900], n_nodes=[40, 7]),  # M tiles without a node
     dict(T=9, Hq=16, Hkv=8, cap=1024, lens=[1000, 800, 513, 64], listed=[3, 0]),
+    dict(T=9, Hq=16, Hkv=8, cap=512, lens=[512], d=4096, V=16000),         # 16 + 125 CTAs in clusters of two
+    dict(T=9, Hq=16, Hkv=8, cap=512, lens=[500], d=4096, V=16000, entropy=False),
     dict(T=61, Hq=16, Hkv=8, cap=8192, lens=[8192]),                       # 16 splits through the workspace: not in turn
     dict(T=61, Hq=16, Hkv=8, cap=16384, lens=[16000]),
 ])
@@ -170,6 +188,7 @@ def test_fused_pass_gives_the_attentions_own_bits(kw):
 
 CHAINS = dict(T=9, Hq=32, Hkv=8, cap=256, lens=[256, 100, 31], d=2048, V=40000)      # 27 rows, 24 CTAs
 ONE = dict(T=9, Hq=16, Hkv=8, cap=512, lens=[512], d=2048, V=32000)
+TWO = dict(T=9, Hq=8, Hkv=1, cap=8192, lens=[8000], d=2048, V=32000)                 # 16 splits through the workspace
 
 
 def _want(p):
@@ -178,10 +197,12 @@ def _want(p):
     return p.snapshot()
 
 
-@pytest.mark.parametrize("call", ["fused", "from_host"])
-def test_a_pass_does_not_wait_for_another_callers_stream(call):
+@pytest.mark.parametrize("call,kw,saved", [("fused", CHAINS, ONE_LAUNCH), ("from_host", CHAINS, SECOND_STREAM),
+                                           ("fused", TWO, SECOND_STREAM), ("from_host", TWO, SECOND_STREAM)])
+def test_a_pass_does_not_wait_for_another_callers_stream(call, kw, saved):
     import torch
-    a, b = Pass(**CHAINS), Pass(**dict(CHAINS, seed=4))
+    a, b = Pass(**kw), Pass(**dict(kw, seed=4))
+    assert launches(a.separate) - launches(getattr(a, call)) == saved
     sa, sb = torch.cuda.Stream(), torch.cuda.Stream()
     want = [_want(a), _want(b)]
     for p, s in ((a, sa), (b, sb)):
@@ -202,23 +223,26 @@ def test_a_pass_does_not_wait_for_another_callers_stream(call):
     assert_same_attention(got[1], want[1])
 
 
-@pytest.mark.parametrize("kw", [CHAINS, ONE, dict(T=61, Hq=16, Hkv=8, cap=4096, lens=[4096])])
-def test_captured_pass_beside_an_eager_one(kw):
+@pytest.mark.parametrize("call,kw,saved", [
+    ("fused", CHAINS, ONE_LAUNCH), ("fused", ONE, ONE_LAUNCH), ("fused", dict(T=61, Hq=16, Hkv=8, cap=4096, lens=[4096]), ONE_LAUNCH),
+    ("fused", TWO, SECOND_STREAM), ("from_host", CHAINS, SECOND_STREAM), ("from_host", TWO, SECOND_STREAM),
+])
+def test_captured_pass_beside_an_eager_one(call, kw, saved):
     """A pass under capture, and between two of its calls an eager pass on another stream: neither disturbs the other."""
     import torch
-    p, q = Pass(**kw), Pass(**dict(CHAINS, seed=4))
+    p, q = Pass(**kw), Pass(**dict(TWO if kw is TWO else CHAINS, seed=4))
     want_p, want_q = _want(p), _want(q)
     sp, sq = torch.cuda.Stream(), torch.cuda.Stream()
     for x, s in ((p, sp), (q, sq)):
-        x.fused(s)
+        assert launches(x.separate, s) - launches(getattr(x, call), s) == saved
     torch.cuda.synchronize()
     graph = torch.cuda.CUDAGraph()
     q.spoil()
     torch.cuda.synchronize()
     with torch.cuda.graph(graph, stream=sp):
-        p.fused(sp)
-        q.fused(sq)
-        p.fused(sp)
+        getattr(p, call)(sp)
+        getattr(q, call)(sq)
+        getattr(p, call)(sp)
     assert_same_attention(q.snapshot(), want_q)
     for _ in range(3):
         p.spoil()
@@ -227,12 +251,12 @@ def test_captured_pass_beside_an_eager_one(kw):
         assert_same_attention(p.snapshot(), want_p)
     p.spoil()
     torch.cuda.synchronize()
-    p.fused(sp)                                    # the stream's second stream is usable again after the capture
+    getattr(p, call)(sp)                                    # the stream's second stream is usable again after the capture
     assert_same_attention(p.snapshot(), want_p)
     first = torch.cuda.CUDAGraph()
     fresh = torch.cuda.Stream()                    # a stream that the library meets under capture
     with torch.cuda.graph(first, stream=fresh):
-        p.fused(fresh)
+        getattr(p, call)(fresh)
     p.spoil()
     torch.cuda.synchronize()
     first.replay()
@@ -246,6 +270,7 @@ def test_more_busy_streams_than_second_streams():
     tiny = dict(T=9, Hq=8, Hkv=8, cap=128, lens=[100], d=64, V=3000)
     passes = [Pass(**dict(tiny, seed=i)) for i in range(20)]
     want = [_want(p) for p in passes]
+    assert launches(passes[0].separate) - launches(passes[0].fused) == SECOND_STREAM
     for rounds in range(2):
         for p in passes:
             p.spoil()
@@ -266,10 +291,10 @@ def test_more_busy_streams_than_second_streams():
 def test_threads_on_streams_of_their_own_and_on_a_shared_one():
     import threading
     import torch
-    passes = [Pass(**dict(kw, seed=i)) for i, kw in enumerate((CHAINS, ONE, CHAINS, ONE))]
+    passes = [Pass(**dict(kw, seed=i)) for i, kw in enumerate((CHAINS, ONE, CHAINS, ONE, TWO, TWO))]
     want = [_want(p) for p in passes]
     shared = torch.cuda.Stream()
-    streams = [torch.cuda.Stream(), torch.cuda.Stream(), shared, shared]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream(), shared, shared, torch.cuda.Stream(), shared]
     for p in passes:
         p.spoil()
     torch.cuda.synchronize()
@@ -283,7 +308,7 @@ def test_threads_on_streams_of_their_own_and_on_a_shared_one():
             errors.append(e)
 
     threads = [threading.Thread(target=work, args=(p, s, c))
-               for p, s, c in zip(passes, streams, ("fused", "from_host", "from_host", "fused"))]
+               for p, s, c in zip(passes, streams, ("fused", "from_host", "from_host", "fused", "fused", "fused"))]
     for t in threads:
         t.start()
     for t in threads:
@@ -390,4 +415,46 @@ def test_stochastic_pass_beside(kw):
     for _ in range(3):
         p.spoil()
         p.fused()
+        assert_same_attention(p.snapshot(), want)
+
+
+@pytest.mark.parametrize("kw", [CHAINS, ONE, dict(T=61, Hq=16, Hkv=8, cap=4096, lens=[3000]),
+                                dict(T=61, Hq=64, Hkv=8, cap=2048, lens=[1999], target=True)])
+def test_malformed_tree_in_one_launch(kw):
+    """A parent that comes later, in the last sequence: its node and all below it see nothing of the tree, and the status says so."""
+    import torch
+    p = Pass(**kw)
+    p.parent[-1, 2] = 5
+    want = None
+    for call in (p.separate, p.fused, p.fused):
+        p.spoil()
+        p.status.zero_()
+        n = launches(call)
+        got = p.snapshot(status=11)
+        if want is not None:
+            assert want_n - n == ONE_LAUNCH
+            assert_same_attention(got, want)
+        want, want_n = want or got, n if want is None else want_n
+    assert int(p.mask[-1, 2].item()) == 0 and int(p.depth[-1, 2].item()) == -1 and (p.mask[:, 0] == 1).all()
+
+
+@pytest.mark.parametrize("kw", [
+    dict(ONE, other_mask=True), dict(CHAINS, other_mask=True), dict(T=61, Hq=16, Hkv=8, cap=4096, lens=[3000], other_mask=True),
+    dict(T=9, Hq=16, Hkv=8, cap=64, lens=[64] * 2048, listed=[5, 1999], V=32000),     # more trees than the launch takes along
+])
+def test_masks_of_a_launch_of_their_own(kw):
+    import torch
+    from paper_2601_23180_b200 import binding as ts
+    kw = dict(kw)
+    other = kw.pop("other_mask", False)
+    p = Pass(**kw)
+    if other:                                      # the attention follows chains, whatever the trees are
+        chain = torch.tensor([(2 << i) - 1 for i in range(p.T)], dtype=torch.int64, device="cuda").repeat(p.B, 1).contiguous()
+        p.attn_args.mask = chain.data_ptr()
+    p.spoil()
+    n = launches(p.separate)
+    want = p.snapshot()
+    for _ in range(3):
+        p.spoil()
+        assert n - launches(p.fused) == MASKS_APART
         assert_same_attention(p.snapshot(), want)
