@@ -914,6 +914,7 @@ lmhead_rows_beside_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gr
 // that a range still is one row block of the partials. Up to 8 stages of 16 KB of W and up to 12 KB of H per CTA.
 // ---------------------------------------------------------------------------------------
 constexpr int LC_EPI_WARPS = 8, LC_THREADS = 32 * (LC_EPI_WARPS + 2), LC_MAX_STAGES = 8, LC_MAX_COLS = 256;
+constexpr int LC_MIN_V = 96 << 10;                                // vocabulary from which it is taken
 constexpr int LC_A_BYTES = 128 * LM_BK * 2;                        // 16 KB: this CTA's half of the W tile
 constexpr int LC_RING_BYTES = LW_SMEM_BYTES - 1024 - LC_EPI_WARPS * LW_XPOSE_BYTES - 256;
 
@@ -1153,10 +1154,14 @@ static void lm_plan_rows(const trispec_lmhead_args* a, int n_seq, bool slots, si
   int tail = pairs - pl->n_mt * r;
   if (pl->n_mt < 2 || tail < 1 || pl->n_mt * r > pairs) tail = 0;
   while (tail > 0 && static_cast<size_t>(r + tail) * pl->part_rows * sizeof(LmPartial) > max_ws) --tail;
-  // Rows as columns where the M tiles would be a quarter padding or more, over rows long enough to hide the heavier statistics
-  // (LM head alone, pair kernel against this one: 183 rows of 5120 345 and 327 us, 312 of 4096 394 and 368, 576 of 4096 575 and
-  // 563, 150 of 2048 137 and 133; 784 of 4096, a fifth padding, 752 and 749; 488 of 2048 262 and 278; 150 of 1024 31 and 42).
-  pl->cols = !slots && pl->tile_rows <= 192 && a->d >= 2048 && lm_long_stream(a);
+  // Rows as columns where the M tiles would be a quarter padding or more, over rows long enough to hide the heavier statistics and
+  // a vocabulary of five tiles and more per pair and M tile, behind which the last tile's do not count. Such a call costs less energy, not
+  // fewer clocks. LM head alone, pair kernel and this one, in loops at the power limit: 183 rows of 5120 x 151936 weights 386 and
+  // 362 us, 312 of 4096 x 128256 426 and 394, 576 of 4096 x 128256 619 and 580, 150 of 2048 x 151936 144 and 135; one call now and
+  // then: 314 and 303, 352 and 333, 501 and 513, 124 and 127. Shorter vocabularies, loops and single calls: 183 of 5120 x 32000 91 and 97,
+  // 77 and 87; 576 of 4096 x 33000 173 and 177, 144 and 154; 150 of 2048 x 65600 73 and 75, 63 and 70; 150 of 3072 x 100000 153
+  // and 148, 124 and 127. Without padding or over short rows it loses: 488 of 2048 262 and 278, 150 of 1024 31 and 42.
+  pl->cols = !slots && pl->tile_rows <= 192 && a->d >= 2048 && a->V >= LC_MIN_V;
   if (pl->cols) tail = 0;
   if (tail > 0) {
     int best_slice = 0, best_cost = (V32 / r + 7) / 8 + 1;    // without a tail: the longest main range

@@ -55,17 +55,17 @@ def test_tail_slices_over_several_m_tiles(B, T, V, entropy):
 
 
 @pytest.mark.parametrize("B,T,V", [
-    (3, 43, 70001),      # 129 rows: 144 columns, an odd vocabulary
-    (3, 61, 70000),      # 183: 192 columns, most of a tile of each CTA's last range missing
-    (32, 6, 68003),      # 192 exactly
-    (1, 64, 70001),      # (64: the small-row kernel, for comparison)
-    (43, 6, 66000),      # 258: two tiles of 144 columns, the second with 114 rows
-    (12, 26, 70007),     # 312
-    (8, 48, 70007),      # 384
-    (9, 57, 65600),      # 513: three tiles of 176
-    (64, 9, 65553),      # 576
+    (3, 43, 100001),      # 129 rows: 144 columns, an odd vocabulary
+    (3, 61, 100000),      # 183: 192 columns, most of a tile of each CTA's last range missing
+    (32, 6, 98307),      # 192 exactly
+    (1, 64, 100001),      # (64: the small-row kernel, for comparison)
+    (43, 6, 98304),      # 258: two tiles of 144 columns, the second with 114 rows
+    (12, 26, 100007),     # 312
+    (8, 48, 100007),      # 384
+    (9, 57, 98400),      # 513: three tiles of 176
+    (64, 9, 98333),      # 576
 ])
 @pytest.mark.parametrize("entropy", [False, True])
 def test_rows_as_columns_of_a_pair(B, T, V, entropy):
-    """From 2048 x 65536 weights on, rows that would leave a quarter of an M tile empty are the N side."""
+    """From 98304 entries on, rows that would leave a quarter of an M tile empty are the N side."""
     _check(B, T, 2048, V, entropy)

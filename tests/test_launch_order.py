@@ -93,3 +93,17 @@ def test_masks_come_first_where_the_tree_step_shares_memory_with_the_attention(t
         kernels = [x.kernel for what, _, x in log if what == "launch"]
         assert ["tree_mask" in k for k in kernels].index(False) == (0 if name == "apart" else 1), name
         assert any("rows_beside" in k for k in kernels), name
+
+
+COLUMNS = """
+for rows, d, V, cols in ((150, 2048, 98304, 1), (150, 2048, 98303, 0), (150, 1984, 151936, 0), (312, 4096, 128256, 1), (386, 4096, 128256, 0),
+                         (513, 5120, 98304, 1), (576, 2048, 65600, 0), (784, 4096, 151936, 0)):
+    p = Args(B=rows, T=1, d=d, V=V)
+    call("%d_%d_%d:%d" % (rows, d, V, cols), lib.trispec_lmhead_stats(r(p.lm), 77))
+"""
+
+
+def test_which_lm_heads_take_rows_as_columns(tmp_path):
+    for name, log in requests(tmp_path, COLUMNS).items():
+        kernels = [x.kernel for what, _, x in log if what == "launch"]
+        assert any("lmhead_cols" in k for k in kernels) == (name[-1] == "1"), name
