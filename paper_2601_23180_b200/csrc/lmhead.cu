@@ -1396,9 +1396,11 @@ static int trispec::lmhead_stats_planned(const trispec_lmhead_args* a, const LmP
     }
     count_launch();
     f.stride = pl.part_rows;
-    // one row per block: as many SMs as rows fetch the merge's operands (LM head alone, 9 rows: 31.7 -> 30.1 us, 61: 110.7 -> 107.3)
-    TRISPEC_CUDA_OK(launch_dependent(beside ? lmhead_finalize_kernel<true> : lmhead_finalize_kernel<false>, static_cast<unsigned>(n_rows),
-                                     32, 0, st, 1, f, n_seq));
+    // One row per block: as many SMs as rows fetch the merge's operands (LM head alone, 151936 x 2048 weights, 9 rows 102.1 -> 101.0
+    // us, 61 rows 105.2 -> 104.2; 61 rows, 32000 x 1024, 27.0 -> 26.5). More rows than 64 are eight per block (122 rows 138.8 -> 136.8).
+    const unsigned per_block = sp.n_rows > 64 ? LM_FIN_THREADS / 32 : 1;
+    TRISPEC_CUDA_OK(launch_dependent(beside ? lmhead_finalize_kernel<true> : lmhead_finalize_kernel<false>,
+                                     (static_cast<unsigned>(n_rows) + per_block - 1) / per_block, 32 * per_block, 0, st, 1, f, n_seq));
     count_launch();
     return TRISPEC_OK;
   }
