@@ -172,7 +172,7 @@ accept_scan_small_kernel(trispec_scan_args a, int rehearse) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int esc = 0;
   // Behind another kernel of the same call the scan runs twice, the first time before the wait and without writing: that
-  // brings its code into the instruction cache (the loads bypass L1).
+  // brings its code into the instruction cache (the loads bypass L1). One chain 36.0 -> 35.1 us a pass, five short sequences 59.0 -> 57.4.
 #pragma unroll 1
   for (int run = rehearse ? 0 : 1; run < 2; ++run) {
     if (run == 1) pdl_wait();

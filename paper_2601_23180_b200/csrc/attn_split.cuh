@@ -88,7 +88,6 @@ __device__ __forceinline__ void attn_merge_row(const AttnParams& p, const uint4 
     p.lse[(static_cast<size_t>(b) * p.Hq + hq) * p.T + node] = (M + log2f(Lsum)) * kLn2;
 }
 
-// CTA `block` of the launch, its first AT_THREADS threads (a kernel that hosts it may have more)
 // The seventh warp of a CTA in turn that computes the mask of its tree: into shared memory, for the softmax threads.
 template <bool kPair>
 __device__ __forceinline__ void attn_mask_warp(const AttnParams& p, int block) {
@@ -107,6 +106,7 @@ __device__ __forceinline__ void attn_mask_warp(const AttnParams& p, int block) {
   asm volatile("bar.arrive 4, %0;" ::"r"(32 * ((n_rows + 31) >> 5) + 32) : "memory");
 }
 
+// CTA `block` of the launch, its first AT_THREADS threads (a kernel that hosts it may have more)
 template <int kMerge, int NP>
 __device__ __forceinline__ void attn_split_cta(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const CUtensorMap& tm_kt,
                                                const CUtensorMap& tm_vt, const AttnParams& p, int block) {
