@@ -13,12 +13,17 @@ namespace trispec {
 
 constexpr int kScanThreads = 256;  // 8 sequences per block
 
+// kTwice: a run of the scan came before what it reads was complete, so that nothing may be left of it in L1. A large batch runs
+// once (524288 sequences of 61 nodes: 180 us with the loads that bypass L1, 175 without).
+template <bool kTwice, class V>
+__device__ __forceinline__ V scan_load(const V* p) { return kTwice ? __ldcg(p) : __ldg(p); }
+
 // the proxy feature the routing criterion looks at (margin of Eq. 8 by default)
-template <int kCrit>
+template <int kCrit, bool kTwice>
 __device__ __forceinline__ float scan_feature(const trispec_scan_args& a, long long idx) {
-  if (kCrit == TRISPEC_CRIT_TOP1) return __ldcg(a.in.p_top1 + idx);
-  if (kCrit == TRISPEC_CRIT_ENTROPY) return __ldcg(a.in.entropy + idx);
-  return __ldcg(a.in.p_top1 + idx) - __ldcg(a.in.p_top2 + idx);
+  if (kCrit == TRISPEC_CRIT_TOP1) return scan_load<kTwice>(a.in.p_top1 + idx);
+  if (kCrit == TRISPEC_CRIT_ENTROPY) return scan_load<kTwice>(a.in.entropy + idx);
+  return scan_load<kTwice>(a.in.p_top1 + idx) - scan_load<kTwice>(a.in.p_top2 + idx);
 }
 
 // The walk of one sequence by one warp; writes the sequence's outputs and returns its escalation flag.
@@ -26,14 +31,14 @@ __device__ __forceinline__ float scan_feature(const trispec_scan_args& a, long l
 // latency-bound, and the plain case (margin rule, greedy acceptance) pays for nothing else.
 // kAccept: TRISPEC_ACCEPT_GREEDY (arg-max match), _STOCHASTIC (Eq. 6 at temperature 1) or
 // _TOKEN_SPECIFIC (the token-specific deferral rule of the SpecCascade baselines).
-template <int kCrit, int kAccept>
+template <int kCrit, int kAccept, bool kTwice>
 __device__ __forceinline__ int scan_sequence(const trispec_scan_args& a, const long long b, const int lane, const bool write = true) {
   const int T = a.T;
   const long long base = b * T;
   int32_t* path = a.path + base;
   const bool has0 = lane < T, has1 = lane + 32 < T;
 
-  if (a.active && __ldcg(a.active + b) == 0) {
+  if (a.active && (kTwice ? __ldcg(a.active + b) : a.active[b]) == 0) {
     if (!write) return 0;
     if (has0) path[lane] = -1;
     if (has1) path[lane + 32] = -1;
@@ -58,23 +63,23 @@ __device__ __forceinline__ int scan_sequence(const trispec_scan_args& a, const l
   // (1 - alpha) times its parent's) and the probability of the nodes' own drafted tokens
   float pt0 = 0.f, pt1 = 0.f, pd0 = -1.f, pd1 = -1.f;
   if (token_rule) {
-    if (has0) { pt0 = __ldcg(a.in.p_top1 + base + lane); if (lane > 0) pd0 = __ldcg(a.in.p_draft + base + lane); }
-    if (has1) { pt1 = __ldcg(a.in.p_top1 + base + lane + 32); pd1 = __ldcg(a.in.p_draft + base + lane + 32); }
+    if (has0) { pt0 = scan_load<kTwice>(a.in.p_top1 + base + lane); if (lane > 0) pd0 = scan_load<kTwice>(a.in.p_draft + base + lane); }
+    if (has1) { pt1 = scan_load<kTwice>(a.in.p_top1 + base + lane + 32); pd1 = scan_load<kTwice>(a.in.p_draft + base + lane + 32); }
   }
   if (has0) {
-    par0 = __ldcg(a.parent + base + lane); tok0 = __ldcg(a.tok + base + lane);
-    top0 = __ldcg(a.in.top1_idx + base + lane);
+    par0 = scan_load<kTwice>(a.parent + base + lane); tok0 = scan_load<kTwice>(a.tok + base + lane);
+    top0 = scan_load<kTwice>(a.in.top1_idx + base + lane);
     if (proxy) {
-      const float f = scan_feature<kCrit>(a, base + lane);
+      const float f = scan_feature<kCrit, kTwice>(a, base + lane);
       tr0 = (kCrit == TRISPEC_CRIT_ENTROPY) ? (f <= a.lambda) : (f >= a.lambda);
       nr0 = fabsf(f - a.lambda) < 1e-3f;
     }
   }
   if (has1) {
-    par1 = __ldcg(a.parent + base + lane + 32); tok1 = __ldcg(a.tok + base + lane + 32);
-    top1v = __ldcg(a.in.top1_idx + base + lane + 32);
+    par1 = scan_load<kTwice>(a.parent + base + lane + 32); tok1 = scan_load<kTwice>(a.tok + base + lane + 32);
+    top1v = scan_load<kTwice>(a.in.top1_idx + base + lane + 32);
     if (proxy) {
-      const float f = scan_feature<kCrit>(a, base + lane + 32);
+      const float f = scan_feature<kCrit, kTwice>(a, base + lane + 32);
       tr1 = (kCrit == TRISPEC_CRIT_ENTROPY) ? (f <= a.lambda) : (f >= a.lambda);
       nr1 = fabsf(f - a.lambda) < 1e-3f;
     }
@@ -88,19 +93,19 @@ __device__ __forceinline__ int scan_sequence(const trispec_scan_args& a, const l
   if (stochastic) {
     bool ps0 = false, ps1 = false;
     if (has0 && lane > 0) {
-      const float q = __ldcg(a.q_draft + base + lane), pd = __ldcg(a.in.p_draft + base + lane);
-      ps0 = __ldcg(a.u_accept + base + lane) < ((q > 0.f) ? fminf(1.f, pd / q) : 1.f);
+      const float q = scan_load<kTwice>(a.q_draft + base + lane), pd = scan_load<kTwice>(a.in.p_draft + base + lane);
+      ps0 = scan_load<kTwice>(a.u_accept + base + lane) < ((q > 0.f) ? fminf(1.f, pd / q) : 1.f);
     }
     if (has1) {
-      const float q = __ldcg(a.q_draft + base + lane + 32), pd = __ldcg(a.in.p_draft + base + lane + 32);
-      ps1 = __ldcg(a.u_accept + base + lane + 32) < ((q > 0.f) ? fminf(1.f, pd / q) : 1.f);
+      const float q = scan_load<kTwice>(a.q_draft + base + lane + 32), pd = scan_load<kTwice>(a.in.p_draft + base + lane + 32);
+      ps1 = scan_load<kTwice>(a.u_accept + base + lane + 32) < ((q > 0.f) ? fminf(1.f, pd / q) : 1.f);
     }
     passes = __ballot_sync(0xffffffffu, ps0) | (static_cast<unsigned long long>(__ballot_sync(0xffffffffu, ps1)) << 32);
   }
   // the compaction kernel only writes the leading entries of esc_index
   if (write && a.esc_index && lane == 0) a.esc_index[b] = -1;
 
-  int cur = a.start_node ? __ldcg(a.start_node + b) : 0;
+  int cur = a.start_node ? (kTwice ? __ldcg(a.start_node + b) : a.start_node[b]) : 0;
   if (cur < 0 || cur >= T) cur = 0;
   int n = 0, esc = 0, bonus = -1, near = 0;
   int path0 = -1, path1 = -1;   // entries `lane` and `lane + 32` of the accepted path
@@ -157,7 +162,7 @@ accept_scan_kernel(trispec_scan_args a) {
   const int lane = threadIdx.x & 31;
   const long long b = static_cast<long long>(blockIdx.x) * (kScanThreads / 32) + (threadIdx.x >> 5);
   if (b >= a.B) return;
-  scan_sequence<kCrit, kAccept>(a, b, lane);
+  scan_sequence<kCrit, kAccept, false>(a, b, lane);
 }
 
 // Up to 32 sequences (a decode batch): one block, one warp per sequence, and the ordered list of
@@ -176,7 +181,7 @@ accept_scan_small_kernel(trispec_scan_args a, int rehearse) {
 #pragma unroll 1
   for (int run = rehearse ? 0 : 1; run < 2; ++run) {
     if (run == 1) pdl_wait();
-    if (warp < a.B) esc = scan_sequence<kCrit, kAccept>(a, warp, lane, run == 1);
+    if (warp < a.B) esc = scan_sequence<kCrit, kAccept, true>(a, warp, lane, run == 1);
   }
   if (lane == 0) s_esc[warp] = esc;
   __syncthreads();
