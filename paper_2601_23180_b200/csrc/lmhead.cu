@@ -775,7 +775,7 @@ __device__ __forceinline__ void lm_rows_cta(const CUtensorMap& tmap_w, const CUt
       }
       // The kernels after this one may start when its last copies are on their way. Earlier their blocks keep an attention on
       // a second stream off the SMs left to it (a pass of one sequence behind other work: 197 us, now 133), and their
-      // first loads, behind the stream of W, take longer than it saves (LM head alone, 9 rows: 36.8 -> 30.1 us).
+      // first loads, behind the stream of W, take longer than it saves (LM head alone, 9 rows: 34.2 -> 32.8 us).
       pdl_launch_dependents();
     }
   } else if (warp == LW_EPI_WARPS + 1) {
